@@ -252,11 +252,13 @@ def kernel_bytes_per_step(name, sizes, quants, sum_q, tuning, with_matrices):
     us = sum_q["unique_links"] if sum_q else 0
     rs = sum_q["unique_sources"] if sum_q else 0
     rounds = max(1, (len(sizes) - 1).bit_length()) if len(sizes) > 1 else 0
-    # the windows' order from the packet sort: the packets carry 16-bit window ids
-    regroup = bool(tuning) and tuning.get("agg_path") == 3 and sum_q is not None and 2 <= len(sizes) <= 1 << 16
+    # packets sorted: the windows', and (sum_path 2, agg_path 3) the batch's as one segment
+    pk = bool(tuning) and sum_q is not None and (tuning.get("sum_path") == 2 or tuning.get("agg_path") == 3)
+    p_ss = p_os + (p_all if pk else 0)
     rules = {
-        "pack_hist": 16 * p_os,                        # read pairs, write keys
-        "onesweep": 8 * 16 * p_os,                     # 8 passes: read + write a key
+        "ss_count": 10 * p_ss,                         # read pairs, write a 16-bit bucket id
+        "ss_scatter": 18 * p_ss,                       # read pairs and ids, write keys
+        "ss_local": 16 * p_ss,                         # read keys, write them sorted
         "cluster_sort": 16 * p_cl,                     # read pairs, write sorted keys
         "hash_insert": 8 * p_all,                      # read pairs
         "hash_compact": 32 * u,                        # slot in, (key, count) out
@@ -270,10 +272,6 @@ def kernel_bytes_per_step(name, sizes, quants, sum_q, tuning, with_matrices):
         "merge": rounds * 32 * u,                      # each round: read both runs, write the merge
         "onesweep_sum": 8 * 32 * u,                    # 8 passes over (key, count)
         "scan_u64": 16 * us,
-        "pack_hist_sum": 16 * p_all,                   # the time sum's packets: read pairs, write keys
-        "onesweep_pk": 8 * (20 if regroup else 16) * p_all,  # 8 passes over the batch's packets (+ window ids)
-        "wid_fill": 2 * p_all,                         # a window id per packet
-        "regroup": 20 * p_all + 18 * p_all,            # (id, key) in and out; then (id, key) in, key out
         "colhash_part": 24 * u,                        # regroup (read twice, write) + count (read) per link
         "hq_split": 24 * p_all,                        # regroup packets: read twice, write once
         "hq_links": 8 * p_all + 12 * u,                # read packets, append distinct links
@@ -640,11 +638,11 @@ def main(argv=None):
             ls_ms.append(a.elapsed_time(b))
         del keys
         torch.cuda.empty_cache()
-        own = prof.get("onesweep_pk") or prof.get("onesweep")
+        own = [prof[k][1] for k in ("ss_sample", "ss_count", "ss_scatter", "ss_plan", "ss_local") if k in prof]
         lib_sort = {"what": "torch.sort(stable=True) of the step's packets as int64 keys (CUB radix sort, "
                             "keys + int64 indices)", "ms": round(min(ls_ms), 3),
-                    "own_sort_ms": round(own[1] / args.steps, 3) if own else None,
-                    "own_sort": "the path's eight digit passes per step (onesweep_pk or onesweep)"}
+                    "own_sort_ms": round(sum(own) / args.steps, 3) if own else None,
+                    "own_sort": "every sample sort of the step (ss_*): the windows' and, on most paths, the batch's"}
 
     # ---- end to end through the C ABI with host buffers
     e2e = None

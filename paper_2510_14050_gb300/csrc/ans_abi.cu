@@ -759,18 +759,112 @@ T* at(char* m, size_t off) {
   return reinterpret_cast<T*>(m + off);
 }
 
-// Sort keys (and values) of the segments of `p` in place: 8 stable digit
+// Sort the (key, value) pairs of the segments of `p` in place: 8 stable digit
 // passes ping-ponging between a and b; the result ends in a.
 int sort_segments(ans_ctx* c, const SegPlan& p, uint64_t* ka, uint64_t* kb, uint64_t* va, uint64_t* vb,
                   const uint32_t* seg_hist, uint64_t* st0, uint64_t* st1, uint32_t* tickets, cudaStream_t st,
-                  const char* name = nullptr) {
+                  const char* name = "onesweep_sum") {
   for (int pass = 0; pass < kPasses; ++pass) {
     const bool even = (pass % 2) == 0;
-    KTime kt(c, name ? name : va ? "onesweep_sum" : "onesweep", st);
-    ANS_CUDA(launch_onesweep(p, pass, even ? ka : kb, even ? kb : ka, va ? (even ? va : vb) : nullptr,
-                             va ? (even ? vb : va) : nullptr, seg_hist, even ? st0 : st1,
-                             even ? st1 : st0, tickets + pass, c->d_err, va ? c->cfg_kv : c->cfg_keys, st));
+    KTime kt(c, name, st);
+    ANS_CUDA(launch_onesweep(p, pass, even ? ka : kb, even ? kb : ka, even ? va : vb, even ? vb : va, seg_hist,
+                             even ? st0 : st1, even ? st1 : st0, tickets + pass, c->d_err, c->cfg_kv, st));
   }
+  return ANS_OK;
+}
+
+// Scratch of a segmented sample sort (ans_ssort.cu) over plans of up to
+// `ntiles` tiles and `nseg` segments; with `two` also for a first split of
+// the segments too long for one.
+struct SsScratch {
+  size_t tree[2] = {0, 0}, cnt[2] = {0, 0}, cur[2] = {0, 0}, bstart[2] = {0, 0}, eq[2] = {0, 0};
+  size_t start2 = 0, len2 = 0, parent2 = 0, first_tile2 = 0, tile_seg2 = 0, count2 = 0;
+  uint32_t nseg2 = 0, ntiles2 = 0;
+  void reserve(Layout& L, uint32_t nseg, uint32_t ntiles, bool two) {
+    const uint64_t l1 = two ? ss_level1_buckets((uint64_t)ntiles * kTile, nseg) : 0;
+    nseg2 = (uint32_t)(nseg + l1);
+    ntiles2 = (uint32_t)(ntiles + l1);
+    for (int lv = 0; lv < (two ? 2 : 1); ++lv) {
+      const size_t nb = (size_t)kSsPerTile * (lv ? ntiles : ntiles2);
+      tree[lv] = L.add(nb * 2 * 8);
+      cnt[lv] = L.add(nb * 4);
+      cur[lv] = L.add(nb * 4);
+      bstart[lv] = L.add(nb * 4);
+      eq[lv] = L.add(nb);
+    }
+    if (two) {
+      start2 = L.add((size_t)nseg2 * 8);
+      len2 = L.add((size_t)nseg2 * 8);
+      parent2 = L.add((size_t)nseg2 * 4);
+      first_tile2 = L.add(((size_t)nseg2 + 1) * 4);
+      tile_seg2 = L.add((size_t)ntiles2 * 4);
+      count2 = L.add(8);
+    }
+  }
+};
+
+// The raw packets of the segments of `p`, packed and sorted into ka (kb and
+// ids are scratch).  total and max_len bound the keys in all and the longest
+// segment; `two`: some segments may be too long for one split (the scratch
+// was reserved for it).
+int sample_sort(ans_ctx* c, char* m, const SsScratch& ss, const SegPlan& p, const uint32_t* d_src,
+                const uint32_t* d_dst, uint64_t total, uint64_t max_len, bool two, uint64_t* ka, uint64_t* kb,
+                uint16_t* ids, cudaStream_t st) {
+  SsArgs a;
+  a.one_level = ss_one_level(total);
+  a.plan = p;
+  a.src = d_src;
+  a.dst = d_dst;
+  a.start = p.base;
+  a.len = p.len;
+  a.first_tile = p.first_tile;
+  a.tile_seg = p.tile_seg;
+  a.nseg = p.nseg;
+  a.ntiles = p.ntiles;
+  a.keys_split = kb;
+  a.keys_out = ka;
+  a.ids = ids;
+  auto level = [&](int lv) {
+    a.tree = at<uint64_t>(m, ss.tree[lv]);
+    a.cnt = at<uint32_t>(m, ss.cnt[lv]);
+    a.cur = at<uint32_t>(m, ss.cur[lv]);
+    a.bstart = at<uint32_t>(m, ss.bstart[lv]);
+    a.eq = at<uint8_t>(m, ss.eq[lv]);
+  };
+  if (two) {  // long segments into buckets of keys_a first
+    level(1);
+    a.level1 = true;
+    a.keys_split = ka;
+    SsSeg2 o;
+    o.start = at<uint64_t>(m, ss.start2);
+    o.len = at<uint64_t>(m, ss.len2);
+    o.parent = at<uint32_t>(m, ss.parent2);
+    o.first_tile = at<uint32_t>(m, ss.first_tile2);
+    o.tile_seg = at<uint32_t>(m, ss.tile_seg2);
+    o.count = at<uint32_t>(m, ss.count2);
+    ANS_CUDA(timed(c, "ss_sample", st, [&] { return launch_ss_sample(a, max_len, st); }));
+    ANS_CUDA(timed(c, "ss_count", st, [&] { return launch_ss_count(a, st); }));
+    ANS_CUDA(timed(c, "ss_scatter", st, [&] { return launch_ss_scatter(a, st); }));
+    ANS_CUDA(timed(c, "ss_plan", st, [&] { return launch_ss_plan2(a, o, st); }));
+    a.level1 = false;
+    a.keys_in = ka;
+    a.keys_split = kb;
+    a.start = o.start;
+    a.len = o.len;
+    a.first_tile = o.first_tile;
+    a.tile_seg = o.tile_seg;
+    a.parent = o.parent;
+    a.nseg_d = o.count;
+    a.ntiles_d = o.count + 1;
+    a.nseg = ss.nseg2;
+    a.ntiles = ss.ntiles2;
+    max_len = a.one_level;
+  }
+  level(0);
+  ANS_CUDA(timed(c, "ss_sample", st, [&] { return launch_ss_sample(a, max_len, st); }));
+  ANS_CUDA(timed(c, "ss_count", st, [&] { return launch_ss_count(a, st); }));
+  ANS_CUDA(timed(c, "ss_scatter", st, [&] { return launch_ss_scatter(a, st); }));
+  ANS_CUDA(timed(c, "ss_local", st, [&] { return launch_ss_local(a, st); }));
   return ANS_OK;
 }
 
@@ -1028,67 +1122,28 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
   return column_pass(c, s, a.ulen, blk->col_ids, blk->vals, ps, m, col_tickets, blk->q, st, narrow, a.col_hkeys);
 }
 
-// The windows of a batch whose sorted keys come from its packet sort
-// (agg_path 3): their plan, the packets' window ids (two buffers of one id
-// per packet: the second is the column keys' buffer, free until the sum's
-// column pass) and each window's offset from the batch sorted by window to
-// its padded base.
-struct Regroup {
-  SegPlan win;
-  uint16_t* wid = nullptr;
-  uint16_t* wid_b = nullptr;
-  uint64_t* shift = nullptr;
-};
-
 // Time sum of a batch from its packets (sum_path 2): every packet of the
-// batch, as the one segment of `pk`, is packed and sorted again, and the
-// sorted keys are reduced like a window (counts = run lengths) into `blk`,
-// with the sum's row and column statistics.  Runs after the window
-// statistics, whose key buffers, status words and tickets it reuses -- or,
-// with `rg`, before them: the packets then carry their window ids through
-// the sort, which leaves the sorted keys in keys_a and their ids in
-// rg->wid for regroup_windows.  Only queues work on `st`.
+// batch, as the one segment of `pk`, is sorted again, and the sorted keys are
+// reduced like a window (counts = run lengths) into `blk`, with the sum's row
+// and column statistics.  Runs after the window statistics, whose key
+// buffers, status words and tickets it reuses.  Only queues work on `st`.
 int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, const uint32_t* d_src,
-                const uint32_t* d_dst, Block* blk, cudaStream_t st, bool narrow, const Regroup* rg = nullptr) {
+                const uint32_t* d_dst, Block* blk, cudaStream_t st, bool narrow, const SsScratch& ss, uint64_t total,
+                bool two) {
   uint64_t* ka = at<uint64_t>(m, ps.keys_a);
   uint64_t* kb = at<uint64_t>(m, ps.keys_b);
-  uint32_t* seg_hist = at<uint32_t>(m, ps.seg_hist);
   uint32_t* tickets = at<uint32_t>(m, ps.tickets);
   auto cu = [&](cudaError_t e, const char* what) -> int {
     if (e == cudaSuccess) return ANS_OK;
     return fail(ANS_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
   };
   int rc;
-  // with window ids, their two digit histograms follow the packets' eight
-  if ((rc = cu(launch_zero(seg_hist, (rg ? kPasses + 2 : kPasses) * kRadix * 4, st), "memset")) ||
-      (rc = cu(launch_zero(m + ps.lb, (size_t)pk.ntiles * 8, st), "memset")) ||
+  if ((rc = cu(launch_zero(m + ps.lb, (size_t)pk.ntiles * 8, st), "memset")) ||
       (rc = cu(launch_zero(m + ps.col_hist, kColPasses * kRadix * 4, st), "memset")) ||
-      (rc = cu(launch_zero(blk->q, sizeof(ans_quantities), st), "memset")))
+      (rc = cu(launch_zero(blk->q, sizeof(ans_quantities), st), "memset")) ||
+      (rc = cu(launch_zero(tickets, 32 * 4, st), "memset")) ||
+      (rc = sample_sort(c, m, ss, pk, d_src, d_dst, total, total, two, ka, kb, at<uint16_t>(m, ps.ck_a), st)))
     return rc;
-  if (rg && (rc = cu(timed(c, "wid_fill", st, [&] {
-                       return launch_wid_fill(rg->win, pk.in_off, rg->wid, rg->shift, seg_hist + kPasses * kRadix, st);
-                     }), "window ids")))
-    return rc;
-  // (the kv passes with window ids run two sub-tiles per tile)
-  if ((rc = cu(timed(c, "pack_hist_sum", st, [&] {
-                 return launch_pack_hist(pk, d_src, d_dst, ka, seg_hist, at<uint64_t>(m, ps.st0), tickets, st,
-                                         rg ? 2u : key_subtiles(c->cfg_keys));
-               }), "pack")))
-    return rc;
-  if (rg) {
-    uint64_t* st0 = at<uint64_t>(m, ps.st0);
-    uint64_t* st1 = at<uint64_t>(m, ps.st1);
-    for (int pass = 0; pass < kPasses; ++pass) {
-      const bool even = (pass % 2) == 0;
-      KTime kt(c, "onesweep_pk", st);
-      ANS_CUDA(launch_onesweep_wid(pk, pass, even ? ka : kb, even ? kb : ka, even ? rg->wid : rg->wid_b,
-                                   even ? rg->wid_b : rg->wid, seg_hist, even ? st0 : st1, even ? st1 : st0,
-                                   tickets + pass, c->d_err, c->cfg_keys, st));
-    }
-  } else {
-    ANS_TRY(sort_segments(c, pk, ka, kb, nullptr, nullptr, seg_hist, at<uint64_t>(m, ps.st0),
-                          at<uint64_t>(m, ps.st1), tickets, st, "onesweep_pk"));
-  }
   StatsArgs a;
   a.plan = pk;
   a.hdr = blk->hdr;
@@ -1102,7 +1157,7 @@ int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, c
   a.row_pos = at<uint64_t>(m, ps.row_pos);
   if (narrow) a.vals32 = (uint32_t*)at<uint64_t>(m, ps.cv_b);
   a.lookback = at<uint64_t>(m, ps.lb);
-  a.ticket = tickets + kPasses;  // zeroed by the pack kernel
+  a.ticket = tickets + kPasses;
   a.col_hist = at<uint32_t>(m, ps.col_hist);
   a.ulen = at<uint64_t>(m, ps.ulen);
   a.col_st0 = at<uint64_t>(m, ps.st0);
@@ -1114,39 +1169,6 @@ int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, c
   if ((rc = cu(timed(c, "finish", st, [&] { return launch_finish(a, st); }), "finish"))) return rc;
   return column_pass(c, pk, a.ulen, blk->col_ids, blk->vals, ps, m, a.col_tickets, blk->q, st, narrow,
                      a.col_hkeys);
-}
-
-// The windows' sorted keys from the batch's packet sort (agg_path 3, after
-// sum_packets with `rg`): the sorted packets are sorted again by window id
-// in two stable digit passes (keys_a -> keys_b -> keys_a), the second of
-// which moves each window's packets to its padded base.  Within a window
-// the packets keep the key order of the packet sort, so keys_a ends as the
-// window sort would leave it.  The scratch words the sum's reduction used
-// (status words, tickets, look-back and column histograms) are cleared
-// again for the window statistics.  Only queues work on `st`.
-int regroup_windows(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, const Regroup& rg,
-                    uint64_t win_tiles, cudaStream_t st) {
-  uint64_t* ka = at<uint64_t>(m, ps.keys_a);
-  uint64_t* kb = at<uint64_t>(m, ps.keys_b);
-  uint64_t* st0 = at<uint64_t>(m, ps.st0);
-  uint64_t* st1 = at<uint64_t>(m, ps.st1);
-  uint32_t* tickets = at<uint32_t>(m, ps.tickets);
-  const uint32_t* hist = at<uint32_t>(m, ps.seg_hist) + kPasses * kRadix;
-  ANS_CUDA(launch_zero(st0, (size_t)pk.ntiles * 2 * kRadix * 8, st));
-  ANS_CUDA(launch_zero(tickets, 32 * 4, st));  // these passes' and the window statistics
-  ANS_CUDA(launch_zero(m + ps.lb, (size_t)win_tiles * 8, st));
-  ANS_CUDA(launch_zero(m + ps.col_hist, (size_t)rg.win.nseg * kColPasses * kRadix * 4, st));
-  {
-    KTime kt(c, "regroup", st);
-    ANS_CUDA(launch_onesweep_regroup(pk, 0 | kPassStable, rg.wid, rg.wid_b, ka, kb, hist, st0, st1, tickets,
-                                     c->d_err, c->cfg_keys, nullptr, 0, st));
-  }
-  {
-    KTime kt(c, "regroup", st);
-    ANS_CUDA(launch_onesweep_regroup(pk, 1, rg.wid_b, nullptr, kb, ka, hist, st1, st0, tickets + 1, c->d_err,
-                                     c->cfg_keys, rg.shift, rg.win.nseg, st));
-  }
-  return ANS_OK;
 }
 
 // Snapshot the device error word into `dst` (device); reset_err clears it.
@@ -1269,12 +1291,11 @@ void plan_tables(const std::vector<uint64_t>& lens, std::vector<uint32_t>* lg, H
   tab->build(slots, nullptr);
 }
 
-// agg_path 3: the windows' sorted keys come from the batch's one packet sort
-// (which then also gives the time sum), for batches with a time sum, two or
-// more windows (at most 2^16: the ids travel as 16-bit values) and the
-// packets in one stream.
-bool regroup_windows_ok(const ans_ctx* c, uint32_t nseg, bool want_sum, bool addrs) {
-  return c->agg_path == 3 && want_sum && nseg >= 2 && nseg <= kMaxRegroupWindows && !addrs;
+// agg_path 3: the time sum comes from the batch's packets, sorted as one
+// segment, for batches with a time sum, two or more windows (at most 2^16)
+// and the packets in one stream.
+bool agg_packets(const ans_ctx* c, uint32_t nseg, bool want_sum, bool addrs) {
+  return c->agg_path == 3 && want_sum && nseg >= 2 && nseg <= kMaxPacketWindows && !addrs;
 }
 
 // Scratch layout of one batch (shared by run_windows and ans_batch_bytes).
@@ -1288,14 +1309,17 @@ struct WinLayout {
   size_t off_hqwin = 0, off_lstart = 0, off_kstart = 0, off_sortlen = 0, off_items = 0;  // hashed window statistics
   DevPlan dp_tab;        // hash path: the windows' tables as segments
   DevPlan dp_pk;         // sum_path 2: all packets of the batch as one segment
-  size_t off_wid = 0, off_wshift = 0;  // agg_path 3: packets' window ids, windows' offsets to their bases
   size_t off_tlg = 0, off_special = 0, off_hulen = 0, off_nclaim = 0, off_claims = 0;
   PipeScratch ps;
+  SsScratch ss;
+  bool ss_two_win = false, ss_two_pk = false;  // windows, or the batch as one segment, beyond one split
   size_t s_col = 0, s_vals = 0, s_row = 0, s_rp = 0, s_hdr = 0, s_q = 0;
   size_t off_mats = 0, off_gplan = 0, off_splan = 0, off_catoff = 0, off_lens = 0, off_total = 0;
   size_t size = 0;
-  void reserve(const HostPlan& hp, uint32_t nseg, bool want_mats, bool want_sum, bool hash = false,
-               bool regroup = false) {
+  // total, max_len: the batch's packets, its longest window (bounds, when
+  // the batch is planned on the device).
+  void reserve(const HostPlan& hp, uint32_t nseg, bool want_mats, bool want_sum, uint64_t total, uint64_t max_len,
+               bool hash = false) {
     Layout L;
     const bool addrs = !hp.src_at.empty();
     dp.reserve(L, nseg, addrs);
@@ -1311,10 +1335,6 @@ struct WinLayout {
     off_sortlen = L.add((size_t)nseg * 8);
     off_items = L.add(((size_t)2 * nseg + 2) * 4);
     dp_pk.reserve(L, 1);
-    if (regroup) {
-      off_wid = L.add(hp.pad * 2);
-      off_wshift = L.add((size_t)nseg * 8);
-    }
     if (hash) {
       dp_tab.reserve(L, nseg);
       off_tlg = L.add((size_t)nseg * 4);
@@ -1324,6 +1344,9 @@ struct WinLayout {
       off_claims = L.add(hp.pad * 4);
     }
     ps.reserve(L, hp.pad, std::max<uint32_t>(nseg, 1), hp.ntiles, want_sum || hash);
+    ss_two_win = max_len > ss_one_level(total);
+    ss_two_pk = want_sum && total > ss_one_level(total);
+    ss.reserve(L, std::max<uint32_t>(nseg, 1), hp.ntiles, ss_two_win || ss_two_pk);
     if (!want_mats) {  // the DCSR arrays are intermediate: keep them in scratch
       s_col = L.add(hp.pad * 4);
       s_vals = L.add(hp.pad * 8);
@@ -1365,6 +1388,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
     }
     total = h_offsets[nwin] - h_offsets[0];
   }
+  uint64_t max_len = dev ? total : 0;
+  for (uint64_t l : lens) max_len = std::max(max_len, l);
   if (total && !h_srcs && (!d_src || !d_dst)) return fail(ANS_ERR_INVALID_ARG, "NULL packet arrays");
   const bool want_mats = (flags & ANS_BATCH_MATRICES) != 0;
   const bool want_sum = (flags & ANS_BATCH_SUM) != 0;
@@ -1400,9 +1425,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   const SortCfg cfg_win = c->cfg_win;
   // (hashed window statistics, agg_path 2, sort only the windows the hash
   // gives up on: those take the key passes)
-  // (the windows of the packet sort, agg_path 3, take no window sort at all)
-  const bool regroup = regroup_windows_ok(c, nseg, want_sum, h_srcs != nullptr);
-  const bool on_chip = !dev && win_path == 0 && !(c->agg_path == 2 && !want_mats) && !regroup &&
+  const bool packets = agg_packets(c, nseg, want_sum, h_srcs != nullptr);
+  const bool on_chip = !dev && win_path == 0 && !(c->agg_path == 2 && !want_mats) && !packets &&
                        cluster_sort_clusters(c->device) > 0;
   for (uint32_t s = 0; s < nseg; ++s) {
     if (on_chip && lens[s] <= kClusterWindowMax) small_ids.push_back(s);
@@ -1427,7 +1451,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   std::vector<size_t> guard_off;
   {
     GuardSink gs(c->guards ? &guard_off : nullptr);
-    wl.reserve(hp, nseg, want_mats, want_sum, hash, regroup);
+    wl.reserve(hp, nseg, want_mats, want_sum, total, max_len, hash);
   }
   const DevPlan& dp = wl.dp;
   const PipeScratch& ps = wl.ps;
@@ -1483,7 +1507,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   // sum_path 2: all packets of the batch as one segment (device-planned
   // batches: its offset and length come from the planner, the tile count is
   // the capacity's)
-  const bool sum_pk = want_sum && nseg && (c->sum_path == 2 || regroup) && !h_srcs;
+  const bool sum_pk = want_sum && nseg && (c->sum_path == 2 || packets) && !h_srcs;
   // agg_path 2: the windows' quantities by on-chip hashing, when no window
   // DCSR is returned and the time sum (if any) comes from the packets
   const bool hq = c->agg_path == 2 && nseg && !want_mats && (!want_sum || sum_pk);
@@ -1671,24 +1695,11 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
                      }), "cluster sort")))
           return rc;
       }
-      if (regroup) {  // the time sum first; its packet sort yields the windows' order
-        Regroup rg;
-        rg.win = p;
-        rg.wid = at<uint16_t>(m, wl.off_wid);
-        rg.wid_b = at<uint16_t>(m, ps.ck_a);
-        rg.shift = at<uint64_t>(m, wl.off_wshift);
-        const SegPlan pk = wl.dp_pk.bind(m, hp_pk);
-        if ((rc = sum_packets(c, m, ps, pk, d_src, d_dst, sump.blk, ls, total < (1ull << 32), &rg))) return rc;
-        if ((rc = regroup_windows(c, m, ps, pk, rg, hp.ntiles, ls))) return rc;
-      } else if (!hash && !big_ids.empty()) {
+      if (!hash && !big_ids.empty()) {
         const SegPlan pb = dev || big_ids.size() == nseg ? pwin : wl.dp_big.bind(m, hp_big);
-        const size_t nb = big_ids.size();
-        if ((rc = cu(launch_zero(seg_hist, nb * kPasses * kRadix * 4, ls), "memset hist"))) return rc;
-        if ((rc = cu(timed(c, "pack_hist", ls, [&] { return launch_pack_hist(pb, d_src, d_dst, ka, seg_hist, at<uint64_t>(m, ps.st0), tickets, ls,
-                                                                                         key_subtiles(c->cfg_keys)); }), "pack")))
-          return rc;
-        if ((rc = sort_segments(c, pb, ka, kb, nullptr, nullptr, seg_hist, at<uint64_t>(m, ps.st0),
-                                at<uint64_t>(m, ps.st1), tickets, ls)))
+        if ((rc = cu(launch_zero(tickets, 32 * 4, ls), "memset")) ||
+            (rc = sample_sort(c, m, wl.ss, pb, d_src, d_dst, total, max_len, wl.ss_two_win, ka, kb,
+                              at<uint16_t>(m, ps.ck_a), ls)))
           return rc;
       }
       StatsArgs a;
@@ -1715,7 +1726,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       // With merge rounds, the run reduction also writes each link's key
       // beside its stored value (keys_b at the window's padded base): the
       // windows' links are then the time sum's sorted input runs in place.
-      const bool in_place = want_sum && c->sum_path == 0 && !regroup;
+      const bool in_place = want_sum && c->sum_path == 0 && !packets;
       if (in_place) a.sum_keys = kb;
       if ((rc = cu(timed(c, "empty_fixup", ls, [&] { return launch_empty_fixup(a, ls); }), "empty"))) return rc;
       if ((rc = cu(timed(c, "rle", ls, [&] { return launch_rle(a, ls); }), "rle"))) return rc;
@@ -1764,10 +1775,9 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
         if ((rc = cu(launch_zero(sblk->q, sizeof(ans_quantities), ls), "memset"))) return rc;
       } else if (forked) {  // a sum of window counts stays below the batch's packets
         if ((rc = links_to_block(c, m, ps, sump.s, sfk, sfv, sump.blk, ls, total < (1ull << 32)))) return rc;
-      } else if (regroup) {
-        // (the sum came first, from the packet sort that ordered the windows)
       } else if (sum_pk) {
-        if ((rc = sum_packets(c, m, ps, wl.dp_pk.bind(m, hp_pk), d_src, d_dst, sump.blk, ls, total < (1ull << 32))))
+        if ((rc = sum_packets(c, m, ps, wl.dp_pk.bind(m, hp_pk), d_src, d_dst, sump.blk, ls, total < (1ull << 32),
+                              wl.ss, total, wl.ss_two_pk)))
           return rc;
       } else {
         rc = sum_launch(c, m, ps, at<MatDesc>(m, off_mats), nseg, &sump, off_catoff, off_lens, off_total, ls,
@@ -1782,7 +1792,9 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   // the column hash's cluster shape changes with the window count: a cached
   // graph must not be updated to another one
   const std::string sig = launch_sig(flags, hp.ntiles > 0, !small_ids.empty(), !big_ids.empty(), rounds, c) + "/h" +
-                          std::to_string(c->col_hash && nseg ? colhash_ctas(nseg) : 0u) + (dev ? "/d" : "");
+                          std::to_string(c->col_hash && nseg ? colhash_ctas(nseg) : 0u) + (dev ? "/d" : "") + "/s" +
+                          std::to_string(wl.ss_two_win) + std::to_string(wl.ss_two_pk) +
+                          std::to_string(ss_shape(hp.ntiles)) + std::to_string(ss_shape(wl.ss.ntiles2));
   if ((rc = run_launches(c, st, sig, launch_all))) return bail(rc);
   if (sump.blk) {  // the time sum's block is filled
     sblk = sump.blk;
@@ -2639,11 +2651,12 @@ int ans_ctx_memory(ans_ctx* c, size_t* live_bytes, size_t* budget_bytes) {
 int ans_batch_bytes(ans_ctx* c, const uint64_t* h_offsets, size_t nwin, uint32_t flags, size_t* bytes) {
   if (!c || !h_offsets || !bytes) return fail(ANS_ERR_INVALID_ARG, "NULL argument");
   std::vector<uint64_t> lens(nwin);
-  uint64_t total = 0;
+  uint64_t total = 0, max_len = 0;
   for (size_t w = 0; w < nwin; ++w) {
     if (h_offsets[w + 1] < h_offsets[w]) return fail(ANS_ERR_INVALID_ARG, "offsets must be nondecreasing");
     lens[w] = h_offsets[w + 1] - h_offsets[w];
     total += lens[w];
+    max_len = std::max(max_len, lens[w]);
   }
   HostPlan hp;
   hp.build(lens, nullptr);
@@ -2651,8 +2664,7 @@ int ans_batch_bytes(ans_ctx* c, const uint64_t* h_offsets, size_t nwin, uint32_t
   std::lock_guard<std::mutex> g(c->mu);
   const bool hash = c->agg_path == 1 && nwin > 0;
   WinLayout wl;
-  wl.reserve(hp, (uint32_t)nwin, want_mats, want_sum, hash,
-             nwin <= 0xFFFFFFF0ull && regroup_windows_ok(c, (uint32_t)nwin, want_sum, false));
+  wl.reserve(hp, (uint32_t)nwin, want_mats, want_sum, total, max_len, hash);
   size_t need = 0;
   if (wl.size > c->scratch_size)  // the scratch is replaced by a larger one
     need += std::max(wl.size, c->scratch_size + c->scratch_size / 4) - c->scratch_size;
@@ -2736,9 +2748,10 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
   if (!c || !h_offsets || nwin == 0) return fail(ANS_ERR_INVALID_ARG, "NULL argument or empty batch");
   if (flags & ~(ANS_BATCH_MATRICES | ANS_BATCH_SUM | ANS_BATCH_SYNC)) return fail(ANS_ERR_INVALID_ARG, "unknown flag");
   flags &= ANS_BATCH_MATRICES | ANS_BATCH_SUM;
-  // The last kKeyOnly shapes exist for the key and column passes only (not
-  // for the kv passes).
-  constexpr int kVariants = 12, kKeyOnly = 3;
+  // The last kColOnly shapes exist for the column passes only (not for the
+  // kv passes).  Packets are sorted without digit passes: the key_* shape
+  // stays as it is set.
+  constexpr int kVariants = 12, kColOnly = 3;
   const SortCfg variants[kVariants] = {{512, kRankMatch, 1}, {512, kRankBallot, 1}, {512, kRankTable, 1},
                                        {512, kRankMatch, 2}, {512, kRankBallot, 2}, {512, kRankTable, 2},
                                        {1024, kRankMatch, 1}, {1024, kRankBallot, 1}, {1024, kRankTable, 1},
@@ -2840,23 +2853,26 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
     return it == p.end() ? 0.0 : it->second;
   };
   constexpr double kNever = 1e300;
+  auto sort_time = [&](const Prof& p) {
+    return get(p, "ss_sample") + get(p, "ss_count") + get(p, "ss_scatter") + get(p, "ss_plan") + get(p, "ss_local");
+  };
 
   // Radix-pass launch shapes, per family, on the paths that use them all.
-  double t_keys[kVariants], t_kv[kVariants], t_col[kVariants];
+  double t_keys = kNever, t_kv[kVariants], t_col[kVariants];
   for (int v = 0; v < kVariants; ++v) {
-    const bool key_only = v >= kVariants - kKeyOnly;
+    const bool col_only = v >= kVariants - kColOnly;
     Prof pr;
     bool ran = false;
     ANS_TRY(trial([&] {
-      c->cfg_keys = c->cfg_kv = c->cfg_col = variants[key_only ? 0 : v];
-      c->cfg_keys = c->cfg_col = variants[v];
-      c->win_path = 1;  // the key passes on every window
+      c->cfg_kv = variants[col_only ? 0 : v];
+      c->cfg_col = variants[v];
+      c->win_path = 1;  // the sample sort on every window
       c->sum_path = 1;  // the kv passes on the time sum
       c->agg_path = 0;
     }, &pr, &ran));
     if (!ran) return fail(ANS_ERR_OOM, "autotune: the batch does not fit the device with the default paths");
-    t_keys[v] = get(pr, "onesweep") + get(pr, "pack_hist");
-    t_kv[v] = key_only ? kNever : get(pr, "onesweep_sum") + get(pr, "gather");
+    t_keys = std::min(t_keys, sort_time(pr));
+    t_kv[v] = col_only ? kNever : get(pr, "onesweep_sum") + get(pr, "gather");
     t_col[v] = get(pr, "onesweep_col");
   }
   auto best = [&](const double* t) {
@@ -2865,18 +2881,17 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
       if (t[v] < t[b]) b = v;
     return b;
   };
-  const int bk_i = best(t_keys), bv_i = best(t_kv), bc_i = best(t_col);
+  const int bv_i = best(t_kv), bc_i = best(t_col);
   auto base = [&] {
-    c->cfg_keys = variants[bk_i];
     c->cfg_kv = variants[bv_i];
     c->cfg_col = variants[bc_i];
   };
 
-  // The on-chip window sort (windows that fit a cluster) against the key
-  // passes plus their histogram sweep.
+  // The on-chip window sort (windows that fit a cluster) against the sample
+  // sort.
   int win_path = 1;
   SortCfg win_cfg{1024, kRankMatch, 1};
-  double best_win = t_keys[bk_i];
+  double best_win = t_keys;
   if (cluster_sort_clusters(c->device) > 0) {
     const SortCfg wv[3] = {{1024, kRankMatch, 1}, {1024, kRankBallot, 1}, {512, kRankMatch, 1}};
     for (const SortCfg& w : wv) {
@@ -2889,7 +2904,7 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
         c->sum_path = 1;
         c->agg_path = 0;
       }, &pr, &ran));
-      const double t = ran ? get(pr, "cluster_sort") + get(pr, "onesweep") + get(pr, "pack_hist") : kNever;
+      const double t = ran ? get(pr, "cluster_sort") + sort_time(pr) : kNever;
       if (t < best_win) {
         best_win = t;
         win_path = 0;
@@ -2952,7 +2967,7 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
     // it from the packets)
     const bool want_sum = (flags & ANS_BATCH_SUM) != 0;
     const bool ok[4] = {true, true, !(flags & ANS_BATCH_MATRICES),
-                        want_sum && nwin >= 2 && nwin <= kMaxRegroupWindows};
+                        want_sum && nwin >= 2 && nwin <= kMaxPacketWindows};
     const int sum_for[4] = {sum_path, sum_path, want_sum ? 2 : sum_path, 2};
     double wall[4] = {kNever, kNever, kNever, kNever};
     for (int a = 0; a < 4; ++a) {
@@ -2974,15 +2989,13 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
   }
 
   // With the paths chosen, the column passes' shape (on the large time sums
-  // they order the summed links by destination hash) and, when the windows
-  // come from the packet sort, the ranking of its passes: each by the
-  // batch's device time as the production path runs it.
-  SortCfg bk = variants[bk_i], bc = variants[bc_i];
+  // they order the summed links by destination hash) by the batch's device
+  // time as the production path runs it.
+  SortCfg bc = variants[bc_i];
   const SortCfg bv = variants[bv_i];
   {
     auto chosen_paths = [&] {
       base();
-      c->cfg_keys = bk;
       c->cfg_col = bc;
       c->win_path = win_path;
       c->cfg_win = win_cfg;
@@ -3006,23 +3019,12 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
         }
       }
     }
-    if (agg_path == 3) {
-      for (int r = kRankMatch; r <= kRankBallot; ++r) {
-        if (r == bk.rank) continue;
-        const SortCfg v{bk.threads, r, bk.blocks};
-        ANS_TRY(trial([&] { chosen_paths(); c->cfg_keys = v; }, &pr, &ran));
-        if (ran && pr[kWall] < best_wall) {
-          best_wall = pr[kWall];
-          bk = v;
-        }
-      }
-    }
   }
 
   ans_tuning res{};
-  res.key_threads = (uint32_t)bk.threads;
-  res.key_rank = (uint32_t)bk.rank;
-  res.key_blocks = (uint32_t)bk.blocks;
+  res.key_threads = (uint32_t)c->cfg_keys.threads;
+  res.key_rank = (uint32_t)c->cfg_keys.rank;
+  res.key_blocks = (uint32_t)c->cfg_keys.blocks;
   res.kv_threads = (uint32_t)bv.threads;
   res.kv_rank = (uint32_t)bv.rank;
   res.kv_blocks = (uint32_t)bv.blocks;

@@ -48,14 +48,12 @@ enum ErrBits : uint32_t {
   kErrGuard = 16u,     // a scratch guard (debug mode) was overwritten
 };
 constexpr uint64_t kMaxWindowItems = (1ull << 31) - 1;  // packets of one window, links of one time sum
-constexpr int kPassStable = 0x100;  // digit-pass flag: pass 0 keeps the input order of equal digits
-constexpr int kPassMask = 0xFF;
-constexpr uint32_t kMaxRegroupWindows = 1u << 16;  // window ids carried as 16-bit values
+constexpr uint32_t kMaxPacketWindows = 1u << 16;  // windows of a batch that agg_path 3 takes
 
 // How a onesweep pass is launched (chosen per context by the autotuner):
-// threads per 8192-key tile (512 or 1024; for the 64-bit key passes and the
-// column passes with 32-bit counts also 256, which splits every tile into
-// two 4096-key sub-tiles with one CTA each and four resident CTAs per SM), how lanes with equal digits are found (one
+// threads per 8192-key tile (512 or 1024; for the column passes with 32-bit
+// counts also 256, which splits every tile into two 4096-key sub-tiles with
+// one CTA each and four resident CTAs per SM), how lanes with equal digits are found (one
 // __match_any_sync; eight ballots; or a per-warp shared-memory table where
 // each lane ORs its bit into its digit's entry, which also holds the digit's
 // running count), and whether a 512-thread tile is compiled to leave room for
@@ -254,38 +252,11 @@ cudaError_t launch_plan(const uint64_t* d_offsets, uint32_t nseg, uint64_t cap, 
 int set_last_error(int code, const std::string& msg);
 
 // ---- launchers (ans_sort.cu) ---------------------------------------------
-// Pack (src, dst) into keys src << 32 | dst, build per-segment digit
-// histograms of all passes, zero the pass-0 status words (sub * kRadix per
-// tile, for key passes over `sub` sub-tiles per tile) and the tickets.
-cudaError_t launch_pack_hist(const SegPlan& p, const uint32_t* src, const uint32_t* dst,
-                             uint64_t* keys, uint32_t* seg_hist, uint64_t* status0,
-                             uint32_t* tickets, cudaStream_t st, uint32_t sub = 1);
-// Sub-tiles per tile of a key-pass configuration.
-constexpr uint32_t key_subtiles(const SortCfg& cfg) { return cfg.threads == 256 ? 2u : 1u; }
-// One onesweep digit pass (stable), optionally carrying uint64 values.
+// One onesweep digit pass (stable) over 64-bit keys carrying uint64 values.
 cudaError_t launch_onesweep(const SegPlan& p, int pass, const uint64_t* kin, uint64_t* kout,
                             const uint64_t* vin, uint64_t* vout, const uint32_t* seg_hist,
                             uint64_t* st_cur, uint64_t* st_next, uint32_t* ticket,
                             uint32_t* err, const SortCfg& cfg, cudaStream_t st);
-// The one packet sort of a batch that also yields its windows' order
-// (agg_path 3): a digit pass over the 64-bit keys carrying each packet's
-// 16-bit window id, and a stable digit pass over the window ids carrying the
-// keys (pass | kPassStable for its first pass; with `remap`, a key whose
-// window is w lands at its sorted place + remap[w]; a null kout drops the
-// ids).  Both in the 4096-key sub-tile shape with cfg's ranking mode.
-cudaError_t launch_onesweep_wid(const SegPlan& p, int pass, const uint64_t* kin, uint64_t* kout,
-                                const uint16_t* vin, uint16_t* vout, const uint32_t* seg_hist, uint64_t* st_cur,
-                                uint64_t* st_next, uint32_t* ticket, uint32_t* err, const SortCfg& cfg,
-                                cudaStream_t st);
-cudaError_t launch_onesweep_regroup(const SegPlan& p, int pass, const uint16_t* kin, uint16_t* kout,
-                                    const uint64_t* vin, uint64_t* vout, const uint32_t* seg_hist,
-                                    uint64_t* st_cur, uint64_t* st_next, uint32_t* ticket, uint32_t* err,
-                                    const SortCfg& cfg, const uint64_t* remap, uint32_t nremap, cudaStream_t st);
-// Window ids of the windows of `p` over their packets in the batch's
-// one-segment packet order, each window's offset from that order (sorted by
-// window) to its padded base, and the ids' two digit histograms.
-cudaError_t launch_wid_fill(const SegPlan& p, const uint64_t* pk_in_off, uint16_t* wid, uint64_t* shift,
-                            uint32_t* hist, cudaStream_t st);
 // One digit pass over 32-bit destination keys carrying uint64 counts.
 cudaError_t launch_onesweep_col(const SegPlan& p, int pass, const uint32_t* kin, uint32_t* kout,
                                 const uint64_t* vin, uint64_t* vout, const uint32_t* seg_hist,
@@ -307,6 +278,61 @@ cudaError_t launch_gather(const SegPlan& p, const MatDesc* mats, const uint64_t*
 // lens, their sum -> *total and cat_off[k].
 cudaError_t launch_count_prefix(const MatDesc* mats, uint32_t k, uint64_t* cat_off, uint64_t* lens,
                                 uint64_t* total, cudaStream_t st);
+
+// ---- launchers (ans_ssort.cu) ----------------------------------------------
+// Segmented sample sort of link keys (see ans_ssort.cu): sample, count,
+// scatter, local over the segments of `plan` (raw packets), or over the
+// level-2 segments that launch_ss_plan2 lists after a first split of the
+// segments longer than one_level.
+constexpr uint32_t kSsPerTile = 3;  // buckets per tile of keys
+// Longest segment that one split takes, in a plan of `total` keys.  One CTA
+// sorts a segment's sample: 23 us for 2^17 keys, 148 us for 2^20 (measured),
+// which a large batch hides behind its other segments and a small one does
+// not; a second split costs two more reads and a write of the keys.
+constexpr uint64_t ss_one_level(uint64_t total) { return total >= (1ull << 24) ? 1ull << 21 : 1ull << 18; }
+struct SsArgs {
+  SegPlan plan;                         // raw packets: window_inputs(plan, s, src, dst)
+  const uint32_t* src = nullptr;
+  const uint32_t* dst = nullptr;
+  const uint64_t* start = nullptr;      // segments: first place in the key buffers, length,
+  const uint64_t* len = nullptr;        // first tile, and (optional) each tile's segment
+  const uint32_t* first_tile = nullptr;
+  const uint32_t* tile_seg = nullptr;
+  const uint32_t* parent = nullptr;     // level 2: where the segment's keys are (null: raw)
+  const uint32_t* nseg_d = nullptr;     // level 2: segments and tiles in use, on the device
+  const uint32_t* ntiles_d = nullptr;
+  uint32_t nseg = 0, ntiles = 0;        // or a bound on them
+  bool level1 = false;                  // the first of two splits
+  uint64_t one_level = 0;
+  const uint64_t* keys_in = nullptr;    // level 2: the first split's output
+  uint64_t* keys_split = nullptr;       // this split's output
+  uint64_t* keys_out = nullptr;         // the sorted keys
+  uint16_t* ids = nullptr;              // bucket of every key, at its place
+  uint64_t* tree = nullptr;             // [2 * kSsPerTile * ntiles] splitter trees
+  uint32_t* cnt = nullptr;              // [kSsPerTile * ntiles] each: bucket sizes, cursors, starts,
+  uint32_t* cur = nullptr;              //     one-value marks
+  uint32_t* bstart = nullptr;
+  uint8_t* eq = nullptr;
+  uint32_t sample_max = 0;
+};
+struct SsSeg2 {
+  uint64_t* start = nullptr;
+  uint64_t* len = nullptr;
+  uint32_t* parent = nullptr;
+  uint32_t* first_tile = nullptr;  // one more entry
+  uint32_t* tile_seg = nullptr;
+  uint32_t* count = nullptr;       // [2] segments, tiles
+};
+// Bound on the buckets of the first splits of at most nseg segments of `total` keys in all.
+uint64_t ss_level1_buckets(uint64_t total, uint64_t nseg);
+cudaError_t launch_ss_sample(const SsArgs& a, uint64_t max_len, cudaStream_t st);
+cudaError_t launch_ss_count(const SsArgs& a, cudaStream_t st);
+cudaError_t launch_ss_scatter(const SsArgs& a, cudaStream_t st);
+cudaError_t launch_ss_local(const SsArgs& a, cudaStream_t st);
+// Launch shape of count and scatter for a plan of this many tiles (part of
+// the key of a cached batch graph).
+int ss_shape(uint32_t ntiles);
+cudaError_t launch_ss_plan2(const SsArgs& a, const SsSeg2& o, cudaStream_t st);
 
 // ---- launchers (ans_cluster.cu) ------------------------------------------
 // Sort the keys src << 32 | dst of every segment seg_ids[0..nclusters) (or

@@ -42,10 +42,8 @@ constexpr uint32_t kNoAllocTiles = (uint32_t)(kNoAllocMaxPackets / kTile);
 // The buffers below are sized for kNoAllocMaxPackets items, which must cover
 // the padded index space (whole tiles) of the largest window.
 static_assert(kNoAllocMaxPackets % kTile == 0, "the packet limit must be a whole number of tiles");
-// The key passes run with the default launch shape; its sub-tiles' status
-// words must fit the two per tile reserved at oSt0 / oSt1.
-constexpr SortCfg kNoAllocSort{};
-static_assert(key_subtiles(kNoAllocSort) <= 2, "status words hold at most two sub-tiles per tile");
+constexpr SortCfg kNoAllocSort{};  // the column passes' launch shape
+static_assert(ss_one_level(kNoAllocMaxPackets) >= kNoAllocMaxPackets, "the packets take one split");
 constexpr size_t kAl = 256;
 constexpr size_t al(size_t x) { return (x + kAl - 1) / kAl * kAl; }
 
@@ -53,10 +51,14 @@ constexpr size_t al(size_t x) { return (x + kAl - 1) / kAl * kAl; }
 constexpr size_t oPlan = 0;                                        // in_off, len, base, first_tile[2]
 constexpr size_t oKeysA = al(oPlan + 64);
 constexpr size_t oKeysB = al(oKeysA + kNoAllocMaxPackets * 8);
-constexpr size_t oHist = al(oKeysB + kNoAllocMaxPackets * 8);
+constexpr size_t oTree = al(oKeysB + kNoAllocMaxPackets * 8);      // the packet sort's splitters and buckets
+constexpr size_t oCnt = al(oTree + (size_t)kNoAllocTiles * kSsPerTile * 16);
+constexpr size_t oCur = al(oCnt + (size_t)kNoAllocTiles * kSsPerTile * 4);
+constexpr size_t oBstart = al(oCur + (size_t)kNoAllocTiles * kSsPerTile * 4);
+constexpr size_t oEq = al(oBstart + (size_t)kNoAllocTiles * kSsPerTile * 4);
 // look-back status words: two sub-tiles' worth per tile (k_finish clears
 // that many for the column passes)
-constexpr size_t oSt0 = al(oHist + (size_t)kPasses * kRadix * 4);
+constexpr size_t oSt0 = al(oEq + (size_t)kNoAllocTiles * kSsPerTile);
 constexpr size_t oSt1 = al(oSt0 + (size_t)kNoAllocTiles * 2 * kRadix * 8);
 constexpr size_t oLb = al(oSt1 + (size_t)kNoAllocTiles * 2 * kRadix * 8);
 constexpr size_t oTickets = al(oLb + (size_t)kNoAllocTiles * 8);
@@ -142,7 +144,7 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
   if ((rc = cu(cudaMemsetAsync(err, 0, 8, st), "memset"))) return rc;  // error bits; default poll limit
   const uint32_t ntiles = (uint32_t)((n + kTile - 1) / kTile);
   if (ntiles) {
-    if ((rc = cu(cudaMemsetAsync(m + oHist, 0, (size_t)kPasses * kRadix * 4, st), "memset"))) return rc;
+    if ((rc = cu(cudaMemsetAsync(m + oTickets, 0, 32 * 4, st), "memset"))) return rc;
     if ((rc = cu(cudaMemsetAsync(m + oLb, 0, (size_t)ntiles * 8, st), "memset"))) return rc;
     if ((rc = cu(cudaMemsetAsync(m + oColHist, 0, (size_t)kColPasses * kRadix * 4, st), "memset"))) return rc;
     k_noalloc_plan<<<1, 32, 0, st>>>(n, ntiles);
@@ -159,16 +161,28 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     uint64_t* kb = reinterpret_cast<uint64_t*>(m + oKeysB);
     uint64_t* st0 = reinterpret_cast<uint64_t*>(m + oSt0);
     uint64_t* st1 = reinterpret_cast<uint64_t*>(m + oSt1);
-    uint32_t* hist = reinterpret_cast<uint32_t*>(m + oHist);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(m + oTickets);
-    if ((rc = cu(launch_pack_hist(p, d_src, d_dst, ka, hist, st0, tickets, st, key_subtiles(kNoAllocSort)), "pack"))) return rc;
-    for (int pass = 0; pass < kPasses; ++pass) {
-      const bool even = (pass % 2) == 0;
-      if ((rc = cu(launch_onesweep(p, pass, even ? ka : kb, even ? kb : ka, nullptr, nullptr, hist,
-                                   even ? st0 : st1, even ? st1 : st0, tickets + pass, err, kNoAllocSort, st),
-                   "onesweep")))
-        return rc;
-    }
+    SsArgs ss;
+    ss.one_level = kNoAllocMaxPackets;
+    ss.plan = p;
+    ss.src = d_src;
+    ss.dst = d_dst;
+    ss.start = p.base;
+    ss.len = p.len;
+    ss.first_tile = p.first_tile;
+    ss.nseg = 1;
+    ss.ntiles = ntiles;
+    ss.keys_split = kb;
+    ss.keys_out = ka;
+    ss.ids = reinterpret_cast<uint16_t*>(m + oCkA);  // free until the column passes
+    ss.tree = reinterpret_cast<uint64_t*>(m + oTree);
+    ss.cnt = reinterpret_cast<uint32_t*>(m + oCnt);
+    ss.cur = reinterpret_cast<uint32_t*>(m + oCur);
+    ss.bstart = reinterpret_cast<uint32_t*>(m + oBstart);
+    ss.eq = reinterpret_cast<uint8_t*>(m + oEq);
+    if ((rc = cu(launch_ss_sample(ss, n, st), "sample")) || (rc = cu(launch_ss_count(ss, st), "count")) ||
+        (rc = cu(launch_ss_scatter(ss, st), "scatter")) || (rc = cu(launch_ss_local(ss, st), "local sort")))
+      return rc;
     StatsArgs a;
     a.plan = p;
     a.hdr = reinterpret_cast<uint64_t*>(m + oHdr);

@@ -1,0 +1,700 @@
+// Segmented sample sort of 64-bit link keys.
+//
+// Grouping equal (src, dst) pairs (Table I caption: A(i, j) = #packets i -> j)
+// needs the packed keys src << 32 | dst of every window, or of a whole batch,
+// in order (Sec. IV-B: rows ascending, columns ascending within a row).  Equal
+// keys are indistinguishable, so the sort need not be stable, and it works
+// from the most significant end:
+//
+//   sample   one CTA per segment sorts ~32 sampled keys per bucket on chip and
+//            takes every 32nd as a splitter; a key that fills several buckets
+//            gets one of its own (its copies need no sorting at all);
+//   count    every key's bucket by a search tree of splitters in shared
+//            memory (ids kept as 16-bit words), bucket sizes;
+//   scatter  keys moved to their buckets: ranks by one shared-memory atomic
+//            per key, space by one global atomic per bucket and tile -- no
+//            chain of tiles waiting for one another;
+//   local    every bucket (~2048 keys) sorted by one CTA on chip: 16 keys per
+//            thread in registers, then merge-path rounds in shared memory.
+//
+// Buckets hold equal numbers of packets whatever the addresses look like, so
+// heavy sources and links cost nothing extra.  A segment too long for one
+// split is first split into about as many buckets as each of them will have,
+// which then are the segments of the steps above.
+//
+// Against eight least-significant-digit passes (each bound by its chain of
+// tiles and by 150 instructions per key; 53 us for 64 windows of 2^17 keys,
+// 930 us for 2^27 keys with 16-bit window ids) this reads and writes the keys
+// four times instead of nine: 64 windows in 274 us against 491, one window
+// of 2^17 in 60 us against 82, 2^27 keys as one segment in 4.9 ms.  On one
+// GB300 the local sort is bound by shared-memory wavefronts (75% of peak, 341
+// instructions per key), count by issue slots (72%), scatter by the latency
+// of its loads.
+#include "ans_internal.cuh"
+
+namespace ans {
+
+namespace {
+
+constexpr uint32_t kSsBucket = (kTile + kSsPerTile - 1) / kSsPerTile;  // keys per bucket aimed at
+constexpr uint32_t kSsLocal = 4096;         // keys one CTA sorts on chip
+constexpr uint32_t kSsMaxBuckets = 1024;    // buckets of one split
+constexpr uint32_t kSsSampleMax = 16384;    // sampled keys of one segment
+constexpr uint32_t kSsOversample = 32;      // sampled keys per bucket
+constexpr uint32_t kSsRawBit = 0x80000000u; // level-2 parent: the segment itself, still unsplit input
+constexpr uint32_t kSsDone = 0xFFFFFFFFu;   // level-2 parent: nothing to sort
+
+// Buckets of an n-key split.  Level 1, the first of two splits: as many as
+// the second split will make of each of its buckets.
+__host__ __device__ __forceinline__ uint32_t ss_buckets(uint64_t n, bool level1, uint64_t one_level) {
+  if (level1) {
+    if (n <= one_level) return 0u;
+    const uint64_t want = (n + kSsBucket - 1) / kSsBucket;
+    uint32_t r = 2;
+    while ((uint64_t)r * r < want && r < kSsMaxBuckets) r += r < 64 ? 1 : 16;
+    return r;
+  }
+  return n <= kSsLocal ? 1u : (uint32_t)umin64((n + kSsBucket - 1) / kSsBucket, kSsMaxBuckets);
+}
+__device__ __forceinline__ uint32_t ss_levels(uint32_t nb) { return nb <= 1 ? 0u : 32u - __clz(nb - 1); }
+
+// Where the keys of segment s come from.
+struct SsIn {
+  const uint32_t* src = nullptr;
+  const uint32_t* dst = nullptr;
+  const uint64_t* keys = nullptr;
+  __device__ __forceinline__ uint64_t get(uint64_t i) const {
+    return keys ? keys[i] : ((uint64_t)src[i] << 32) | dst[i];
+  }
+};
+
+// One split's segments: the plan's own (raw packets), or, after a first
+// split, the list seg2 (keys of the first split's buckets, or a raw segment
+// that was small enough).
+__device__ __forceinline__ SsIn ss_input(const SsArgs& a, uint32_t s, uint64_t start) {
+  SsIn in;
+  uint32_t raw = s;
+  if (a.parent) {
+    const uint32_t p = a.parent[s];
+    if (!(p & kSsRawBit)) {
+      in.keys = a.keys_in + start;
+      return in;
+    }
+    raw = p & ~kSsRawBit;
+  }
+  window_inputs(a.plan, raw, a.src, a.dst, &in.src, &in.dst);
+  return in;
+}
+
+struct SsSeg {
+  uint32_t s, b0, nb, ft;
+  uint64_t start, n;
+};
+__device__ __forceinline__ SsSeg ss_seg(const SsArgs& a, uint32_t s) {
+  SsSeg g;
+  g.s = s;
+  g.ft = a.first_tile[s];
+  g.b0 = g.ft * kSsPerTile;
+  g.n = a.len[s];
+  g.start = a.start[s];
+  g.nb = ss_buckets(g.n, a.level1, a.one_level);
+  if (a.parent && a.parent[s] == kSsDone) g.nb = 0;
+  return g;
+}
+__device__ __forceinline__ uint32_t ss_find(const SsArgs& a, uint32_t t) {
+  if (a.tile_seg) return a.tile_seg[t];
+  uint32_t lo = 0, hi = a.nseg_d ? *a.nseg_d : a.nseg;
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (a.first_tile[mid] <= t) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+__device__ __forceinline__ uint32_t mix32(uint32_t h) {  // MurmurHash3's finalizer
+  h ^= h >> 16;
+  h *= 0x85ebca6bu;
+  h ^= h >> 13;
+  h *= 0xc2b2ae35u;
+  return h ^ (h >> 16);
+}
+
+constexpr int kSsSampleThreads = 1024;
+
+// Bitonic sort of sm[0 .. R * 1024) by 1024 threads, R keys per thread in
+// registers (key r of thread t is element r * 1024 + t): strides below a warp
+// by shuffles, above the CTA's width in registers, the rest through sm.
+template <int R>
+__device__ __forceinline__ void ss_bitonic_r(uint64_t* sm) {
+  const uint32_t t = threadIdx.x;
+  uint64_t v[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) v[r] = sm[r * 1024 + t];
+  for (uint32_t k = 2; k <= R * 1024u; k <<= 1) {
+#pragma unroll
+    for (int lr = 4; lr >= 0; --lr) {  // strides of whole register rows
+      const int jr = 1 << lr;
+      if (jr < R && (uint32_t)jr * 1024u < k) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if ((r & jr) == 0 && r + jr < R) {
+            const bool up = (((uint32_t)r * 1024u + t) & k) == 0;
+            const uint64_t x = v[r], y = v[(r + jr) % R];
+            const bool sw = (x > y) == up;
+            v[r] = sw ? y : x;
+            v[(r + jr) % R] = sw ? x : y;
+          }
+        }
+      }
+    }
+    for (uint32_t j = min(k >> 1, 512u); j > 0; j >>= 1) {
+      if (j >= 32) {
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < R; ++r) sm[r * 1024 + t] = v[r];
+        __syncthreads();
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint64_t o = j >= 32 ? sm[(r * 1024 + t) ^ j] : __shfl_xor_sync(0xffffffffu, v[r], j);
+        const bool up = (((uint32_t)r * 1024u + t) & k) == 0, low = (t & j) == 0;
+        v[r] = (v[r] > o) == (up == low) ? o : v[r];
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < R; ++r) sm[r * 1024 + t] = v[r];
+  __syncthreads();
+}
+__device__ __forceinline__ void ss_bitonic(uint64_t* sm, uint32_t S) {
+  if (S == 1024) ss_bitonic_r<1>(sm);
+  else if (S == 2048) ss_bitonic_r<2>(sm);
+  else if (S == 4096) ss_bitonic_r<4>(sm);
+  else if (S == 8192) ss_bitonic_r<8>(sm);
+  else ss_bitonic_r<16>(sm);
+}
+
+
+// The segment's splitters as a search tree: tree[1 .. 2^lv) in breadth-first
+// order over the sorted splitters (padded with all-ones).  Bucket b holds the
+// keys k with exactly b splitters <= k.  A splitter value drawn twice or more
+// is one that fills at least a bucket: it is kept together with its
+// successor, so that the bucket between the two holds copies of it alone.
+__global__ void __launch_bounds__(kSsSampleThreads) k_ss_sample(SsArgs a) {
+  extern __shared__ __align__(16) uint64_t sm[];
+  __shared__ uint32_t s_w[kSsSampleThreads / 32], s_tot;
+  const uint32_t nseg = a.nseg_d ? *a.nseg_d : a.nseg;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (uint32_t s = blockIdx.x; s < nseg; s += gridDim.x) {
+    const SsSeg g = ss_seg(a, s);
+    for (uint32_t i = tid; i < g.nb; i += kSsSampleThreads) {
+      a.cnt[g.b0 + i] = 0;
+      a.cur[g.b0 + i] = 0;
+    }
+    if (g.nb <= 1) continue;
+    const SsIn in = ss_input(a, s, g.start);
+    const uint32_t lv = ss_levels(g.nb);
+    uint32_t S = 1024;
+    while (S < g.nb * kSsOversample && S < a.sample_max) S <<= 1;
+    // one key from each of S equal stretches of the segment
+    for (uint32_t i = tid; i < S; i += kSsSampleThreads) {
+      const uint64_t at = (((uint64_t)i << 16 | (mix32(i + 1) & 0xFFFFu)) * g.n) >> (16 + (31 - __clz(S)));
+      sm[i] = in.get(at);
+    }
+    __syncthreads();
+    ss_bitonic(sm, S);
+    // splitter candidates 1 .. nb - 1 (at most 1023: one per thread)
+    auto cand = [&](uint32_t i) { return sm[(uint32_t)(((uint64_t)i * S) / g.nb)]; };
+    const uint32_t c = tid + 1;
+    const bool in_range = c < g.nb;
+    const uint64_t v = in_range ? cand(c) : 0ull;
+    const bool first = in_range && (c == 1 || cand(c - 1) != v);
+    const bool twice = first && c + 1 < g.nb && cand(c + 1) == v && v != ~0ull;
+    // the successor is dropped if it is itself the next splitter
+    bool succ = twice;
+    if (twice) {
+      uint32_t lo = c + 1, hi = g.nb;  // the next different candidate
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (cand(mid) > v) hi = mid; else lo = mid + 1;
+      }
+      if (lo < g.nb && cand(lo) == v + 1) succ = false;
+    }
+    const uint32_t mine = (first ? 1u : 0u) + (succ ? 1u : 0u);
+    uint32_t x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    uint32_t off = 0;
+    for (int w = 0; w < warp; ++w) off += s_w[w];
+    if (tid == kSsSampleThreads - 1) s_tot = off + x;
+    __syncthreads();  // every candidate has been read: sm is rewritten below
+    const uint32_t at = off + x - mine, m = s_tot;
+    if (first) sm[at] = v;
+    if (succ) sm[at + 1] = v + 1;
+    __syncthreads();
+    const uint32_t full = 1u << lv;
+    uint64_t* tree = a.tree + (uint64_t)g.b0 * 2;
+    for (uint32_t i = 1 + tid; i < full; i += kSsSampleThreads) {
+      const uint32_t l = 31u - __clz(i), j = i - (1u << l);
+      const uint32_t at2 = (2 * j + 1) * (full >> (l + 1)) - 1;
+      tree[i] = at2 < m ? sm[at2] : ~0ull;
+    }
+    // buckets that hold one value: between neighbours that differ by one
+    for (uint32_t b = tid; b < g.nb; b += kSsSampleThreads)
+      a.eq[g.b0 + b] = b >= 1 && (b < m ? sm[b] == sm[b - 1] + 1 : b == m && sm[b - 1] == ~0ull) ? 1 : 0;
+    if (tid == 0) tree[0] = m;  // splitters: buckets 0 .. m
+    __syncthreads();
+  }
+}
+
+// kT threads take kP keys each.
+template <int kT, int kP>
+__global__ void __launch_bounds__(kT) k_ss_count(SsArgs a) {
+  constexpr uint32_t kTT = kT * kP, kSub = kTile / kTT;
+  __shared__ uint64_t s_tree[kSsMaxBuckets];
+  __shared__ uint32_t s_h[kSsMaxBuckets];
+  const uint32_t t = blockIdx.x / kSub;
+  if (a.ntiles_d && t >= *a.ntiles_d) return;
+  const SsSeg g = ss_seg(a, ss_find(a, t));
+  const uint64_t off = (uint64_t)(t - g.ft) * kTile + (uint64_t)(blockIdx.x % kSub) * kTT;
+  if (g.nb <= 1 || off >= g.n) return;
+  const uint32_t count = (uint32_t)umin64(kTT, g.n - off);
+  const uint32_t lv = ss_levels(g.nb);
+  const uint64_t* tree = a.tree + (uint64_t)g.b0 * 2;
+  for (uint32_t i = threadIdx.x; i < (1u << lv); i += kT) {
+    s_tree[i] = tree[i];
+    s_h[i] = 0;
+  }
+  const SsIn in = ss_input(a, g.s, g.start);
+  uint64_t k[kP];
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    const uint32_t x = i * kT + threadIdx.x;
+    k[i] = x < count ? in.get(off + x) : 0ull;
+  }
+  __syncthreads();
+  const uint32_t last = (uint32_t)s_tree[0];
+  uint32_t node[kP];
+#pragma unroll
+  for (int i = 0; i < kP; ++i) node[i] = 1;
+  for (uint32_t l = 0; l < lv; ++l) {
+#pragma unroll
+    for (int i = 0; i < kP; ++i) node[i] = 2 * node[i] + (k[i] >= s_tree[node[i]] ? 1u : 0u);
+  }
+  uint16_t* ids = a.ids + g.start + off;
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    const uint32_t x = i * kT + threadIdx.x;
+    if (x < count) {
+      // (a key of all ones passes the padding too)
+      const uint32_t b = min(node[i] - (1u << lv), last);
+      ids[x] = (uint16_t)b;
+      atomicAdd(&s_h[b], 1u);
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < g.nb; i += kT) {
+    const uint32_t c = s_h[i];
+    if (c) atomicAdd(&a.cnt[g.b0 + i], c);
+  }
+}
+
+template <int kT, int kP>
+constexpr size_t ss_scatter_smem() {
+  return (size_t)kT * kP * 10;
+}
+
+template <int kT, int kP, int kMinB>
+__global__ void __launch_bounds__(kT, kMinB) k_ss_scatter(SsArgs a) {
+  constexpr uint32_t kTT = kT * kP, kSub = kTile / kTT;
+  constexpr int kPer = kSsMaxBuckets / kT;  // buckets per thread
+  static_assert(kPer * kT == kSsMaxBuckets, "");
+  extern __shared__ __align__(16) uint8_t smem[];
+  uint64_t* s_keys = reinterpret_cast<uint64_t*>(smem);
+  uint16_t* s_ids = reinterpret_cast<uint16_t*>(smem + (size_t)kTT * 8);
+  __shared__ uint32_t s_h[kSsMaxBuckets];    // count, then the bucket's first slot in the tile
+  __shared__ uint32_t s_rel[kSsMaxBuckets];  // tile slot -> segment position
+  __shared__ uint64_t s_w[kT / 32];
+  const uint32_t t = blockIdx.x / kSub;
+  if (a.ntiles_d && t >= *a.ntiles_d) return;
+  const SsSeg g = ss_seg(a, ss_find(a, t));
+  const uint64_t off = (uint64_t)(t - g.ft) * kTile + (uint64_t)(blockIdx.x % kSub) * kTT;
+  if (g.nb <= 1 || off >= g.n) return;
+  const uint32_t count = (uint32_t)umin64(kTT, g.n - off);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (uint32_t i = threadIdx.x; i < kSsMaxBuckets; i += kT) s_h[i] = 0;
+  const SsIn in = ss_input(a, g.s, g.start);
+  const uint16_t* ids = a.ids + g.start + off;
+  uint64_t k[kP];
+  uint32_t r[kP];  // bucket << 16 | rank
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    const uint32_t x = i * kT + threadIdx.x;
+    r[i] = x < count ? (uint32_t)ids[x] << 16 : 0u;
+    k[i] = x < count ? in.get(off + x) : 0ull;
+  }
+  uint32_t all[kPer];  // the segment's bucket sizes
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const uint32_t b = threadIdx.x * kPer + j;
+    all[j] = b < g.nb ? a.cnt[g.b0 + b] : 0u;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kP; ++i)
+    if (i * kT + threadIdx.x < count) r[i] |= atomicAdd(&s_h[r[i] >> 16], 1u);
+  __syncthreads();
+  // exclusive prefixes of the tile's counts (low) and the segment's (high)
+  uint32_t got[kPer];
+  uint64_t run = 0;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const uint32_t b = threadIdx.x * kPer + j;
+    const uint32_t c = s_h[b];
+    // space in the bucket; the answer is not needed before the write-out
+    got[j] = c ? atomicAdd(&a.cur[g.b0 + b], c) : 0u;
+    run += (uint64_t)all[j] << 32 | c;
+  }
+  uint64_t x = run;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  uint64_t before = x - run;
+#pragma unroll
+  for (int w = 0; w < kT / 32; ++w) before += w < warp ? s_w[w] : 0ull;
+  const bool lead = t == g.ft && blockIdx.x % kSub == 0;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const uint32_t b = threadIdx.x * kPer + j, c = s_h[b];
+    s_h[b] = (uint32_t)before;
+    s_rel[b] = (uint32_t)(before >> 32) - (uint32_t)before;
+    if (lead && b < g.nb) a.bstart[g.b0 + b] = (uint32_t)(before >> 32);
+    before += (uint64_t)all[j] << 32 | c;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    if (i * kT + threadIdx.x < count) {
+      const uint32_t b = r[i] >> 16, pos = s_h[b] + (r[i] & 0xFFFFu);
+      s_keys[pos] = k[i];
+      s_ids[pos] = (uint16_t)b;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) s_rel[threadIdx.x * kPer + j] += got[j];
+  __syncthreads();
+  uint64_t* out = a.keys_split + g.start;
+#pragma unroll 4
+  for (uint32_t i = threadIdx.x; i < count; i += kT) out[s_rel[s_ids[i]] + i] = s_keys[i];
+}
+
+// ---- local sort --------------------------------------------------------------
+constexpr int kSsLT = 256;  // threads
+constexpr int kSsLP = 16;   // keys per thread
+constexpr uint32_t kSsWarpKeys = 32 * kSsLP;
+static_assert(kSsLT * kSsLP == kSsLocal, "one CTA sorts kSsLocal keys");
+// one word of padding per run of a thread keeps threads that walk their runs
+// off each other's banks
+__device__ __forceinline__ uint32_t ss_pad(uint32_t i) { return i + i / kSsLP; }
+
+__device__ __forceinline__ void ss_cx(uint64_t& x, uint64_t& y) {
+  const bool sw = x > y;
+  const uint64_t lo = sw ? y : x, hi = sw ? x : y;
+  x = lo;
+  y = hi;
+}
+
+// Batcher's odd-even merge sort of a thread's keys (Batcher 1968).
+__device__ __forceinline__ void ss_sort_run(uint64_t (&k)[kSsLP]) {
+#pragma unroll
+  for (int lp = 0; (1 << lp) < kSsLP; ++lp) {
+#pragma unroll
+    for (int lq = lp; lq >= 0; --lq) {
+      const int q = 1 << lq, j0 = lq == lp ? 0 : q;
+#pragma unroll
+      for (int i = 0; i < kSsLP; ++i) {  // i: the lower index of a comparator, if it is one
+        const int x = i - j0;
+        if (x >= 0 && (x & q) == 0 && i + q < kSsLP && (i >> (lp + 1)) == ((i + q) >> (lp + 1))) ss_cx(k[i], k[i + q]);
+      }
+    }
+  }
+}
+
+// Sort in.get(at .. at + m), 0 < m <= kSsLocal, into out[0 .. m); every
+// thread of the CTA calls it.  sm: ss_pad(kSsLocal) + 1 keys.
+__device__ __forceinline__ void ss_sort_block(const SsIn& in, uint64_t at, uint32_t m, uint64_t* out, uint64_t* sm) {
+  const uint32_t tid = threadIdx.x;
+  uint64_t k[kSsLP];
+  // any assignment of keys to threads will do: coalesced loads.  Threads
+  // 0 .. T - 1 hold a run each, missing keys all ones (sorted last).
+  const uint32_t T = (m + kSsLP - 1) / kSsLP, m16 = T * kSsLP;
+  if (tid < T) {
+#pragma unroll
+    for (int j = 0; j < kSsLP; ++j) {
+      const uint32_t i = j * T + tid;
+      k[j] = i < m ? in.get(at + i) : ~0ull;
+    }
+    ss_sort_run(k);
+#pragma unroll
+    for (int j = 0; j < kSsLP; ++j) sm[tid * (kSsLP + 1) + j] = k[j];
+  }
+  for (uint32_t R = kSsLP; R < m16; R <<= 1) {
+    const bool wide = 2 * R > kSsWarpKeys;  // a pair of runs spans warps
+    if (wide) __syncthreads(); else __syncwarp();
+    const uint32_t o = tid * kSsLP, g0 = o & ~(2 * R - 1);
+    const bool act = o < m16 && g0 + R < m16;
+    if (act) {
+      const uint32_t A = g0, B = g0 + R, na = R, nb = min(R, m16 - B), diag = o - g0;
+      uint32_t lo = diag > nb ? diag - nb : 0u, hi = diag < na ? diag : na;
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (sm[ss_pad(A + mid)] <= sm[ss_pad(B + diag - 1 - mid)]) lo = mid + 1; else hi = mid;
+      }
+      uint32_t ai = A + lo, bi = B + diag - lo;
+      const uint32_t ae = A + na, be = B + nb;
+      uint64_t ka = sm[ss_pad(min(ai, ae - 1))], kb = sm[ss_pad(min(bi, be - 1))];
+#pragma unroll
+      for (int j = 0; j < kSsLP; ++j) {
+        const bool pa = bi >= be || (ai < ae && ka <= kb);
+        k[j] = pa ? ka : kb;
+        const uint32_t nx = (pa ? ai : bi) + 1;
+        if (pa) ai = nx; else bi = nx;
+        // (one past a run's end is inside the buffer and never used)
+        const uint64_t kn = sm[ss_pad(nx)];
+        if (pa) ka = kn; else kb = kn;
+      }
+    }
+    if (wide) __syncthreads(); else __syncwarp();
+    if (act) {
+#pragma unroll
+      for (int j = 0; j < kSsLP; ++j) sm[tid * (kSsLP + 1) + j] = k[j];
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = tid; i < m; i += kSsLT) out[i] = sm[ss_pad(i)];
+  __syncthreads();  // sm may be reused
+}
+
+// How many of the first `diag` keys of merge(A, B) come from A.
+__device__ __forceinline__ uint32_t ss_merge_path(const uint64_t* A, uint32_t na, const uint64_t* B, uint32_t nb,
+                                                  uint32_t diag) {
+  uint32_t lo = diag > nb ? diag - nb : 0u, hi = diag < na ? diag : na;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (A[mid] <= B[diag - 1 - mid]) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+__global__ void __launch_bounds__(kSsLT, 4) k_ss_local(SsArgs a) {
+  __shared__ uint64_t sm[kSsLocal + kSsLocal / kSsLP + 1];
+  const uint32_t t = blockIdx.x / kSsPerTile;
+  if (a.ntiles_d && t >= *a.ntiles_d) return;
+  const SsSeg g = ss_seg(a, ss_find(a, t));
+  const uint32_t b = blockIdx.x - g.b0;
+  if (b >= g.nb || g.n == 0) return;
+  if (g.nb == 1) {  // never split: the whole segment
+    ss_sort_block(ss_input(a, g.s, g.start), 0, (uint32_t)g.n, a.keys_out + g.start, sm);
+    return;
+  }
+  const uint32_t m = a.cnt[g.b0 + b];
+  if (m == 0) return;
+  const uint64_t at = g.start + a.bstart[g.b0 + b];
+  uint64_t* from = a.keys_split + at;
+  uint64_t* to = a.keys_out + at;
+  if (a.eq[g.b0 + b]) {  // copies of one key
+    const uint64_t v = from[0];
+    for (uint32_t i = threadIdx.x; i < m; i += kSsLT) to[i] = v;
+    return;
+  }
+  SsIn in;
+  in.keys = from;
+  if (m <= kSsLocal) {
+    ss_sort_block(in, 0, m, to, sm);
+    return;
+  }
+  // A bucket the sample misjudged: kSsLocal keys at a time, then merge rounds
+  // between the two buffers, ending in keys_out.
+  int rounds = 0;
+  for (uint64_t r = kSsLocal; r < m; r <<= 1) ++rounds;
+  uint64_t* x = rounds % 2 ? from : to;
+  for (uint32_t c = 0; c < m; c += kSsLocal) ss_sort_block(in, c, min(kSsLocal, m - c), x + c, sm);
+  __syncthreads();
+  for (uint64_t R = kSsLocal; R < m; R <<= 1) {
+    uint64_t* y = x == from ? to : from;
+    for (uint64_t o = (uint64_t)threadIdx.x * kSsLP; o < m; o += (uint64_t)kSsLT * kSsLP) {
+      const uint64_t g0 = o / (2 * R) * (2 * R);
+      const uint64_t na = umin64(R, m - g0), nb = umin64(R, m - g0 - na);
+      const uint64_t *A = x + g0, *B = A + na;
+      const uint32_t diag = (uint32_t)(o - g0), end = (uint32_t)umin64(kSsLP, m - o);
+      uint32_t ai = ss_merge_path(A, (uint32_t)na, B, (uint32_t)nb, diag);
+      uint32_t bi = diag - ai;
+      for (uint32_t j = 0; j < end; ++j) {
+        const bool pa = bi >= nb || (ai < na && A[ai] <= B[bi]);
+        y[o + j] = pa ? A[ai++] : B[bi++];
+      }
+    }
+    __syncthreads();
+    x = y;
+  }
+}
+
+// The second split's segments after a first one (one CTA): every bucket of a
+// segment that was split, every other segment as it is.  seg2 arrays hold
+// their starts, lengths, parents and first tiles.
+__global__ void __launch_bounds__(1024) k_ss_plan2(SsArgs a, SsSeg2 o) {
+  __shared__ uint32_t s_w[32], s_carry;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto scan = [&](uint32_t v) -> uint32_t {  // exclusive, carried from call to call
+    uint32_t x = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
+    }
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    uint32_t off = 0, tot = 0;
+    for (int w = 0; w < 32; ++w) {
+      off += w < warp ? s_w[w] : 0u;
+      tot += s_w[w];
+    }
+    const uint32_t r = s_carry + off + x - v;
+    __syncthreads();
+    if (tid == 0) s_carry += tot;
+    __syncthreads();
+    return r;
+  };
+  if (tid == 0) s_carry = 0;
+  __syncthreads();
+  for (uint32_t s0 = 0; s0 < a.nseg; s0 += 1024) {
+    const uint32_t s = s0 + tid;
+    const bool in = s < a.nseg;
+    const SsSeg g = ss_seg(a, in ? s : 0);
+    const uint32_t at = scan(!in ? 0u : g.nb ? g.nb : 1u);
+    if (in && !g.nb) {
+      o.start[at] = g.start;
+      o.len[at] = g.n;
+      o.parent[at] = s | kSsRawBit;
+    } else if (in) {
+      for (uint32_t b = 0; b < g.nb; ++b) {
+        const uint32_t c = a.cnt[g.b0 + b];
+        o.start[at + b] = g.start + (c ? a.bstart[g.b0 + b] : 0u);
+        o.len[at + b] = c;
+        o.parent[at + b] = c && a.eq[g.b0 + b] ? kSsDone : 0u;
+      }
+    }
+  }
+  const uint32_t n2 = s_carry;
+  __syncthreads();
+  if (tid == 0) s_carry = 0;
+  __syncthreads();
+  for (uint32_t s0 = 0; s0 < n2; s0 += 1024) {
+    const uint32_t s = s0 + tid;
+    const uint32_t at = scan(s < n2 ? (uint32_t)((o.len[s] + kTile - 1) / kTile) : 0u);
+    if (s < n2) o.first_tile[s] = at;
+  }
+  if (tid == 0) {
+    o.first_tile[n2] = s_carry;
+    o.count[0] = n2;
+    o.count[1] = s_carry;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_ss_tile_seg(SsSeg2 o) {
+  const uint32_t n2 = o.count[0];
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < o.count[1]; t += gridDim.x * blockDim.x) {
+    uint32_t lo = 0, hi = n2;
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (o.first_tile[mid] <= t) lo = mid; else hi = mid;
+    }
+    o.tile_seg[t] = lo;
+  }
+}
+
+template <typename F>
+cudaError_t set_smem_once(F* f, size_t bytes, unsigned long long* done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((*done >> dev) & 1ull)) return cudaSuccess;
+  e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess && dev < 64) *done |= 1ull << dev;
+  return e;
+}
+
+}  // namespace
+
+// (r <= sqrt(n / kSsBucket) + 17 buckets of an n-key segment longer than
+// 2^18 keys: at most n / 2^13, and 1024)
+uint64_t ss_level1_buckets(uint64_t total, uint64_t nseg) {
+  const uint64_t by_len = total / (1u << 13) + 1, by_seg = nseg * kSsMaxBuckets;
+  return by_len < by_seg ? by_len : by_seg;
+}
+
+cudaError_t launch_ss_sample(const SsArgs& a0, uint64_t max_len, cudaStream_t st) {
+  if (a0.ntiles == 0 || a0.nseg == 0) return cudaSuccess;
+  static unsigned long long done = 0;
+  cudaError_t e = set_smem_once(k_ss_sample, kSsSampleMax * 8, &done);
+  if (e != cudaSuccess) return e;
+  SsArgs a = a0;
+  a.sample_max = 1024;
+  const uint64_t want = (uint64_t)umin64(kSsSampleMax, (uint64_t)umax64(1, ss_buckets(max_len, a.level1, a.one_level)) * kSsOversample);
+  while (a.sample_max < want) a.sample_max <<= 1;
+  // (nb - 1 splitters are compacted in the same buffer: sample_max >= 32 nb)
+  const uint32_t grid = a.nseg < 65536u ? a.nseg : 65536u;
+  k_ss_sample<<<grid, kSsSampleThreads, (size_t)a.sample_max * 8, st>>>(a);
+  return cudaGetLastError();
+}
+
+// Tiles below this many are cut into four: 2048 keys per CTA fill the 152
+// SMs from 2^18 keys on.
+constexpr uint32_t kSsSmallTiles = 608;
+int ss_shape(uint32_t ntiles) { return ntiles <= kSsSmallTiles ? 0 : 1; }
+
+cudaError_t launch_ss_count(const SsArgs& a, cudaStream_t st) {
+  if (a.ntiles == 0) return cudaSuccess;
+  if (ss_shape(a.ntiles) == 0) k_ss_count<256, 8><<<a.ntiles * 4, 256, 0, st>>>(a);
+  else k_ss_count<512, 8><<<a.ntiles * 2, 512, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_ss_scatter(const SsArgs& a, cudaStream_t st) {
+  if (a.ntiles == 0) return cudaSuccess;
+  if (ss_shape(a.ntiles) == 0) {
+    k_ss_scatter<256, 8, 4><<<a.ntiles * 4, 256, ss_scatter_smem<256, 8>(), st>>>(a);
+  } else {
+    static unsigned long long done = 0;
+    cudaError_t e = set_smem_once(k_ss_scatter<512, 16, 2>, ss_scatter_smem<512, 16>(), &done);
+    if (e != cudaSuccess) return e;
+    k_ss_scatter<512, 16, 2><<<a.ntiles, 512, ss_scatter_smem<512, 16>(), st>>>(a);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_ss_local(const SsArgs& a, cudaStream_t st) {
+  if (a.ntiles == 0) return cudaSuccess;
+  k_ss_local<<<a.ntiles * kSsPerTile, kSsLT, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_ss_plan2(const SsArgs& a, const SsSeg2& o, cudaStream_t st) {
+  k_ss_plan2<<<1, 1024, 0, st>>>(a, o);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_ss_tile_seg<<<512, 256, 0, st>>>(o);
+  return cudaGetLastError();
+}
+
+}  // namespace ans
