@@ -147,9 +147,8 @@ int ans_network_quantities(ans_ctx* ctx, const ans_matrix* m, ans_quantities* ou
  *                  host memory that the device addresses (cudaHostAlloc or
  *                  cudaHostRegister): the kernels then read the pairs in
  *                  place over the host link, so the host-to-device transfer
- *                  happens inside the batch, without a staging copy.  With
- *                  agg_path 3 the pairs are read exactly once (by the packet
- *                  pack); the other paths read them once or twice.
+ *                  happens inside the batch, without a staging copy.  Every
+ *                  packet sort reads the pairs twice.
  *   d_offsets    : DEVICE array of nwin + 1 nondecreasing uint64 offsets
  *                  (d_offsets[0] may be nonzero).  The batch is planned on the
  *                  device (window lengths, tile table, padded starts: one
@@ -165,8 +164,8 @@ int ans_network_quantities(ans_ctx* ctx, const ans_matrix* m, ans_quantities* ou
  *                  ans_matrix_view and ans_matrix_quantities report
  *                  ANS_ERR_INVALID_ARG.  Per-window matrices of such a batch
  *                  learn their layout when the batch completes: summing or
- *                  re-analysing them waits for it.  Every window is sorted by
- *                  the radix passes (win_path is not consulted).
+ *                  re-analysing them waits for it.  Every window takes
+ *                  the sample sort (win_path is not consulted).
  *   flags        : ANS_BATCH_* bits.
  *   out          : nwin ans_quantities (host or device memory; pageable host
  *                  memory makes the call blocking).  May be NULL.
@@ -310,28 +309,29 @@ int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
 int ans_ctx_memory(ans_ctx* ctx, size_t* live_bytes, size_t* budget_bytes);
 int ans_batch_bytes(ans_ctx* ctx, const uint64_t* h_offsets, size_t nwin, uint32_t flags, size_t* bytes);
 
-/* Launch configuration of the three families of radix passes: the 64-bit link
- * keys of window sorts (key_*), the 64-bit keys with counts of time sums
- * (kv_*), and the 32-bit destination keys of the column pass (col_*).
+/* Launch configuration of the families of radix passes -- the 64-bit keys
+ * with counts of time sums (kv_*), the 32-bit destination keys of the column
+ * pass (col_*) -- and the paths of a batch.  Packets are sorted by a sample
+ * sort without digit passes: key_* are checked and kept, and have no effect.
  * *_threads: threads per 8192-key tile, 512 or 1024.  *_rank: how lanes
  * holding equal digits find each other, 0 = one __match_any_sync per key,
  * 1 = eight ballots per key, 2 = a per-warp shared-memory table (each lane
- * ORs its bit into its digit's entry, which also carries the digit's count).  *_blocks: CTAs per SM the kernel is compiled
- * for, 1, or 2 (512 threads only: registers capped at 64).  The key passes
- * and the column passes also take 256 threads with blocks 4: every 8192-key
- * tile is split into two 4096-key sub-tiles, one CTA each, four CTAs
- * resident per SM (column passes carrying 64-bit counts then run the
- * 512-thread shape).
+ * ORs its bit into its digit's entry, which also carries the digit's count).
+ * *_blocks: CTAs per SM the kernel is compiled for, 1, or 2 (512 threads
+ * only: registers capped at 64).  key_* and col_* also take 256 threads with
+ * blocks 4: for column passes every 8192-key tile is then split into two
+ * 4096-key sub-tiles, one CTA each, four CTAs resident per SM (column passes
+ * carrying 64-bit counts then run the 512-thread shape).
  * win_path: how window keys are sorted, 0 = on chip, one 8-CTA thread-block
  * cluster per window of at most 2^17 packets sorting it in distributed shared
  * memory (larger windows, and every window when the device cannot host such
- * a cluster, take the key_* passes), 1 = the key_* passes for every window.
+ * a cluster, take the sample sort), 1 = the sample sort for every window.
  * win_threads (512 or 1024) and win_rank (0 or 1, as *_rank) configure the
  * cluster kernel.  sum_path: how time sums order the links of their input matrices,
  * 0 = ceil(log2 k) rounds of pairwise merges of the matrices' already sorted
  * links, 1 = the kv_* radix passes over all gathered links, 2 = (a batch's
  * own time sum, windows stored back to back) every packet of the batch
- * sorted again as one segment by the key_* passes and reduced like a window
+ * sorted again as one segment and reduced like a window
  * -- the sum of Table I's A_t is the matrix of the concatenated packets;
  * batches of windows in their own arrays then take the kv_* passes, and sums
  * of k given matrices merge them (k <= 256) or take the kv_* passes.  agg_path: how
@@ -346,13 +346,8 @@ int ans_batch_bytes(ans_ctx* ctx, const uint64_t* h_offsets, size_t nwin, uint32
  * distinct links grouped by source and by destination, one table of 16384
  * keys per partition -- with no sort; a window whose table overflows, or of
  * more than 2^18 packets, is sorted instead (other batches sort as agg_path 0);
- * 3 = for batches with a time sum, 2 to 2^16 windows and the packets in one
- * stream: no window sort -- the time sum always comes from the batch's
- * packets sorted as one segment (sum_path 2's sort), each packet carrying
- * its 16-bit window id through the key_* passes, and a stable sort of the
- * sorted packets by window id (two digit passes, the second writing each
- * window at its padded base) leaves every window's packets in key order,
- * as the window sort would (other batches sort as agg_path 0).  Setting
+ * 3 = as agg_path 0, and for batches with a time sum, 2 to 2^16 windows and
+ * the packets in one stream the sum takes sum_path 2.  Setting
  * agg_path 0 waits for the device and releases the tables.  graph: 1 = a batch's launch sequence is recorded into a CUDA
  * graph and replayed through a cached executable graph of the same shape
  * (updated in place with the call's pointers), 0 = launched directly; per-
@@ -391,7 +386,7 @@ int ans_set_tuning(ans_ctx* ctx, const ans_tuning* tuning);
  * every pass family runs), and keeps, per family, the configuration with the
  * least total pass time; it then times the on-chip window sort (win_path 0,
  * three cluster configurations) and keeps it if the batch's windows sort
- * faster that way than by the best key passes plus their histogram sweep, and
+ * faster that way than by the sample sort, and
  * finally picks sum_path, merge_tile (with merge rounds), then agg_path (2
  * only without ANS_BATCH_MATRICES in `flags`, together with sum_path 2 when
  * the batch has a time sum; 3 only with ANS_BATCH_SUM and 2 to 2^16
@@ -399,8 +394,8 @@ int ans_set_tuning(ans_ctx* ctx, const ans_tuning* tuning);
  * `flags` (ANS_BATCH_* bits of the batches the context will run; one CUDA
  * graph with its concurrent branches, between CUDA events on `stream`, the
  * host's planning included).  With those paths fixed, it last retries the
- * column passes' shape (when the chosen paths run column passes) and, with
- * agg_path 3, the key passes' ranking mode, by the same device time.  An
+ * column passes' shape (when the chosen paths run column passes) by the same
+ * device time; key_* stay as they are.  An
  * optional path whose trial cannot get its
  * device memory (ANS_ERR_OOM / ANS_ERR_BUDGET) is skipped; the call fails
  * with ANS_ERR_OOM only if the default paths do not fit.  The choice is
