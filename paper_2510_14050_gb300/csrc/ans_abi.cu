@@ -713,6 +713,8 @@ struct DevPlan {
 struct PipeScratch {
   size_t keys_a, keys_b, vals_a, vals_b, seg_hist, st0, st1, lb, lb2, tickets, run_start, row_pos, pre;
   size_t ck_a, ck_b, cv_a, cv_b, col_hist, ulen, bnd;
+  size_t cp_cnt, cp_cur, cp_start, cp_hkey, cp_hsum;  // hash partitions of the links by destination
+  uint32_t cp_entries = 0;
   // hash-group column statistics of a time sum (buffers for up to
   // hgroup_links links, when reserved)
   size_t hbnd = 0, hitem = 0, hpart = 0, hheavy = 0, hmeta = 0, hcnt = 0, hbuf = 0, hacc = 0;
@@ -726,6 +728,12 @@ struct PipeScratch {
     col_hist = L.add((size_t)nseg * kColPasses * kRadix * 4);
     ulen = L.add((size_t)nseg * 8);
     bnd = L.add((size_t)ntiles * sizeof(ColBnd));
+    cp_entries = kColPerTile * ntiles;
+    cp_cnt = L.add((size_t)cp_entries * 4);
+    cp_cur = L.add((size_t)cp_entries * 4);
+    cp_start = L.add((size_t)cp_entries * 4);
+    cp_hkey = L.add((size_t)ntiles * kColHeavyPerTile * 4);
+    cp_hsum = L.add((size_t)ntiles * kColHeavyPerTile * 16);
     if (with_vals && pad >= kHGroupMinLinks) {
       hgroup_links = pad;
       hgroup_cap = (uint32_t)(2 * (pad / kHGroupPartLinks) + 1);
@@ -868,21 +876,61 @@ int sample_sort(ans_ctx* c, char* m, const SsScratch& ss, const SegPlan& p, cons
   return ANS_OK;
 }
 
-// Column statistics of the segments of `p` (the transpose-free column pass):
-// the stored links (col_ids, vals) are sorted by destination in four 8-bit
+// The segments whose links are grouped by hash partitions for the column
+// statistics: of at most 2^25 links (max_len bounds them; known: on the host).
+// Longer ones would meet more than kColMaxParts partitions' worth of
+// destinations and be read in several classes (a batch planned on the device
+// may hold such windows; the result stays exact).  With `narrow` counts, one
+// segment of 2^24 links or more takes the hash groups instead.
+bool col_parts_ok(const ans_ctx* c, uint64_t max_len, bool known = true) {
+  return c->col_hash && (!known || max_len <= (1ull << 25));
+}
+// Their partition counts cleared and their heavy destinations listed, between
+// the run reduction (a->hdr, a->col_ids) and k_finish over the plan `p`.
+int col_parts_begin(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& p, uint64_t max_len, StatsArgs* a,
+                    cudaStream_t st) {
+  a->cp.cnt = at<uint32_t>(m, ps.cp_cnt);
+  a->cp.cur = at<uint32_t>(m, ps.cp_cur);
+  a->cp.start = at<uint32_t>(m, ps.cp_start);
+  a->cp.max_parts = col_parts(max_len, std::min<uint64_t>(kColMaxParts, (uint64_t)kColPerTile * p.ntiles));
+  ANS_CUDA(launch_zero(a->cp.cnt, (size_t)kColPerTile * p.ntiles * 4, st));
+  ANS_CUDA(launch_zero(a->cp.cur, (size_t)kColPerTile * p.ntiles * 4, st));
+  a->cp.hkey = at<uint32_t>(m, ps.cp_hkey);
+  a->cp.hsum = at<unsigned long long>(m, ps.cp_hsum);
+  if (max_len >= kColHeavyLinks) {
+    ANS_CUDA(launch_zero(a->cp.hsum, (size_t)kColHeavyPerTile * p.ntiles * 16, st));
+    ANS_CUDA(timed(c, "col_heavy", st, [&] { return launch_col_heavy(p, a->cp, a->col_ids, a->hdr, st); }));
+  }
+  return ANS_OK;
+}
+
+// Column statistics of the segments of a.plan after k_finish: by hash
+// partitions (a.cp), or by the transpose-free column sort: the stored links
+// (a.col_ids, a.vals) are sorted by destination in four 8-bit
 // passes (in -> A -> B -> A -> B) and the destination runs reduced.  Expects
 // k_finish to have filled col_hist and ulen and zeroed st0 and the tickets.
-// With vals32 (window matrices, whose counts fit 31 bits; k_finish wrote the
-// copy into the value buffer B) the passes carry uint32 counts.  With hkeys
+// With a.vals32 (counts below 2^32; k_finish wrote the copy into the value
+// buffer B) the passes carry uint32 counts.  With a.col_hkeys
 // (one segment, vals32: k_finish wrote the mixed destinations there and
 // counted their bytes), the passes sort the mixed destinations, and after
 // the first two the hash groups are counted (launch_hgroup_stats); if they
 // all fit, the segment's length drops to 0 and the rest finds no work.
-int column_pass(ans_ctx* c, const SegPlan& p, uint64_t* ulen, const uint32_t* col_ids,
-                const uint64_t* vals, const PipeScratch& ps, char* m, uint32_t* tickets,
-                ans_quantities* q, cudaStream_t st, bool vals32 = false, const uint32_t* hkeys = nullptr) {
+int column_pass(ans_ctx* c, const StatsArgs& a, const PipeScratch& ps, char* m, ans_quantities* q, cudaStream_t st) {
+  const SegPlan& p = a.plan;
+  uint64_t* ulen = a.ulen;
+  const uint32_t* col_ids = a.col_ids;
+  const uint64_t* vals = a.vals;
+  const bool vals32 = a.vals32 != nullptr;
+  const uint32_t* hkeys = a.col_hkeys;
+  uint32_t* tickets = a.col_tickets;
   SegPlan cp = p;
   cp.len = ulen;
+  if (a.cp.cnt) {
+    ANS_CUDA(timed(c, "cols", st, [&] {
+      return launch_cols(cp, a.cp, col_ids, a.vals32, a.vals, at<uint32_t>(m, ps.ck_a), at<uint64_t>(m, ps.cv_a), q, st);
+    }));
+    return ANS_OK;
+  }
   uint32_t* ka = at<uint32_t>(m, ps.ck_a);
   uint32_t* kb = at<uint32_t>(m, ps.ck_b);
   uint64_t* va = at<uint64_t>(m, ps.cv_a);
@@ -1118,8 +1166,10 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
   if (hgroup_ok(c, s, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
   if ((e = launch_zero(blk->q, sizeof(ans_quantities), st)) != cudaSuccess) return fail_blk(e, "memset");
   if ((e = timed(c, "rle", st, [&] { return launch_rle(a, st); })) != cudaSuccess) return fail_blk(e, "rle");
+  if (!a.col_hkeys && col_parts_ok(c, (uint64_t)s.ntiles * kTile))
+    ANS_TRY(col_parts_begin(c, m, ps, s, (uint64_t)s.ntiles * kTile, &a, st));
   if ((e = timed(c, "finish", st, [&] { return launch_finish(a, st); })) != cudaSuccess) return fail_blk(e, "finish");
-  return column_pass(c, s, a.ulen, blk->col_ids, blk->vals, ps, m, col_tickets, blk->q, st, narrow, a.col_hkeys);
+  return column_pass(c, a, ps, m, blk->q, st);
 }
 
 // Time sum of a batch from its packets (sum_path 2): every packet of the
@@ -1166,9 +1216,9 @@ int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, c
   a.mode = kModeWindow;
   if (hgroup_ok(c, pk, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
   if ((rc = cu(timed(c, "rle", st, [&] { return launch_rle(a, st); }), "rle"))) return rc;
+  if (!a.col_hkeys && col_parts_ok(c, total)) ANS_TRY(col_parts_begin(c, m, ps, pk, total, &a, st));
   if ((rc = cu(timed(c, "finish", st, [&] { return launch_finish(a, st); }), "finish"))) return rc;
-  return column_pass(c, pk, a.ulen, blk->col_ids, blk->vals, ps, m, a.col_tickets, blk->q, st, narrow,
-                     a.col_hkeys);
+  return column_pass(c, a, ps, m, blk->q, st);
 }
 
 // Snapshot the device error word into `dst` (device); reset_err clears it.
@@ -1302,9 +1352,6 @@ bool agg_packets(const ans_ctx* c, uint32_t nseg, bool want_sum, bool addrs) {
 struct WinLayout {
   DevPlan dp, dp_big;  // every window; the windows sorted by onesweep passes
   size_t off_small = 0;  // ids of the windows sorted on chip
-  size_t off_colacc = 0; // per-window accumulators of the partitioned column hash
-  size_t off_colpart = 0; // its partition starts per window
-  size_t off_colitems = 0; // its (window, partition) work items
   size_t off_tileseg = 0; // the window plan's segment of every tile
   size_t off_hqwin = 0, off_lstart = 0, off_kstart = 0, off_sortlen = 0, off_items = 0;  // hashed window statistics
   DevPlan dp_tab;        // hash path: the windows' tables as segments
@@ -1325,9 +1372,6 @@ struct WinLayout {
     dp.reserve(L, nseg, addrs);
     dp_big.reserve(L, nseg, addrs);
     off_small = L.add((size_t)nseg * 4);
-    off_colacc = L.add(((size_t)nseg + 1) * sizeof(ColPartAcc));
-    off_colpart = L.add((size_t)nseg * 33 * 4);
-    off_colitems = L.add((size_t)nseg * 32 * 4);
     off_tileseg = L.add((size_t)hp.ntiles * 4);
     off_hqwin = L.add((size_t)nseg * sizeof(HqWin));
     off_lstart = L.add((size_t)nseg * 65 * 4);
@@ -1730,6 +1774,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       if (in_place) a.sum_keys = kb;
       if ((rc = cu(timed(c, "empty_fixup", ls, [&] { return launch_empty_fixup(a, ls); }), "empty"))) return rc;
       if ((rc = cu(timed(c, "rle", ls, [&] { return launch_rle(a, ls); }), "rle"))) return rc;
+      if (col_parts_ok(c, max_len, !dev) && (rc = col_parts_begin(c, m, ps, pw, max_len, &a, ls))) return rc;
       if ((rc = cu(timed(c, "finish", ls, [&] { return launch_finish(a, ls); }), "finish"))) return rc;
       if (in_place) {
         if ((rc = cu(cudaEventRecord(c->ev_fork, ls), "event")) ||
@@ -1741,23 +1786,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
         const cudaError_t ej = cudaEventRecord(c->ev_join, c->side);
         if (rc == ANS_OK) rc = cu(ej, "event");
       }
-      if (rc == ANS_OK && c->col_hash)
-        rc = cu(timed(c, "colhash", ls, [&] { return launch_colhash(pw, a.ulen, sb.col_ids, a.vals32, sb.q, ls); }),
-                "colhash");
-      if (rc == ANS_OK && c->col_hash) {  // windows with more destinations than one table holds
-        ColPartAcc* acc = at<ColPartAcc>(m, wl.off_colacc);
-        rc = cu(launch_zero(acc, ((size_t)nseg + 1) * sizeof(ColPartAcc), ls), "memset");
-        if (rc == ANS_OK)
-          rc = cu(timed(c, "colhash_part", ls,
-                        [&] {  // links regrouped into the column sort's buffers, which it overwrites later
-                          return launch_colhash_part(pw, a.ulen, sb.col_ids, a.vals32, at<uint32_t>(m, ps.ck_a),
-                                                     (uint32_t*)at<uint64_t>(m, ps.cv_a),
-                                                     at<uint32_t>(m, wl.off_colpart), acc,
-                                                     at<uint32_t>(m, wl.off_colitems), sb.q, ls);
-                        }),
-                  "colhash part");
-      }
-      if (rc == ANS_OK) rc = column_pass(c, pw, a.ulen, sb.col_ids, sb.vals, ps, m, a.col_tickets, sb.q, ls, true);
+      if (rc == ANS_OK) rc = column_pass(c, a, ps, m, sb.q, ls);
       if (rc == ANS_OK && hq)  // the hashed windows' quantities over the (empty) sorted results
         rc = cu(launch_hq_write(p, at<HqWin>(m, wl.off_hqwin), sb.q, ls), "hash statistics");
       if (forked) {  // join (also after a failure, so that a capture ends joined)
@@ -1789,12 +1818,17 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   };
   int rounds = 0;
   while ((1ull << rounds) < nseg) ++rounds;
-  // the column hash's cluster shape changes with the window count: a cached
-  // graph must not be updated to another one
+  // (what else decides the kernels: one or two splits, the sort's launch
+  // shapes, which column statistics, and theirs)
+  const uint64_t pk_tiles = tiles_for(total);
   const std::string sig = launch_sig(flags, hp.ntiles > 0, !small_ids.empty(), !big_ids.empty(), rounds, c) + "/h" +
-                          std::to_string(c->col_hash && nseg ? colhash_ctas(nseg) : 0u) + (dev ? "/d" : "") + "/s" +
+                          std::to_string(col_parts_ok(c, max_len, !dev)) + std::to_string(col_parts_ok(c, total)) +
+                          std::to_string(max_len > kColPart) + std::to_string(total > kColPart) +
+                          std::to_string(max_len >= kColHeavyLinks) + std::to_string(total >= kColHeavyLinks) +
+                          std::to_string(pk_tiles >= kHGroupMinLinks / kTile) + (dev ? "/d" : "") + "/s" +
                           std::to_string(wl.ss_two_win) + std::to_string(wl.ss_two_pk) +
-                          std::to_string(ss_shape(hp.ntiles)) + std::to_string(ss_shape(wl.ss.ntiles2));
+                          std::to_string(ss_shape(hp.ntiles)) + std::to_string(ss_shape(wl.ss.ntiles2)) +
+                          std::to_string(ss_shape((uint32_t)pk_tiles));
   if ((rc = run_launches(c, st, sig, launch_all))) return bail(rc);
   if (sump.blk) {  // the time sum's block is filled
     sblk = sump.blk;
@@ -1884,8 +1918,9 @@ int matrix_stats(ans_ctx* c, const Block* b, uint32_t seg, ans_quantities* q_out
     a.col_tickets = tickets + 32;
     a.err = c->d_err;
     a.mode = kModeMatrix;
+    if (col_parts_ok(c, cap)) ANS_TRY(col_parts_begin(c, m, ps, p, cap, &a, st));
     ANS_CUDA(timed(c, "finish", st, [&] { return launch_finish(a, st); }));
-    ANS_TRY(column_pass(c, p, a.ulen, a.col_ids, a.vals, ps, m, a.col_tickets, q, st));
+    ANS_TRY(column_pass(c, a, ps, m, q, st));
   }
   return copy_quantities_out(q_out, q, 1, st);
 }

@@ -1,0 +1,398 @@
+// Column statistics of stored links by hash partitions of their destinations
+// (Table I: unique destinations, max fan-in; Sec. IV-C: max destination
+// packets).
+//
+// The three quantities only need equal destinations together, in any order.
+// h = fmix32(destination) is a bijection; a segment of n links is cut into
+// about n / kColPart partitions by the high bits of h.  k_finish, which reads
+// every link anyway, counts the partitions; then
+//   scatter  moves (destination, count) to its partition, ranks by one
+//            shared-memory atomic per link, space by one global atomic per
+//            partition and tile -- no order to keep, no look-back;
+//   count    one CTA per partition counts its destinations in a shared-memory
+//            table and adds the table's three quantities to the segment's.
+// A partition with more destinations than the table holds is read again in
+// 2, 4, ... classes by another mix of the destination, so every input ends
+// here and no sort stands behind.
+//
+// A destination with a large share of the links would make one partition, and
+// one table slot, a queue.  In segments of kColHeavyLinks links or more those
+// with 8 or more of 2048 sampled links are listed first (k_col_heavy) and
+// added up by k_finish (a sum of 4.6 million links of bursty traffic: 127
+// against 381 us).  Shorter segments do without: listing costs 20 us a launch
+// and every link of k_finish a probe, and adding equal destinations of a warp
+// once (__match_any_sync) makes one window of 2^17 packets 47 instead of 24.5 us.
+//
+// The column sorts and the one-CTA-per-window hashes that this replaces took
+// 174 us for that window (24.5 now), 448 us for 64 windows and their sum.
+#include "ans_internal.cuh"
+
+namespace ans {
+
+namespace {
+
+constexpr uint32_t kColSlots = 4096;               // table slots of one CTA
+constexpr uint32_t kColFill = kColSlots / 8 * 7;   // give up above this
+constexpr uint32_t kColNone = 0xFFFFFFFFu;         // empty slot (that destination is counted apart)
+constexpr int kColThreads = 256;
+
+constexpr uint32_t kColSample = 2048;
+constexpr int kColHeavyThreads = 512;
+constexpr uint32_t kColHeavyMin = 8;    // sampled links of a heavy destination
+constexpr uint32_t kColHeavyMost = 48;  // destinations listed
+
+// One CTA per segment: its heavy destinations, as a table of 64 slots
+// (kColNone: empty).
+__global__ void __launch_bounds__(kColHeavyThreads) k_col_heavy(SegPlan p, ColParts c, const uint32_t* __restrict__ col_ids,
+                                                           const uint64_t* __restrict__ hdr) {
+  __shared__ uint32_t t_key[2 * kColSample], t_cnt[2 * kColSample];
+  __shared__ uint32_t s_key[kColHeavySlots], s_n[16];
+  const uint32_t s = blockIdx.x;
+  if (s >= p.nseg) return;
+  const uint64_t n = hdr[2 * (uint64_t)s + 1];
+  if (n < kColHeavyLinks) return;
+  const uint32_t* d0 = col_ids + p.base[s];
+  for (uint32_t i = threadIdx.x; i < 2 * kColSample; i += kColHeavyThreads) {
+    t_key[i] = kColNone;
+    t_cnt[i] = 0;
+  }
+  if (threadIdx.x < kColHeavySlots) s_key[threadIdx.x] = kColNone;
+  if (threadIdx.x < 16) s_n[threadIdx.x] = 0;
+  __syncthreads();
+  for (uint32_t j = threadIdx.x; j < kColSample; j += kColHeavyThreads) {  // one link of each stretch
+    const uint32_t d = d0[(((uint64_t)j << 16 | (fmix32(j + 1) & 0xFFFFu)) * n) / ((uint64_t)kColSample << 16)];
+    if (d == kColNone) continue;  // (the count has a place of its own for it)
+    uint32_t i = fmix32(d) & (2 * kColSample - 1);
+    for (;;) {  // at most half of the slots are taken
+      const uint32_t cur = atomicCAS(&t_key[i], kColNone, d);
+      if (cur == kColNone || cur == d) break;
+      i = (i + 1) & (2 * kColSample - 1);
+    }
+    atomicAdd(&t_cnt[i], 1u);
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < 2 * kColSample; i += kColHeavyThreads)
+    if (t_cnt[i] >= kColHeavyMin) atomicAdd(&s_n[31 - __clz(t_cnt[i])], 1u);
+  __syncthreads();
+  uint32_t lg = 15, most = 0;  // the lowest power of two that lists at most kColHeavyMost
+  while (lg > 3 && most + s_n[lg - 1] <= kColHeavyMost) most += s_n[--lg];
+  for (uint32_t i = threadIdx.x; i < 2 * kColSample; i += kColHeavyThreads) {
+    if (t_cnt[i] < (1u << lg)) continue;
+    uint32_t j = fmix32(t_key[i]) & (kColHeavySlots - 1);
+    while (atomicCAS(&s_key[j], kColNone, t_key[i]) != kColNone) j = (j + 1) & (kColHeavySlots - 1);
+  }
+  __syncthreads();
+  if (threadIdx.x < kColHeavySlots) c.hkey[(uint64_t)p.first_tile[s] * kColHeavyPerTile + threadIdx.x] = s_key[threadIdx.x];
+}
+static_assert(1u << 3 == kColHeavyMin, "the lowest count listed");
+
+struct ColSeg {
+  uint32_t ft, parts;
+  uint64_t n;
+};
+__device__ __forceinline__ ColSeg col_seg(const SegPlan& p, uint32_t s, uint32_t max_parts) {
+  ColSeg g;
+  g.ft = p.first_tile[s];
+  g.n = p.len[s];
+  g.parts = col_parts(g.n, max_parts);
+  return g;
+}
+
+// One sub-tile of kT * kP links per CTA.  kWide: 64-bit counts.
+template <bool kWide, int kT, int kP>
+__global__ void __launch_bounds__(kT) k_col_scatter(SegPlan p, ColParts c, const uint32_t* __restrict__ col_ids,
+                                                    const uint32_t* __restrict__ vals32,
+                                                    const uint64_t* __restrict__ vals64, uint32_t* __restrict__ odst,
+                                                    void* __restrict__ oval) {
+  using V = typename std::conditional<kWide, uint64_t, uint32_t>::type;
+  constexpr uint32_t kTT = kT * kP, kSub = kTile / kTT;
+  extern __shared__ __align__(16) uint8_t smem[];
+  V* s_val = reinterpret_cast<V*>(smem);
+  uint32_t* s_dst = reinterpret_cast<uint32_t*>(smem + (size_t)kTT * sizeof(V));
+  uint32_t* s_h = s_dst + kTT;  // [parts] count, then the partition's first slot in the tile
+  uint32_t* s_rel = s_h + c.max_parts;  // [parts] tile slot -> segment position
+  __shared__ uint64_t s_w[kT / 32];
+  __shared__ uint32_t s_hkey[kColHeavySlots];
+  const uint32_t t = blockIdx.x / kSub;
+  const uint32_t s = find_seg(p, t);
+  const ColSeg g = col_seg(p, s, c.max_parts);
+  const uint64_t off = (uint64_t)(t - g.ft) * kTile + (uint64_t)(blockIdx.x % kSub) * kTT;
+  if (g.parts <= 1 || off >= g.n) return;
+  const uint32_t count = (uint32_t)umin64(kTT, g.n - off);
+  const uint64_t base = p.base[s];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const V* vin = kWide ? (const V*)vals64 : (const V*)vals32;
+  uint32_t d[kP], r[kP];
+  V v[kP];
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    const uint32_t x = i * kT + threadIdx.x;
+    d[i] = x < count ? col_ids[base + off + x] : 0u;
+    v[i] = x < count ? vin[base + off + x] : V(0);
+  }
+  for (uint32_t b = threadIdx.x; b < g.parts; b += kT) s_h[b] = 0;
+  const bool heavy = g.n >= kColHeavyLinks;
+  if (heavy && threadIdx.x < kColHeavySlots) s_hkey[threadIdx.x] = c.hkey[(size_t)g.ft * kColHeavyPerTile + threadIdx.x];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    r[i] = kColNone;  // past the end, or a heavy destination's: not moved
+    if (i * kT + threadIdx.x < count && !(heavy && col_heavy(s_hkey, d[i]) >= 0)) {
+      const uint32_t b = col_part(d[i], g.parts);
+      r[i] = b << 16 | atomicAdd(&s_h[b], 1u);
+    }
+  }
+  __syncthreads();
+  // exclusive prefixes of the tile's counts (low) and the segment's (high);
+  // consecutive partitions per thread
+  const uint32_t* cnt = c.cnt + (size_t)g.ft * kColPerTile;
+  uint32_t* cur = c.cur + (size_t)g.ft * kColPerTile;
+  const uint32_t per = (g.parts + kT - 1) / kT;
+  const uint32_t b0 = min(threadIdx.x * per, g.parts), b1 = min(b0 + per, g.parts);
+  uint64_t run = 0;
+  for (uint32_t b = b0; b < b1; ++b) run += (uint64_t)cnt[b] << 32 | s_h[b];
+  uint64_t x = run;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  uint64_t before = x - run;
+  uint32_t moved = 0;
+#pragma unroll
+  for (int w = 0; w < kT / 32; ++w) {
+    before += w < warp ? s_w[w] : 0ull;
+    moved += (uint32_t)s_w[w];
+  }
+  const bool lead = off == 0;
+  for (uint32_t b = b0; b < b1; ++b) {
+    const uint32_t k = s_h[b], slot = (uint32_t)before, start = (uint32_t)(before >> 32);
+    const uint32_t got = k ? atomicAdd(&cur[b], k) : 0u;
+    s_h[b] = slot;
+    s_rel[b] = start + got - slot;
+    if (lead) c.start[(size_t)g.ft * kColPerTile + b] = start;
+    before += (uint64_t)cnt[b] << 32 | k;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kP; ++i) {
+    if (r[i] != kColNone) {
+      const uint32_t pos = s_h[r[i] >> 16] + (r[i] & 0xFFFFu);
+      s_dst[pos] = d[i];
+      s_val[pos] = v[i];
+    }
+  }
+  __syncthreads();
+  V* ov = reinterpret_cast<V*>(oval) + base;
+#pragma unroll 4
+  for (uint32_t i = threadIdx.x; i < moved; i += kT) {
+    const uint32_t k = s_dst[i], o = s_rel[col_part(k, g.parts)] + i;
+    odst[base + o] = k;
+    ov[o] = s_val[i];
+  }
+}
+
+// One partition per CTA (one that was never split is the whole segment).
+template <bool kWide>
+__global__ void __launch_bounds__(kColThreads) k_col_count(SegPlan p, ColParts c, const uint32_t* __restrict__ col_ids,
+                                                           const uint32_t* __restrict__ vals32,
+                                                           const uint64_t* __restrict__ vals64,
+                                                           const uint32_t* __restrict__ pdst,
+                                                           const void* __restrict__ pval,
+                                                           ans_quantities* __restrict__ q) {
+  using V = typename std::conditional<kWide, uint64_t, uint32_t>::type;
+  extern __shared__ __align__(16) uint32_t t_key[];
+  uint32_t* t_cnt = t_key + kColSlots;
+  uint32_t* t_lo = t_cnt + kColSlots;
+  uint32_t* t_hi = t_lo + kColSlots;  // kWide only
+  __shared__ uint32_t s_fill, s_over, s_spec_cnt, s_spec_lo, s_spec_hi;
+  __shared__ unsigned long long s_red[3][kColThreads / 32];
+  const uint32_t t = blockIdx.x / kColPerTile;
+  const uint32_t s = find_seg(p, t);
+  const ColSeg g = col_seg(p, s, c.max_parts);
+  const uint32_t b = blockIdx.x - g.ft * kColPerTile;
+  if (b >= g.parts || g.n == 0) return;
+  const uint64_t base = p.base[s];
+  const uint32_t* kd = col_ids + base;
+  const V* vd = (kWide ? (const V*)vals64 : (const V*)vals32) + base;
+  uint64_t m = g.n;
+  if (g.parts > 1) {
+    const uint32_t at = c.start[blockIdx.x];
+    m = c.cnt[blockIdx.x];
+    kd = pdst + base + at;
+    vd = reinterpret_cast<const V*>(pval) + base + at;
+  }
+  const bool heavy = b == 0 && g.n >= kColHeavyLinks;  // this CTA adds the heavy destinations
+  if (m == 0 && !heavy) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t slots = 256;
+  while (slots < m + m / 2 && slots < kColSlots) slots <<= 1;
+  auto add = [&](uint32_t* lo, uint32_t* hi, V x) {
+    if constexpr (kWide) add64_shared(lo, hi, x);
+    else atomicAdd(lo, x);
+  };
+  auto sum_of = [&](uint32_t lo, const uint32_t* hi) -> uint64_t { return kWide ? (uint64_t)*hi << 32 | lo : lo; };
+  unsigned long long uniq = 0, mfan = 0, mpk = 0;
+  for (uint32_t R = 1, cls = 0; cls < R;) {
+    for (uint32_t i = threadIdx.x; i < slots; i += kColThreads) {
+      t_key[i] = kColNone;
+      t_cnt[i] = 0;
+      t_lo[i] = 0;
+      if (kWide) t_hi[i] = 0;
+    }
+    if (threadIdx.x == 0) s_fill = s_over = s_spec_cnt = s_spec_lo = s_spec_hi = 0;
+    __syncthreads();
+    constexpr int kU = 4;  // links per thread in flight
+    for (uint64_t u0 = 0; u0 < m; u0 += (uint64_t)kU * kColThreads) {
+      if (*(volatile uint32_t*)&s_over) break;
+      uint32_t d[kU];
+      V v[kU];
+#pragma unroll
+      for (int k = 0; k < kU; ++k) {
+        const uint64_t u = u0 + (uint64_t)k * kColThreads + threadIdx.x;
+        d[k] = u < m ? kd[u] : 0u;
+        v[k] = u < m ? vd[u] : V(0);
+      }
+#pragma unroll
+      for (int k = 0; k < kU; ++k) {
+        if (u0 + (uint64_t)k * kColThreads + threadIdx.x >= m) continue;
+        if (d[k] == kColNone) {
+          if (cls == 0) {
+            atomicAdd(&s_spec_cnt, 1u);
+            add(&s_spec_lo, &s_spec_hi, v[k]);
+          }
+          continue;
+        }
+        const uint32_t h = fmix32(d[k]);
+        if (R > 1 && (fmix32(h ^ 0x9E3779B9u) & (R - 1)) != cls) continue;
+        uint32_t i = h & (slots - 1);
+        for (uint32_t probe = 0; probe < slots; ++probe) {
+          uint32_t cur = *(volatile uint32_t*)&t_key[i];
+          if (cur == kColNone) {
+            cur = atomicCAS(&t_key[i], kColNone, d[k]);
+            if (cur == kColNone) {
+              cur = d[k];
+              if (atomicAdd(&s_fill, 1u) >= kColFill) s_over = 1;
+            }
+          }
+          if (cur == d[k]) {
+            atomicAdd(&t_cnt[i], 1u);
+            add(&t_lo[i], &t_hi[i], v[k]);
+            break;
+          }
+          i = (i + 1) & (slots - 1);
+        }
+      }
+    }
+    __syncthreads();
+    if (s_over) {  // more destinations than the table takes: twice the classes, from the start
+      R <<= 1;
+      cls = 0;
+      uniq = mfan = mpk = 0;
+      __syncthreads();
+      continue;
+    }
+    for (uint32_t i = threadIdx.x; i < slots; i += kColThreads) {
+      if (t_key[i] != kColNone) {
+        ++uniq;
+        mfan = umax64(mfan, t_cnt[i]);
+        mpk = umax64(mpk, sum_of(t_lo[i], &t_hi[i]));
+      }
+    }
+    if (threadIdx.x == 0 && s_spec_cnt) {
+      ++uniq;
+      mfan = umax64(mfan, s_spec_cnt);
+      mpk = umax64(mpk, sum_of(s_spec_lo, &s_spec_hi));
+    }
+    ++cls;
+    __syncthreads();  // the table is cleared for the next class
+  }
+  if (heavy && threadIdx.x < kColHeavySlots) {
+    const size_t at = (size_t)g.ft * kColHeavyPerTile + threadIdx.x;
+    const unsigned long long f = c.hsum[2 * at];
+    if (f) {
+      ++uniq;
+      mfan = umax64(mfan, f);
+      mpk = umax64(mpk, c.hsum[2 * at + 1]);
+    }
+  }
+  uniq = warp_sum(uniq);
+  mfan = warp_max(mfan);
+  mpk = warp_max(mpk);
+  if (lane == 0) {
+    s_red[0][warp] = uniq;
+    s_red[1][warp] = mfan;
+    s_red[2][warp] = mpk;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kColThreads / 32; ++w) {
+      uniq += s_red[0][w];
+      mfan = umax64(mfan, s_red[1][w]);
+      mpk = umax64(mpk, s_red[2][w]);
+    }
+    atomicAdd((unsigned long long*)&q[s].unique_destinations, uniq);
+    atomicMax((unsigned long long*)&q[s].max_destination_fanin, mfan);
+    atomicMax((unsigned long long*)&q[s].max_destination_packets, mpk);
+  }
+}
+
+template <typename F>
+cudaError_t set_smem_once(F* f, size_t bytes, unsigned long long* done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((*done >> dev) & 1ull)) return cudaSuccess;
+  e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e == cudaSuccess && dev < 64) *done |= 1ull << dev;
+  return e;
+}
+
+template <bool kWide, int kT, int kP>
+cudaError_t scatter(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                    const uint64_t* vals64, uint32_t* odst, void* oval, cudaStream_t st) {
+  constexpr size_t kItems = (size_t)kT * kP * (kWide ? 12 : 8);
+  static unsigned long long done = 0;
+  const cudaError_t e = set_smem_once(k_col_scatter<kWide, kT, kP>, kItems + (size_t)kColMaxParts * 8, &done);
+  if (e != cudaSuccess) return e;
+  k_col_scatter<kWide, kT, kP><<<p.ntiles * (kTile / (kT * kP)), kT, kItems + (size_t)c.max_parts * 8, st>>>(
+      p, c, col_ids, vals32, vals64, odst, oval);
+  return cudaGetLastError();
+}
+
+template <bool kWide>
+cudaError_t run_cols(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                     const uint64_t* vals64, uint32_t* odst, void* oval, ans_quantities* q, cudaStream_t st) {
+  cudaError_t e;
+  if (c.max_parts > 1) {
+    // (small plans: 2048 links per CTA fill the SMs sooner)
+    e = p.ntiles <= 608 ? scatter<kWide, 256, 8>(p, c, col_ids, vals32, vals64, odst, oval, st)
+                        : scatter<kWide, 512, 8>(p, c, col_ids, vals32, vals64, odst, oval, st);
+    if (e != cudaSuccess) return e;
+  }
+  constexpr size_t kSmem = (size_t)kColSlots * (kWide ? 16 : 12);
+  static unsigned long long done = 0;
+  if ((e = set_smem_once(k_col_count<kWide>, kSmem, &done)) != cudaSuccess) return e;
+  k_col_count<kWide><<<p.ntiles * kColPerTile, kColThreads, kSmem, st>>>(p, c, col_ids, vals32, vals64, odst, oval, q);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_col_heavy(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint64_t* hdr,
+                             cudaStream_t st) {
+  if (p.ntiles == 0 || p.nseg == 0) return cudaSuccess;
+  k_col_heavy<<<p.nseg, kColHeavyThreads, 0, st>>>(p, c, col_ids, hdr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cols(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                        const uint64_t* vals64, uint32_t* odst, void* oval, ans_quantities* q, cudaStream_t st) {
+  if (p.ntiles == 0) return cudaSuccess;
+  return vals32 ? run_cols<false>(p, c, col_ids, vals32, nullptr, odst, oval, q, st)
+                : run_cols<true>(p, c, col_ids, nullptr, vals64, odst, oval, q, st);
+}
+
+}  // namespace ans

@@ -14,6 +14,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <type_traits>
 
 #include "ans.h"
 
@@ -81,6 +82,33 @@ struct SegPlan {
 };
 
 // Where each phase reads and writes (all device pointers; see the launchers).
+// Partitions of a segment's links by destination hash (ans_cols.cu): their
+// sizes (counted by k_finish), cursors (both zeroed before) and starts, kColPerTile
+// entries per tile of the plan.
+constexpr uint32_t kColPerTile = 3;
+constexpr uint32_t kColMaxParts = 8192;
+constexpr uint32_t kColPart = (kTile + kColPerTile - 1) / kColPerTile;  // links per partition aimed at
+// Hash partitions of a segment of n links.
+constexpr uint32_t col_parts(uint64_t n, uint32_t max_parts) {
+  const uint64_t w = (n + kColPart - 1) / kColPart;
+  return w < 1 ? 1u : w < max_parts ? (uint32_t)w : max_parts;
+}
+// A segment of kColHeavyLinks links or more has a table of its heaviest
+// destinations (found in a sample), whose links are added up apart: 64 slots
+// at kColHeavyPerTile entries per tile, filled by launch_col_heavy; sums
+// (links, packets: two words per slot) zeroed before k_finish.
+constexpr uint32_t kColHeavyLinks = 1u << 18;
+constexpr uint32_t kColHeavySlots = 64;
+constexpr uint32_t kColHeavyPerTile = 2;
+static_assert(kColHeavyLinks / kTile * kColHeavyPerTile >= kColHeavySlots, "room for every table");
+struct ColParts {
+  uint32_t* cnt = nullptr;
+  uint32_t* cur = nullptr;
+  uint32_t* start = nullptr;
+  uint32_t* hkey = nullptr;
+  unsigned long long* hsum = nullptr;
+  uint32_t max_parts = 0;  // most partitions of a segment
+};
 struct StatsArgs {
   SegPlan plan;
   uint64_t* hdr = nullptr;        // [nseg][2] = {nrows, nnz}
@@ -109,6 +137,9 @@ struct StatsArgs {
   // u (the column sort's keys when a time sum's column statistics group
   // destinations by hash); the column histograms then count its bytes.
   uint32_t* col_hkeys = nullptr;
+  // Or (cp.cnt set): k_finish counts the links' hash partitions instead of
+  // their destination digits.
+  ColParts cp;
   int mode = 0;
 };
 
@@ -401,38 +432,28 @@ cudaError_t launch_colstat32(const SegPlan& p, const uint32_t* keys, const uint3
 // Canonical-DCSR check of an imported matrix; ORs failure bits into *bad.
 cudaError_t launch_check_dcsr(uint64_t nrows, uint64_t nnz, const uint32_t* row_ids, const uint64_t* row_ptr,
                               const uint32_t* col_ids, const uint64_t* vals, uint32_t* bad, cudaStream_t st);
-// CTAs per window launch_colhash uses for a batch of nseg windows (its
-// launch shape: part of the key of a cached batch graph).
-uint32_t colhash_ctas(uint32_t nseg);
-// Window column statistics from a shared-memory hash of destinations, one
-// CTA per window of p (links: col_ids / vals32 at base[s], ulen[s] of them);
-// a window whose distinct destinations fit gets its three column quantities
-// in q and ulen[s] = 0 (the column sort then skips it).
-cudaError_t launch_colhash(const SegPlan& p, uint64_t* ulen, const uint32_t* col_ids, const uint32_t* vals32,
-                           ans_quantities* q, cudaStream_t st);
+// The tables of heavy destinations of p's segments (hdr: {nrows, nnz} per
+// segment).
+cudaError_t launch_col_heavy(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint64_t* hdr,
+                             cudaStream_t st);
+// Column statistics of the segments of p (len = links per segment, whose
+// partitions k_finish has counted into c): links grouped by partition into
+// odst / oval (uint32 counts with vals32, uint64 counts with vals64; at the
+// segments' bases) and counted in shared-memory tables; the three column
+// quantities are combined into q.
+cudaError_t launch_cols(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                        const uint64_t* vals64, uint32_t* odst, void* oval, ans_quantities* q, cudaStream_t st);
 // One bounded look-back wait (both forms: the single-thread walk of the
 // radix passes and the warp walk of the run reductions and scans) for the
 // predecessor of tile 1 of a chain whose tile 0 never publishes (st: two
 // words, zero on entry).  Each wait gives up after the context's poll limit
 // and sets kErrLookback in err[0].
 cudaError_t launch_wait_probe(const uint64_t* st, uint32_t* err, cudaStream_t stream);
-// Per-window accumulator of the partitioned column hash (zeroed before it).
+// Accumulator of the hash-group column statistics (zeroed before them).
 struct ColPartAcc {
   unsigned long long count, max_fanin, max_packets;
   uint32_t fail, done;
 };
-// Window column statistics of the windows launch_colhash left (ulen[s] > 0)
-// with more than 8192 and at most 32 x 8192 links (window index below 2^27):
-// their destinations split by a hash into partitions (the links regrouped
-// by partition into pkeys/pvals at the window's base, partition starts in
-// bstart[s][0..33), the (window, partition) items listed in items[nseg *
-// 32]), one shared-memory table per partition, counted by one persistent
-// CTA per SM; windows whose partitions all fit get their three column
-// quantities and ulen[s] = 0.  acc: nseg + 1 zeroed accumulators (the last
-// one counts and hands out the items).
-cudaError_t launch_colhash_part(const SegPlan& p, uint64_t* ulen, const uint32_t* col_ids, const uint32_t* vals32,
-                                uint32_t* pkeys, uint32_t* pvals, uint32_t* bstart, ColPartAcc* acc, uint32_t* items,
-                                ans_quantities* q, cudaStream_t st);
 // Column statistics of one segment of *len links (a time sum) whose mixed
 // destinations `keys` (fmix32 of each destination, with uint32 counts
 // `vals32`) have been sorted by their low 16 bits (two column passes): the
@@ -551,6 +572,37 @@ __device__ __forceinline__ void window_inputs(const SegPlan& p, uint32_t seg, co
     *wd = dst + p.in_off[seg];
   }
 }
+
+// Finalizer of MurmurHash3 (Appleby): a bijective 32-bit mix.
+__device__ __forceinline__ uint32_t fmix32(uint32_t h) {
+  h ^= h >> 16;
+  h *= 0x85ebca6bu;
+  h ^= h >> 13;
+  h *= 0xc2b2ae35u;
+  h ^= h >> 16;
+  return h;
+}
+// Slot of destination d in a heavy table `key` (shared memory), -1 if it is
+// not heavy.  At most 48 of the 64 slots are taken.
+__device__ __forceinline__ int col_heavy(const uint32_t* key, uint32_t d) {
+  uint32_t i = fmix32(d) & (kColHeavySlots - 1);
+  for (uint32_t probe = 0; probe < kColHeavySlots; ++probe) {
+    const uint32_t k = key[i];
+    if (k == 0xFFFFFFFFu) return -1;
+    if (k == d) return (int)i;
+    i = (i + 1) & (kColHeavySlots - 1);
+  }
+  return -1;
+}
+// A 64-bit sum in two shared-memory words (a 64-bit shared atomic is a
+// compare-and-swap loop).
+__device__ __forceinline__ void add64_shared(uint32_t* lo, uint32_t* hi, uint64_t v) {
+  const uint32_t vl = (uint32_t)v, old = atomicAdd(lo, vl);
+  const uint32_t vh = (uint32_t)(v >> 32) + (old + vl < old ? 1u : 0u);
+  if (vh) atomicAdd(hi, vh);
+}
+// A destination's partition of `parts`.
+__device__ __forceinline__ uint32_t col_part(uint32_t dst, uint32_t parts) { return __umulhi(fmix32(dst), parts); }
 
 struct Tile {
   uint32_t seg, j;     // segment and tile index within it

@@ -42,7 +42,6 @@ constexpr uint32_t kNoAllocTiles = (uint32_t)(kNoAllocMaxPackets / kTile);
 // The buffers below are sized for kNoAllocMaxPackets items, which must cover
 // the padded index space (whole tiles) of the largest window.
 static_assert(kNoAllocMaxPackets % kTile == 0, "the packet limit must be a whole number of tiles");
-constexpr SortCfg kNoAllocSort{};  // the column passes' launch shape
 static_assert(ss_one_level(kNoAllocMaxPackets) >= kNoAllocMaxPackets, "the packets take one split");
 constexpr size_t kAl = 256;
 constexpr size_t al(size_t x) { return (x + kAl - 1) / kAl * kAl; }
@@ -56,11 +55,7 @@ constexpr size_t oCnt = al(oTree + (size_t)kNoAllocTiles * kSsPerTile * 16);
 constexpr size_t oCur = al(oCnt + (size_t)kNoAllocTiles * kSsPerTile * 4);
 constexpr size_t oBstart = al(oCur + (size_t)kNoAllocTiles * kSsPerTile * 4);
 constexpr size_t oEq = al(oBstart + (size_t)kNoAllocTiles * kSsPerTile * 4);
-// look-back status words: two sub-tiles' worth per tile (k_finish clears
-// that many for the column passes)
-constexpr size_t oSt0 = al(oEq + (size_t)kNoAllocTiles * kSsPerTile);
-constexpr size_t oSt1 = al(oSt0 + (size_t)kNoAllocTiles * 2 * kRadix * 8);
-constexpr size_t oLb = al(oSt1 + (size_t)kNoAllocTiles * 2 * kRadix * 8);
+constexpr size_t oLb = al(oEq + (size_t)kNoAllocTiles * kSsPerTile);
 constexpr size_t oTickets = al(oLb + (size_t)kNoAllocTiles * 8);
 constexpr size_t oRunStart = al(oTickets + 128 * 4);
 constexpr size_t oRowPos = al(oRunStart + (kNoAllocMaxPackets + 1) * 8);
@@ -71,14 +66,18 @@ constexpr size_t oRowPtr = al(oRowIds + kNoAllocMaxPackets * 4);
 constexpr size_t oHdr = al(oRowPtr + (kNoAllocMaxPackets + 1) * 8);
 constexpr size_t oQ = al(oHdr + 16);
 constexpr size_t oErr = al(oQ + sizeof(ans_quantities));
-constexpr size_t oColHist = al(oErr + 8);                          // destination digit counts
-constexpr size_t oUlen = al(oColHist + (size_t)kColPasses * kRadix * 4);
-constexpr size_t oCkA = al(oUlen + 8);                             // destination-sort ping-pong
-constexpr size_t oCkB = al(oCkA + kNoAllocMaxPackets * 4);
-constexpr size_t oCvA = al(oCkB + kNoAllocMaxPackets * 4);
-constexpr size_t oCvB = al(oCvA + kNoAllocMaxPackets * 8);
-constexpr size_t oBnd = al(oCvB + kNoAllocMaxPackets * 8);
-constexpr size_t kNoAllocBytes = al(oBnd + (size_t)kNoAllocTiles * sizeof(ColBnd));
+// the links' partitions by destination hash (sizes and cursors, cleared
+// together, then starts), their regrouped links and 32-bit counts
+constexpr size_t oCpCnt = al(oErr + 8);
+constexpr size_t oCpCur = oCpCnt + (size_t)kNoAllocTiles * kColPerTile * 4;
+constexpr size_t oCpStart = al(oCpCur + (size_t)kNoAllocTiles * kColPerTile * 4);
+constexpr size_t oCpHkey = al(oCpStart + (size_t)kNoAllocTiles * kColPerTile * 4);
+constexpr size_t oCpHsum = al(oCpHkey + (size_t)kNoAllocTiles * kColHeavyPerTile * 4);
+constexpr size_t oUlen = al(oCpHsum + (size_t)kNoAllocTiles * kColHeavyPerTile * 16);
+constexpr size_t oVals32 = al(oUlen + 8);
+constexpr size_t oCk = al(oVals32 + kNoAllocMaxPackets * 4);
+constexpr size_t oCv = al(oCk + kNoAllocMaxPackets * 4);
+constexpr size_t kNoAllocBytes = al(oCv + kNoAllocMaxPackets * 4);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -146,7 +145,7 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
   if (ntiles) {
     if ((rc = cu(cudaMemsetAsync(m + oTickets, 0, 32 * 4, st), "memset"))) return rc;
     if ((rc = cu(cudaMemsetAsync(m + oLb, 0, (size_t)ntiles * 8, st), "memset"))) return rc;
-    if ((rc = cu(cudaMemsetAsync(m + oColHist, 0, (size_t)kColPasses * kRadix * 4, st), "memset"))) return rc;
+    if ((rc = cu(cudaMemsetAsync(m + oCpCnt, 0, 2 * (size_t)kNoAllocTiles * kColPerTile * 4, st), "memset"))) return rc;
     k_noalloc_plan<<<1, 32, 0, st>>>(n, ntiles);
     if ((rc = cu(cudaGetLastError(), "plan"))) return rc;
     SegPlan p;
@@ -159,8 +158,6 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     p.ntiles = ntiles;
     uint64_t* ka = reinterpret_cast<uint64_t*>(m + oKeysA);
     uint64_t* kb = reinterpret_cast<uint64_t*>(m + oKeysB);
-    uint64_t* st0 = reinterpret_cast<uint64_t*>(m + oSt0);
-    uint64_t* st1 = reinterpret_cast<uint64_t*>(m + oSt1);
     uint32_t* tickets = reinterpret_cast<uint32_t*>(m + oTickets);
     SsArgs ss;
     ss.one_level = kNoAllocMaxPackets;
@@ -174,7 +171,7 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     ss.ntiles = ntiles;
     ss.keys_split = kb;
     ss.keys_out = ka;
-    ss.ids = reinterpret_cast<uint16_t*>(m + oCkA);  // free until the column passes
+    ss.ids = reinterpret_cast<uint16_t*>(m + oCk);  // free until the column statistics
     ss.tree = reinterpret_cast<uint64_t*>(m + oTree);
     ss.cnt = reinterpret_cast<uint32_t*>(m + oCnt);
     ss.cur = reinterpret_cast<uint32_t*>(m + oCur);
@@ -197,31 +194,27 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     a.pre = nullptr;
     a.lookback = reinterpret_cast<uint64_t*>(m + oLb);
     a.ticket = tickets + kPasses;
-    a.col_hist = reinterpret_cast<uint32_t*>(m + oColHist);
+    a.vals32 = reinterpret_cast<uint32_t*>(m + oVals32);
+    a.cp.cnt = reinterpret_cast<uint32_t*>(m + oCpCnt);
+    a.cp.cur = reinterpret_cast<uint32_t*>(m + oCpCur);
+    a.cp.start = reinterpret_cast<uint32_t*>(m + oCpStart);
+    a.cp.hkey = reinterpret_cast<uint32_t*>(m + oCpHkey);
+    a.cp.hsum = reinterpret_cast<unsigned long long*>(m + oCpHsum);
+    a.cp.max_parts = col_parts(n, kNoAllocTiles * kColPerTile);
     a.ulen = reinterpret_cast<uint64_t*>(m + oUlen);
-    a.col_st0 = st0;
-    a.col_tickets = tickets + 32;
     a.err = err;
     a.mode = kModeWindow;
     if ((rc = cu(launch_rle(a, st), "rle"))) return rc;
+    if (n >= kColHeavyLinks &&
+        ((rc = cu(cudaMemsetAsync(a.cp.hsum, 0, (size_t)ntiles * kColHeavyPerTile * 16, st), "memset")) ||
+         (rc = cu(launch_col_heavy(p, a.cp, a.col_ids, a.hdr, st), "heavy destinations"))))
+      return rc;
     if ((rc = cu(launch_finish(a, st), "finish"))) return rc;
-    // Column statistics: sort the stored links by destination, reduce the runs.
     SegPlan cp = p;
     cp.len = a.ulen;
-    uint32_t* cka = reinterpret_cast<uint32_t*>(m + oCkA);
-    uint32_t* ckb = reinterpret_cast<uint32_t*>(m + oCkB);
-    uint64_t* cva = reinterpret_cast<uint64_t*>(m + oCvA);
-    uint64_t* cvb = reinterpret_cast<uint64_t*>(m + oCvB);
-    for (int pass = 0; pass < kColPasses; ++pass) {
-      const uint32_t* kin = pass == 0 ? a.col_ids : (pass % 2 ? cka : ckb);
-      const uint64_t* vin = pass == 0 ? a.vals : (pass % 2 ? cva : cvb);
-      if ((rc = cu(launch_onesweep_col(cp, pass, kin, pass % 2 ? ckb : cka, vin, pass % 2 ? cvb : cva, a.col_hist,
-                                       pass % 2 ? st1 : st0, pass % 2 ? st0 : st1, a.col_tickets + pass, err,
-                                       kNoAllocSort, st),
-                   "onesweep_col")))
-        return rc;
-    }
-    if ((rc = cu(launch_colstat(cp, ckb, cvb, reinterpret_cast<ColBnd*>(m + oBnd), q, st), "colstat"))) return rc;
+    if ((rc = cu(launch_cols(cp, a.cp, a.col_ids, a.vals32, nullptr, reinterpret_cast<uint32_t*>(m + oCk), m + oCv, q, st),
+                 "column statistics")))
+      return rc;
   }
   if ((rc = cu(cudaMemcpyAsync(d_out, q, sizeof(ans_quantities), cudaMemcpyDefault, st), "copy out"))) return rc;
   if (d_status && (rc = cu(cudaMemcpyAsync(d_status, err, 4, cudaMemcpyDefault, st), "copy status"))) return rc;

@@ -111,14 +111,6 @@ __device__ __forceinline__ uint32_t ss_find(const SsArgs& a, uint32_t t) {
   return lo;
 }
 
-__device__ __forceinline__ uint32_t mix32(uint32_t h) {  // MurmurHash3's finalizer
-  h ^= h >> 16;
-  h *= 0x85ebca6bu;
-  h ^= h >> 13;
-  h *= 0xc2b2ae35u;
-  return h ^ (h >> 16);
-}
-
 constexpr int kSsSampleThreads = 1024;
 
 // Bitonic sort of sm[0 .. R * 1024) by 1024 threads, R keys per thread in
@@ -199,7 +191,7 @@ __global__ void __launch_bounds__(kSsSampleThreads) k_ss_sample(SsArgs a) {
     while (S < g.nb * kSsOversample && S < a.sample_max) S <<= 1;
     // one key from each of S equal stretches of the segment
     for (uint32_t i = tid; i < S; i += kSsSampleThreads) {
-      const uint64_t at = (((uint64_t)i << 16 | (mix32(i + 1) & 0xFFFFu)) * g.n) >> (16 + (31 - __clz(S)));
+      const uint64_t at = (((uint64_t)i << 16 | (fmix32(i + 1) & 0xFFFFu)) * g.n) >> (16 + (31 - __clz(S)));
       sm[i] = in.get(at);
     }
     __syncthreads();

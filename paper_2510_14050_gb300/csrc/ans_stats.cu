@@ -10,19 +10,18 @@
 //  * k_scan_u64: exclusive prefix of uint64 values (time sums, imported
 //    matrices), same look-back scheme.
 //  * k_finish: link values A(i,j) (Table I), the link maximum, per-row
-//    nonzero counts (fan-out) and packet sums (Sec. IV-C); it also builds the
-//    digit histograms of the destination keys for the column sort.
+//    nonzero counts (fan-out) and packet sums (Sec. IV-C); it also counts the
+//    links' hash partitions by destination (ans_cols.cu) or, for the column
+//    sort, the digits of their destinations.
 //  * k_colstat / k_colstat_fin: the transpose-free column pass.  Once the
 //    stored links are sorted by destination (32-bit keys carrying the link
 //    counts), every run of equal destinations is one column: its length is the
 //    fan-in and its value sum the destination's packets (Table I, Sec. IV-C).
 //    Runs inside a tile are reduced in place; runs that cross tiles are
 //    completed from per-tile boundary records.
-//  * k_colhash / k_colhash_cl: the same three column quantities of a window
-//    from a shared-memory hash of its destinations (one CTA per window, or a
-//    thread-block cluster per window whose CTAs merge their tables over
-//    distributed shared memory); windows with more distinct destinations than
-//    the table takes are left to the column sort.
+//    Sums of more links than the hash partitions take (ans_cols.cu) use it,
+//    by the bijective mix of the destinations where hash groups can end the
+//    sort after two passes.
 // Maxima are combined with 64-bit atomicMax; every value is an exact integer.
 #include "ans_internal.cuh"
 
@@ -218,32 +217,37 @@ __global__ void __launch_bounds__(kThreads) k_scan_u64(SegPlan p, const uint64_t
   }
 }
 
-// Finalizer of MurmurHash3 (Appleby): a bijective 32-bit mix.
-__device__ __forceinline__ uint32_t fmix32(uint32_t h) {
-  h ^= h >> 16;
-  h *= 0x85ebca6bu;
-  h ^= h >> 13;
-  h *= 0xc2b2ae35u;
-  h ^= h >> 16;
-  return h;
-}
-
-template <int kMode, bool kHKeys>
+// kCol: how the links' destinations are counted for the column statistics.
+enum FinishCols : int {
+  kColDigits = 0,  // digit histograms of the destinations (column sort)
+  kColMixed = 1,   // digit histograms of their mix, written to col_hkeys
+  kColParts = 2,   // hash partitions
+};
+template <int kMode, int kCol>
 __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
   __shared__ Tile s_tile;
   __shared__ uint64_t s_red[3][kWarps];
-  __shared__ uint32_t s_h[kColPasses * kRadix];
+  extern __shared__ uint32_t s_h[];  // digit counts, or the segment's partitions
+  __shared__ uint32_t s_hkey[kColHeavySlots], s_hfan[kColHeavySlots], s_hlo[kColHeavySlots], s_hhi[kColHeavySlots];
   const uint32_t t = blockIdx.x;
   const Tile tl = block_tile(a.plan, t, &s_tile);
   const uint32_t s = tl.seg;
   const uint64_t nrows = a.hdr[2 * s], nnz = a.hdr[2 * s + 1];
   const uint64_t bs = tl.base + s;
-  for (int i = threadIdx.x; i < kColPasses * kRadix; i += kThreads) s_h[i] = 0;
-  // Prepare the column sort: its first-pass status words, its tickets and
-  // the number of links per segment.
-  if (t == 0 && threadIdx.x < 32) a.col_tickets[threadIdx.x] = 0;
-  // (two sub-tiles' worth per tile: the column passes may run sub-tiles)
-  for (uint32_t i = threadIdx.x; i < 2 * kRadix; i += kThreads) a.col_st0[(uint64_t)t * 2 * kRadix + i] = 0;
+  const uint32_t nh = kCol == kColParts ? col_parts(nnz, a.cp.max_parts) : (uint32_t)(kColPasses * kRadix);
+  if (kCol != kColParts || tl.start < nnz)
+    for (uint32_t i = threadIdx.x; i < nh; i += kThreads) s_h[i] = 0;
+  const bool heavy = kCol == kColParts && nnz >= kColHeavyLinks && tl.start < nnz;
+  if (heavy && threadIdx.x < kColHeavySlots) {
+    s_hkey[threadIdx.x] = a.cp.hkey[(size_t)(t - tl.j) * kColHeavyPerTile + threadIdx.x];
+    s_hfan[threadIdx.x] = s_hlo[threadIdx.x] = s_hhi[threadIdx.x] = 0;
+  }
+  if constexpr (kCol != kColParts) {
+    // Prepare the column sort: its first-pass status words and its tickets
+    // (two sub-tiles' worth per tile: the column passes may run sub-tiles).
+    if (t == 0 && threadIdx.x < 32) a.col_tickets[threadIdx.x] = 0;
+    for (uint32_t i = threadIdx.x; i < 2 * kRadix; i += kThreads) a.col_st0[(uint64_t)t * 2 * kRadix + i] = 0;
+  }
   if (tl.j == 0 && threadIdx.x == 0) a.ulen[s] = nnz;
   __syncthreads();
 
@@ -291,16 +295,26 @@ __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
         if (a.vals32) a.vals32[tl.base + u] = (uint32_t)v;
       }
       mlink = v > mlink ? v : mlink;
-      // the column sort's key: the destination, or its bijective mix when
-      // the sum's column statistics group destinations by hash
-      uint32_t ck = dst[j];
-      if constexpr (kHKeys) {
-        ck = fmix32(ck);
-        a.col_hkeys[tl.base + u] = ck;
-      }
+      if constexpr (kCol == kColParts) {
+        const int hs = heavy ? col_heavy(s_hkey, dst[j]) : -1;
+        if (hs >= 0) {
+          atomicAdd(&s_hfan[hs], 1u);
+          add64_shared(&s_hlo[hs], &s_hhi[hs], v);
+        } else {
+          atomicAdd(&s_h[col_part(dst[j], nh)], 1u);
+        }
+      } else {
+        // the column sort's key: the destination, or its bijective mix when
+        // the sum's column statistics group destinations by hash
+        uint32_t ck = dst[j];
+        if constexpr (kCol == kColMixed) {
+          ck = fmix32(ck);
+          a.col_hkeys[tl.base + u] = ck;
+        }
 #pragma unroll
-      for (int p = 0; p < kColPasses; ++p)
-        atomicAdd(&s_h[p * kRadix + ((ck >> (p * kRadixBits)) & 0xffu)], 1u);
+        for (int p = 0; p < kColPasses; ++p)
+          atomicAdd(&s_h[p * kRadix + ((ck >> (p * kRadixBits)) & 0xffu)], 1u);
+      }
     }
   }
   const uint64_t r_end = umin64(tl.start + kTile, nrows);
@@ -322,10 +336,18 @@ __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
     s_red[2][warp] = mrow;
   }
   __syncthreads();
-  uint32_t* gh = a.col_hist + (size_t)s * kColPasses * kRadix;
-  for (int i = threadIdx.x; i < kColPasses * kRadix; i += kThreads) {
-    const uint32_t c = s_h[i];
-    if (c) atomicAdd(&gh[i], c);
+  if (heavy && threadIdx.x < kColHeavySlots && s_hfan[threadIdx.x]) {
+    unsigned long long* g = a.cp.hsum + 2 * ((size_t)(t - tl.j) * kColHeavyPerTile + threadIdx.x);
+    atomicAdd(g, (unsigned long long)s_hfan[threadIdx.x]);
+    atomicAdd(g + 1, (unsigned long long)s_hhi[threadIdx.x] << 32 | s_hlo[threadIdx.x]);
+  }
+  if (kCol != kColParts || tl.start < nnz) {
+    uint32_t* gh = kCol == kColParts ? a.cp.cnt + (size_t)(t - tl.j) * kColPerTile
+                                     : a.col_hist + (size_t)s * kColPasses * kRadix;
+    for (uint32_t i = threadIdx.x; i < nh; i += kThreads) {
+      const uint32_t c = s_h[i];
+      if (c) atomicAdd(&gh[i], c);
+    }
   }
   if (threadIdx.x == 0) {
     for (int w = 1; w < kWarps; ++w) {
@@ -665,514 +687,6 @@ __global__ void k_scatter_nonzero(SegPlan p, const uint64_t* __restrict__ kin, c
   }
 }
 
-// ---- window column statistics by a shared-memory hash of destinations -----
-//
-// One CTA per window counts, per distinct destination, its links (fan-in)
-// and their packets (destination packets) in a shared-memory open-addressing
-// table, then reduces the table to the three column quantities (Table I;
-// Sec. IV-C).  This replaces the four column-sort passes for every window
-// whose distinct destinations fit the table: once the table passes three
-// quarters full the CTA gives up and leaves the window to the sort; a window
-// it finished gets ulen = 0, so the column sort and its run reduction skip it.
-
-constexpr int kColHashThreads = 1024;
-constexpr uint32_t kColHashSlots = 1u << 14;                 // 16384
-constexpr uint32_t kColHashMaxFill = kColHashSlots / 4 * 3;  // give up above this
-constexpr size_t kColHashSmem = (size_t)kColHashSlots * 12;  // key, links, packets (uint32 each)
-constexpr uint32_t kColEmpty = 0xFFFFFFFFu;                  // empty slot (that destination is counted apart)
-
-__global__ void __launch_bounds__(kColHashThreads, 1) k_colhash(SegPlan p, uint64_t* __restrict__ ulen,
-                                                                 const uint32_t* __restrict__ col_ids,
-                                                                 const uint32_t* __restrict__ vals32,
-                                                                 ans_quantities* __restrict__ q) {
-  extern __shared__ __align__(16) uint32_t sm[];
-  uint32_t* t_key = sm;
-  uint32_t* t_cnt = sm + kColHashSlots;
-  uint32_t* t_sum = sm + 2 * kColHashSlots;
-  __shared__ uint32_t s_fill, s_over, s_spec_cnt, s_spec_sum;
-  __shared__ unsigned long long s_red[3][kColHashThreads / 32];
-  const uint32_t s = blockIdx.x;
-  if (s >= p.nseg) return;
-  const uint64_t n = ulen[s];
-  const uint64_t b = p.base[s];
-  for (uint32_t i = threadIdx.x; i < kColHashSlots; i += kColHashThreads) {
-    t_key[i] = kColEmpty;
-    t_cnt[i] = 0;
-    t_sum[i] = 0;
-  }
-  if (threadIdx.x == 0) s_fill = s_over = s_spec_cnt = s_spec_sum = 0;
-  __syncthreads();
-  for (uint64_t u = threadIdx.x; u < n; u += kColHashThreads) {
-    if (*(volatile uint32_t*)&s_over) break;
-    const uint32_t d = col_ids[b + u];
-    const uint32_t v = vals32[b + u];
-    if (d == kColEmpty) {
-      atomicAdd(&s_spec_cnt, 1u);
-      atomicAdd(&s_spec_sum, v);
-      continue;
-    }
-    uint32_t h = fmix32(d) & (kColHashSlots - 1);
-    for (uint32_t probe = 0; probe < kColHashSlots; ++probe) {
-      uint32_t cur = *(volatile uint32_t*)&t_key[h];
-      if (cur == kColEmpty) {
-        cur = atomicCAS(&t_key[h], kColEmpty, d);
-        if (cur == kColEmpty) {
-          cur = d;
-          if (atomicAdd(&s_fill, 1u) + 1 > kColHashMaxFill) s_over = 1;
-        }
-      }
-      if (cur == d) {
-        atomicAdd(&t_cnt[h], 1u);
-        atomicAdd(&t_sum[h], v);
-        break;
-      }
-      h = (h + 1) & (kColHashSlots - 1);
-    }
-  }
-  __syncthreads();
-  if (s_over) return;  // the column sort takes this window
-  unsigned long long c = 0, mcnt = 0, msum = 0;
-  for (uint32_t i = threadIdx.x; i < kColHashSlots; i += kColHashThreads) {
-    if (t_key[i] != kColEmpty) {
-      ++c;
-      mcnt = t_cnt[i] > mcnt ? t_cnt[i] : mcnt;
-      msum = t_sum[i] > msum ? t_sum[i] : msum;
-    }
-  }
-  c = warp_sum(c);
-  mcnt = warp_max(mcnt);
-  msum = warp_max(msum);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_red[0][warp] = c;
-    s_red[1][warp] = mcnt;
-    s_red[2][warp] = msum;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    c = 0;
-    mcnt = msum = 0;
-    for (int w = 0; w < kColHashThreads / 32; ++w) {
-      c += s_red[0][w];
-      mcnt = s_red[1][w] > mcnt ? s_red[1][w] : mcnt;
-      msum = s_red[2][w] > msum ? s_red[2][w] : msum;
-    }
-    if (s_spec_cnt) {
-      ++c;
-      mcnt = s_spec_cnt > mcnt ? s_spec_cnt : mcnt;
-      msum = s_spec_sum > msum ? s_spec_sum : msum;
-    }
-    q[s].unique_destinations = c;
-    q[s].max_destination_fanin = mcnt;
-    q[s].max_destination_packets = msum;
-    ulen[s] = 0;  // done: the column sort skips this window
-  }
-}
-
-// The same statistics with one cluster of C CTAs per window (launched with
-// clusters along x; cluster i takes window i; C a power of two): CTA r
-// counts links [r, r + 1) * ceil(n / C) of the window in its own table;
-// then, in log2(C) rounds, CTA r pulls the table of CTA r + 2^k (for r a
-// multiple of 2^(k+1)) over distributed shared memory and adds it into its
-// own, so CTA 0 ends with the window's table and reduces it.  A table that
-// passes kColHashMaxFill -- its own links, or a pulled table -- marks its CTA
-// overflowing, and the mark travels with the pulls: the window gives up
-// (ulen kept) exactly when it has more distinct destinations than that.
-// Every CTA of a cluster passes the same cluster barriers.
-__global__ void __launch_bounds__(kColHashThreads, 1) k_colhash_cl(SegPlan p, uint64_t* __restrict__ ulen,
-                                                                    const uint32_t* __restrict__ col_ids,
-                                                                    const uint32_t* __restrict__ vals32,
-                                                                    ans_quantities* __restrict__ q) {
-  extern __shared__ __align__(16) uint32_t sm[];
-  uint32_t* t_key = sm;
-  uint32_t* t_cnt = sm + kColHashSlots;
-  uint32_t* t_sum = sm + 2 * kColHashSlots;
-  __shared__ uint32_t s_fill, s_over, s_spec_cnt, s_spec_sum;
-  __shared__ unsigned long long s_red[3][kColHashThreads / 32];
-  const uint32_t me = cta_rank(), nc = cluster_nctarank();
-  const uint32_t s = cluster_id();
-  // A launch whose grid is not one cluster per window (the same for every
-  // CTA, so all leave before any cluster barrier) counts nothing: its
-  // windows keep their ulen and the column sort takes them.
-  if (gridDim.x != p.nseg * nc || gridDim.y != 1 || gridDim.z != 1) return;
-  const uint64_t n = s < p.nseg ? ulen[s] : 0;
-  const uint64_t b = s < p.nseg ? p.base[s] : 0;
-  for (uint32_t i = threadIdx.x; i < kColHashSlots; i += kColHashThreads) {
-    t_key[i] = kColEmpty;
-    t_cnt[i] = 0;
-    t_sum[i] = 0;
-  }
-  if (threadIdx.x == 0) s_fill = s_over = s_spec_cnt = s_spec_sum = 0;
-  __syncthreads();
-  // Adds (d, c links, v packets) to this CTA's table.
-  auto insert = [&](uint32_t d, uint32_t c, uint32_t v) {
-    uint32_t h = fmix32(d) & (kColHashSlots - 1);
-    for (uint32_t probe = 0; probe < kColHashSlots; ++probe) {
-      uint32_t cur = *(volatile uint32_t*)&t_key[h];
-      if (cur == kColEmpty) {
-        cur = atomicCAS(&t_key[h], kColEmpty, d);
-        if (cur == kColEmpty) {
-          cur = d;
-          if (atomicAdd(&s_fill, 1u) + 1 > kColHashMaxFill) s_over = 1;
-        }
-      }
-      if (cur == d) {
-        atomicAdd(&t_cnt[h], c);
-        atomicAdd(&t_sum[h], v);
-        return;
-      }
-      h = (h + 1) & (kColHashSlots - 1);
-    }
-  };
-  const uint64_t chunk = (n + nc - 1) / nc;
-  const uint64_t lo = umin64((uint64_t)me * chunk, n), hi = umin64(lo + chunk, n);
-  for (uint64_t u = lo + threadIdx.x; u < hi; u += kColHashThreads) {
-    if (*(volatile uint32_t*)&s_over) break;
-    const uint32_t d = col_ids[b + u];
-    const uint32_t v = vals32[b + u];
-    if (d == kColEmpty) {
-      atomicAdd(&s_spec_cnt, 1u);
-      atomicAdd(&s_spec_sum, v);
-      continue;
-    }
-    insert(d, 1u, v);
-  }
-  cluster_sync();  // every local table is complete
-  for (uint32_t step = 1; step < nc; step <<= 1) {
-    if ((me & (2 * step - 1)) == 0 && me + step < nc) {
-      const uint32_t r = me + step;
-      const uint32_t key_r = map_rank(smem_addr(t_key), r), cnt_r = map_rank(smem_addr(t_cnt), r),
-                     sum_r = map_rank(smem_addr(t_sum), r);
-      if (ld_cluster(map_rank(smem_addr(&s_over), r)) != 0) {
-        if (threadIdx.x == 0) s_over = 1;
-      } else {
-        constexpr int kU = 4;  // slots read per round trip
-        for (uint32_t i0 = threadIdx.x; i0 < kColHashSlots; i0 += kU * kColHashThreads) {
-          if (*(volatile uint32_t*)&s_over) break;
-          uint32_t d[kU];
-#pragma unroll
-          for (int j = 0; j < kU; ++j) d[j] = ld_cluster(key_r + 4 * (i0 + j * kColHashThreads));
-#pragma unroll
-          for (int j = 0; j < kU; ++j) {
-            if (d[j] == kColEmpty) continue;
-            const uint32_t i = i0 + j * kColHashThreads;
-            insert(d[j], ld_cluster(cnt_r + 4 * i), ld_cluster(sum_r + 4 * i));
-          }
-        }
-        if (threadIdx.x == 0) {
-          s_spec_cnt += ld_cluster(map_rank(smem_addr(&s_spec_cnt), r));
-          s_spec_sum += ld_cluster(map_rank(smem_addr(&s_spec_sum), r));
-        }
-      }
-    }
-    cluster_sync();  // this round's pulls are done: their sources are read no more
-  }
-  if (me != 0 || s_over || s >= p.nseg) return;  // an overflowing window is left to the column sort
-  unsigned long long c = 0, mcnt = 0, msum = 0;
-  for (uint32_t i = threadIdx.x; i < kColHashSlots; i += kColHashThreads) {
-    if (t_key[i] != kColEmpty) {
-      ++c;
-      mcnt = t_cnt[i] > mcnt ? t_cnt[i] : mcnt;
-      msum = t_sum[i] > msum ? t_sum[i] : msum;
-    }
-  }
-  c = warp_sum(c);
-  mcnt = warp_max(mcnt);
-  msum = warp_max(msum);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_red[0][warp] = c;
-    s_red[1][warp] = mcnt;
-    s_red[2][warp] = msum;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    c = 0;
-    mcnt = msum = 0;
-    for (int w = 0; w < kColHashThreads / 32; ++w) {
-      c += s_red[0][w];
-      mcnt = s_red[1][w] > mcnt ? s_red[1][w] : mcnt;
-      msum = s_red[2][w] > msum ? s_red[2][w] : msum;
-    }
-    if (s_spec_cnt) {
-      ++c;
-      mcnt = s_spec_cnt > mcnt ? s_spec_cnt : mcnt;
-      msum = s_spec_sum > msum ? s_spec_sum : msum;
-    }
-    q[s].unique_destinations = c;
-    q[s].max_destination_fanin = mcnt;
-    q[s].max_destination_packets = msum;
-    ulen[s] = 0;  // done: the column sort skips this window
-  }
-}
-
-// Windows with more destinations than one table holds: the destinations
-// are split between up to kColParts partitions by a hash, and each
-// partition's links are counted by its own CTA in its own shared-memory
-// table.  A window of n links gets ceil(n / kColPartLinks) partitions (n
-// bounds its distinct destinations).  First one CTA per window groups the
-// window's links by partition (a counting pass and a scatter pass, both
-// warp-aggregated); then CTA r of the window counts partition r's links.
-// Partial results meet in a per-window accumulator; the last CTA of a
-// window to finish writes the window's three quantities and marks it done
-// (ulen = 0) -- unless some partition overflowed its table, in which case
-// the window is left, untouched, to the column sort.
-constexpr uint32_t kColParts = 32;
-constexpr uint32_t kColPartLinks = 8192;
-constexpr int kSplitThreads = 1024;
-constexpr int kSplitUnroll = 4;
-
-// Finalizer-derived partition of a destination: the high bits of its mix
-// (the table slot uses the low bits), scaled to [0, parts).
-__device__ __forceinline__ uint32_t col_part(uint32_t d, uint32_t parts) {
-  return (uint32_t)(((uint64_t)(fmix32(d) >> 14) * parts) >> 18);
-}
-
-// Partitions of window s of n links, or 0 if the partitioned hash does not
-// take it (empty, finished, within one table, too large, or an index past
-// the 2^27 windows whose (window, partition) items fit 32 bits).
-__device__ __forceinline__ uint32_t col_parts_of(uint64_t n, uint32_t s) {
-  const uint64_t parts = (n + kColPartLinks - 1) / kColPartLinks;
-  return parts >= 2 && parts <= kColParts && s < (1u << 27) ? (uint32_t)parts : 0u;
-}
-
-// One CTA per window: the window's (destination, count) links regrouped by
-// partition into okeys/ovals at the window's base; the partition starts in
-// bstart[s][0..parts]; the window's (window, partition) items s * 32 + r
-// appended to `items` (their count in work->count).
-__global__ void __launch_bounds__(kSplitThreads, 2) k_colpart_split(SegPlan p, const uint64_t* __restrict__ ulen,
-                                                                    const uint32_t* __restrict__ col_ids,
-                                                                    const uint32_t* __restrict__ vals32,
-                                                                    uint32_t* __restrict__ okeys,
-                                                                    uint32_t* __restrict__ ovals,
-                                                                    uint32_t* __restrict__ bstart,
-                                                                    ColPartAcc* __restrict__ work,
-                                                                    uint32_t* __restrict__ items) {
-  __shared__ uint32_t s_cnt[kColParts], s_cur[kColParts];
-  const uint32_t s = blockIdx.x;
-  if (s >= p.nseg) return;
-  const uint64_t n = ulen[s];
-  const uint32_t parts = col_parts_of(n, s);
-  if (!parts) return;
-  const uint64_t b = p.base[s];
-  const uint32_t* ci = col_ids + b;
-  const uint32_t* vi = vals32 + b;
-  const int lane = threadIdx.x & 31;
-  if (threadIdx.x < kColParts) s_cnt[threadIdx.x] = 0;
-  __syncthreads();
-  // pass 1: links per partition
-  for (uint64_t w0 = threadIdx.x & ~31u; w0 < n; w0 += (uint64_t)kSplitUnroll * kSplitThreads) {
-    const uint64_t u0 = w0 + (threadIdx.x & 31);  // the loop bound is the same for the whole warp
-    uint32_t d[kSplitUnroll];
-#pragma unroll
-    for (int k = 0; k < kSplitUnroll; ++k) {
-      const uint64_t u = u0 + (uint64_t)k * kSplitThreads;
-      d[k] = u < n ? ci[u] : 0u;
-    }
-#pragma unroll
-    for (int k = 0; k < kSplitUnroll; ++k) {
-      const bool valid = u0 + (uint64_t)k * kSplitThreads < n;
-      const uint32_t pt = valid ? col_part(d[k], parts) : kColParts;
-      const uint32_t peers = __match_any_sync(0xffffffffu, pt);
-      if (valid && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[pt], __popc(peers));
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t run = 0;
-    for (uint32_t r = 0; r < parts; ++r) {
-      s_cur[r] = run;
-      bstart[(uint64_t)s * (kColParts + 1) + r] = run;
-      run += s_cnt[r];
-    }
-    bstart[(uint64_t)s * (kColParts + 1) + parts] = run;
-    const uint32_t first = (uint32_t)atomicAdd(&work->count, (unsigned long long)parts);
-    for (uint32_t r = 0; r < parts; ++r) items[first + r] = s * kColParts + r;
-  }
-  __syncthreads();
-  // pass 2: scatter each link to its partition (order within a partition is free)
-  uint32_t* ko = okeys + b;
-  uint32_t* vo = ovals + b;
-  for (uint64_t w0 = threadIdx.x & ~31u; w0 < n; w0 += (uint64_t)kSplitUnroll * kSplitThreads) {
-    const uint64_t u0 = w0 + (threadIdx.x & 31);  // the loop bound is the same for the whole warp
-    uint32_t d[kSplitUnroll], v[kSplitUnroll];
-#pragma unroll
-    for (int k = 0; k < kSplitUnroll; ++k) {
-      const uint64_t u = u0 + (uint64_t)k * kSplitThreads;
-      d[k] = u < n ? ci[u] : 0u;
-      v[k] = u < n ? vi[u] : 0u;
-    }
-#pragma unroll
-    for (int k = 0; k < kSplitUnroll; ++k) {
-      const bool valid = u0 + (uint64_t)k * kSplitThreads < n;
-      const uint32_t pt = valid ? col_part(d[k], parts) : kColParts;
-      const uint32_t peers = __match_any_sync(0xffffffffu, pt);
-      const int leader = __ffs(peers) - 1;
-      uint32_t pos = 0;
-      if (valid && lane == leader) pos = atomicAdd(&s_cur[pt], __popc(peers));
-      pos = __shfl_sync(0xffffffffu, pos, leader) + __popc(peers & lanemask_lt());
-      if (valid) {
-        ko[pos] = d[k];
-        vo[pos] = v[k];
-      }
-    }
-  }
-}
-
-// Partitions counted by persistent CTAs (one per SM: the table takes the
-// SM's shared memory), each taking the next (window s, partition r) item
-// that k_colpart_split listed and counting partition r's links.  The links
-// are read in chunks of kColPartChunk per thread, the first chunk's loads
-// issued before the table is cleared; the table's fill is counted once per
-// warp.
-constexpr int kColPartChunk = 8;
-__global__ void __launch_bounds__(kColHashThreads, 1) k_colhash_part(SegPlan p, uint64_t* __restrict__ ulen,
-                                                                      const uint32_t* __restrict__ pkeys,
-                                                                      const uint32_t* __restrict__ pvals,
-                                                                      const uint32_t* __restrict__ bstart,
-                                                                      ColPartAcc* __restrict__ acc,
-                                                                      const uint32_t* __restrict__ items,
-                                                                      ans_quantities* __restrict__ q) {
-  extern __shared__ __align__(16) uint32_t sm[];
-  uint32_t* t_key = sm;
-  uint32_t* t_cnt = sm + kColHashSlots;
-  uint32_t* t_sum = sm + 2 * kColHashSlots;
-  __shared__ uint32_t s_fill, s_over, s_spec_cnt, s_spec_sum, s_last, s_item;
-  __shared__ unsigned long long s_red[3][kColHashThreads / 32];
-  ColPartAcc* work = acc + p.nseg;
-  const uint32_t nitems = (uint32_t)work->count;  // written by k_colpart_split
-  for (;;) {
-    if (threadIdx.x == 0) {
-      const uint32_t i = atomicAdd(&work->done, 1u);
-      s_item = i < nitems ? items[i] : 0xFFFFFFFFu;
-    }
-    __syncthreads();
-    const uint32_t item = s_item;
-    if (item == 0xFFFFFFFFu) break;
-    const uint32_t s = item / kColParts, r = item % kColParts;
-    const uint32_t parts = col_parts_of(ulen[s], s);
-    const uint64_t b = p.base[s];
-    const uint32_t lo = bstart[(uint64_t)s * (kColParts + 1) + r], hi = bstart[(uint64_t)s * (kColParts + 1) + r + 1];
-    const uint32_t* pk = pkeys + b;
-    const uint32_t* pv = pvals + b;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t d[kColPartChunk], v[kColPartChunk];
-    auto load = [&](uint32_t u0) {
-#pragma unroll
-      for (int j = 0; j < kColPartChunk; ++j) {
-        const uint32_t u = u0 + (uint32_t)j * kColHashThreads + threadIdx.x;
-        d[j] = u < hi ? __ldg(pk + u) : 0u;
-        v[j] = u < hi ? __ldg(pv + u) : 0u;
-      }
-    };
-    load(lo);
-    {
-      uint4* k4 = reinterpret_cast<uint4*>(t_key);
-      uint4* c4 = reinterpret_cast<uint4*>(t_cnt);  // t_cnt and t_sum, back to back
-      const uint4 empty = make_uint4(kColEmpty, kColEmpty, kColEmpty, kColEmpty), zero = make_uint4(0, 0, 0, 0);
-      for (uint32_t i = threadIdx.x; i < kColHashSlots / 4; i += kColHashThreads) k4[i] = empty;
-      for (uint32_t i = threadIdx.x; i < kColHashSlots / 2; i += kColHashThreads) c4[i] = zero;
-    }
-    if (threadIdx.x == 0) s_fill = s_over = s_spec_cnt = s_spec_sum = 0;
-    __syncthreads();
-    constexpr uint32_t kStep = (uint32_t)kColPartChunk * kColHashThreads;
-    for (uint32_t u0 = lo; u0 < hi; u0 += kStep) {  // the same trip count for every thread
-      if (u0 != lo) load(u0);
-      if (__any_sync(0xffffffffu, *(volatile uint32_t*)&s_over != 0)) break;  // warp-uniform
-#pragma unroll
-      for (int j = 0; j < kColPartChunk; ++j) {
-        const uint32_t u = u0 + (uint32_t)j * kColHashThreads + threadIdx.x;
-        bool claimed = false;
-        if (u < hi) {
-          if (d[j] == kColEmpty) {
-            atomicAdd(&s_spec_cnt, 1u);
-            atomicAdd(&s_spec_sum, v[j]);
-          } else {
-            uint32_t h = fmix32(d[j]) & (kColHashSlots - 1);
-            for (uint32_t probe = 0; probe < kColHashSlots; ++probe) {
-              uint32_t cur = *(volatile uint32_t*)&t_key[h];
-              if (cur == kColEmpty) {
-                cur = atomicCAS(&t_key[h], kColEmpty, d[j]);
-                if (cur == kColEmpty) {
-                  cur = d[j];
-                  claimed = true;
-                }
-              }
-              if (cur == d[j]) {
-                atomicAdd(&t_cnt[h], 1u);
-                atomicAdd(&t_sum[h], v[j]);
-                break;
-              }
-              h = (h + 1) & (kColHashSlots - 1);
-            }
-          }
-        }
-        // new slots counted once per warp; past three quarters the table gives
-        // up (at most one slot per thread more can still be claimed meanwhile)
-        const uint32_t nc = __popc(__ballot_sync(0xffffffffu, claimed));
-        if (lane == 0 && nc && atomicAdd(&s_fill, nc) + nc > kColHashMaxFill) s_over = 1;
-      }
-    }
-    __syncthreads();
-    ColPartAcc* a = acc + s;
-    if (!s_over) {
-      unsigned long long c = 0, mcnt = 0, msum = 0;
-      for (uint32_t i = threadIdx.x; i < kColHashSlots; i += kColHashThreads) {
-        if (t_key[i] != kColEmpty) {
-          ++c;
-          mcnt = t_cnt[i] > mcnt ? t_cnt[i] : mcnt;
-          msum = t_sum[i] > msum ? t_sum[i] : msum;
-        }
-      }
-      c = warp_sum(c);
-      mcnt = warp_max(mcnt);
-      msum = warp_max(msum);
-      if (lane == 0) {
-        s_red[0][warp] = c;
-        s_red[1][warp] = mcnt;
-        s_red[2][warp] = msum;
-      }
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        c = 0;
-        mcnt = msum = 0;
-        for (int w = 0; w < kColHashThreads / 32; ++w) {
-          c += s_red[0][w];
-          mcnt = s_red[1][w] > mcnt ? s_red[1][w] : mcnt;
-          msum = s_red[2][w] > msum ? s_red[2][w] : msum;
-        }
-        if (s_spec_cnt) {
-          ++c;
-          mcnt = s_spec_cnt > mcnt ? s_spec_cnt : mcnt;
-          msum = s_spec_sum > msum ? s_spec_sum : msum;
-        }
-        if (c) atomicAdd(&a->count, c);
-        if (mcnt) atomicMax(&a->max_fanin, mcnt);
-        if (msum) atomicMax(&a->max_packets, msum);
-      }
-    } else if (threadIdx.x == 0) {
-      atomicOr(&a->fail, 1u);
-    }
-    // The last partition of the window to arrive publishes the result.
-    if (threadIdx.x == 0) {
-      __threadfence();
-      s_last = atomicAdd(&a->done, 1u) == parts - 1 ? 1u : 0u;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && s_last) {
-      __threadfence();
-      const volatile ColPartAcc* va = a;
-      if (va->fail == 0) {
-        q[s].unique_destinations = va->count;
-        q[s].max_destination_fanin = va->max_fanin;
-        q[s].max_destination_packets = va->max_packets;
-        ulen[s] = 0;  // done: the column sort skips this window
-      }
-    }
-    __syncthreads();  // the table and the shared words are reused by the next item
-  }
-}
-
 // ---- column statistics of one large segment (a time sum) by hash groups ---
 //
 // The column statistics only need equal destinations grouped, in any order,
@@ -1193,6 +707,7 @@ constexpr uint32_t kHGroupMaxFill = kHGroupSlots / 4 * 3;     // give up above t
 constexpr size_t kHGroupSmem = (size_t)kHGroupSlots * 12;     // key, links, packets
 constexpr int kHGroupChunk = 8;
 constexpr uint32_t kHNone = 0xFFFFFFFFu;
+constexpr uint32_t kColEmpty = 0xFFFFFFFFu;  // empty slot (that mix is counted apart)
 static_assert(kHGroupPartWords == 3 * (kHGroupMaxFill + 1), "a part's entries: its table's fill and the key apart");
 
 // bnd[g] = first position of group g (g in [0, 2^16]; bnd[2^16] = n) in the
@@ -1514,105 +1029,7 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_merge(HGroupBufs b
   }
 }
 
-// CTAs per window for the cluster form (1 = the one-CTA kernel): enough to
-// cover the SMs with the batch's windows, if the device hosts such clusters.
-uint32_t colhash_cluster_size(uint32_t nseg) {
-  static int ok[4][64];  // per size index and device: 0 unknown, 1 yes, 2 no
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev >= 64) return 1;
-  int sms = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-  for (uint32_t c = 8, k = 3; c >= 2; c >>= 1, --k) {
-    if ((uint64_t)nseg * c > (uint64_t)sms) continue;
-    if (ok[k][dev] == 0) {
-      cudaLaunchConfig_t lc = {};
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = c;
-      attr.val.clusterDim.y = 1;
-      attr.val.clusterDim.z = 1;
-      lc.attrs = &attr;
-      lc.numAttrs = 1;
-      lc.gridDim = dim3(c, 1, 1);
-      lc.blockDim = dim3(kColHashThreads, 1, 1);
-      lc.dynamicSmemBytes = kColHashSmem;
-      int n = 0;
-      ok[k][dev] = cudaFuncSetAttribute(k_colhash_cl, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)kColHashSmem) == cudaSuccess &&
-                           cudaOccupancyMaxActiveClusters(&n, k_colhash_cl, &lc) == cudaSuccess && n > 0
-                       ? 1
-                       : 2;
-      cudaGetLastError();
-    }
-    if (ok[k][dev] == 1) return c;
-  }
-  return 1;
-}
-
 }  // namespace
-
-uint32_t colhash_ctas(uint32_t nseg) { return nseg ? colhash_cluster_size(nseg) : 1u; }
-
-cudaError_t launch_colhash(const SegPlan& p, uint64_t* ulen, const uint32_t* col_ids, const uint32_t* vals32,
-                           ans_quantities* q, cudaStream_t st) {
-  if (p.nseg == 0) return cudaSuccess;
-  static unsigned long long configured = 0;  // one bit per device ordinal
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev >= 64 || !((configured >> dev) & 1ull)) {
-    e = cudaFuncSetAttribute(k_colhash, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColHashSmem);
-    if (e != cudaSuccess) return e;
-    if (dev < 64) configured |= 1ull << dev;
-  }
-  const uint32_t c = colhash_cluster_size(p.nseg);
-  if (c > 1) {
-    cudaLaunchConfig_t lc = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = c;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
-    lc.gridDim = dim3(p.nseg * c, 1, 1);
-    lc.blockDim = dim3(kColHashThreads, 1, 1);
-    lc.dynamicSmemBytes = kColHashSmem;
-    lc.stream = st;
-    return cudaLaunchKernelEx(&lc, k_colhash_cl, p, ulen, col_ids, vals32, q);
-  }
-  k_colhash<<<p.nseg, kColHashThreads, kColHashSmem, st>>>(p, ulen, col_ids, vals32, q);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_colhash_part(const SegPlan& p, uint64_t* ulen, const uint32_t* col_ids, const uint32_t* vals32,
-                                uint32_t* pkeys, uint32_t* pvals, uint32_t* bstart, ColPartAcc* acc, uint32_t* items,
-                                ans_quantities* q, cudaStream_t st) {
-  if (p.nseg == 0) return cudaSuccess;
-  static unsigned long long configured = 0;  // one bit per device ordinal
-  static int sms[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev >= 64 || !((configured >> dev) & 1ull)) {
-    e = cudaFuncSetAttribute(k_colhash_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColHashSmem);
-    if (e != cudaSuccess) return e;
-    int n = 0;
-    e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 64) {
-      sms[dev] = n;
-      configured |= 1ull << dev;
-    }
-  }
-  const unsigned ctas = dev < 64 && sms[dev] > 0 ? (unsigned)sms[dev] : 1u;
-  k_colpart_split<<<p.nseg, kSplitThreads, 0, st>>>(p, ulen, col_ids, vals32, pkeys, pvals, bstart, acc + p.nseg,
-                                                    items);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_colhash_part<<<ctas, kColHashThreads, kColHashSmem, st>>>(p, ulen, pkeys, pvals, bstart, acc, items, q);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_hgroup_stats(const uint32_t* keys, const uint32_t* vals32, uint64_t* len, const HGroupBufs& b,
                                 uint32_t max_hparts, ans_quantities* q, cudaStream_t st) {
@@ -1704,18 +1121,20 @@ cudaError_t launch_scan_u64(const SegPlan& p, const uint64_t* in, uint64_t* out,
 
 cudaError_t launch_finish(const StatsArgs& a, cudaStream_t st) {
   if (a.plan.ntiles == 0) return cudaSuccess;
-  const bool h = a.col_hkeys != nullptr;
-  switch (a.mode) {
-    case kModeWindow:
-      if (h) k_finish<kModeWindow, true><<<a.plan.ntiles, kThreads, 0, st>>>(a);
-      else k_finish<kModeWindow, false><<<a.plan.ntiles, kThreads, 0, st>>>(a);
-      break;
-    case kModeSum:
-      if (h) k_finish<kModeSum, true><<<a.plan.ntiles, kThreads, 0, st>>>(a);
-      else k_finish<kModeSum, false><<<a.plan.ntiles, kThreads, 0, st>>>(a);
-      break;
-    default: k_finish<kModeMatrix, false><<<a.plan.ntiles, kThreads, 0, st>>>(a); break;
+  const int col = a.cp.cnt ? kColParts : a.col_hkeys ? kColMixed : kColDigits;
+  const size_t sm = (size_t)(col == kColParts ? a.cp.max_parts : kColPasses * kRadix) * 4;
+#define ANS_FINISH(M)                                                                              \
+  if (col == kColParts) k_finish<M, kColParts><<<a.plan.ntiles, kThreads, sm, st>>>(a);            \
+  else if (col == kColMixed) k_finish<M, kColMixed><<<a.plan.ntiles, kThreads, sm, st>>>(a);       \
+  else k_finish<M, kColDigits><<<a.plan.ntiles, kThreads, sm, st>>>(a)
+  if (a.mode == kModeWindow) {
+    ANS_FINISH(kModeWindow);
+  } else if (a.mode == kModeSum) {
+    ANS_FINISH(kModeSum);
+  } else {
+    ANS_FINISH(kModeMatrix);
   }
+#undef ANS_FINISH
   return cudaGetLastError();
 }
 
