@@ -852,8 +852,8 @@ int sample_sort(ans_ctx* c, char* m, const SsScratch& ss, const SegPlan& p, cons
     o.count = at<uint32_t>(m, ss.count2);
     ANS_CUDA(timed(c, "ss_sample", st, [&] { return launch_ss_sample(a, max_len, st); }));
     ANS_CUDA(timed(c, "ss_count", st, [&] { return launch_ss_count(a, st); }));
-    ANS_CUDA(timed(c, "ss_scatter", st, [&] { return launch_ss_scatter(a, st); }));
     ANS_CUDA(timed(c, "ss_plan", st, [&] { return launch_ss_plan2(a, o, st); }));
+    ANS_CUDA(timed(c, "ss_scatter", st, [&] { return launch_ss_scatter(a, st); }));
     a.level1 = false;
     a.keys_in = ka;
     a.keys_split = kb;

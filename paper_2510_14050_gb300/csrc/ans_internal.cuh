@@ -315,7 +315,7 @@ cudaError_t launch_count_prefix(const MatDesc* mats, uint32_t k, uint64_t* cat_o
 // scatter, local over the segments of `plan` (raw packets), or over the
 // level-2 segments that launch_ss_plan2 lists after a first split of the
 // segments longer than one_level.
-constexpr uint32_t kSsPerTile = 3;  // buckets per tile of keys
+constexpr uint32_t kSsPerTile = 6;  // buckets per tile of keys
 // Longest segment that one split takes, in a plan of `total` keys.  One CTA
 // sorts a segment's sample: 23 us for 2^17 keys, 148 us for 2^20 (measured),
 // which a large batch hides behind its other segments and a small one does

@@ -6,15 +6,15 @@
 // keys are indistinguishable, so the sort need not be stable, and it works
 // from the most significant end:
 //
-//   sample   one CTA per segment sorts ~32 sampled keys per bucket on chip and
-//            takes every 32nd as a splitter; a key that fills several buckets
+//   sample   one CTA per segment sorts ~16 sampled keys per bucket on chip and
+//            takes every 16th as a splitter; a key that fills several buckets
 //            gets one of its own (its copies need no sorting at all);
 //   count    every key's bucket by a search tree of splitters in shared
 //            memory (ids kept as 16-bit words), bucket sizes;
 //   scatter  keys moved to their buckets: ranks by one shared-memory atomic
 //            per key, space by one global atomic per bucket and tile -- no
 //            chain of tiles waiting for one another;
-//   local    every bucket (~2048 keys) sorted by one CTA on chip: 16 keys per
+//   local    every bucket (~1366 keys) sorted by one CTA on chip: 16 keys per
 //            thread in registers, then merge-path rounds in shared memory.
 //
 // Buckets hold equal numbers of packets whatever the addresses look like, so
@@ -25,11 +25,13 @@
 // Against eight least-significant-digit passes (each bound by its chain of
 // tiles and by 150 instructions per key; 53 us for 64 windows of 2^17 keys,
 // 930 us for 2^27 keys with 16-bit window ids) this reads and writes the keys
-// four times instead of nine: 64 windows in 274 us against 491, one window
-// of 2^17 in 60 us against 82, 2^27 keys as one segment in 4.9 ms.  On one
-// GB300 the local sort is bound by shared-memory wavefronts (75% of peak, 341
-// instructions per key), count by issue slots (72%), scatter by the latency
-// of its loads.
+// four times instead of nine: 64 windows in 242 us against 491, one window
+// of 2^17 in 60-67 us against 82, 2^27 keys as one segment in 4.5 ms.  On one
+// GB300, 2^27 keys in windows of 2^17: sample 0.17, count 0.38 (bound by issue
+// slots, 72%), scatter 0.62 (by the latency of its loads: 0.93 with one 4-byte
+// load per address instead of 16-byte vectors), local 1.7 ms (by
+// shared-memory wavefronts, 75% of peak, 340 instructions per key; buckets of
+// 2731 keys and 256 threads: 1.93 ms).
 #include "ans_internal.cuh"
 
 namespace ans {
@@ -37,10 +39,10 @@ namespace ans {
 namespace {
 
 constexpr uint32_t kSsBucket = (kTile + kSsPerTile - 1) / kSsPerTile;  // keys per bucket aimed at
-constexpr uint32_t kSsLocal = 4096;         // keys one CTA sorts on chip
+constexpr uint32_t kSsLocal = 2048;         // keys one CTA sorts on chip
 constexpr uint32_t kSsMaxBuckets = 1024;    // buckets of one split
 constexpr uint32_t kSsSampleMax = 16384;    // sampled keys of one segment
-constexpr uint32_t kSsOversample = 32;      // sampled keys per bucket
+constexpr uint32_t kSsOversample = 16;      // sampled keys per bucket
 constexpr uint32_t kSsRawBit = 0x80000000u; // level-2 parent: the segment itself, still unsplit input
 constexpr uint32_t kSsDone = 0xFFFFFFFFu;   // level-2 parent: nothing to sort
 
@@ -49,10 +51,9 @@ constexpr uint32_t kSsDone = 0xFFFFFFFFu;   // level-2 parent: nothing to sort
 __host__ __device__ __forceinline__ uint32_t ss_buckets(uint64_t n, bool level1, uint64_t one_level) {
   if (level1) {
     if (n <= one_level) return 0u;
-    const uint64_t want = (n + kSsBucket - 1) / kSsBucket;
-    uint32_t r = 2;
-    while ((uint64_t)r * r < want && r < kSsMaxBuckets) r += r < 64 ? 1 : 16;
-    return r;
+    // (sqrtf is correctly rounded on both sides)
+    const uint32_t r = (uint32_t)sqrtf((float)((n + kSsBucket - 1) / kSsBucket)) + 1;
+    return r < kSsMaxBuckets ? r : kSsMaxBuckets;
   }
   return n <= kSsLocal ? 1u : (uint32_t)umin64((n + kSsBucket - 1) / kSsBucket, kSsMaxBuckets);
 }
@@ -66,7 +67,19 @@ struct SsIn {
   __device__ __forceinline__ uint64_t get(uint64_t i) const {
     return keys ? keys[i] : ((uint64_t)src[i] << 32) | dst[i];
   }
+  // Raw packets from `at` on can be read four at a time (get4).
+  __device__ __forceinline__ bool vectors(uint64_t at) const {
+    return !keys && (((uintptr_t)(src + at) | (uintptr_t)(dst + at)) & 15u) == 0;
+  }
+  __device__ __forceinline__ void get4(uint64_t at, uint32_t v, uint64_t* k) const {
+    const uint4 x = reinterpret_cast<const uint4*>(src + at)[v], y = reinterpret_cast<const uint4*>(dst + at)[v];
+    k[0] = (uint64_t)x.x << 32 | y.x;
+    k[1] = (uint64_t)x.y << 32 | y.y;
+    k[2] = (uint64_t)x.z << 32 | y.z;
+    k[3] = (uint64_t)x.w << 32 | y.w;
+  }
 };
+constexpr uint32_t kSsNone = 0xFFFFFFFFu;
 
 // One split's segments: the plan's own (raw packets), or, after a first
 // split, the list seg2 (keys of the first split's buckets, or a raw segment
@@ -180,10 +193,7 @@ __global__ void __launch_bounds__(kSsSampleThreads) k_ss_sample(SsArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (uint32_t s = blockIdx.x; s < nseg; s += gridDim.x) {
     const SsSeg g = ss_seg(a, s);
-    for (uint32_t i = tid; i < g.nb; i += kSsSampleThreads) {
-      a.cnt[g.b0 + i] = 0;
-      a.cur[g.b0 + i] = 0;
-    }
+    for (uint32_t i = tid; i < g.nb; i += kSsSampleThreads) a.cnt[g.b0 + i] = a.cur[g.b0 + i] = 0;
     if (g.nb <= 1) continue;
     const SsIn in = ss_input(a, s, g.start);
     const uint32_t lv = ss_levels(g.nb);
@@ -247,7 +257,7 @@ __global__ void __launch_bounds__(kSsSampleThreads) k_ss_sample(SsArgs a) {
 
 // kT threads take kP keys each.
 template <int kT, int kP>
-__global__ void __launch_bounds__(kT) k_ss_count(SsArgs a) {
+__global__ void __launch_bounds__(kT, 1536 / kT) k_ss_count(SsArgs a) {
   constexpr uint32_t kTT = kT * kP, kSub = kTile / kTT;
   __shared__ uint64_t s_tree[kSsMaxBuckets];
   __shared__ uint32_t s_h[kSsMaxBuckets];
@@ -265,10 +275,20 @@ __global__ void __launch_bounds__(kT) k_ss_count(SsArgs a) {
   }
   const SsIn in = ss_input(a, g.s, g.start);
   uint64_t k[kP];
+  const bool vec = count == kTT && in.vectors(off);
+  if (vec) {
 #pragma unroll
-  for (int i = 0; i < kP; ++i) {
-    const uint32_t x = i * kT + threadIdx.x;
-    k[i] = x < count ? in.get(off + x) : 0ull;
+    for (int i = 0; i < kP; i += 4) in.get4(off, (i / 4) * kT + threadIdx.x, &k[i]);
+  } else if (count == kTT && in.keys) {
+    const uint64_t* kk = in.keys + off;
+#pragma unroll
+    for (int i = 0; i < kP; ++i) k[i] = kk[i * kT + threadIdx.x];
+  } else {
+#pragma unroll
+    for (int i = 0; i < kP; ++i) {
+      const uint32_t x = i * kT + threadIdx.x;
+      k[i] = x < count ? in.get(off + x) : 0ull;
+    }
   }
   __syncthreads();
   const uint32_t last = (uint32_t)s_tree[0];
@@ -280,14 +300,21 @@ __global__ void __launch_bounds__(kT) k_ss_count(SsArgs a) {
     for (int i = 0; i < kP; ++i) node[i] = 2 * node[i] + (k[i] >= s_tree[node[i]] ? 1u : 0u);
   }
   uint16_t* ids = a.ids + g.start + off;
+  // (a key of all ones passes the padding too)
+#pragma unroll
+  for (int i = 0; i < kP; ++i) node[i] = min(node[i] - (1u << lv), last);
+  if (vec) {
+#pragma unroll
+    for (int i = 0; i < kP; i += 4)
+      reinterpret_cast<ushort4*>(ids)[(i / 4) * kT + threadIdx.x] =
+          make_ushort4((uint16_t)node[i], (uint16_t)node[i + 1], (uint16_t)node[i + 2], (uint16_t)node[i + 3]);
+  }
 #pragma unroll
   for (int i = 0; i < kP; ++i) {
     const uint32_t x = i * kT + threadIdx.x;
-    if (x < count) {
-      // (a key of all ones passes the padding too)
-      const uint32_t b = min(node[i] - (1u << lv), last);
-      ids[x] = (uint16_t)b;
-      atomicAdd(&s_h[b], 1u);
+    if (vec || x < count) {
+      if (!vec) ids[x] = (uint16_t)node[i];
+      atomicAdd(&s_h[node[i]], 1u);
     }
   }
   __syncthreads();
@@ -324,23 +351,42 @@ __global__ void __launch_bounds__(kT, kMinB) k_ss_scatter(SsArgs a) {
   const SsIn in = ss_input(a, g.s, g.start);
   const uint16_t* ids = a.ids + g.start + off;
   uint64_t k[kP];
-  uint32_t r[kP];  // bucket << 16 | rank
+  uint32_t r[kP];  // bucket << 16 | rank; kSsNone: past the end
+  if (count == kTT && in.vectors(off)) {
 #pragma unroll
-  for (int i = 0; i < kP; ++i) {
-    const uint32_t x = i * kT + threadIdx.x;
-    r[i] = x < count ? (uint32_t)ids[x] << 16 : 0u;
-    k[i] = x < count ? in.get(off + x) : 0ull;
+    for (int i = 0; i < kP; i += 4) {
+      const uint32_t v = (i / 4) * kT + threadIdx.x;
+      const ushort4 b = reinterpret_cast<const ushort4*>(ids)[v];
+      in.get4(off, v, &k[i]);
+      r[i] = (uint32_t)b.x << 16;
+      r[i + 1] = (uint32_t)b.y << 16;
+      r[i + 2] = (uint32_t)b.z << 16;
+      r[i + 3] = (uint32_t)b.w << 16;
+    }
+  } else if (count == kTT && in.keys) {
+    const uint64_t* kk = in.keys + off;
+#pragma unroll
+    for (int i = 0; i < kP; ++i) k[i] = kk[i * kT + threadIdx.x];
+#pragma unroll
+    for (int i = 0; i < kP; ++i) r[i] = (uint32_t)ids[i * kT + threadIdx.x] << 16;
+  } else {
+#pragma unroll
+    for (int i = 0; i < kP; ++i) {
+      const uint32_t x = i * kT + threadIdx.x;
+      r[i] = x < count ? (uint32_t)ids[x] << 16 : kSsNone;
+      k[i] = x < count ? in.get(off + x) : 0ull;
+    }
   }
-  uint32_t all[kPer];  // the segment's bucket sizes
+  uint32_t all[kPer];  // the segment's bucket sizes (a first split's cursors are places already)
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
     const uint32_t b = threadIdx.x * kPer + j;
-    all[j] = b < g.nb ? a.cnt[g.b0 + b] : 0u;
+    all[j] = !a.level1 && b < g.nb ? a.cnt[g.b0 + b] : 0u;
   }
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < kP; ++i)
-    if (i * kT + threadIdx.x < count) r[i] |= atomicAdd(&s_h[r[i] >> 16], 1u);
+    if (r[i] != kSsNone) r[i] |= atomicAdd(&s_h[r[i] >> 16], 1u);
   __syncthreads();
   // exclusive prefixes of the tile's counts (low) and the segment's (high)
   uint32_t got[kPer];
@@ -364,7 +410,7 @@ __global__ void __launch_bounds__(kT, kMinB) k_ss_scatter(SsArgs a) {
   uint64_t before = x - run;
 #pragma unroll
   for (int w = 0; w < kT / 32; ++w) before += w < warp ? s_w[w] : 0ull;
-  const bool lead = t == g.ft && blockIdx.x % kSub == 0;
+  const bool lead = !a.level1 && off == 0;
 #pragma unroll
   for (int j = 0; j < kPer; ++j) {
     const uint32_t b = threadIdx.x * kPer + j, c = s_h[b];
@@ -376,7 +422,7 @@ __global__ void __launch_bounds__(kT, kMinB) k_ss_scatter(SsArgs a) {
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < kP; ++i) {
-    if (i * kT + threadIdx.x < count) {
+    if (r[i] != kSsNone) {
       const uint32_t b = r[i] >> 16, pos = s_h[b] + (r[i] & 0xFFFFu);
       s_keys[pos] = k[i];
       s_ids[pos] = (uint16_t)b;
@@ -391,7 +437,7 @@ __global__ void __launch_bounds__(kT, kMinB) k_ss_scatter(SsArgs a) {
 }
 
 // ---- local sort --------------------------------------------------------------
-constexpr int kSsLT = 256;  // threads
+constexpr int kSsLT = 128;  // threads
 constexpr int kSsLP = 16;   // keys per thread
 constexpr uint32_t kSsWarpKeys = 32 * kSsLP;
 static_assert(kSsLT * kSsLP == kSsLocal, "one CTA sorts kSsLocal keys");
@@ -488,7 +534,7 @@ __device__ __forceinline__ uint32_t ss_merge_path(const uint64_t* A, uint32_t na
   return lo;
 }
 
-__global__ void __launch_bounds__(kSsLT, 4) k_ss_local(SsArgs a) {
+__global__ void __launch_bounds__(kSsLT, 8) k_ss_local(SsArgs a) {
   __shared__ uint64_t sm[kSsLocal + kSsLocal / kSsLP + 1];
   const uint32_t t = blockIdx.x / kSsPerTile;
   if (a.ntiles_d && t >= *a.ntiles_d) return;
@@ -541,9 +587,10 @@ __global__ void __launch_bounds__(kSsLT, 4) k_ss_local(SsArgs a) {
   }
 }
 
-// The second split's segments after a first one (one CTA): every bucket of a
-// segment that was split, every other segment as it is.  seg2 arrays hold
-// their starts, lengths, parents and first tiles.
+// Between count and scatter of a first split (one CTA): the starts of its
+// buckets (their cursors), and the second split's segments: every bucket of a
+// segment that is split, every other segment as it is.  seg2 arrays hold their
+// starts, lengths, parents and first tiles.
 __global__ void __launch_bounds__(1024) k_ss_plan2(SsArgs a, SsSeg2 o) {
   __shared__ uint32_t s_w[32], s_carry;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -567,25 +614,42 @@ __global__ void __launch_bounds__(1024) k_ss_plan2(SsArgs a, SsSeg2 o) {
     __syncthreads();
     return r;
   };
+  __shared__ uint2 s_big[1024];  // (segment, its first bucket's place in the list)
+  __shared__ uint32_t s_nbig;
   if (tid == 0) s_carry = 0;
   __syncthreads();
   for (uint32_t s0 = 0; s0 < a.nseg; s0 += 1024) {
     const uint32_t s = s0 + tid;
     const bool in = s < a.nseg;
     const SsSeg g = ss_seg(a, in ? s : 0);
+    if (tid == 0) s_nbig = 0;
     const uint32_t at = scan(!in ? 0u : g.nb ? g.nb : 1u);
     if (in && !g.nb) {
       o.start[at] = g.start;
       o.len[at] = g.n;
       o.parent[at] = s | kSsRawBit;
     } else if (in) {
-      for (uint32_t b = 0; b < g.nb; ++b) {
-        const uint32_t c = a.cnt[g.b0 + b];
-        o.start[at + b] = g.start + (c ? a.bstart[g.b0 + b] : 0u);
-        o.len[at + b] = c;
-        o.parent[at + b] = c && a.eq[g.b0 + b] ? kSsDone : 0u;
-      }
+      s_big[atomicAdd(&s_nbig, 1u)] = make_uint2(s, at);
     }
+    __syncthreads();
+    const uint32_t carry = s_carry;
+    for (uint32_t e = 0; e < s_nbig; ++e) {  // one thread per bucket
+      const SsSeg h = ss_seg(a, s_big[e].x);
+      const uint32_t sum = tid < h.nb ? a.cnt[h.b0 + tid] : 0u;
+      if (tid == 0) s_carry = 0;
+      __syncthreads();
+      const uint32_t run = scan(sum);
+      if (tid < h.nb) {
+        const uint32_t i = s_big[e].y + tid;
+        o.start[i] = h.start + run;
+        o.len[i] = sum;
+        o.parent[i] = sum && a.eq[h.b0 + tid] ? kSsDone : 0u;
+        a.cur[h.b0 + tid] = run;
+      }
+      __syncthreads();
+    }
+    if (tid == 0) s_carry = carry;
+    __syncthreads();
   }
   const uint32_t n2 = s_carry;
   __syncthreads();
@@ -628,8 +692,8 @@ cudaError_t set_smem_once(F* f, size_t bytes, unsigned long long* done) {
 
 }  // namespace
 
-// (r <= sqrt(n / kSsBucket) + 17 buckets of an n-key segment longer than
-// 2^18 keys: at most n / 2^13, and 1024)
+// (about sqrt(n / kSsBucket) + 1 buckets of an n-key segment, which is longer
+// than 2^18 keys: at most n / 2^13, and 1024)
 uint64_t ss_level1_buckets(uint64_t total, uint64_t nseg) {
   const uint64_t by_len = total / (1u << 13) + 1, by_seg = nseg * kSsMaxBuckets;
   return by_len < by_seg ? by_len : by_seg;
@@ -657,8 +721,7 @@ int ss_shape(uint32_t ntiles) { return ntiles <= kSsSmallTiles ? 0 : 1; }
 
 cudaError_t launch_ss_count(const SsArgs& a, cudaStream_t st) {
   if (a.ntiles == 0) return cudaSuccess;
-  if (ss_shape(a.ntiles) == 0) k_ss_count<256, 8><<<a.ntiles * 4, 256, 0, st>>>(a);
-  else k_ss_count<512, 8><<<a.ntiles * 2, 512, 0, st>>>(a);
+  k_ss_count<256, 8><<<a.ntiles * 4, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 

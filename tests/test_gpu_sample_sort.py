@@ -9,7 +9,8 @@ import oracle
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-LOCAL = 4096          # keys one CTA sorts on chip
+LOCAL = 2048          # keys one CTA sorts on chip
+BUCKET = 1366         # keys of a bucket aimed at
 ONE_LEVEL = 1 << 18   # longest segment of one split (plans below 2^24 keys)
 
 
@@ -72,10 +73,10 @@ def _check(wins, flags_sum=True, path=0):
 
 
 @pytest.mark.parametrize("kind", ["random", "few", "ones", "zero", "sorted", "misjudged"])
-@pytest.mark.parametrize("n", [1, 2, 2731, LOCAL, LOCAL + 1, 8191, 8193, 20011, 131072, ONE_LEVEL, ONE_LEVEL + 1])
+@pytest.mark.parametrize("n", [1, 2, BUCKET, LOCAL, LOCAL + 1, 2 * LOCAL, 8191, 8193, 20011, 131072, ONE_LEVEL, ONE_LEVEL + 1])
 def test_one_window(kind, n):
     if kind == "misjudged" and n <= LOCAL:
-        n += 2 * LOCAL
+        n += 4 * LOCAL
     _check([_window(kind, n, np.random.default_rng(n))])
 
 
@@ -84,7 +85,7 @@ def test_mixed_windows(path):
     rng = np.random.default_rng(5)
     sizes = [0, 1, LOCAL, LOCAL + 1, 0, 100003, ONE_LEVEL, ONE_LEVEL + 12345, 3 * ONE_LEVEL + 1, 8192]
     kinds = ["random", "few", "ones", "misjudged"]
-    _check([_window(kinds[i % 4] if n > 2 * LOCAL else "random", n, rng) for i, n in enumerate(sizes)], path=path)
+    _check([_window(kinds[i % 4] if n > 4 * LOCAL else "random", n, rng) for i, n in enumerate(sizes)], path=path)
 
 
 def test_long_windows_of_a_large_batch():
