@@ -290,7 +290,7 @@ int ans_matrix_retain(const ans_matrix* m, ans_matrix** out);
  *   d_out    : device memory (or pinned host memory) for one ans_quantities.
  *   d_status : optional device word receiving 0, or nonzero if a bounded
  *              device wait gave up (the result is then invalid).
- * All intermediate data lives in one fixed device array of about 5 MiB,
+ * All intermediate data lives in one fixed device array of about 3 MiB,
  * present on every GPU that loads the library until the process exits.
  * Every call shares that array and it keeps the previous call's contents (the
  * call clears what must start at zero); calls whose work overlaps on the GPU

@@ -885,22 +885,23 @@ int sample_sort(ans_ctx* c, char* m, const SsScratch& ss, const SegPlan& p, cons
 bool col_parts_ok(const ans_ctx* c, uint64_t max_len, bool known = true) {
   return c->col_hash && (!known || max_len <= (1ull << 25));
 }
-// Their partition counts cleared and their heavy destinations listed, between
-// the run reduction (a->hdr, a->col_ids) and k_finish over the plan `p`.
-int col_parts_begin(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& p, uint64_t max_len, StatsArgs* a,
-                    cudaStream_t st) {
+// Their partition counts and heavy sums over the plan `p` (to be cleared
+// before k_finish).
+void col_parts_begin(char* m, const PipeScratch& ps, const SegPlan& p, uint64_t max_len, StatsArgs* a, ZeroBatch* z) {
   a->cp.cnt = at<uint32_t>(m, ps.cp_cnt);
   a->cp.cur = at<uint32_t>(m, ps.cp_cur);
   a->cp.start = at<uint32_t>(m, ps.cp_start);
   a->cp.max_parts = col_parts(max_len, std::min<uint64_t>(kColMaxParts, (uint64_t)kColPerTile * p.ntiles));
-  ANS_CUDA(launch_zero(a->cp.cnt, (size_t)kColPerTile * p.ntiles * 4, st));
-  ANS_CUDA(launch_zero(a->cp.cur, (size_t)kColPerTile * p.ntiles * 4, st));
   a->cp.hkey = at<uint32_t>(m, ps.cp_hkey);
   a->cp.hsum = at<unsigned long long>(m, ps.cp_hsum);
-  if (max_len >= kColHeavyLinks) {
-    ANS_CUDA(launch_zero(a->cp.hsum, (size_t)kColHeavyPerTile * p.ntiles * 16, st));
-    ANS_CUDA(timed(c, "col_heavy", st, [&] { return launch_col_heavy(p, a->cp, a->col_ids, a->hdr, st); }));
-  }
+  z->add(a->cp.cnt, (size_t)kColPerTile * p.ntiles * 4);
+  z->add(a->cp.cur, (size_t)kColPerTile * p.ntiles * 4);
+  if (max_len >= kColHeavyLinks) z->add(a->cp.hsum, (size_t)kColHeavyPerTile * p.ntiles * 16);
+}
+// Their heavy destinations, between the run reduction and k_finish.
+int col_parts_heavy(ans_ctx* c, const SegPlan& p, uint64_t max_len, const StatsArgs& a, cudaStream_t st) {
+  if (!a.cp.cnt || max_len < kColHeavyLinks) return ANS_OK;
+  ANS_CUDA(timed(c, "col_heavy", st, [&] { return launch_col_heavy(p, a.cp, a.col_ids, a.hdr, st); }));
   return ANS_OK;
 }
 
@@ -1065,9 +1066,6 @@ int sum_order(ans_ctx* c, char* m, const PipeScratch& ps, const MatDesc* d_mats,
   if ((e = timed(c, "count_prefix", st, [&] { return launch_count_prefix(d_mats, k, at<uint64_t>(m, off_catoff), at<uint64_t>(m, off_lens),
                                at<uint64_t>(m, off_total), st); })) != cudaSuccess)
     return fail_blk(e, "count_prefix");
-  if ((e = launch_zero(seg_hist, kPasses * kRadix * 4, st)) != cudaSuccess) return fail_blk(e, "memset");
-  if ((e = launch_zero(m + ps.lb, (size_t)sp.ntiles * 8, st)) != cudaSuccess) return fail_blk(e, "memset");
-  if ((e = launch_zero(m + ps.lb2, (size_t)sp.ntiles * 8, st)) != cudaSuccess) return fail_blk(e, "memset");
   // gather zeroes the tickets and, for the radix path, builds the sum
   // segment's histograms and zeroes the sort's first status words (the
   // gather plan has at least as many tiles as the sum plan)
@@ -1077,8 +1075,13 @@ int sum_order(ans_ctx* c, char* m, const PipeScratch& ps, const MatDesc* d_mats,
   const bool merge = c->sum_path == 0 || (c->sum_path == 2 && k <= 256);
   const uint64_t* cat_off = at<uint64_t>(m, off_catoff);
   const bool in_place = merge && run_base;
+  ZeroBatch z;
+  z.add(m + ps.lb, (size_t)sp.ntiles * 8);
+  z.add(m + ps.lb2, (size_t)sp.ntiles * 8);
+  if (!merge) z.add(seg_hist, kPasses * kRadix * 4);
+  if (in_place) z.add(tickets, 32 * 4);
+  if ((e = launch_zero_batch(z, st)) != cudaSuccess) return fail_blk(e, "memset");
   if (in_place) {
-    if ((e = launch_zero(tickets, 32 * 4, st)) != cudaSuccess) return fail_blk(e, "memset");
   } else if ((e = timed(c, "gather", st, [&] {
                 return launch_gather(g, d_mats, cat_off, ka, va, merge ? nullptr : seg_hist,
                                      merge ? nullptr : at<uint64_t>(m, ps.st0), tickets, st);
@@ -1135,8 +1138,6 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
     return fail(ANS_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
   };
   cudaError_t e;
-  if ((e = launch_zero(m + ps.col_hist, kColPasses * kRadix * 4, st)) != cudaSuccess)
-    return fail_blk(e, "memset");
   uint64_t* pre = at<uint64_t>(m, ps.pre);
   if ((e = timed(c, "scan_u64", st, [&] { return launch_scan_u64(s, fv, pre, at<uint64_t>(m, ps.lb2), tickets + kPasses + 1, c->d_err, st); })) !=
       cudaSuccess)
@@ -1150,8 +1151,8 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
   a.vals = blk->vals;
   a.row_ids = blk->row_ids;
   a.row_ptr = blk->row_ptr;
-  a.run_start = at<uint64_t>(m, ps.run_start);
-  a.row_pos = at<uint64_t>(m, ps.row_pos);
+  a.run_start = at<uint32_t>(m, ps.run_start);
+  a.row_pos = at<uint32_t>(m, ps.row_pos);
   a.pre = pre;
   a.lookback = at<uint64_t>(m, ps.lb);
   a.ticket = tickets + kPasses;
@@ -1164,10 +1165,14 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
   a.mode = kModeSum;
   if (narrow) a.vals32 = (uint32_t*)at<uint64_t>(m, ps.cv_b);
   if (hgroup_ok(c, s, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
-  if ((e = launch_zero(blk->q, sizeof(ans_quantities), st)) != cudaSuccess) return fail_blk(e, "memset");
+  const uint64_t most = (uint64_t)s.ntiles * kTile;
+  ZeroBatch z;
+  z.add(blk->q, sizeof(ans_quantities));
+  if (!a.col_hkeys && col_parts_ok(c, most)) col_parts_begin(m, ps, s, most, &a, &z);
+  else z.add(m + ps.col_hist, kColPasses * kRadix * 4);
+  if ((e = launch_zero_batch(z, st)) != cudaSuccess) return fail_blk(e, "memset");
   if ((e = timed(c, "rle", st, [&] { return launch_rle(a, st); })) != cudaSuccess) return fail_blk(e, "rle");
-  if (!a.col_hkeys && col_parts_ok(c, (uint64_t)s.ntiles * kTile))
-    ANS_TRY(col_parts_begin(c, m, ps, s, (uint64_t)s.ntiles * kTile, &a, st));
+  ANS_TRY(col_parts_heavy(c, s, most, a, st));
   if ((e = timed(c, "finish", st, [&] { return launch_finish(a, st); })) != cudaSuccess) return fail_blk(e, "finish");
   return column_pass(c, a, ps, m, blk->q, st);
 }
@@ -1188,13 +1193,17 @@ int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, c
     return fail(ANS_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
   };
   int rc;
-  if ((rc = cu(launch_zero(m + ps.lb, (size_t)pk.ntiles * 8, st), "memset")) ||
-      (rc = cu(launch_zero(m + ps.col_hist, kColPasses * kRadix * 4, st), "memset")) ||
-      (rc = cu(launch_zero(blk->q, sizeof(ans_quantities), st), "memset")) ||
-      (rc = cu(launch_zero(tickets, 32 * 4, st), "memset")) ||
+  StatsArgs a;
+  if (hgroup_ok(c, pk, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
+  ZeroBatch z;
+  z.add(m + ps.lb, (size_t)pk.ntiles * 8);
+  z.add(blk->q, sizeof(ans_quantities));
+  z.add(tickets, 32 * 4);
+  if (!a.col_hkeys && col_parts_ok(c, total)) col_parts_begin(m, ps, pk, total, &a, &z);
+  else z.add(m + ps.col_hist, kColPasses * kRadix * 4);
+  if ((rc = cu(launch_zero_batch(z, st), "memset")) ||
       (rc = sample_sort(c, m, ss, pk, d_src, d_dst, total, total, two, ka, kb, at<uint16_t>(m, ps.ck_a), st)))
     return rc;
-  StatsArgs a;
   a.plan = pk;
   a.hdr = blk->hdr;
   a.q = blk->q;
@@ -1203,8 +1212,8 @@ int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, c
   a.vals = blk->vals;
   a.row_ids = blk->row_ids;
   a.row_ptr = blk->row_ptr;
-  a.run_start = at<uint64_t>(m, ps.run_start);
-  a.row_pos = at<uint64_t>(m, ps.row_pos);
+  a.run_start = at<uint32_t>(m, ps.run_start);
+  a.row_pos = at<uint32_t>(m, ps.row_pos);
   if (narrow) a.vals32 = (uint32_t*)at<uint64_t>(m, ps.cv_b);
   a.lookback = at<uint64_t>(m, ps.lb);
   a.ticket = tickets + kPasses;
@@ -1214,9 +1223,8 @@ int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, c
   a.col_tickets = tickets + 3 * 32;
   a.err = c->d_err;
   a.mode = kModeWindow;
-  if (hgroup_ok(c, pk, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
   if ((rc = cu(timed(c, "rle", st, [&] { return launch_rle(a, st); }), "rle"))) return rc;
-  if (!a.col_hkeys && col_parts_ok(c, total)) ANS_TRY(col_parts_begin(c, m, ps, pk, total, &a, st));
+  ANS_TRY(col_parts_heavy(c, pk, total, a, st));
   if ((rc = cu(timed(c, "finish", st, [&] { return launch_finish(a, st); }), "finish"))) return rc;
   return column_pass(c, a, ps, m, blk->q, st);
 }
@@ -1232,34 +1240,51 @@ int reset_err(ans_ctx* c, cudaStream_t st) {
   return ANS_OK;
 }
 
-int new_ticket(ans_ctx* c, cudaStream_t st, ans_ticket* out) {
+// A ticket's word in the pinned ring, to receive the device error word before
+// the ticket's event.
+uint32_t take_err_slot(ans_ctx* c) {
+  const uint32_t slot = (uint32_t)c->err_next;
+  c->err_next = (c->err_next + 1) % kErrSlots;
+  c->h_err_slots[slot] = 0;
+  return slot;
+}
+int add_ticket(ans_ctx* c, cudaStream_t st, uint32_t slot, ans_ticket* out) {
   ans_ctx::Ticket t;
   ANS_CUDA(cudaEventCreateWithFlags(&t.ev, cudaEventDisableTiming));
-  t.slot = c->err_next;
-  c->err_next = (c->err_next + 1) % kErrSlots;
-  c->h_err_slots[t.slot] = 0;
-  ANS_CUDA(cudaMemcpyAsync(c->h_err_slots + t.slot, c->d_err, 4, cudaMemcpyDeviceToHost, st));
+  t.slot = (int)slot;
   ANS_CUDA(cudaEventRecord(t.ev, st));
   const uint64_t id = c->next_ticket++;
   c->tickets[id] = t;
   *out = id;
   return ANS_OK;
 }
+int new_ticket(ans_ctx* c, cudaStream_t st, ans_ticket* out) {
+  const uint32_t slot = take_err_slot(c);
+  ANS_CUDA(cudaMemcpyAsync(c->h_err_slots + slot, c->d_err, 4, cudaMemcpyDeviceToHost, st));
+  return add_ticket(c, st, slot, out);
+}
 
-// The quantities to the caller's array: by a kernel when the device can
-// address it (its own memory, page-locked or managed host memory; see
-// UploadSet for why not the copy engines), else by cudaMemcpyAsync.
-int copy_quantities_out(ans_quantities* out, const ans_quantities* src, size_t n, cudaStream_t st) {
-  if (!out || n == 0) return ANS_OK;
+// `ptr` as kernels of this device can address it (its own memory, page-locked
+// or managed host memory), or null.
+void* addressable(void* ptr) {
   cudaPointerAttributes pa{};
   int dev = -1;
-  const bool known = cudaPointerGetAttributes(&pa, out) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess;
+  const bool known = cudaPointerGetAttributes(&pa, ptr) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess;
   if (!known) cudaGetLastError();
-  const bool addressable = known && (pa.type == cudaMemoryTypeHost || pa.type == cudaMemoryTypeManaged ||
-                                     (pa.type == cudaMemoryTypeDevice && pa.device == dev));
-  if (addressable) {
+  const bool ok = known && (pa.type == cudaMemoryTypeHost || pa.type == cudaMemoryTypeManaged ||
+                            (pa.type == cudaMemoryTypeDevice && pa.device == dev));
+  if (!ok) return nullptr;
+  return pa.devicePointer ? pa.devicePointer : ptr;
+}
+
+// The quantities to the caller's array: by a kernel when the device can
+// address it (see UploadSet for why not the copy engines), else by
+// cudaMemcpyAsync.
+int copy_quantities_out(ans_quantities* out, const ans_quantities* src, size_t n, cudaStream_t st) {
+  if (!out || n == 0) return ANS_OK;
+  if (void* dst = addressable(out)) {
     SmallCopyBatch b;
-    b.it[b.n++] = SmallCopyItem{pa.devicePointer ? pa.devicePointer : out, src, n * sizeof(ans_quantities)};
+    b.it[b.n++] = SmallCopyItem{dst, src, n * sizeof(ans_quantities)};
     ANS_CUDA(launch_small_copy(b, st));
     return ANS_OK;
   }
@@ -1433,7 +1458,11 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
     total = h_offsets[nwin] - h_offsets[0];
   }
   uint64_t max_len = dev ? total : 0;
-  for (uint64_t l : lens) max_len = std::max(max_len, l);
+  bool maybe_empty = dev;  // segments without a tile, whose outputs no tile writes
+  for (uint64_t l : lens) {
+    max_len = std::max(max_len, l);
+    maybe_empty = maybe_empty || l == 0;
+  }
   if (total && !h_srcs && (!d_src || !d_dst)) return fail(ANS_ERR_INVALID_ARG, "NULL packet arrays");
   const bool want_mats = (flags & ANS_BATCH_MATRICES) != 0;
   const bool want_sum = (flags & ANS_BATCH_SUM) != 0;
@@ -1657,10 +1686,15 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
     if (p.tile_seg && (rc = cu(launch_tile_seg(p, at<uint32_t>(m, wl.off_tileseg), ls), "tile segments")))
       return rc;
     if (nseg) {
-      if ((rc = cu(launch_zero(sb.q, (size_t)nseg * sizeof(ans_quantities), ls), "memset q"))) return rc;
-      if ((rc = cu(launch_zero(m + ps.lb, (size_t)hp.ntiles * 8, ls), "memset lb"))) return rc;
-      if ((rc = cu(launch_zero(m + ps.col_hist, (size_t)nseg * kColPasses * kRadix * 4, ls), "memset")))
-        return rc;
+      StatsArgs a;
+      ZeroBatch z;
+      z.add(sb.q, (size_t)nseg * sizeof(ans_quantities));
+      z.add(m + ps.lb, (size_t)hp.ntiles * 8);
+      z.add(tickets, 32 * 4);
+      if (col_parts_ok(c, max_len, !dev)) col_parts_begin(m, ps, p, max_len, &a, &z);
+      else z.add(m + ps.col_hist, (size_t)nseg * kColPasses * kRadix * 4);
+      if (hq) z.add(m + wl.off_hqwin, (size_t)nseg * sizeof(HqWin));
+      if ((rc = cu(launch_zero_batch(z, ls), "memset"))) return rc;
       // The window plan of the sort path: with hashed statistics, the windows
       // the hash finished get length 0 there (only failed windows are sorted).
       SegPlan pwin = p;
@@ -1680,7 +1714,6 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
         hb.sort_len = at<uint64_t>(m, wl.off_sortlen);
         hb.items = at<uint32_t>(m, wl.off_items);
         hb.counter = hb.items + 2 * (size_t)nseg + 1;
-        if ((rc = cu(launch_zero(hb.win, (size_t)nseg * sizeof(HqWin), ls), "memset"))) return rc;
         static const char* const kHqNames[5] = {"hq_split", "hq_links", "hq_keysplit", "hq_keyhash", "hq_mask"};
         for (int stage = 0; stage < 5; ++stage)
           if ((rc = cu(timed(c, kHqNames[stage], ls,
@@ -1741,12 +1774,10 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       }
       if (!hash && !big_ids.empty()) {
         const SegPlan pb = dev || big_ids.size() == nseg ? pwin : wl.dp_big.bind(m, hp_big);
-        if ((rc = cu(launch_zero(tickets, 32 * 4, ls), "memset")) ||
-            (rc = sample_sort(c, m, wl.ss, pb, d_src, d_dst, total, max_len, wl.ss_two_win, ka, kb,
+        if ((rc = sample_sort(c, m, wl.ss, pb, d_src, d_dst, total, max_len, wl.ss_two_win, ka, kb,
                               at<uint16_t>(m, ps.ck_a), ls)))
           return rc;
       }
-      StatsArgs a;
       a.plan = pw;
       a.hdr = sb.hdr;
       a.q = sb.q;
@@ -1755,8 +1786,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       a.vals = sb.vals;
       a.row_ids = sb.row_ids;
       a.row_ptr = sb.row_ptr;
-      a.run_start = at<uint64_t>(m, ps.run_start);
-      a.row_pos = at<uint64_t>(m, ps.row_pos);
+      a.run_start = at<uint32_t>(m, ps.run_start);
+      a.row_pos = at<uint32_t>(m, ps.row_pos);
       a.pre = pre;
       a.vals32 = (uint32_t*)at<uint64_t>(m, ps.cv_b);  // window counts fit 31 bits
       a.lookback = at<uint64_t>(m, ps.lb);
@@ -1770,11 +1801,17 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       // With merge rounds, the run reduction also writes each link's key
       // beside its stored value (keys_b at the window's padded base): the
       // windows' links are then the time sum's sorted input runs in place.
+      // (windows whose matrices nobody reads keep neither counts nor row ids)
+      if (!want_mats && (!want_sum || sum_pk)) {
+        a.vals = nullptr;
+        a.row_ids = nullptr;
+      }
       const bool in_place = want_sum && c->sum_path == 0 && !packets;
       if (in_place) a.sum_keys = kb;
-      if ((rc = cu(timed(c, "empty_fixup", ls, [&] { return launch_empty_fixup(a, ls); }), "empty"))) return rc;
+      if (maybe_empty && (rc = cu(timed(c, "empty_fixup", ls, [&] { return launch_empty_fixup(a, ls); }), "empty")))
+        return rc;
       if ((rc = cu(timed(c, "rle", ls, [&] { return launch_rle(a, ls); }), "rle"))) return rc;
-      if (col_parts_ok(c, max_len, !dev) && (rc = col_parts_begin(c, m, ps, pw, max_len, &a, ls))) return rc;
+      if ((rc = col_parts_heavy(c, pw, max_len, a, ls))) return rc;
       if ((rc = cu(timed(c, "finish", ls, [&] { return launch_finish(a, ls); }), "finish"))) return rc;
       if (in_place) {
         if ((rc = cu(cudaEventRecord(c->ev_fork, ls), "event")) ||
@@ -1825,7 +1862,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
                           std::to_string(col_parts_ok(c, max_len, !dev)) + std::to_string(col_parts_ok(c, total)) +
                           std::to_string(max_len > kColPart) + std::to_string(total > kColPart) +
                           std::to_string(max_len >= kColHeavyLinks) + std::to_string(total >= kColHeavyLinks) +
-                          std::to_string(pk_tiles >= kHGroupMinLinks / kTile) + (dev ? "/d" : "") + "/s" +
+                          std::to_string(pk_tiles >= kHGroupMinLinks / kTile) + std::to_string(maybe_empty) + (dev ? "/d" : "") + "/s" +
                           std::to_string(wl.ss_two_win) + std::to_string(wl.ss_two_pk) +
                           std::to_string(ss_shape(hp.ntiles)) + std::to_string(ss_shape(wl.ss.ntiles2)) +
                           std::to_string(ss_shape((uint32_t)pk_tiles));
@@ -1841,19 +1878,26 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       if (b) guard_addr.insert(guard_addr.end(), b->guards.begin(), b->guards.end());
     if ((rc = cu(run_guards(guard_addr, c->d_err, st), "guards"))) return bail(rc);
   }
-  if (blk) {
-    if ((rc = capture_err(c, blk->status, st))) return bail(rc);
+  BatchEnd end;
+  end.err = c->d_err;
+  if (blk) end.status[0] = blk->status;
+  if (sblk) end.status[1] = sblk->status;
+  if (out && nseg) {
+    end.dst = (uint64_t*)addressable(out);
+    if (end.dst) {
+      end.src = (const uint64_t*)sb.q;
+      end.words = (uint64_t)nseg * sizeof(ans_quantities) / 8;
+    } else {
+      ANS_CUDA(cudaMemcpyAsync(out, sb.q, (size_t)nseg * sizeof(ans_quantities), cudaMemcpyDefault, st));
+    }
   }
-  if (sblk) {
-    if ((rc = capture_err(c, sblk->status, st))) return bail(rc);
-  }
-  if (out) {
-    if ((rc = copy_quantities_out(out, sb.q, nseg, st))) return bail(rc);
-  }
+  uint32_t slot = 0;
   if (ticket) {
-    if ((rc = new_ticket(c, st, ticket))) return bail(rc);
+    slot = take_err_slot(c);
+    end.status[2] = c->h_err_slots + slot;
   }
-  if ((rc = reset_err(c, st))) return bail(rc);
+  if ((rc = cu(launch_batch_end(end, st), "batch end"))) return bail(rc);
+  if (ticket && (rc = add_ticket(c, st, slot, ticket))) return bail(rc);
   if (blk) {
     if ((rc = cu(cudaEventRecord(blk->done, st), "record"))) return bail(rc);
     blk->refs = (int)nseg;
@@ -1896,14 +1940,17 @@ int matrix_stats(ans_ctx* c, const Block* b, uint32_t seg, ans_quantities* q_out
   p.len = hdr + 1;  // nnz, on the device
   ans_quantities* q = at<ans_quantities>(m, off_q);
   uint32_t* tickets = at<uint32_t>(m, ps.tickets);
-  ANS_CUDA(cudaMemsetAsync(q, 0, sizeof(ans_quantities), st));
-  ANS_CUDA(cudaMemsetAsync(m + off_lb, 0, (size_t)std::max<uint32_t>(hp.ntiles, 1) * 8, st));
-  ANS_CUDA(cudaMemsetAsync(tickets, 0, 32 * 4, st));
-  ANS_CUDA(cudaMemsetAsync(m + ps.col_hist, 0, kColPasses * kRadix * 4, st));
+  StatsArgs a;
+  ZeroBatch z;
+  z.add(q, sizeof(ans_quantities));
+  z.add(m + off_lb, (size_t)std::max<uint32_t>(hp.ntiles, 1) * 8);
+  z.add(tickets, 32 * 4);
+  if (hp.ntiles && col_parts_ok(c, cap)) col_parts_begin(m, ps, p, cap, &a, &z);
+  else z.add(m + ps.col_hist, kColPasses * kRadix * 4);
+  ANS_CUDA(launch_zero_batch(z, st));
   uint64_t* pre = at<uint64_t>(m, off_pre);
   if (hp.ntiles) {
     ANS_CUDA(timed(c, "scan_u64", st, [&] { return launch_scan_u64(p, b->vals + bs, pre, at<uint64_t>(m, off_lb), tickets, c->d_err, st); }));
-    StatsArgs a;
     a.plan = p;
     a.hdr = hdr;
     a.q = q;
@@ -1918,7 +1965,7 @@ int matrix_stats(ans_ctx* c, const Block* b, uint32_t seg, ans_quantities* q_out
     a.col_tickets = tickets + 32;
     a.err = c->d_err;
     a.mode = kModeMatrix;
-    if (col_parts_ok(c, cap)) ANS_TRY(col_parts_begin(c, m, ps, p, cap, &a, st));
+    ANS_TRY(col_parts_heavy(c, p, cap, a, st));
     ANS_CUDA(timed(c, "finish", st, [&] { return launch_finish(a, st); }));
     ANS_TRY(column_pass(c, a, ps, m, q, st));
   }

@@ -115,12 +115,12 @@ struct StatsArgs {
   ans_quantities* q = nullptr;    // [nseg]
   const uint64_t* keys = nullptr; // sorted keys (padded space)
   uint32_t* col_ids = nullptr;    // at base[s]
-  uint64_t* vals = nullptr;       // at base[s]
+  uint64_t* vals = nullptr;       // at base[s]; null (with vals32): not kept
   uint32_t* vals32 = nullptr;     // optional uint32 copy of vals (column pass input), at base[s]
-  uint32_t* row_ids = nullptr;    // at base[s]
+  uint32_t* row_ids = nullptr;    // at base[s]; null: not kept
   uint64_t* row_ptr = nullptr;    // at base[s] + s  (nrows + 1 entries)
-  uint64_t* run_start = nullptr;  // at base[s] + s  (nnz + 1 entries); null = identity
-  uint64_t* row_pos = nullptr;    // at base[s] + s  (nrows + 1 entries); null = row_ptr
+  uint32_t* run_start = nullptr;  // at base[s] + s  (nnz + 1 entries); null = identity
+  uint32_t* row_pos = nullptr;    // at base[s] + s  (nrows + 1 entries); null = row_ptr
   const uint64_t* pre = nullptr;  // exclusive value prefix at base[s] + s; null = identity
   uint64_t* lookback = nullptr;   // [ntiles] status words (zeroed)
   uint32_t* ticket = nullptr;     // zeroed counter
@@ -485,6 +485,20 @@ cudaError_t launch_hgroup_stats(const uint32_t* keys, const uint32_t* vals32, ui
 cudaError_t launch_tile_seg(const SegPlan& p, uint32_t* tile_seg, cudaStream_t st);
 // Zero `bytes` bytes at p (4-byte aligned pointer); a kernel, unlike a memset.
 cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st);
+// Several arrays of whole words zeroed by one launch (a small batch is a chain
+// of launches of two to four microseconds each).
+struct ZeroBatch {
+  static constexpr uint32_t kMost = 8;
+  uint32_t n = 0;
+  uint32_t* p[kMost];
+  uint64_t words[kMost];
+  void add(void* ptr, size_t bytes) {  // at most kMost times
+    if (!bytes) return;
+    p[n] = static_cast<uint32_t*>(ptr);
+    words[n++] = bytes / 4;
+  }
+};
+cudaError_t launch_zero_batch(const ZeroBatch& z, cudaStream_t st);
 // Copies of small arrays by a kernel instead of the copy engines (so they
 // never queue behind other streams' bulk transfers): item i copies bytes from
 // src to dst, either of which may be page-locked host memory (read or written
@@ -524,6 +538,17 @@ cudaError_t launch_guards(const GuardList& g, uint32_t* err, cudaStream_t st);
 cudaError_t launch_guard_probe_write(uint64_t* guard, cudaStream_t st);
 // *dst = *src for one device word, by a kernel.
 cudaError_t launch_copy_word(uint32_t* dst, const uint32_t* src, cudaStream_t st);
+// The end of a batch in one launch: the error word err[0] to up to three words
+// (null: skipped; device or page-locked host memory), then cleared; `words`
+// 64-bit words of src to dst.
+struct BatchEnd {
+  uint32_t* err = nullptr;
+  uint32_t* status[3] = {nullptr, nullptr, nullptr};
+  uint64_t* dst = nullptr;
+  const uint64_t* src = nullptr;
+  uint64_t words = 0;
+};
+cudaError_t launch_batch_end(const BatchEnd& e, cudaStream_t st);
 // Zero-length segments: row_ptr[0] = 0 and hdr = {0, 0}.
 cudaError_t launch_empty_fixup(const StatsArgs& a, cudaStream_t st);
 

@@ -13,7 +13,7 @@
 // Limits and sharing:
 //  * at most kNoAllocMaxPackets (65,536) packets per call; larger windows are
 //    rejected with ANS_ERR_INVALID_ARG;
-//  * the array (kNoAllocBytes, about 5 MiB) exists on every GPU that loads
+//  * the array (kNoAllocBytes, about 3 MiB) exists on every GPU that loads
 //    the library and is held until the process exits;
 //  * every call uses the same array, and the array keeps the previous call's
 //    contents: the call clears what must start at zero itself, and calls
@@ -58,11 +58,9 @@ constexpr size_t oEq = al(oBstart + (size_t)kNoAllocTiles * kSsPerTile * 4);
 constexpr size_t oLb = al(oEq + (size_t)kNoAllocTiles * kSsPerTile);
 constexpr size_t oTickets = al(oLb + (size_t)kNoAllocTiles * 8);
 constexpr size_t oRunStart = al(oTickets + 128 * 4);
-constexpr size_t oRowPos = al(oRunStart + (kNoAllocMaxPackets + 1) * 8);
-constexpr size_t oColIds = al(oRowPos + (kNoAllocMaxPackets + 1) * 8);
-constexpr size_t oVals = al(oColIds + kNoAllocMaxPackets * 4);
-constexpr size_t oRowIds = al(oVals + kNoAllocMaxPackets * 8);
-constexpr size_t oRowPtr = al(oRowIds + kNoAllocMaxPackets * 4);
+constexpr size_t oRowPos = al(oRunStart + (kNoAllocMaxPackets + 1) * 4);
+constexpr size_t oColIds = al(oRowPos + (kNoAllocMaxPackets + 1) * 4);
+constexpr size_t oRowPtr = al(oColIds + kNoAllocMaxPackets * 4);
 constexpr size_t oHdr = al(oRowPtr + (kNoAllocMaxPackets + 1) * 8);
 constexpr size_t oQ = al(oHdr + 16);
 constexpr size_t oErr = al(oQ + sizeof(ans_quantities));
@@ -139,13 +137,16 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     return set_last_error(ANS_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(x));
   };
   int rc;
-  if ((rc = cu(cudaMemsetAsync(q, 0, sizeof(ans_quantities), st), "memset"))) return rc;
-  if ((rc = cu(cudaMemsetAsync(err, 0, 8, st), "memset"))) return rc;  // error bits; default poll limit
   const uint32_t ntiles = (uint32_t)((n + kTile - 1) / kTile);
+  ZeroBatch z;
+  z.add(q, sizeof(ans_quantities));
+  z.add(err, 8);  // error bits; default poll limit
+  z.add(m + oTickets, 32 * 4);
+  z.add(m + oLb, (size_t)ntiles * 8);
+  if (ntiles) z.add(m + oCpCnt, 2 * (size_t)kNoAllocTiles * kColPerTile * 4);
+  if (n >= kColHeavyLinks) z.add(m + oCpHsum, (size_t)ntiles * kColHeavyPerTile * 16);
+  if ((rc = cu(launch_zero_batch(z, st), "memset"))) return rc;
   if (ntiles) {
-    if ((rc = cu(cudaMemsetAsync(m + oTickets, 0, 32 * 4, st), "memset"))) return rc;
-    if ((rc = cu(cudaMemsetAsync(m + oLb, 0, (size_t)ntiles * 8, st), "memset"))) return rc;
-    if ((rc = cu(cudaMemsetAsync(m + oCpCnt, 0, 2 * (size_t)kNoAllocTiles * kColPerTile * 4, st), "memset"))) return rc;
     k_noalloc_plan<<<1, 32, 0, st>>>(n, ntiles);
     if ((rc = cu(cudaGetLastError(), "plan"))) return rc;
     SegPlan p;
@@ -186,11 +187,9 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     a.q = q;
     a.keys = ka;
     a.col_ids = reinterpret_cast<uint32_t*>(m + oColIds);
-    a.vals = reinterpret_cast<uint64_t*>(m + oVals);
-    a.row_ids = reinterpret_cast<uint32_t*>(m + oRowIds);
     a.row_ptr = reinterpret_cast<uint64_t*>(m + oRowPtr);
-    a.run_start = reinterpret_cast<uint64_t*>(m + oRunStart);
-    a.row_pos = reinterpret_cast<uint64_t*>(m + oRowPos);
+    a.run_start = reinterpret_cast<uint32_t*>(m + oRunStart);
+    a.row_pos = reinterpret_cast<uint32_t*>(m + oRowPos);
     a.pre = nullptr;
     a.lookback = reinterpret_cast<uint64_t*>(m + oLb);
     a.ticket = tickets + kPasses;
@@ -205,10 +204,7 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     a.err = err;
     a.mode = kModeWindow;
     if ((rc = cu(launch_rle(a, st), "rle"))) return rc;
-    if (n >= kColHeavyLinks &&
-        ((rc = cu(cudaMemsetAsync(a.cp.hsum, 0, (size_t)ntiles * kColHeavyPerTile * 16, st), "memset")) ||
-         (rc = cu(launch_col_heavy(p, a.cp, a.col_ids, a.hdr, st), "heavy destinations"))))
-      return rc;
+    if (n >= kColHeavyLinks && (rc = cu(launch_col_heavy(p, a.cp, a.col_ids, a.hdr, st), "heavy destinations"))) return rc;
     if ((rc = cu(launch_finish(a, st), "finish"))) return rc;
     SegPlan cp = p;
     cp.len = a.ulen;

@@ -210,6 +210,17 @@ __global__ void __launch_bounds__(256) k_gather_windows(const GatherWin* __restr
 }
 
 // One 32-bit word copied on the device (error-word snapshots).
+__global__ void __launch_bounds__(256) k_batch_end(BatchEnd e) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const uint32_t v = *e.err;
+    for (uint32_t* s : e.status)
+      if (s) *s = v;
+    *e.err = 0;
+  }
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < e.words; i += (uint64_t)gridDim.x * 256)
+    e.dst[i] = e.src[i];
+}
+
 __global__ void k_copy_word(uint32_t* dst, const uint32_t* src) { *dst = *src; }
 
 }  // namespace
@@ -245,6 +256,12 @@ cudaError_t launch_gather_windows(const GatherWin* wins, uint32_t nwin, uint32_t
 
 cudaError_t launch_guard_probe_write(uint64_t* guard, cudaStream_t st) {
   k_guard_probe_write<<<1, 1, 0, st>>>(guard);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_end(const BatchEnd& e, cudaStream_t st) {
+  const uint64_t want = (e.words + 1023) / 1024;
+  k_batch_end<<<(unsigned)(want < 1 ? 1 : (want > 1024 ? 1024 : want)), 256, 0, st>>>(e);
   return cudaGetLastError();
 }
 

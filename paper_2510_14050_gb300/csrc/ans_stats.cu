@@ -116,8 +116,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_rle(StatsArgs a) {
       s_er = er;
       if (tl.start + tl.count == tl.len) {  // last tile: terminators and header
         const uint64_t u = eh + th, r = er + tr;
-        if (a.run_start) a.run_start[bs + u] = tl.len;
-        if (a.row_pos) a.row_pos[bs + r] = tl.len;
+        if (a.run_start) a.run_start[bs + u] = (uint32_t)tl.len;
+        if (a.row_pos) a.row_pos[bs + r] = (uint32_t)tl.len;
         a.row_ptr[bs + r] = u;
         a.hdr[2 * tl.seg] = r;
         a.hdr[2 * tl.seg + 1] = u;
@@ -134,12 +134,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_rle(StatsArgs a) {
       const uint64_t u = uh + __popc(hb[i] & lt);
       a.col_ids[tl.base + u] = (uint32_t)k[i];
       if (a.sum_keys) a.sum_keys[tl.base + u] = k[i];
-      if (a.run_start) a.run_start[bs + u] = tl.start + idx;
+      if (a.run_start) a.run_start[bs + u] = (uint32_t)tl.start + idx;
       if ((rb[i] >> lane) & 1u) {
         const uint64_t r = ur + __popc(rb[i] & lt);
-        a.row_ids[tl.base + r] = (uint32_t)(k[i] >> 32);
+        if (a.row_ids) a.row_ids[tl.base + r] = (uint32_t)(k[i] >> 32);
         a.row_ptr[bs + r] = u;
-        if (a.row_pos) a.row_pos[bs + r] = tl.start + idx;
+        if (a.row_pos) a.row_pos[bs + r] = (uint32_t)tl.start + idx;
       }
     }
     uh += __popc(hb[i]);
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
       if (u >= u_end) continue;
       const uint64_t v = kMode == kModeMatrix ? x0[j] : (x1[j] - x0[j]) & kValMask;
       if (kMode != kModeMatrix) {
-        a.vals[tl.base + u] = v;
+        if (a.vals) a.vals[tl.base + u] = v;
         if (a.vals32) a.vals32[tl.base + u] = (uint32_t)v;
       }
       mlink = v > mlink ? v : mlink;
@@ -622,6 +622,12 @@ __global__ void k_wait_probe(const uint64_t* st, uint32_t* err) {
 
 // Zero `bytes` bytes at p (4-byte aligned): a kernel instead of a memset so
 // that a recorded launch sequence keeps its topology when sizes change.
+__global__ void __launch_bounds__(256) k_zero_batch(ZeroBatch z) {
+  uint32_t* p = z.p[blockIdx.y];
+  const uint64_t n = z.words[blockIdx.y];
+  for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) p[i] = 0u;
+}
+
 __global__ void k_zero(uint32_t* __restrict__ p, size_t words, uint8_t* __restrict__ tail, uint32_t ntail) {
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += stride) p[i] = 0u;
@@ -1094,6 +1100,15 @@ cudaError_t launch_tile_seg(const SegPlan& p, uint32_t* tile_seg, cudaStream_t s
 
 cudaError_t launch_wait_probe(const uint64_t* st, uint32_t* err, cudaStream_t stream) {
   k_wait_probe<<<1, 64, 0, stream>>>(st, err);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_zero_batch(const ZeroBatch& z, cudaStream_t st) {
+  if (z.n == 0) return cudaSuccess;
+  uint64_t most = 0;
+  for (uint32_t i = 0; i < z.n; ++i) most = z.words[i] > most ? z.words[i] : most;
+  const uint64_t want = (most + 1023) / 1024;
+  k_zero_batch<<<dim3((unsigned)(want < 1 ? 1 : (want > 2048 ? 2048 : want)), z.n), 256, 0, st>>>(z);
   return cudaGetLastError();
 }
 
