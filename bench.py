@@ -266,17 +266,13 @@ def kernel_bytes_per_step(name, sizes, quants, sum_q, tuning, with_matrices):
         "rle": 8 * p_all + 12 * u + 20 * r + 8 * u + 12 * us + 20 * rs,
         "finish": 32 * u + 32 * r + 28 * us + 32 * rs,
         "onesweep_col": 4 * 16 * u + 4 * 16 * us,      # (dst, u32 count) per digit pass
-        "colhash": 8 * u,
+        "col_scatter": 16 * u,                         # (dst, count) in and out
+        "col_count": 8 * u,
         "colstat": 8 * u + 8 * us,
         "gather": 28 * u,                              # link + its row in, (key, count) out
         "merge": rounds * 32 * u,                      # each round: read both runs, write the merge
         "onesweep_sum": 8 * 32 * u,                    # 8 passes over (key, count)
         "scan_u64": 16 * us,
-        "colhash_part": 24 * u,                        # regroup (read twice, write) + count (read) per link
-        "hq_split": 24 * p_all,                        # regroup packets: read twice, write once
-        "hq_links": 8 * p_all + 12 * u,                # read packets, append distinct links
-        "hq_keysplit": 2 * 3 * 8 * u,                  # two stages: read links twice, write once
-        "hq_keyhash": 2 * 8 * u,                       # two stages: read links
     }
     return rules.get(name)
 
@@ -618,8 +614,7 @@ def main(argv=None):
 
     # ---- optional comparator: a library radix sort of the same packed keys
     # (torch.sort on int64, stable: CUB's radix sort of keys with int64
-    # indices), against the path's own packet sort (eight passes carrying
-    # 16-bit window ids)
+    # indices), against the path's own packet sorts
     lib_sort = None
     if args.library_sort:
         keys = (src_d.to(torch.int64) & 0xFFFFFFFF) << 32 | (dst_d.to(torch.int64) & 0xFFFFFFFF)

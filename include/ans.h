@@ -339,13 +339,7 @@ int ans_batch_bytes(ans_ctx* ctx, const uint64_t* h_offsets, size_t nwin, uint32
  * 1 = counting links in a per-window hash table (2^k >= 2 x packets slots of
  * 12 bytes, kept by the context between calls) and sorting only the distinct
  * links with their counts (kv_* passes); worth it when windows repeat links
- * heavily; 2 = for batches that return no per-window matrix (and whose time
- * sum, if any, takes sum_path 2): every quantity of a window by counting in
- * shared-memory hash tables -- its packets grouped by link hash into
- * partitions of ~4096, one table of 8192 links per partition, then its
- * distinct links grouped by source and by destination, one table of 16384
- * keys per partition -- with no sort; a window whose table overflows, or of
- * more than 2^18 packets, is sorted instead (other batches sort as agg_path 0);
+ * heavily; 2 = as agg_path 0;
  * 3 = as agg_path 0, and for batches with a time sum, 2 to 2^16 windows and
  * the packets in one stream the sum takes sum_path 2.  Setting
  * agg_path 0 waits for the device and releases the tables.  graph: 1 = a batch's launch sequence is recorded into a CUDA
@@ -387,10 +381,8 @@ int ans_set_tuning(ans_ctx* ctx, const ans_tuning* tuning);
  * least total pass time; it then times the on-chip window sort (win_path 0,
  * three cluster configurations) and keeps it if the batch's windows sort
  * faster that way than by the sample sort, and
- * finally picks sum_path, merge_tile (with merge rounds), then agg_path (2
- * only without ANS_BATCH_MATRICES in `flags`, together with sum_path 2 when
- * the batch has a time sum; 3 only with ANS_BATCH_SUM and 2 to 2^16
- * windows, together with sum_path 2) by the batch's device time as submitted with
+ * finally picks sum_path, merge_tile (with merge rounds), then agg_path (0 or
+ * 1) by the batch's device time as submitted with
  * `flags` (ANS_BATCH_* bits of the batches the context will run; one CUDA
  * graph with its concurrent branches, between CUDA events on `stream`, the
  * host's planning included).  With those paths fixed, it last retries the

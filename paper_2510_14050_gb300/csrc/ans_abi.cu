@@ -717,7 +717,7 @@ struct PipeScratch {
   uint32_t cp_entries = 0;
   // hash-group column statistics of a time sum (buffers for up to
   // hgroup_links links, when reserved)
-  size_t hbnd = 0, hitem = 0, hpart = 0, hheavy = 0, hmeta = 0, hcnt = 0, hbuf = 0, hacc = 0;
+  size_t hbnd = 0, hitem = 0, higrp = 0, hpart = 0, hheavy = 0, hmeta = 0, hcnt = 0, hbuf = 0, hacc = 0;
   uint64_t hgroup_links = 0;
   uint32_t hgroup_cap = 0;  // parts of cut groups the buffers hold
   void reserve(Layout& L, uint64_t pad, uint32_t nseg, uint32_t ntiles, bool with_vals) {
@@ -739,6 +739,7 @@ struct PipeScratch {
       hgroup_cap = (uint32_t)(2 * (pad / kHGroupPartLinks) + 1);
       hbnd = L.add((size_t)kHGroupBounds * 4);
       hitem = L.add((size_t)kHGroupBounds * 4);
+      higrp = L.add(((size_t)kHGroups + hgroup_cap) * 4);
       hpart = L.add((size_t)kHGroupBounds * 4);
       hheavy = L.add((size_t)kHGroups * 4);
       hmeta = L.add(16);
@@ -927,8 +928,13 @@ int column_pass(ans_ctx* c, const StatsArgs& a, const PipeScratch& ps, char* m, 
   SegPlan cp = p;
   cp.len = ulen;
   if (a.cp.cnt) {
-    ANS_CUDA(timed(c, "cols", st, [&] {
-      return launch_cols(cp, a.cp, col_ids, a.vals32, a.vals, at<uint32_t>(m, ps.ck_a), at<uint64_t>(m, ps.cv_a), q, st);
+    uint32_t* pdst = at<uint32_t>(m, ps.ck_a);
+    uint64_t* pval = at<uint64_t>(m, ps.cv_a);
+    ANS_CUDA(timed(c, "col_scatter", st, [&] {
+      return launch_col_scatter(cp, a.cp, col_ids, a.vals32, a.vals, pdst, pval, st);
+    }));
+    ANS_CUDA(timed(c, "col_count", st, [&] {
+      return launch_col_count(cp, a.cp, col_ids, a.vals32, a.vals, pdst, pval, q, st);
     }));
     return ANS_OK;
   }
@@ -945,6 +951,7 @@ int column_pass(ans_ctx* c, const StatsArgs& a, const PipeScratch& ps, char* m, 
       HGroupBufs hb;
       hb.bnd = at<uint32_t>(m, ps.hbnd);
       hb.item_start = at<uint32_t>(m, ps.hitem);
+      hb.item_group = at<uint32_t>(m, ps.higrp);
       hb.hpart = at<uint32_t>(m, ps.hpart);
       hb.heavy = at<uint32_t>(m, ps.hheavy);
       hb.meta = at<uint32_t>(m, ps.hmeta);
@@ -1031,7 +1038,7 @@ int sum_prepare(ans_ctx* c, char* m, uint32_t k, const std::vector<uint64_t>& ca
 // caller at `m` / `ps` (which must provide vals buffers).  Only queues work
 // on `st` (it may be capturing); on failure the caller discards plan->blk.
 int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s, const uint64_t* fk,
-                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow = false);
+                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow = false, bool cols = true);
 
 // First half of the time sum: the input links gathered and ordered (merge
 // rounds, or the kv passes with sum_path 1), left in (*fk, *fv).  Touches
@@ -1121,18 +1128,20 @@ int sum_order(ans_ctx* c, char* m, const PipeScratch& ps, const MatDesc* d_mats,
 // narrow: every count of the sum is known to stay below 2^32 (the column
 // pass then carries 32-bit counts).
 int sum_launch(ans_ctx* c, char* m, const PipeScratch& ps, const MatDesc* d_mats, uint32_t k, SumPlan* plan,
-               size_t off_catoff, size_t off_lens, size_t off_total, cudaStream_t st, bool narrow = false) {
+               size_t off_catoff, size_t off_lens, size_t off_total, cudaStream_t st, bool narrow = false,
+               bool cols = true) {
   const uint64_t *fk = nullptr, *fv = nullptr;
   ANS_TRY(sum_order(c, m, ps, d_mats, k, plan, off_catoff, off_lens, off_total, st, &fk, &fv));
-  return links_to_block(c, m, ps, plan->s, fk, fv, plan->blk, st, narrow);
+  return links_to_block(c, m, ps, plan->s, fk, fv, plan->blk, st, narrow, cols);
 }
 
 // From sorted (key, value) links (equal keys adjacent) of the single segment
 // of `s` to a DCSR block: value prefix, run-length reduction, values as
 // prefix differences, row statistics and the column pass (the time sum's
-// statistics half).  Only queues work on `st`.
+// statistics half).  cols false: without column statistics (a block that is
+// only gathered again).  Only queues work on `st`.
 int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s, const uint64_t* fk,
-                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow) {
+                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow, bool cols) {
   uint32_t* tickets = at<uint32_t>(m, ps.tickets) + 32;
   auto fail_blk = [&](cudaError_t e, const char* what) {
     return fail(ANS_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
@@ -1164,17 +1173,18 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
   a.err = c->d_err;
   a.mode = kModeSum;
   if (narrow) a.vals32 = (uint32_t*)at<uint64_t>(m, ps.cv_b);
-  if (hgroup_ok(c, s, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
+  a.no_cols = !cols;
+  if (cols && hgroup_ok(c, s, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
   const uint64_t most = (uint64_t)s.ntiles * kTile;
   ZeroBatch z;
   z.add(blk->q, sizeof(ans_quantities));
-  if (!a.col_hkeys && col_parts_ok(c, most)) col_parts_begin(m, ps, s, most, &a, &z);
+  if (cols && !a.col_hkeys && col_parts_ok(c, most)) col_parts_begin(m, ps, s, most, &a, &z);
   else z.add(m + ps.col_hist, kColPasses * kRadix * 4);
   if ((e = launch_zero_batch(z, st)) != cudaSuccess) return fail_blk(e, "memset");
   if ((e = timed(c, "rle", st, [&] { return launch_rle(a, st); })) != cudaSuccess) return fail_blk(e, "rle");
   ANS_TRY(col_parts_heavy(c, s, most, a, st));
   if ((e = timed(c, "finish", st, [&] { return launch_finish(a, st); })) != cudaSuccess) return fail_blk(e, "finish");
-  return column_pass(c, a, ps, m, blk->q, st);
+  return cols ? column_pass(c, a, ps, m, blk->q, st) : ANS_OK;
 }
 
 // Time sum of a batch from its packets (sum_path 2): every packet of the
@@ -1378,7 +1388,6 @@ struct WinLayout {
   DevPlan dp, dp_big;  // every window; the windows sorted by onesweep passes
   size_t off_small = 0;  // ids of the windows sorted on chip
   size_t off_tileseg = 0; // the window plan's segment of every tile
-  size_t off_hqwin = 0, off_lstart = 0, off_kstart = 0, off_sortlen = 0, off_items = 0;  // hashed window statistics
   DevPlan dp_tab;        // hash path: the windows' tables as segments
   DevPlan dp_pk;         // sum_path 2: all packets of the batch as one segment
   size_t off_tlg = 0, off_special = 0, off_hulen = 0, off_nclaim = 0, off_claims = 0;
@@ -1398,11 +1407,6 @@ struct WinLayout {
     dp_big.reserve(L, nseg, addrs);
     off_small = L.add((size_t)nseg * 4);
     off_tileseg = L.add((size_t)hp.ntiles * 4);
-    off_hqwin = L.add((size_t)nseg * sizeof(HqWin));
-    off_lstart = L.add((size_t)nseg * 65 * 4);
-    off_kstart = L.add((size_t)nseg * 2 * 65 * 4);
-    off_sortlen = L.add((size_t)nseg * 8);
-    off_items = L.add(((size_t)2 * nseg + 2) * 4);
     dp_pk.reserve(L, 1);
     if (hash) {
       dp_tab.reserve(L, nseg);
@@ -1496,10 +1500,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   std::vector<uint32_t> small_ids, big_ids;
   const int win_path = c->win_path;  // the caller holds c->mu
   const SortCfg cfg_win = c->cfg_win;
-  // (hashed window statistics, agg_path 2, sort only the windows the hash
-  // gives up on: those take the key passes)
   const bool packets = agg_packets(c, nseg, want_sum, h_srcs != nullptr);
-  const bool on_chip = !dev && win_path == 0 && !(c->agg_path == 2 && !want_mats) && !packets &&
+  const bool on_chip = !dev && win_path == 0 && !packets &&
                        cluster_sort_clusters(c->device) > 0;
   for (uint32_t s = 0; s < nseg; ++s) {
     if (on_chip && lens[s] <= kClusterWindowMax) small_ids.push_back(s);
@@ -1581,9 +1583,6 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   // batches: its offset and length come from the planner, the tile count is
   // the capacity's)
   const bool sum_pk = want_sum && nseg && (c->sum_path == 2 || packets) && !h_srcs;
-  // agg_path 2: the windows' quantities by on-chip hashing, when no window
-  // DCSR is returned and the time sum (if any) comes from the packets
-  const bool hq = c->agg_path == 2 && nseg && !want_mats && (!want_sum || sum_pk);
   HostPlan hp_pk;
   if (sum_pk) {
     std::vector<uint64_t> pk_off{dev ? 0 : h_offsets[0]};
@@ -1693,36 +1692,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       z.add(tickets, 32 * 4);
       if (col_parts_ok(c, max_len, !dev)) col_parts_begin(m, ps, p, max_len, &a, &z);
       else z.add(m + ps.col_hist, (size_t)nseg * kColPasses * kRadix * 4);
-      if (hq) z.add(m + wl.off_hqwin, (size_t)nseg * sizeof(HqWin));
       if ((rc = cu(launch_zero_batch(z, ls), "memset"))) return rc;
-      // The window plan of the sort path: with hashed statistics, the windows
-      // the hash finished get length 0 there (only failed windows are sorted).
-      SegPlan pwin = p;
-      if (hq) {
-        HqBufs hb;
-        hb.keys = kb;
-        hb.lsrc = at<uint32_t>(m, ps.ck_a);
-        hb.ldst = at<uint32_t>(m, ps.ck_b);
-        hb.lcnt = (uint32_t*)at<uint64_t>(m, ps.cv_a);
-        hb.pkey[0] = (uint32_t*)at<uint64_t>(m, ps.cv_b);
-        hb.pval[0] = hb.pkey[0] + hp.pad;
-        hb.pkey[1] = (uint32_t*)ka;  // the window sort's keys: free until the failed windows are sorted
-        hb.pval[1] = hb.pkey[1] + hp.pad;
-        hb.lstart = at<uint32_t>(m, wl.off_lstart);
-        hb.kstart = at<uint32_t>(m, wl.off_kstart);
-        hb.win = at<HqWin>(m, wl.off_hqwin);
-        hb.sort_len = at<uint64_t>(m, wl.off_sortlen);
-        hb.items = at<uint32_t>(m, wl.off_items);
-        hb.counter = hb.items + 2 * (size_t)nseg + 1;
-        static const char* const kHqNames[5] = {"hq_split", "hq_links", "hq_keysplit", "hq_keyhash", "hq_mask"};
-        for (int stage = 0; stage < 5; ++stage)
-          if ((rc = cu(timed(c, kHqNames[stage], ls,
-                             [&] { return launch_hq_stage(stage, p, d_src, d_dst, hb, ls); }),
-                       "hash statistics")))
-            return rc;
-        pwin.len = hb.sort_len;
-      }
-      SegPlan pw = pwin;  // the plan of the statistics phases
+      SegPlan pw = p;  // the plan of the statistics phases
       int mode = kModeWindow;
       uint64_t* pre = nullptr;
       if (hash) {
@@ -1767,13 +1738,13 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
       if (!hash && !small_ids.empty()) {
         const uint32_t* ids = small_ids.size() == nseg ? nullptr : at<uint32_t>(m, wl.off_small);
         if ((rc = cu(timed(c, "cluster_sort", ls, [&] {
-                       return launch_cluster_sort(pwin, ids, (uint32_t)small_ids.size(), d_src, d_dst, ka, tickets,
+                       return launch_cluster_sort(p, ids, (uint32_t)small_ids.size(), d_src, d_dst, ka, tickets,
                                                   cfg_win, ls);
                      }), "cluster sort")))
           return rc;
       }
       if (!hash && !big_ids.empty()) {
-        const SegPlan pb = dev || big_ids.size() == nseg ? pwin : wl.dp_big.bind(m, hp_big);
+        const SegPlan pb = dev || big_ids.size() == nseg ? p : wl.dp_big.bind(m, hp_big);
         if ((rc = sample_sort(c, m, wl.ss, pb, d_src, d_dst, total, max_len, wl.ss_two_win, ka, kb,
                               at<uint16_t>(m, ps.ck_a), ls)))
           return rc;
@@ -1824,8 +1795,6 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
         if (rc == ANS_OK) rc = cu(ej, "event");
       }
       if (rc == ANS_OK) rc = column_pass(c, a, ps, m, sb.q, ls);
-      if (rc == ANS_OK && hq)  // the hashed windows' quantities over the (empty) sorted results
-        rc = cu(launch_hq_write(p, at<HqWin>(m, wl.off_hqwin), sb.q, ls), "hash statistics");
       if (forked) {  // join (also after a failure, so that a capture ends joined)
         const cudaError_t ew = cudaStreamWaitEvent(ls, c->ev_join, 0);
         if (rc == ANS_OK) rc = cu(ew, "event");
@@ -1861,6 +1830,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   const std::string sig = launch_sig(flags, hp.ntiles > 0, !small_ids.empty(), !big_ids.empty(), rounds, c) + "/h" +
                           std::to_string(col_parts_ok(c, max_len, !dev)) + std::to_string(col_parts_ok(c, total)) +
                           std::to_string(max_len > kColPart) + std::to_string(total > kColPart) +
+                          std::to_string(max_len > 512 * (uint64_t)kColPart) + std::to_string(total > 512 * (uint64_t)kColPart) +
                           std::to_string(max_len >= kColHeavyLinks) + std::to_string(total >= kColHeavyLinks) +
                           std::to_string(pk_tiles >= kHGroupMinLinks / kTile) + std::to_string(maybe_empty) + (dev ? "/d" : "") + "/s" +
                           std::to_string(wl.ss_two_win) + std::to_string(wl.ss_two_pk) +
@@ -1973,10 +1943,10 @@ int matrix_stats(ans_ctx* c, const Block* b, uint32_t seg, ans_quantities* q_out
 }
 
 // Drop the stored zeros of a signed combination: the links of `blk` (one
-// matrix, at most cap links) are gathered as (key, value), the nonzero ones
-// compacted in order, and the statistics rebuilt into a new block *out.  A
+// matrix, at most cap links; narrow: the result's counts stay below 2^32) are
+// gathered as (key, value), the nonzero ones compacted in order, and the statistics rebuilt into a new block *out.  A
 // negative count sets kErrNegative in the context's error word.
-int drop_zeros(ans_ctx* c, Block* blk, uint64_t cap, cudaStream_t st, Block** out) {
+int drop_zeros(ans_ctx* c, Block* blk, uint64_t cap, bool narrow, cudaStream_t st, Block** out) {
   *out = nullptr;
   HostPlan sp;
   sp.build(std::vector<uint64_t>{cap}, nullptr);
@@ -2033,7 +2003,7 @@ int drop_zeros(ans_ctx* c, Block* blk, uint64_t cap, cudaStream_t st, Block** ou
     return bail(rc);
   SegPlan s2 = s;
   s2.len = count;
-  if ((rc = links_to_block(c, m, ps, s2, kb, vb, plan.blk, st))) return bail(rc);
+  if ((rc = links_to_block(c, m, ps, s2, kb, vb, plan.blk, st, narrow))) return bail(rc);
   *out = plan.blk;
   return ANS_OK;
 }
@@ -2050,6 +2020,10 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
   std::vector<MatDesc> md;
   uint64_t total_cap = 0;
   bool any_neg = false;
+  // every count of the result stays below 2^32 if the inputs hold fewer
+  // packets in all (known once they have been computed)
+  uint64_t packets = 0;
+  bool narrow = true;
   for (size_t i = 0; i < k; ++i) {
     const ans_matrix* x = mats[i];
     if (!x) return fail(ANS_ERR_INVALID_ARG, "NULL matrix");
@@ -2067,8 +2041,12 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
     if (cudaEventQuery(b->done) == cudaSuccess) {
       ANS_TRY(block_fill_cache(const_cast<Block*>(b)));
       cap = std::min<uint64_t>(cap, b->h_hdr[2 * (size_t)x->seg + 1]);
+      const uint64_t held = b->h_q[x->seg].valid_packets;
+      narrow = narrow && held < (1ull << 32) - packets;
+      if (narrow) packets += held;
     } else {
       cudaGetLastError();
+      narrow = false;
     }
     caps.push_back(cap);
     total_cap += cap;
@@ -2107,7 +2085,8 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
       block_discard(sump.blk, st);
       return rc;
     }
-    rc = sum_launch(c, m, ps, at<MatDesc>(m, off_mats), (uint32_t)k, &sump, off_catoff, off_lens, off_total, st);
+    rc = sum_launch(c, m, ps, at<MatDesc>(m, off_mats), (uint32_t)k, &sump, off_catoff, off_lens, off_total, st,
+                    narrow && !any_neg, !any_neg);
     if (rc) {
       block_discard(sump.blk, st);
       return rc;
@@ -2115,7 +2094,7 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
     sblk = sump.blk;
     if (any_neg) {  // cancelled links are stored as zeros: compact them away
       Block* clean = nullptr;
-      rc = drop_zeros(c, sblk, total_cap, st, &clean);
+      rc = drop_zeros(c, sblk, total_cap, narrow, st, &clean);
       block_discard(sblk, st);
       if (rc) return rc;
       sblk = clean;
@@ -2351,9 +2330,9 @@ int ans_batch_submit_windows(ans_ctx* c, const uint32_t* const* srcs, const uint
       }
     }
   }
-  // The paths that sort all of a batch's packets as one segment (the windows
-  // from the packet sort, the time sum by re-sorting the packets, the hashed
-  // statistics) read the packets as one stream: the windows' pairs are first
+  // The paths that sort all of a batch's packets as one segment (the time sum
+  // by re-sorting the packets) read the packets as one stream, and every sort
+  // of packets reads them twice: the windows' pairs are first
   // gathered into one device buffer by a kernel (reading each window in
   // place), then analysed like contiguous windows.  If that buffer cannot be
   // had, the windows are analysed in place on the other paths.
@@ -2997,8 +2976,7 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
 
   // Time sums (pairwise merges, whose ordering runs beside the window column
   // pass, against the kv passes and the packet re-sort) and then window
-  // aggregation (sorting every packet, hash counting of links, or -- without
-  // per-window matrices -- every quantity by on-chip hashing): each by the
+  // aggregation (sorting every packet, or hash counting of links): each by the
   // batch's device time as the production path runs it with the caller's
   // flags, everything else as chosen.
   run_flags = flags;
@@ -3042,32 +3020,24 @@ int ans_autotune(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const
     merge_tile = wall[1] < wall[0] ? 2048 : 4096;
     c->merge_tile = merge_tile;
   }
+  // (agg_path 2 is agg_path 0, and agg_path 3 is that with sum_path 2: both
+  // have been timed)
   int agg_path = 0;
   {
-    // hashed statistics need no window DCSR, and a time sum from the packets;
-    // the windows' order from the packet sort needs a time sum (and takes
-    // it from the packets)
-    const bool want_sum = (flags & ANS_BATCH_SUM) != 0;
-    const bool ok[4] = {true, true, !(flags & ANS_BATCH_MATRICES),
-                        want_sum && nwin >= 2 && nwin <= kMaxPacketWindows};
-    const int sum_for[4] = {sum_path, sum_path, want_sum ? 2 : sum_path, 2};
-    double wall[4] = {kNever, kNever, kNever, kNever};
-    for (int a = 0; a < 4; ++a) {
-      if (!ok[a]) continue;
+    double wall[2] = {kNever, kNever};
+    for (int a = 0; a < 2; ++a) {
       Prof pr;
       bool ran = false;
       ANS_TRY(trial([&] {
         base();
         c->win_path = win_path;
         c->cfg_win = win_cfg;
-        c->sum_path = sum_for[a];
+        c->sum_path = sum_path;
         c->agg_path = a;
       }, &pr, &ran));
       if (ran) wall[a] = pr[kWall];
     }
-    for (int a = 1; a < 4; ++a)
-      if (wall[a] < wall[agg_path]) agg_path = a;
-    sum_path = sum_for[agg_path];
+    if (wall[1] < wall[0]) agg_path = 1;
   }
 
   // With the paths chosen, the column passes' shape (on the large time sums

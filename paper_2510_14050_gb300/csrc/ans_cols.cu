@@ -100,7 +100,7 @@ __device__ __forceinline__ ColSeg col_seg(const SegPlan& p, uint32_t s, uint32_t
 
 // One sub-tile of kT * kP links per CTA.  kWide: 64-bit counts.
 template <bool kWide, int kT, int kP>
-__global__ void __launch_bounds__(kT) k_col_scatter(SegPlan p, ColParts c, const uint32_t* __restrict__ col_ids,
+__global__ void __launch_bounds__(kT, kP == 16 ? (kWide ? 1 : 2) : kT == 512 ? 3 : 4) k_col_scatter(SegPlan p, ColParts c, const uint32_t* __restrict__ col_ids,
                                                     const uint32_t* __restrict__ vals32,
                                                     const uint64_t* __restrict__ vals64, uint32_t* __restrict__ odst,
                                                     void* __restrict__ oval) {
@@ -149,8 +149,16 @@ __global__ void __launch_bounds__(kT) k_col_scatter(SegPlan p, ColParts c, const
   uint32_t* cur = c.cur + (size_t)g.ft * kColPerTile;
   const uint32_t per = (g.parts + kT - 1) / kT;
   const uint32_t b0 = min(threadIdx.x * per, g.parts), b1 = min(b0 + per, g.parts);
+  constexpr int kB = kP == 16 ? 4 : 1;  // partitions whose loads and atomics are in flight together
   uint64_t run = 0;
-  for (uint32_t b = b0; b < b1; ++b) run += (uint64_t)cnt[b] << 32 | s_h[b];
+  for (uint32_t c0 = b0; c0 < b1; c0 += kB) {
+    uint32_t all[kB];
+#pragma unroll
+    for (int j = 0; j < kB; ++j) all[j] = c0 + j < b1 ? cnt[c0 + j] : 0u;
+#pragma unroll
+    for (int j = 0; j < kB; ++j)
+      if (c0 + j < b1) run += (uint64_t)all[j] << 32 | s_h[c0 + j];
+  }
   uint64_t x = run;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -167,13 +175,25 @@ __global__ void __launch_bounds__(kT) k_col_scatter(SegPlan p, ColParts c, const
     moved += (uint32_t)s_w[w];
   }
   const bool lead = off == 0;
-  for (uint32_t b = b0; b < b1; ++b) {
-    const uint32_t k = s_h[b], slot = (uint32_t)before, start = (uint32_t)(before >> 32);
-    const uint32_t got = k ? atomicAdd(&cur[b], k) : 0u;
-    s_h[b] = slot;
-    s_rel[b] = start + got - slot;
-    if (lead) c.start[(size_t)g.ft * kColPerTile + b] = start;
-    before += (uint64_t)cnt[b] << 32 | k;
+  for (uint32_t c0 = b0; c0 < b1; c0 += kB) {
+    uint32_t all[kB], k[kB], got[kB];
+#pragma unroll
+    for (int j = 0; j < kB; ++j) {
+      const bool in = c0 + j < b1;
+      all[j] = in ? cnt[c0 + j] : 0u;
+      k[j] = in ? s_h[c0 + j] : 0u;
+      got[j] = k[j] ? atomicAdd(&cur[c0 + j], k[j]) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kB; ++j) {
+      if (c0 + j < b1) {
+        const uint32_t slot = (uint32_t)before, start = (uint32_t)(before >> 32);
+        s_h[c0 + j] = slot;
+        s_rel[c0 + j] = start + got[j] - slot;
+        if (lead) c.start[(size_t)g.ft * kColPerTile + c0 + j] = start;
+        before += (uint64_t)all[j] << 32 | k[j];
+      }
+    }
   }
   __syncthreads();
 #pragma unroll
@@ -363,18 +383,27 @@ cudaError_t scatter(const SegPlan& p, const ColParts& c, const uint32_t* col_ids
 }
 
 template <bool kWide>
-cudaError_t run_cols(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
-                     const uint64_t* vals64, uint32_t* odst, void* oval, ans_quantities* q, cudaStream_t st) {
-  cudaError_t e;
-  if (c.max_parts > 1) {
-    // (small plans: 2048 links per CTA fill the SMs sooner)
-    e = p.ntiles <= 608 ? scatter<kWide, 256, 8>(p, c, col_ids, vals32, vals64, odst, oval, st)
-                        : scatter<kWide, 512, 8>(p, c, col_ids, vals32, vals64, odst, oval, st);
-    if (e != cudaSuccess) return e;
-  }
+cudaError_t run_scatter(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                        const uint64_t* vals64, uint32_t* odst, void* oval, cudaStream_t st) {
+  if (c.max_parts <= 1) return cudaSuccess;
+  // With many partitions a CTA pays an atomic for nearly every one of them, so
+  // it takes a whole tile (3 million links, 1108 partitions, 64-bit counts: 48
+  // us, 85 by 2048 links); else 4096 links per CTA are faster (2^28 packets in
+  // windows of 2^17: 1.30 against 1.63 ms), and 2048 fill the SMs sooner for
+  // small plans.
+  if (c.max_parts > 512) return scatter<kWide, 512, 16>(p, c, col_ids, vals32, vals64, odst, oval, st);
+  return p.ntiles <= 608 ? scatter<kWide, 256, 8>(p, c, col_ids, vals32, vals64, odst, oval, st)
+                         : scatter<kWide, 512, 8>(p, c, col_ids, vals32, vals64, odst, oval, st);
+}
+
+template <bool kWide>
+cudaError_t run_count(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                      const uint64_t* vals64, const uint32_t* odst, const void* oval, ans_quantities* q,
+                      cudaStream_t st) {
   constexpr size_t kSmem = (size_t)kColSlots * (kWide ? 16 : 12);
   static unsigned long long done = 0;
-  if ((e = set_smem_once(k_col_count<kWide>, kSmem, &done)) != cudaSuccess) return e;
+  const cudaError_t e = set_smem_once(k_col_count<kWide>, kSmem, &done);
+  if (e != cudaSuccess) return e;
   k_col_count<kWide><<<p.ntiles * kColPerTile, kColThreads, kSmem, st>>>(p, c, col_ids, vals32, vals64, odst, oval, q);
   return cudaGetLastError();
 }
@@ -388,11 +417,19 @@ cudaError_t launch_col_heavy(const SegPlan& p, const ColParts& c, const uint32_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_cols(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
-                        const uint64_t* vals64, uint32_t* odst, void* oval, ans_quantities* q, cudaStream_t st) {
+cudaError_t launch_col_scatter(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                               const uint64_t* vals64, uint32_t* odst, void* oval, cudaStream_t st) {
   if (p.ntiles == 0) return cudaSuccess;
-  return vals32 ? run_cols<false>(p, c, col_ids, vals32, nullptr, odst, oval, q, st)
-                : run_cols<true>(p, c, col_ids, nullptr, vals64, odst, oval, q, st);
+  return vals32 ? run_scatter<false>(p, c, col_ids, vals32, nullptr, odst, oval, st)
+                : run_scatter<true>(p, c, col_ids, nullptr, vals64, odst, oval, st);
+}
+
+cudaError_t launch_col_count(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                             const uint64_t* vals64, const uint32_t* odst, const void* oval, ans_quantities* q,
+                             cudaStream_t st) {
+  if (p.ntiles == 0) return cudaSuccess;
+  return vals32 ? run_count<false>(p, c, col_ids, vals32, nullptr, odst, oval, q, st)
+                : run_count<true>(p, c, col_ids, nullptr, vals64, odst, oval, q, st);
 }
 
 }  // namespace ans

@@ -86,7 +86,7 @@ struct SegPlan {
 // sizes (counted by k_finish), cursors (both zeroed before) and starts, kColPerTile
 // entries per tile of the plan.
 constexpr uint32_t kColPerTile = 3;
-constexpr uint32_t kColMaxParts = 8192;
+constexpr uint32_t kColMaxParts = 2048;
 constexpr uint32_t kColPart = (kTile + kColPerTile - 1) / kColPerTile;  // links per partition aimed at
 // Hash partitions of a segment of n links.
 constexpr uint32_t col_parts(uint64_t n, uint32_t max_parts) {
@@ -140,6 +140,7 @@ struct StatsArgs {
   // Or (cp.cnt set): k_finish counts the links' hash partitions instead of
   // their destination digits.
   ColParts cp;
+  bool no_cols = false;  // or nothing of the two
   int mode = 0;
 };
 
@@ -205,48 +206,6 @@ struct DevPlanOut {
   const uint64_t* vals = nullptr;
   const uint64_t* hdr = nullptr;
 };
-
-// ---- window quantities by on-chip hashing (ans_winhash.cu) -----------------
-constexpr uint32_t kHqMaxPackets = 1u << 18;  // larger windows are sorted
-// Per-window accumulator of the hashed statistics (zeroed before the batch):
-// the link stage's distinct links and largest count, then per stage (0 =
-// sources, 1 = destinations) the distinct keys, the largest number of links
-// of a key (fan-out / fan-in) and the largest packet count of a key; fail =
-// some table overflowed (the window is sorted instead); nlinks = the
-// window's distinct links appended so far.
-struct HqWin {
-  unsigned long long links, max_link;
-  unsigned long long keys[2], max_links[2], max_packets[2];
-  uint32_t fail, nlinks;
-};
-// Device buffers of the hashed statistics (keys: packets regrouped by link
-// partition, at each window's padded base; lsrc / ldst / lcnt: the windows'
-// distinct links; pkey[st] / pval[st]: links regrouped by source (st = 0) or
-// destination (1) partition; lstart: 65 link-partition starts per window;
-// kstart: 65 key-partition starts per window and stage, stage 0 first;
-// sort_len: the plan lengths the sort path then uses).
-struct HqBufs {
-  uint64_t* keys = nullptr;
-  uint32_t* lsrc = nullptr;
-  uint32_t* ldst = nullptr;
-  uint32_t* lcnt = nullptr;
-  uint32_t* pkey[2] = {nullptr, nullptr};
-  uint32_t* pval[2] = {nullptr, nullptr};
-  uint32_t* lstart = nullptr;
-  uint32_t* kstart = nullptr;
-  HqWin* win = nullptr;
-  uint64_t* sort_len = nullptr;
-  uint32_t* items = nullptr;    // work-item prefix of the counting steps (2 * nseg + 1)
-  uint32_t* counter = nullptr;  // their queue counter
-};
-// The hashed statistics of every window of p (win zeroed by the caller), in
-// five launches, stage 0 .. 4: regroup packets by link partition, count
-// links, regroup the distinct links by source and destination partition,
-// count sources and destinations, set sort_len.  The quantities are written
-// by launch_hq_write once the sort path has run over sort_len.
-cudaError_t launch_hq_stage(int stage, const SegPlan& p, const uint32_t* src, const uint32_t* dst, const HqBufs& b,
-                            cudaStream_t st);
-cudaError_t launch_hq_write(const SegPlan& p, const HqWin* win, ans_quantities* q, cudaStream_t st);
 
 // ---- row partition across ranks (ans_split.cu) ----------------------------
 constexpr uint32_t kMaxSplitParts = 64;
@@ -441,8 +400,11 @@ cudaError_t launch_col_heavy(const SegPlan& p, const ColParts& c, const uint32_t
 // odst / oval (uint32 counts with vals32, uint64 counts with vals64; at the
 // segments' bases) and counted in shared-memory tables; the three column
 // quantities are combined into q.
-cudaError_t launch_cols(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
-                        const uint64_t* vals64, uint32_t* odst, void* oval, ans_quantities* q, cudaStream_t st);
+cudaError_t launch_col_scatter(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                               const uint64_t* vals64, uint32_t* odst, void* oval, cudaStream_t st);
+cudaError_t launch_col_count(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
+                             const uint64_t* vals64, const uint32_t* odst, const void* oval, ans_quantities* q,
+                             cudaStream_t st);
 // One bounded look-back wait (both forms: the single-thread walk of the
 // radix passes and the warp walk of the run reductions and scans) for the
 // predecessor of tile 1 of a chain whose tile 0 never publishes (st: two
@@ -471,6 +433,7 @@ constexpr uint32_t kHGroupPartWords = 3 * ((1u << 13) / 4 * 3 + 1);  // a part's
 struct HGroupBufs {
   uint32_t* bnd = nullptr;         // [kHGroupBounds] group starts
   uint32_t* item_start = nullptr;  // [kHGroupBounds] first work item of each group
+  uint32_t* item_group = nullptr;  // [kHGroups + max_hparts] the group of each work item
   uint32_t* hpart = nullptr;       // [kHGroupBounds] first part (of cut groups) of each group
   uint32_t* heavy = nullptr;       // [kHGroups] the cut groups
   uint32_t* meta = nullptr;        // [4] items, cut groups, their parts

@@ -208,8 +208,9 @@ extern "C" int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32
     if ((rc = cu(launch_finish(a, st), "finish"))) return rc;
     SegPlan cp = p;
     cp.len = a.ulen;
-    if ((rc = cu(launch_cols(cp, a.cp, a.col_ids, a.vals32, nullptr, reinterpret_cast<uint32_t*>(m + oCk), m + oCv, q, st),
-                 "column statistics")))
+    uint32_t* pdst = reinterpret_cast<uint32_t*>(m + oCk);
+    if ((rc = cu(launch_col_scatter(cp, a.cp, a.col_ids, a.vals32, nullptr, pdst, m + oCv, st), "column statistics")) ||
+        (rc = cu(launch_col_count(cp, a.cp, a.col_ids, a.vals32, nullptr, pdst, m + oCv, q, st), "column statistics")))
       return rc;
   }
   if ((rc = cu(cudaMemcpyAsync(d_out, q, sizeof(ans_quantities), cudaMemcpyDefault, st), "copy out"))) return rc;

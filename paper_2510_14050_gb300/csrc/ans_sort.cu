@@ -323,22 +323,30 @@ __global__ void __launch_bounds__(kThreads) k_gather(SegPlan p, const MatDesc* _
   __syncthreads();
   const uint64_t o = cat_off[tl.seg] + tl.start;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // A warp's links are consecutive and every row holds one at least: after a
+  // search of all rows for its first link, the rows of its next 32 links are
+  // among the 33 from the last one's (5 steps instead of up to 13).
+  uint32_t from = 0, span = nr;
   for (int it = 0; it < kPerThread; ++it) {
     const uint32_t i = warp * (kPerThread * 32) + it * 32 + lane;
     const bool valid = i < tl.count;
     const uint32_t vmask = __ballot_sync(0xffffffffu, valid);
     uint64_t key = 0;
+    uint32_t row = 0;
     if (valid) {
-      uint32_t lo = 0, hi = nr;  // last row r with s_rp[r] <= i
+      uint32_t lo = from, hi = min(from + span, nr);  // last row r with s_rp[r] <= i
       while (hi - lo > 1) {
         const uint32_t mid = (lo + hi) >> 1;
         if (s_rp[mid] <= i) lo = mid; else hi = mid;
       }
       key = ((uint64_t)s_ri[lo] << 32) | m.col_ids[tl.start + i];
+      row = lo;
       keys[o + i] = key;
       vals[o + i] = m.neg ? 0ull - m.vals[tl.start + i] : m.vals[tl.start + i];
     }
     if (sum_hist) hist_add(h, key, valid, vmask);
+    from = __shfl_sync(0xffffffffu, row, 31);  // (used only while whole warps remain)
+    span = 33;
   }
   if (!sum_hist) return;
   __syncthreads();

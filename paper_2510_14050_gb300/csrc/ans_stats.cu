@@ -222,6 +222,7 @@ enum FinishCols : int {
   kColDigits = 0,  // digit histograms of the destinations (column sort)
   kColMixed = 1,   // digit histograms of their mix, written to col_hkeys
   kColParts = 2,   // hash partitions
+  kColSkip = 3,    // not at all
 };
 template <int kMode, int kCol>
 __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
@@ -234,7 +235,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
   const uint32_t s = tl.seg;
   const uint64_t nrows = a.hdr[2 * s], nnz = a.hdr[2 * s + 1];
   const uint64_t bs = tl.base + s;
-  const uint32_t nh = kCol == kColParts ? col_parts(nnz, a.cp.max_parts) : (uint32_t)(kColPasses * kRadix);
+  const uint32_t nh = kCol == kColSkip    ? 0u
+                      : kCol == kColParts ? col_parts(nnz, a.cp.max_parts)
+                                          : (uint32_t)(kColPasses * kRadix);
   if (kCol != kColParts || tl.start < nnz)
     for (uint32_t i = threadIdx.x; i < nh; i += kThreads) s_h[i] = 0;
   const bool heavy = kCol == kColParts && nnz >= kColHeavyLinks && tl.start < nnz;
@@ -242,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
     s_hkey[threadIdx.x] = a.cp.hkey[(size_t)(t - tl.j) * kColHeavyPerTile + threadIdx.x];
     s_hfan[threadIdx.x] = s_hlo[threadIdx.x] = s_hhi[threadIdx.x] = 0;
   }
-  if constexpr (kCol != kColParts) {
+  if constexpr (kCol == kColDigits || kCol == kColMixed) {
     // Prepare the column sort: its first-pass status words and its tickets
     // (two sub-tiles' worth per tile: the column passes may run sub-tiles).
     if (t == 0 && threadIdx.x < 32) a.col_tickets[threadIdx.x] = 0;
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_finish(StatsArgs a) {
         } else {
           atomicAdd(&s_h[col_part(dst[j], nh)], 1u);
         }
-      } else {
+      } else if constexpr (kCol != kColSkip) {
         // the column sort's key: the destination, or its bijective mix when
         // the sum's column statistics group destinations by hash
         uint32_t ck = dst[j];
@@ -768,6 +771,7 @@ __global__ void __launch_bounds__(1024) k_hgroup_plan(HGroupBufs b, uint32_t max
     const uint32_t parts = n > kHGroupPartLinks ? (n + kHGroupPartLinks - 1) / kHGroupPartLinks : 1u;
     b.item_start[g] = ia;
     b.hpart[g] = ib;
+    for (uint32_t j = 0; j < parts && ia + j < kHGroups + max_hparts; ++j) b.item_group[ia + j] = g;
     ia += parts;
     if (parts > 1) {
       b.heavy[ic++] = g;
@@ -788,10 +792,10 @@ __global__ void __launch_bounds__(1024) k_hgroup_plan(HGroupBufs b, uint32_t max
 // a new slot.  The fill stays below the table size (the callers give up at
 // three quarters, and each thread takes at most one slot meanwhile), so a
 // slot is always found.
-__device__ __forceinline__ bool hg_insert(uint32_t* t_key, uint32_t* t_cnt, uint32_t* t_sum, uint32_t key,
-                                          uint32_t cnt, uint32_t sum) {
-  uint32_t h = (key >> 16) & (kHGroupSlots - 1);  // the group fixes the low 16 bits
-  for (uint32_t probe = 0; probe < kHGroupSlots; ++probe) {
+__device__ __forceinline__ bool hg_insert(uint32_t* t_key, uint32_t* t_cnt, uint32_t* t_sum, uint32_t slots,
+                                          uint32_t key, uint32_t cnt, uint32_t sum) {
+  uint32_t h = (key >> 16) & (slots - 1);  // the group fixes the low 16 bits
+  for (uint32_t probe = 0; probe < slots; ++probe) {
     uint32_t cur = *(volatile uint32_t*)&t_key[h];
     bool claimed = false;
     if (cur == kColEmpty) {
@@ -806,22 +810,28 @@ __device__ __forceinline__ bool hg_insert(uint32_t* t_key, uint32_t* t_cnt, uint
       atomicAdd(&t_sum[h], sum);
       return claimed;
     }
-    h = (h + 1) & (kHGroupSlots - 1);
+    h = (h + 1) & (slots - 1);
   }
   return false;
 }
 
 struct HGroupShared {
   uint32_t fill, over, spec_cnt, spec_sum, item, nflush;
+  uint32_t g, lo, hi, parts, k;  // the drawn item's group, links, parts of the group, and which it is
   unsigned long long red[3][kHGroupThreads / 32];
 };
 
-__device__ __forceinline__ void hg_clear(uint32_t* t_key, HGroupShared& sh) {
+// The first `slots` slots of the three arrays emptied.
+__device__ __forceinline__ void hg_clear(uint32_t* t_key, uint32_t slots, HGroupShared& sh) {
   uint4* k4 = reinterpret_cast<uint4*>(t_key);
-  uint4* c4 = reinterpret_cast<uint4*>(t_key + kHGroupSlots);  // t_cnt and t_sum, back to back
+  uint4* c4 = reinterpret_cast<uint4*>(t_key + kHGroupSlots);
+  uint4* s4 = reinterpret_cast<uint4*>(t_key + 2 * kHGroupSlots);
   const uint4 empty = make_uint4(kColEmpty, kColEmpty, kColEmpty, kColEmpty), zero = make_uint4(0, 0, 0, 0);
-  for (uint32_t i = threadIdx.x; i < kHGroupSlots / 4; i += kHGroupThreads) k4[i] = empty;
-  for (uint32_t i = threadIdx.x; i < kHGroupSlots / 2; i += kHGroupThreads) c4[i] = zero;
+  for (uint32_t i = threadIdx.x; i < slots / 4; i += kHGroupThreads) {
+    k4[i] = empty;
+    c4[i] = zero;
+    s4[i] = zero;
+  }
   if (threadIdx.x == 0) sh.fill = sh.over = sh.spec_cnt = sh.spec_sum = sh.nflush = 0;
 }
 
@@ -834,10 +844,10 @@ __device__ __forceinline__ void hg_count_fill(bool claimed, HGroupShared& sh) {
 
 // The table's (distinct keys, most links, most packets), the key counted
 // apart included, added into acc (call with the whole CTA).
-__device__ void hg_reduce(const uint32_t* t_key, const uint32_t* t_cnt, const uint32_t* t_sum, HGroupShared& sh,
-                          ColPartAcc* acc) {
+__device__ void hg_reduce(const uint32_t* t_key, const uint32_t* t_cnt, const uint32_t* t_sum, uint32_t slots,
+                          HGroupShared& sh, ColPartAcc* acc) {
   unsigned long long c = 0, mcnt = 0, msum = 0;
-  for (uint32_t i = threadIdx.x; i < kHGroupSlots; i += kHGroupThreads) {
+  for (uint32_t i = threadIdx.x; i < slots; i += kHGroupThreads) {
     if (t_key[i] != kColEmpty) {
       ++c;
       mcnt = t_cnt[i] > mcnt ? t_cnt[i] : mcnt;
@@ -886,27 +896,37 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_hash(const uint32_
   uint32_t* t_sum = sm + 2 * kHGroupSlots;
   __shared__ HGroupShared sh;
   const uint32_t nitems = b.meta[0];
+  // Thread 0 draws the next item while the CTA counts the current one: the
+  // draw, its group and the group's bounds are three dependent reads of a
+  // microsecond in all, as long as counting a group of a thousand links takes
+  // (1.94 ms for the 67 million links of 1024 windows' sum when a search over
+  // all groups followed every draw, 1.49 now).
+  auto draw = [&]() -> uint32_t {
+    const uint32_t i = atomicAdd(&b.acc[1].done, 1u);
+    return i < nitems && *(volatile uint32_t*)&b.acc[0].fail == 0 ? i : kHNone;
+  };
+  auto publish = [&](uint32_t i, uint32_t g) {
+    sh.item = i;
+    if (i == kHNone) return;
+    const uint32_t i0 = b.item_start[g], i1 = b.item_start[g + 1], n0 = b.bnd[g], n1 = b.bnd[g + 1];
+    sh.g = g;
+    sh.parts = i1 - i0;
+    sh.k = i - i0;
+    sh.lo = n0 + (i - i0) * kHGroupPartLinks;
+    sh.hi = min(sh.lo + kHGroupPartLinks, n1);
+  };
+  if (threadIdx.x == 0) {
+    const uint32_t i = draw();
+    publish(i, i == kHNone ? 0u : b.item_group[i]);
+  }
   for (;;) {
-    if (threadIdx.x == 0) {
-      const uint32_t i = atomicAdd(&b.acc[1].done, 1u);
-      sh.item = i < nitems && *(volatile uint32_t*)&b.acc[0].fail == 0 ? i : kHNone;
-    }
     __syncthreads();
-    const uint32_t i = sh.item;
-    if (i == kHNone) break;
-    uint32_t lo_g = 0, hi_g = kHGroups;  // the group: the last g with item_start[g] <= i
-    while (hi_g - lo_g > 1) {
-      const uint32_t mid = (lo_g + hi_g) >> 1;
-      if (b.item_start[mid] <= i) lo_g = mid; else hi_g = mid;
-    }
-    const uint32_t g = lo_g;
-    const uint32_t parts = b.item_start[g + 1] - b.item_start[g], k = i - b.item_start[g];
-    const uint32_t lo = b.bnd[g] + k * kHGroupPartLinks;
-    const uint32_t hi = min(lo + kHGroupPartLinks, b.bnd[g + 1]);
-    if (lo == hi) {  // an empty group (never cut in parts): nothing to count
-      __syncthreads();
-      continue;
-    }
+    if (sh.item == kHNone) break;
+    const uint32_t g = sh.g, parts = sh.parts, k = sh.k, lo = sh.lo, hi = sh.hi;
+    uint32_t next = 0, next_g = 0;
+    if (threadIdx.x == 0) next = draw();
+    uint32_t slots = 512;  // at most two thirds taken, unless it is the whole table
+    while (slots < kHGroupSlots && 2 * slots < 3 * (hi - lo)) slots <<= 1;
     uint32_t d[kHGroupChunk], v[kHGroupChunk];
     auto load = [&](uint32_t u0) {
 #pragma unroll
@@ -917,8 +937,9 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_hash(const uint32_
       }
     };
     load(lo);
-    hg_clear(t_key, sh);
+    hg_clear(t_key, slots, sh);
     __syncthreads();
+    if (threadIdx.x == 0 && next != kHNone) next_g = b.item_group[next];
     constexpr uint32_t kStep = (uint32_t)kHGroupChunk * kHGroupThreads;
     for (uint32_t u0 = lo; u0 < hi; u0 += kStep) {  // the same trip count for every thread
       if (u0 != lo) load(u0);
@@ -932,7 +953,7 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_hash(const uint32_
             atomicAdd(&sh.spec_cnt, 1u);
             atomicAdd(&sh.spec_sum, v[j]);
           } else {
-            claimed = hg_insert(t_key, t_cnt, t_sum, d[j], 1u, v[j]);
+            claimed = hg_insert(t_key, t_cnt, t_sum, slots, d[j], 1u, v[j]);
           }
         }
         hg_count_fill(claimed, sh);
@@ -942,11 +963,11 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_hash(const uint32_
     if (sh.over) {
       if (threadIdx.x == 0) atomicOr(&b.acc[0].fail, 1u);
     } else if (parts == 1) {
-      hg_reduce(t_key, t_cnt, t_sum, sh, &b.acc[0]);
+      hg_reduce(t_key, t_cnt, t_sum, slots, sh, &b.acc[0]);
     } else {  // a part of a cut group: its entries out
       const uint64_t pidx = (uint64_t)b.hpart[g] + k;
       uint32_t* out = b.hbuf + pidx * kHGroupPartWords;
-      for (uint32_t e = threadIdx.x; e < kHGroupSlots; e += kHGroupThreads) {
+      for (uint32_t e = threadIdx.x; e < slots; e += kHGroupThreads) {
         if (t_key[e] != kColEmpty) {
           const uint32_t at = atomicAdd(&sh.nflush, 1u);
           out[3 * at] = t_key[e];
@@ -967,6 +988,7 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_hash(const uint32_
       }
     }
     __syncthreads();  // the table and the shared words are reused by the next item
+    if (threadIdx.x == 0) publish(next, next_g);
   }
 }
 
@@ -990,7 +1012,7 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_merge(HGroupBufs b
     const uint32_t g = sh.item;
     if (g == kHNone) break;
     const uint32_t parts = b.item_start[g + 1] - b.item_start[g];
-    hg_clear(t_key, sh);
+    hg_clear(t_key, kHGroupSlots, sh);
     __syncthreads();
     for (uint32_t k = 0; k < parts; ++k) {
       const uint64_t pidx = (uint64_t)b.hpart[g] + k;
@@ -1006,7 +1028,7 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_merge(HGroupBufs b
             atomicAdd(&sh.spec_cnt, cnt);
             atomicAdd(&sh.spec_sum, sum);
           } else {
-            claimed = hg_insert(t_key, t_cnt, t_sum, key, cnt, sum);
+            claimed = hg_insert(t_key, t_cnt, t_sum, kHGroupSlots, key, cnt, sum);
           }
         }
         hg_count_fill(claimed, sh);
@@ -1016,7 +1038,7 @@ __global__ void __launch_bounds__(kHGroupThreads, 2) k_hgroup_merge(HGroupBufs b
     if (sh.over) {
       if (threadIdx.x == 0) atomicOr(&b.acc[0].fail, 1u);
     } else {
-      hg_reduce(t_key, t_cnt, t_sum, sh, &b.acc[0]);
+      hg_reduce(t_key, t_cnt, t_sum, kHGroupSlots, sh, &b.acc[0]);
     }
     __syncthreads();  // the table and the shared words are reused by the next group
   }
@@ -1136,11 +1158,12 @@ cudaError_t launch_scan_u64(const SegPlan& p, const uint64_t* in, uint64_t* out,
 
 cudaError_t launch_finish(const StatsArgs& a, cudaStream_t st) {
   if (a.plan.ntiles == 0) return cudaSuccess;
-  const int col = a.cp.cnt ? kColParts : a.col_hkeys ? kColMixed : kColDigits;
+  const int col = a.no_cols ? kColSkip : a.cp.cnt ? kColParts : a.col_hkeys ? kColMixed : kColDigits;
   const size_t sm = (size_t)(col == kColParts ? a.cp.max_parts : kColPasses * kRadix) * 4;
 #define ANS_FINISH(M)                                                                              \
   if (col == kColParts) k_finish<M, kColParts><<<a.plan.ntiles, kThreads, sm, st>>>(a);            \
   else if (col == kColMixed) k_finish<M, kColMixed><<<a.plan.ntiles, kThreads, sm, st>>>(a);       \
+  else if (col == kColSkip) k_finish<M, kColSkip><<<a.plan.ntiles, kThreads, sm, st>>>(a);         \
   else k_finish<M, kColDigits><<<a.plan.ntiles, kThreads, sm, st>>>(a)
   if (a.mode == kModeWindow) {
     ANS_FINISH(kModeWindow);
