@@ -445,15 +445,17 @@ static_assert(kSsLT * kSsLP == kSsLocal, "one CTA sorts kSsLocal keys");
 // off each other's banks
 __device__ __forceinline__ uint32_t ss_pad(uint32_t i) { return i + i / kSsLP; }
 
-__device__ __forceinline__ void ss_cx(uint64_t& x, uint64_t& y) {
+template <typename K>
+__device__ __forceinline__ void ss_cx(K& x, K& y) {
   const bool sw = x > y;
-  const uint64_t lo = sw ? y : x, hi = sw ? x : y;
+  const K lo = sw ? y : x, hi = sw ? x : y;
   x = lo;
   y = hi;
 }
 
 // Batcher's odd-even merge sort of a thread's keys (Batcher 1968).
-__device__ __forceinline__ void ss_sort_run(uint64_t (&k)[kSsLP]) {
+template <typename K>
+__device__ __forceinline__ void ss_sort_run(K (&k)[kSsLP]) {
 #pragma unroll
   for (int lp = 0; (1 << lp) < kSsLP; ++lp) {
 #pragma unroll
@@ -468,20 +470,11 @@ __device__ __forceinline__ void ss_sort_run(uint64_t (&k)[kSsLP]) {
   }
 }
 
-// Sort in.get(at .. at + m), 0 < m <= kSsLocal, into out[0 .. m); every
-// thread of the CTA calls it.  sm: ss_pad(kSsLocal) + 1 keys.
-__device__ __forceinline__ void ss_sort_block(const SsIn& in, uint64_t at, uint32_t m, uint64_t* out, uint64_t* sm) {
-  const uint32_t tid = threadIdx.x;
-  uint64_t k[kSsLP];
-  // any assignment of keys to threads will do: coalesced loads.  Threads
-  // 0 .. T - 1 hold a run each, missing keys all ones (sorted last).
-  const uint32_t T = (m + kSsLP - 1) / kSsLP, m16 = T * kSsLP;
+// The keys k of threads 0 .. T - 1, 16 each, sorted into sm[ss_pad(0 ..)].
+template <typename K>
+__device__ __forceinline__ void ss_sort_keys(K (&k)[kSsLP], uint32_t T, K* sm) {
+  const uint32_t tid = threadIdx.x, m16 = T * kSsLP;
   if (tid < T) {
-#pragma unroll
-    for (int j = 0; j < kSsLP; ++j) {
-      const uint32_t i = j * T + tid;
-      k[j] = i < m ? in.get(at + i) : ~0ull;
-    }
     ss_sort_run(k);
 #pragma unroll
     for (int j = 0; j < kSsLP; ++j) sm[tid * (kSsLP + 1) + j] = k[j];
@@ -500,7 +493,7 @@ __device__ __forceinline__ void ss_sort_block(const SsIn& in, uint64_t at, uint3
       }
       uint32_t ai = A + lo, bi = B + diag - lo;
       const uint32_t ae = A + na, be = B + nb;
-      uint64_t ka = sm[ss_pad(min(ai, ae - 1))], kb = sm[ss_pad(min(bi, be - 1))];
+      K ka = sm[ss_pad(min(ai, ae - 1))], kb = sm[ss_pad(min(bi, be - 1))];
 #pragma unroll
       for (int j = 0; j < kSsLP; ++j) {
         const bool pa = bi >= be || (ai < ae && ka <= kb);
@@ -508,7 +501,7 @@ __device__ __forceinline__ void ss_sort_block(const SsIn& in, uint64_t at, uint3
         const uint32_t nx = (pa ? ai : bi) + 1;
         if (pa) ai = nx; else bi = nx;
         // (one past a run's end is inside the buffer and never used)
-        const uint64_t kn = sm[ss_pad(nx)];
+        const K kn = sm[ss_pad(nx)];
         if (pa) ka = kn; else kb = kn;
       }
     }
@@ -519,7 +512,41 @@ __device__ __forceinline__ void ss_sort_block(const SsIn& in, uint64_t at, uint3
     }
   }
   __syncthreads();
-  for (uint32_t i = tid; i < m; i += kSsLT) out[i] = sm[ss_pad(i)];
+}
+
+// Sort in.get(at .. at + m), 0 < m <= kSsLocal, into out[0 .. m); every
+// thread of the CTA calls it.  sm: ss_pad(kSsLocal) + 1 keys.  Keys that share
+// their high word (one source: half of the buckets of 2^30 packets of Zipf
+// traffic) are sorted by their low words: half the shared-memory traffic and a
+// third of the instructions of a comparison.
+__device__ __forceinline__ void ss_sort_block(const SsIn& in, uint64_t at, uint32_t m, uint64_t* out, uint64_t* sm) {
+  const uint32_t tid = threadIdx.x;
+  uint64_t k[kSsLP];
+  // any assignment of keys to threads will do: coalesced loads.  Threads
+  // 0 .. T - 1 hold a run each, missing keys all ones (sorted last).
+  const uint32_t T = (m + kSsLP - 1) / kSsLP;
+  uint32_t high = 0, differ = 0;
+  if (tid < T) {
+    high = (uint32_t)(in.get(at) >> 32);
+#pragma unroll
+    for (int j = 0; j < kSsLP; ++j) {
+      const uint32_t i = j * T + tid;
+      k[j] = i < m ? in.get(at + i) : ~0ull;
+      differ |= i < m ? (uint32_t)(k[j] >> 32) ^ high : 0u;
+    }
+  }
+  if (__syncthreads_or((int)differ)) {
+    ss_sort_keys(k, T, sm);
+    for (uint32_t i = tid; i < m; i += kSsLT) out[i] = sm[ss_pad(i)];
+  } else {
+    uint32_t* s32 = reinterpret_cast<uint32_t*>(sm);
+    uint32_t l[kSsLP];
+#pragma unroll
+    for (int j = 0; j < kSsLP; ++j) l[j] = (uint32_t)k[j];
+    ss_sort_keys(l, T, s32);
+    high = (uint32_t)(in.get(at) >> 32);
+    for (uint32_t i = tid; i < m; i += kSsLT) out[i] = (uint64_t)high << 32 | s32[ss_pad(i)];
+  }
   __syncthreads();  // sm may be reused
 }
 
