@@ -145,10 +145,14 @@ int ans_network_quantities(ans_ctx* ctx, const ans_matrix* m, ans_quantities* ou
  *   d_src, d_dst : device arrays; window w is packets [d_offsets[w],
  *                  d_offsets[w+1]) of them.  They may also be page-locked
  *                  host memory that the device addresses (cudaHostAlloc or
- *                  cudaHostRegister): the kernels then read the pairs in
- *                  place over the host link, so the host-to-device transfer
- *                  happens inside the batch, without a staging copy.  Every
- *                  packet sort reads the pairs twice.
+ *                  cudaHostRegister): the host-to-device transfer then
+ *                  happens inside the batch, every pair crossing the host
+ *                  link once: on-chip window sorts and hash tables read the
+ *                  pairs in place, and batches whose packet sorts would read
+ *                  them more than once are first copied by a kernel into
+ *                  device memory held for the call (8 bytes per packet,
+ *                  counted against the budget; where it does not fit the
+ *                  pairs are read in place, twice per packet sort).
  *   d_offsets    : DEVICE array of nwin + 1 nondecreasing uint64 offsets
  *                  (d_offsets[0] may be nonzero).  The batch is planned on the
  *                  device (window lengths, tile table, padded starts: one

@@ -2118,6 +2118,70 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
   return ANS_OK;
 }
 
+// Whether a batch's pairs are first copied to the device by a kernel: they lie
+// in page-locked host memory, the offsets (offs null: on the device, at most
+// `total` packets) are good, and the batch's sorts read the pairs more than
+// once -- a packet sort reads them twice, and the batch's sum by re-sorting
+// (sum_path 2) as often again -- which over the host link costs more than the
+// copy's 8 bytes a packet written and read on the device (2^24 packets in 128
+// windows: 1.27 ms against 1.95, with sum_path 2 2.98 against 4.84; 2^18 in one
+// window 184 us against 204).  On-chip window sorts and the hash tables read
+// them once, in place.
+bool gather_pays(const ans_ctx* c, const uint32_t* src, const uint32_t* dst, const uint64_t* offs, uint64_t total,
+                 size_t nwin, bool want_sum) {
+  if (!src || !dst || !nwin || nwin > 0xFFFFFFF0ull) return false;
+  bool big = !offs;  // (a batch planned on the device is never sorted on chip)
+  for (size_t w = 0; offs && w < nwin; ++w) {
+    if (offs[w + 1] < offs[w] || offs[w + 1] - offs[w] > kMaxWindow) return false;
+    big = big || offs[w + 1] - offs[w] > kClusterWindowMax;
+  }
+  if (!total || (want_sum && total > kMaxWindow)) return false;
+  const bool again = want_sum && (c->sum_path == 2 || c->agg_path == 3);
+  const bool sorted = c->agg_path != 1 && (big || c->win_path != 0 || cluster_sort_clusters(c->device) <= 0);
+  if (!again && !sorted) return false;
+  for (const uint32_t* p : {src, dst}) {
+    cudaPointerAttributes pa{};
+    if (cudaPointerGetAttributes(&pa, offs ? p + offs[0] : p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (pa.type != cudaMemoryTypeHost) return false;
+  }
+  return true;
+}
+
+// A batch of windows stored back to back, offsets on the host or (h_offsets
+// null) on the device with at most `total` packets: analysed from where the
+// pairs lie, or (gather_pays) from a copy made on the device, given back when
+// the batch has been queued.  Where that copy or the batch beside it does not
+// fit in memory, the pairs are read in place.
+int run_pairs(ans_ctx* c, const uint32_t* src, const uint32_t* dst, const uint64_t* h_offsets,
+              const uint64_t* d_offsets, uint64_t total, size_t nwin, uint32_t flags, ans_quantities* out,
+              ans_matrix** per_window, ans_matrix** sum, ans_ticket* ticket, cudaStream_t st) {
+  if (gather_pays(c, src, dst, h_offsets, total, nwin, (flags & ANS_BATCH_SUM) != 0)) {
+    const size_t pairs = align_up((size_t)total * 4), bytes = 2 * pairs + (nwin + 3) * 8;
+    void* mem = nullptr;
+    int rc = dev_alloc(c, bytes, st, &mem);
+    if (rc == ANS_OK) {
+      uint32_t *gsrc = (uint32_t*)mem, *gdst = (uint32_t*)((char*)mem + pairs);
+      uint64_t* span = (uint64_t*)((char*)mem + 2 * pairs);  // first packet, packets, offsets from the first
+      cudaError_t e = d_offsets ? launch_gather_offsets(d_offsets, nwin, total, span, st) : cudaSuccess;
+      if (e == cudaSuccess)
+        e = launch_gather_span(src, dst, h_offsets ? h_offsets[0] : 0, total, d_offsets ? span : nullptr, gsrc, gdst, st);
+      std::vector<uint64_t> rel(h_offsets ? nwin + 1 : 0);
+      for (size_t w = 0; w < rel.size(); ++w) rel[w] = h_offsets[w] - h_offsets[0];
+      rc = e != cudaSuccess ? fail(ANS_ERR_CUDA, std::string("gather: ") + cudaGetErrorString(e))
+                            : run_windows(c, gsrc, gdst, h_offsets ? rel.data() : nullptr, nwin, flags, out, per_window,
+                                          sum, ticket, st, nullptr, nullptr, d_offsets ? span + 2 : nullptr,
+                                          d_offsets ? total : 0);
+      dev_free(c, mem, bytes, st);
+    }
+    if (rc != ANS_ERR_OOM && rc != ANS_ERR_BUDGET) return rc;
+  }
+  return run_windows(c, src, dst, h_offsets, nwin, flags, out, per_window, sum, ticket, st, nullptr, nullptr, d_offsets,
+                     d_offsets ? total : 0);
+}
+
 }  // namespace
 
 // =========================================================================
@@ -2272,8 +2336,7 @@ int ans_batch_submit(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, c
     if (ends[1] < ends[0]) return fail(ANS_ERR_INVALID_ARG, "offsets must be nondecreasing");
     cap = ends[1] - ends[0];
   }
-  return run_windows(c, d_src, d_dst, nullptr, nwin, flags, out, per_window, sum, ticket, st, nullptr, nullptr,
-                     d_offsets, cap);
+  return run_pairs(c, d_src, d_dst, nullptr, d_offsets, cap, nwin, flags, out, per_window, sum, ticket, st);
 }
 
 int ans_batch_submit_host(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const uint64_t* h_offsets,
@@ -2286,7 +2349,8 @@ int ans_batch_submit_host(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_d
   if ((flags & ANS_BATCH_SUM) && !sum) return fail(ANS_ERR_INVALID_ARG, "sum is NULL");
   std::lock_guard<std::mutex> g(c->mu);
   DeviceGuard dg(c->device);
-  return run_windows(c, d_src, d_dst, h_offsets, nwin, flags, out, per_window, sum, ticket, (cudaStream_t)stream);
+  return run_pairs(c, d_src, d_dst, h_offsets, nullptr, h_offsets[nwin] - h_offsets[0], nwin, flags, out, per_window, sum,
+                   ticket, (cudaStream_t)stream);
 }
 
 int ans_set_batch_capacity(ans_ctx* c, uint64_t max_packets) {

@@ -485,6 +485,15 @@ struct GatherWin {
 };
 cudaError_t launch_gather_windows(const GatherWin* wins, uint32_t nwin, uint32_t* gsrc, uint32_t* gdst,
                                   cudaStream_t st);
+// Packets [base, base + n) of src and dst to gsrc and gdst; span (or null): the
+// device words {base, n} that replace base and n, n then being a bound.
+cudaError_t launch_gather_span(const uint32_t* src, const uint32_t* dst, uint64_t base, uint64_t n,
+                               const uint64_t* span, uint32_t* gsrc, uint32_t* gdst, cudaStream_t st);
+// The span of a batch's nwin + 1 device offsets: span[0] = first packet,
+// span[1] = packets, span[2 ..] = the offsets less the first.  Offsets that
+// decrease or hold more than cap packets: span[1] = 0 and the offsets as they
+// are (for the planner to find).
+cudaError_t launch_gather_offsets(const uint64_t* off, uint64_t nwin, uint64_t cap, uint64_t* span, cudaStream_t st);
 // Scratch guards (debug mode): kGuardBytes after every region of a guarded
 // layout hold a fixed pattern, written before a batch's kernels and compared
 // after them; launch_guards fills (err == NULL) or checks the guards at the

@@ -209,6 +209,35 @@ __global__ void __launch_bounds__(256) k_gather_windows(const GatherWin* __restr
   }
 }
 
+// Packets of one span copied in pieces of kSpanPiece by all CTAs.  Bound by the
+// host link when the pairs lie in page-locked host memory (2^30 pairs: 41 ms,
+// 210 GB/s, the copy engines' rate).
+constexpr uint64_t kSpanPiece = 1ull << 14;
+__global__ void __launch_bounds__(256) k_gather_span(const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
+                                                     uint64_t base, uint64_t n, const uint64_t* __restrict__ span,
+                                                     uint32_t* __restrict__ gsrc, uint32_t* __restrict__ gdst) {
+  if (span) base = span[0], n = umin64(n, span[1]);
+  for (uint64_t p = blockIdx.x * kSpanPiece; p < n; p += gridDim.x * kSpanPiece) {
+    const uint64_t m = umin64(kSpanPiece, n - p);
+    copy_words(gsrc + p, src + base + p, m);
+    copy_words(gdst + p, dst + base + p, m);
+  }
+}
+
+__global__ void __launch_bounds__(1024) k_gather_offsets(const uint64_t* __restrict__ off, uint64_t nwin, uint64_t cap,
+                                                         uint64_t* __restrict__ span) {
+  bool bad = false;
+  for (uint64_t s = threadIdx.x; s < nwin; s += 1024) bad |= off[s + 1] < off[s];
+  bad |= off[nwin] - off[0] > cap;
+  const bool any = __syncthreads_or(bad) != 0;
+  const uint64_t first = off[0];
+  for (uint64_t s = threadIdx.x; s <= nwin; s += 1024) span[2 + s] = any ? off[s] : off[s] - first;
+  if (threadIdx.x == 0) {
+    span[0] = first;
+    span[1] = any ? 0ull : off[nwin] - first;
+  }
+}
+
 // One 32-bit word copied on the device (error-word snapshots).
 __global__ void __launch_bounds__(256) k_batch_end(BatchEnd e) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -251,6 +280,19 @@ cudaError_t launch_gather_windows(const GatherWin* wins, uint32_t nwin, uint32_t
   if (e != cudaSuccess) return e;
   const uint32_t grid = std::min<uint32_t>(nwin, (uint32_t)std::max(sms, 1) * 8u);
   k_gather_windows<<<grid, 256, 0, st>>>(wins, nwin, gsrc, gdst);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gather_span(const uint32_t* src, const uint32_t* dst, uint64_t base, uint64_t n,
+                               const uint64_t* span, uint32_t* gsrc, uint32_t* gdst, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  const unsigned grid = (unsigned)std::min<uint64_t>((n + kSpanPiece - 1) / kSpanPiece, 152 * 8);
+  k_gather_span<<<grid, 256, 0, st>>>(src, dst, base, n, span, gsrc, gdst);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gather_offsets(const uint64_t* off, uint64_t nwin, uint64_t cap, uint64_t* span, cudaStream_t st) {
+  k_gather_offsets<<<1, 1024, 0, st>>>(off, nwin, cap, span);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,93 @@
+"""Batches whose pairs lie in page-locked host memory (run_pairs in
+csrc/ans_abi.cu): copied to the device by a kernel where the sorts read them
+more than once, read in place otherwise and where the copy does not fit; exact
+against the oracle and equal errors, with offsets on the host and on the
+device."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+CHIP = 1 << 17  # largest window sorted on chip
+PIECE = 1 << 14  # packets of a copied piece
+
+
+def _pinned(n, seed):
+    rng = np.random.default_rng(seed)
+    src, dst = rng.zipf(1.4, n).astype(np.uint32), rng.integers(0, 300, n, dtype=np.uint32)
+    return src, dst, *(torch.from_numpy(x.view(np.int32)).pin_memory() for x in (src, dst))
+
+
+def _check(ans, ctx, src, dst, ps, pd, offs, device):
+    o = torch.from_numpy(offs.astype(np.int64)).cuda() if device else offs
+    out = torch.zeros((len(offs) - 1, 9), dtype=torch.int64, device="cuda")
+    mats, summ, tk = ctx.batch_submit(ps, pd, o, ans.BATCH_MATRICES | ans.BATCH_SUM, out=out)
+    ctx.wait(tk)
+    a, b = int(offs[0]), int(offs[-1])
+    emats, eq, esum = oracle.batch(src[a:b], dst[a:b], offs - offs[0])
+    assert ans.quantities_from_tensor(out) == eq
+    for m, e in [*zip(mats, emats), (summ, esum)]:
+        for x, y in zip(m.to_numpy(), e):
+            np.testing.assert_array_equal(x, y)
+        m.free()
+
+
+@pytest.mark.parametrize("device", [False, True])
+@pytest.mark.parametrize("tuning", [{}, {"sum_path": 2}, {"agg_path": 3, "sum_path": 2}, {"agg_path": 1}])
+@pytest.mark.parametrize("lens", [(1,), (PIECE - 1, 0, 2), (PIECE, PIECE), (CHIP,), (5, CHIP + 1), (3 * PIECE + 7,) * 5])
+def test_batches(lens, tuning, device):
+    from paper_2510_14050_gb300 import ans
+    offs = np.concatenate([[3], 3 + np.cumsum(lens)]).astype(np.uint64)  # an odd first packet
+    src, dst, ps, pd = _pinned(int(offs[-1]) + 2, len(lens))
+    ctx = ans.Context(0)
+    ctx.set_tuning(**tuning)
+    _check(ans, ctx, src, dst, ps, pd, offs, device)
+    if device:  # a capacity above the batch, then one below it
+        ctx.set_batch_capacity(2 * int(offs[-1]))
+        _check(ans, ctx, src, dst, ps, pd, offs, device)
+        if lens[0] > 1:
+            ctx.set_batch_capacity(int(offs[-1] - offs[0]) - 1)
+            with pytest.raises(ans.AnsError):
+                _check(ans, ctx, src, dst, ps, pd, offs, device)
+    ctx.close()
+
+
+@pytest.mark.parametrize("device", [False, True])
+def test_decreasing_offsets_stay_refused(device):
+    from paper_2510_14050_gb300 import ans
+    src, dst, ps, pd = _pinned(1000, 1)
+    ctx = ans.Context(0)
+    ctx.set_tuning(sum_path=2)
+    for bad in ([0, 10, 5, 1000], [7, 3, 900]):
+        with pytest.raises(ans.AnsError):
+            _check(ans, ctx, src, dst, ps, pd, np.array(bad, dtype=np.uint64), device)
+    ctx.close()
+
+
+@pytest.mark.parametrize("device", [False, True])
+def test_budget_without_room_for_the_copy(device):
+    """A budget that holds the batch and not the copy beside it."""
+    from paper_2510_14050_gb300 import ans
+    n = 1 << 19
+    src, dst, ps, pd = _pinned(n, 2)
+    offs = np.array([0, n // 2, n], dtype=np.uint64)
+    probe = ans.Context(0)
+    probe.set_tuning(sum_path=2)
+    if device:
+        dev = [x.cuda() for x in (ps, pd)]
+        o = torch.from_numpy(offs.astype(np.int64)).cuda()
+        mats, summ, tk = probe.batch_submit(*dev, o, ans.BATCH_MATRICES | ans.BATCH_SUM)
+        probe.wait(tk)
+        need = probe.memory()[0]
+        for m in [*mats, summ]:
+            m.free()
+    else:
+        need = probe.batch_bytes(offs, ans.BATCH_MATRICES | ans.BATCH_SUM)
+    probe.close()
+    ctx = ans.Context(0, budget_bytes=need + (1 << 20))
+    ctx.set_tuning(sum_path=2)
+    _check(ans, ctx, src, dst, ps, pd, offs, device)
+    ctx.close()
