@@ -201,8 +201,8 @@ int ans_set_batch_capacity(ans_ctx* ctx, uint64_t max_packets);
 
 /* The same analysis with every window in its own arrays: window w is
  * srcs[w][0..lens[w]) and dsts[w][0..lens[w]), in device memory, in
- * page-locked host memory (read by the kernels directly over the host link,
- * no staging copy: the serving path for windows that arrive in pinned
+ * page-locked host memory (read by the kernels over the host link: the
+ * serving path for windows that arrive in pinned
  * buffers), or in any host memory if the device reads pageable memory
  * (cudaDevAttrPageableMemoryAccess).  srcs, dsts and lens are host arrays of
  * nwin entries, read during the call; the windows' arrays must stay valid
@@ -211,7 +211,10 @@ int ans_set_batch_capacity(ans_ctx* ctx, uint64_t max_packets);
  * pairs, read in place, into one context-owned device buffer (8 bytes per
  * packet, kept for later calls and counted against the budget) and the batch
  * is analysed from there; if that buffer cannot be allocated the windows are
- * analysed in place on the other paths.  Every other argument, result and
+ * analysed in place on the other paths.  Other batches that sort packets
+ * gather windows whose first nonempty one lies in page-locked host memory the
+ * same way, into memory given back with the call, or read them in place where
+ * that does not fit.  Every other argument, result and
  * error as ans_batch_submit_host; ANS_ERR_INVALID_ARG also for a window the
  * device cannot read. */
 int ans_batch_submit_windows(ans_ctx* ctx, const uint32_t* const* srcs, const uint32_t* const* dsts,

@@ -411,8 +411,9 @@ class Context:
         """Analyse windows [offsets[w], offsets[w+1]) of (src, dst).
 
         ``src``, ``dst``: int32 tensors on the device, or in page-locked host
-        memory (the kernels then read the pairs in place over the host link,
-        with no staging copy).  ``offsets``: nwin + 1 uint64 offsets -- a CUDA tensor (int64/uint64,
+        memory (the kernels then read every pair over the host link once: in
+        place, or into device memory held for the call where the sorts read
+        the pairs more than once).  ``offsets``: nwin + 1 uint64 offsets -- a CUDA tensor (int64/uint64,
         read on the device: ans_batch_submit) or a host array-like
         (ans_batch_submit_host).  ``out``: optional tensor of nwin x 9 int64
         (device or pinned host) receiving the quantities.  Returns

@@ -160,12 +160,12 @@ struct ans_ctx {
   uint64_t next_ticket = 1;
   cudaStream_t aux = nullptr;  // frees of matrix memory
 
-  // Launch configurations of the three families of onesweep passes (set by
+  // Launch configurations of the families of radix passes (key_*: kept, unused) (set by
   // ans_set_tuning / ans_autotune).
   SortCfg cfg_keys, cfg_kv, cfg_col;
   // Window sort: 0 = on chip (one 8-CTA cluster per window of at most
-  // kClusterWindowMax packets; larger windows take the onesweep passes),
-  // 1 = onesweep passes for every window (the default: faster on every
+  // kClusterWindowMax packets; larger windows take the sample sort),
+  // 1 = the sample sort for every window (the default: faster on every
   // workload measured so far).  cfg_win: the cluster kernel's threads and
   // ranking mode.
   int win_path = 1;
@@ -757,7 +757,7 @@ struct PipeScratch {
     vals_a = with_vals ? L.add(pad * 8) : 0;
     vals_b = with_vals ? L.add(pad * 8) : 0;
     seg_hist = L.add((size_t)nseg * kPasses * kRadix * 4);
-    st0 = L.add((size_t)ntiles * 2 * kRadix * 8);  // key passes may run two sub-tiles per tile
+    st0 = L.add((size_t)ntiles * 2 * kRadix * 8);  // column passes may run two sub-tiles per tile
     st1 = L.add((size_t)ntiles * 2 * kRadix * 8);
     lb = L.add((size_t)ntiles * 8);
     lb2 = L.add((size_t)ntiles * 8);
@@ -1390,7 +1390,7 @@ bool agg_packets(const ans_ctx* c, uint32_t nseg, bool want_sum, bool addrs) {
 
 // Scratch layout of one batch (shared by run_windows and ans_batch_bytes).
 struct WinLayout {
-  DevPlan dp, dp_big;  // every window; the windows sorted by onesweep passes
+  DevPlan dp, dp_big;  // every window; the windows sorted by the sample sort
   size_t off_small = 0;  // ids of the windows sorted on chip
   size_t off_tileseg = 0; // the window plan's segment of every tile
   DevPlan dp_tab;        // hash path: the windows' tables as segments
@@ -1501,7 +1501,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
     }
   }
   // Which windows are sorted on chip (one cluster each) and which by the
-  // onesweep passes.
+  // sample sort.
   std::vector<uint32_t> small_ids, big_ids;
   const int win_path = c->win_path;  // the caller holds c->mu
   const SortCfg cfg_win = c->cfg_win;
@@ -1513,7 +1513,7 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
     else big_ids.push_back(s);
   }
   HostPlan hp_big;
-  if (dev) hp_big = hp;  // planned on the device: the onesweep passes take every window
+  if (dev) hp_big = hp;  // planned on the device: the sample sort takes every window
   else hp_big.subset(hp, big_ids);
   // Hash path: one table per window of 2^lg >= 2 * packets slots (at least
   // one tile; none for an empty window), as segments of the table arena.
@@ -2118,6 +2118,22 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
   return ANS_OK;
 }
 
+// Scratch given back before a batch that did not fit is tried again another
+// way, which may need a little more: growing what is held would take a quarter
+// more than that (ensure_scratch).
+void drop_scratch(ans_ctx* c, cudaStream_t st) {
+  dev_free(c, c->scratch, c->scratch_size, st);
+  c->scratch = nullptr;
+  c->scratch_size = 0;
+}
+
+bool page_locked(const void* p) {
+  cudaPointerAttributes pa{};
+  if (cudaPointerGetAttributes(&pa, p) == cudaSuccess) return pa.type == cudaMemoryTypeHost;
+  cudaGetLastError();
+  return false;
+}
+
 // Whether a batch's pairs are first copied to the device by a kernel: they lie
 // in page-locked host memory, the offsets (offs null: on the device, at most
 // `total` packets) are good, and the batch's sorts read the pairs more than
@@ -2138,16 +2154,27 @@ bool gather_pays(const ans_ctx* c, const uint32_t* src, const uint32_t* dst, con
   if (!total || (want_sum && total > kMaxWindow)) return false;
   const bool again = want_sum && (c->sum_path == 2 || c->agg_path == 3);
   const bool sorted = c->agg_path != 1 && (big || c->win_path != 0 || cluster_sort_clusters(c->device) <= 0);
-  if (!again && !sorted) return false;
-  for (const uint32_t* p : {src, dst}) {
-    cudaPointerAttributes pa{};
-    if (cudaPointerGetAttributes(&pa, offs ? p + offs[0] : p) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
+  const uint64_t first = offs ? offs[0] : 0;
+  return (again || sorted) && page_locked(src + first) && page_locked(dst + first);
+}
+
+// The pieces of windows in their own arrays to be copied to one pair of arrays:
+// at most max(2^14, total / 4096) packets each, so that a few long windows are
+// copied by as many CTAs as many short ones (a served batch of 100 windows of 2^12
+// to 2^17 packets from page-locked memory: 848 us with a CTA per window, 824 so).
+std::vector<GatherWin> gather_pieces(const uint32_t* const* srcs, const uint32_t* const* dsts, const uint64_t* lens,
+                                     size_t nwin, uint64_t total) {
+  const uint64_t most = std::max<uint64_t>(1u << 14, total >> 12);
+  std::vector<GatherWin> table;
+  table.reserve(nwin + (size_t)(total / most));
+  uint64_t off = 0;
+  for (size_t w = 0; w < nwin; ++w)
+    for (uint64_t p = 0; p < lens[w]; p += most) {
+      const uint64_t n = std::min(most, lens[w] - p);
+      table.push_back(GatherWin{(uint64_t)(uintptr_t)(srcs[w] + p), (uint64_t)(uintptr_t)(dsts[w] + p), off, n});
+      off += n;
     }
-    if (pa.type != cudaMemoryTypeHost) return false;
-  }
-  return true;
+  return table;
 }
 
 // A batch of windows stored back to back, offsets on the host or (h_offsets
@@ -2177,6 +2204,7 @@ int run_pairs(ans_ctx* c, const uint32_t* src, const uint32_t* dst, const uint64
       dev_free(c, mem, bytes, st);
     }
     if (rc != ANS_ERR_OOM && rc != ANS_ERR_BUDGET) return rc;
+    drop_scratch(c, st);
   }
   return run_windows(c, src, dst, h_offsets, nwin, flags, out, per_window, sum, ticket, st, nullptr, nullptr, d_offsets,
                      d_offsets ? total : 0);
@@ -2400,20 +2428,37 @@ int ans_batch_submit_windows(ans_ctx* c, const uint32_t* const* srcs, const uint
     }
   }
   // The paths that sort all of a batch's packets as one segment (the time sum
-  // by re-sorting the packets) read the packets as one stream, and every sort
-  // of packets reads them twice: the windows' pairs are first
-  // gathered into one device buffer by a kernel (reading each window in
-  // place), then analysed like contiguous windows.  If that buffer cannot be
-  // had, the windows are analysed in place on the other paths.
+  // by re-sorting the packets) read the packets as one stream: the windows'
+  // pairs are first gathered into one device buffer by a kernel (reading each
+  // window in place), then analysed like contiguous windows.  If that buffer
+  // cannot be had, the windows are analysed in place on the other paths.
+  // Other packet sorts read the pairs twice; where the first window's lie in
+  // page-locked host memory they are gathered too, into memory given back with
+  // the batch (run_pairs; 100 windows of 2^12 to 2^17 packets served with
+  // their sum: 708 us against 920 in place; one of 2^17: 212 against 220).
   const uint64_t total = offs[nwin];
+  cudaStream_t st = (cudaStream_t)stream;
   const bool one_segment = c->agg_path == 2 || c->agg_path == 3 || c->sum_path == 2;
   bool fits = nwin <= 0xFFFFFFF0ull && !((flags & ANS_BATCH_SUM) && total > kMaxWindow);
-  for (size_t w = 0; w < nwin && fits; ++w) fits = lens[w] <= kMaxWindow;
-  if (one_segment && fits && total > 0) {  // (otherwise run_windows reports what does not fit)
+  bool big = false;
+  size_t first = nwin;
+  for (size_t w = 0; w < nwin && fits; ++w) {
+    fits = lens[w] <= kMaxWindow;
+    big = big || lens[w] > kClusterWindowMax;
+    if (lens[w] && first == nwin) first = w;
+  }
+  const bool twice = !one_segment && c->agg_path != 1 &&
+                     (big || c->win_path != 0 || cluster_sort_clusters(c->device) <= 0) && first < nwin &&
+                     page_locked(srcs[first]) && page_locked(dsts[first]);
+  if ((one_segment || twice) && fits && total > 0) {  // (otherwise run_windows reports what does not fit)
+    const std::vector<GatherWin> table = gather_pieces(srcs, dsts, lens, nwin, total);
     const size_t pairs = align_up((size_t)total * 4);
-    const size_t need = 2 * pairs + (size_t)nwin * sizeof(GatherWin);
-    cudaStream_t st = (cudaStream_t)stream;
-    if (need > c->gather_bytes) {
+    const size_t need = 2 * pairs + table.size() * sizeof(GatherWin);
+    void* mem = nullptr;
+    if (twice) {
+      const int rc = dev_alloc(c, need, st, &mem);
+      if (rc != ANS_OK && rc != ANS_ERR_OOM && rc != ANS_ERR_BUDGET) return rc;
+    } else if (need > c->gather_bytes) {
       const size_t want = std::max(need, c->gather_bytes + c->gather_bytes / 4);
       dev_free(c, c->gather_mem, c->gather_bytes, st);
       c->gather_mem = nullptr;
@@ -2427,23 +2472,25 @@ int ans_batch_submit_windows(ans_ctx* c, const uint32_t* const* srcs, const uint
         return rc;
       }
     }
-    if (c->gather_mem) {
-      char* gm = (char*)c->gather_mem;
+    if (char* gm = (char*)(twice ? mem : c->gather_mem)) {
       uint32_t* gsrc = (uint32_t*)gm;
       uint32_t* gdst = (uint32_t*)(gm + pairs);
       GatherWin* gw = (GatherWin*)(gm + 2 * pairs);
-      std::vector<GatherWin> table(nwin);
-      for (size_t w = 0; w < nwin; ++w)
-        table[w] = GatherWin{(uint64_t)(uintptr_t)srcs[w], (uint64_t)(uintptr_t)dsts[w], offs[w], lens[w]};
       UploadSet us;
       us.add(gw, table.data(), table.size() * sizeof(GatherWin));
-      ANS_TRY(us.flush(c, st));
-      ANS_CUDA(launch_gather_windows(gw, (uint32_t)nwin, gsrc, gdst, st));
-      return run_windows(c, gsrc, gdst, offs.data(), nwin, flags, out, per_window, sum, ticket, st);
+      int rc = us.flush(c, st);
+      if (rc == ANS_OK) {
+        const cudaError_t e = launch_gather_windows(gw, (uint32_t)table.size(), gsrc, gdst, st);
+        if (e != cudaSuccess) rc = fail(ANS_ERR_CUDA, std::string("gather: ") + cudaGetErrorString(e));
+      }
+      if (rc == ANS_OK) rc = run_windows(c, gsrc, gdst, offs.data(), nwin, flags, out, per_window, sum, ticket, st);
+      if (!twice) return rc;
+      dev_free(c, mem, need, st);
+      if (rc != ANS_ERR_OOM && rc != ANS_ERR_BUDGET) return rc;
+      drop_scratch(c, st);  // (else in place)
     }
   }
-  return run_windows(c, nullptr, nullptr, offs.data(), nwin, flags, out, per_window, sum, ticket,
-                     (cudaStream_t)stream, srcs, dsts);
+  return run_windows(c, nullptr, nullptr, offs.data(), nwin, flags, out, per_window, sum, ticket, st, srcs, dsts);
 }
 
 int ans_sum_windows(ans_ctx* c, const ans_matrix* const* mats, size_t k, ans_matrix** out, void* stream) {

@@ -55,6 +55,37 @@ def test_batches(lens, tuning, device):
     ctx.close()
 
 
+@pytest.mark.parametrize("tuning", [{}, {"sum_path": 2}])
+@pytest.mark.parametrize("lens", [(1,), (0, PIECE - 1, 0, 2), (PIECE, PIECE + 1, 5), (3 * PIECE + 7,) * 3, (7, CHIP + 1)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_windows_in_their_own_arrays(lens, tuning, mixed):
+    from paper_2510_14050_gb300 import ans
+    offs = np.concatenate([[3], 3 + np.cumsum(lens)]).astype(np.uint64)
+    src, dst, ps, pd = _pinned(int(offs[-1]), len(lens))
+    wins = [(ps[int(a):int(b)], pd[int(a):int(b)]) for a, b in zip(offs[:-1], offs[1:])]
+    if mixed:  # every second window on the device
+        wins = [(s.cuda(), d.cuda()) if i % 2 else (s, d) for i, (s, d) in enumerate(wins)]
+    emats, eq, esum = oracle.batch(src[3:], dst[3:], offs - offs[0])
+    ctx = ans.Context(0)
+    ctx.set_tuning(**tuning)
+    for budget in (0, 1):
+        out = torch.zeros((len(lens), 9), dtype=torch.int64, device="cuda")
+        mats, summ, tk = ctx.batch_submit_windows(wins, ans.BATCH_MATRICES | ans.BATCH_SUM, out=out)
+        ctx.wait(tk)
+        assert ans.quantities_from_tensor(out) == eq
+        for m, e in [*zip(mats, emats), (summ, esum)]:
+            for x, y in zip(m.to_numpy(), e):
+                np.testing.assert_array_equal(x, y)
+            m.free()
+        if budget == 0:  # again without room for a copy beside the batch
+            ctx.close()
+            probe = ans.Context(0)
+            need = probe.batch_bytes(offs, ans.BATCH_MATRICES | ans.BATCH_SUM)
+            probe.close()
+            ctx = ans.Context(0, budget_bytes=need + 4096)
+    ctx.close()
+
+
 @pytest.mark.parametrize("device", [False, True])
 def test_decreasing_offsets_stay_refused(device):
     from paper_2510_14050_gb300 import ans
