@@ -77,9 +77,9 @@ REFERENCE_SAMPLE = {1: 1, 2: 64, 3: 96, 4: 256}
 # for the library sources it was captured with and the paths and launch
 # shapes that decide the traffic (else the bench reports null).
 NCU_TRAFFIC = {
-    4: {"library": "aa3d1cc8fee92455", "matrices": False,
-        "paths": {"agg_path": 3, "sum_path": 2, "col_hash": 1, "key_threads": 256, "key_blocks": 4},
-        "step": 365.65, "kernels": {"onesweep_pk": 19.74, "regroup": 19.73, "rle": 23.18}},
+    4: {"library": "e7be1fcc1b4153ac", "matrices": False,
+        "paths": {"agg_path": 0, "sum_path": 2, "col_hash": 1},
+        "step": 233.8, "kernels": {"ss_local": 14.40, "ss_scatter": 16.63, "ss_count": 9.42, "rle": 17.52}},
 }
 
 
@@ -712,8 +712,8 @@ def main(argv=None):
         del src_e, dst_e
 
         # The same call given the pinned host arrays themselves: the batch's
-        # kernels read the pairs in place over the host link (the packet pack
-        # reads each pair once), so the transfer happens inside the batch.
+        # kernels read each pair over the host link once, so the transfer
+        # happens inside the batch.
         def ip_step():
             return step(src_h, dst_h)
 
