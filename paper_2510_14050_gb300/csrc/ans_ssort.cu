@@ -47,7 +47,9 @@ constexpr uint32_t kSsRawBit = 0x80000000u; // level-2 parent: the segment itsel
 constexpr uint32_t kSsDone = 0xFFFFFFFFu;   // level-2 parent: nothing to sort
 
 // Buckets of an n-key split.  Level 1, the first of two splits: as many as
-// the second split will make of each of its buckets.
+// the second split will make of each of its buckets.  An empty segment has
+// none: it owns no tile, and behind the last tile there is no place for their
+// counts.
 __host__ __device__ __forceinline__ uint32_t ss_buckets(uint64_t n, bool level1, uint64_t one_level) {
   if (level1) {
     if (n <= one_level) return 0u;
@@ -55,6 +57,7 @@ __host__ __device__ __forceinline__ uint32_t ss_buckets(uint64_t n, bool level1,
     const uint32_t r = (uint32_t)sqrtf((float)((n + kSsBucket - 1) / kSsBucket)) + 1;
     return r < kSsMaxBuckets ? r : kSsMaxBuckets;
   }
+  if (n == 0) return 0u;
   return n <= kSsLocal ? 1u : (uint32_t)umin64((n + kSsBucket - 1) / kSsBucket, kSsMaxBuckets);
 }
 __device__ __forceinline__ uint32_t ss_levels(uint32_t nb) { return nb <= 1 ? 0u : 32u - __clz(nb - 1); }
@@ -567,7 +570,7 @@ __global__ void __launch_bounds__(kSsLT, 8) k_ss_local(SsArgs a) {
   if (a.ntiles_d && t >= *a.ntiles_d) return;
   const SsSeg g = ss_seg(a, ss_find(a, t));
   const uint32_t b = blockIdx.x - g.b0;
-  if (b >= g.nb || g.n == 0) return;
+  if (b >= g.nb) return;
   if (g.nb == 1) {  // never split: the whole segment
     ss_sort_block(ss_input(a, g.s, g.start), 0, (uint32_t)g.n, a.keys_out + g.start, sm);
     return;
