@@ -1038,6 +1038,13 @@ int sum_prepare(ans_ctx* c, char* m, uint32_t k, const std::vector<uint64_t>& ca
   return ANS_OK;
 }
 
+// The header and row pointer of a sum without a tile (every window empty),
+// which no kernel of the sum writes.
+void zero_empty(Block* blk, ZeroBatch* z) {
+  z->add(blk->hdr, 16);
+  z->add(blk->row_ptr, 8);
+}
+
 // Device half of the time sum of the matrices described by `d_mats` (device
 // array of k MatDesc), written into plan->blk.  Uses scratch laid out by the
 // caller at `m` / `ps` (which must provide vals buffers).  Only queues work
@@ -1183,6 +1190,7 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
   const uint64_t most = (uint64_t)s.ntiles * kTile;
   ZeroBatch z;
   z.add(blk->q, sizeof(ans_quantities));
+  if (s.ntiles == 0) zero_empty(blk, &z);
   if (cols && !a.col_hkeys && col_parts_ok(c, most)) col_parts_begin(m, ps, s, most, &a, &z);
   else z.add(m + ps.col_hist, kColPasses * kRadix * 4);
   if ((e = launch_zero_batch(z, st)) != cudaSuccess) return fail_blk(e, "memset");
@@ -1214,6 +1222,7 @@ int sum_packets(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& pk, c
   z.add(m + ps.lb, (size_t)pk.ntiles * 8);
   z.add(blk->q, sizeof(ans_quantities));
   z.add(tickets, 32 * 4);
+  if (pk.ntiles == 0) zero_empty(blk, &z);
   if (!a.col_hkeys && col_parts_ok(c, total)) col_parts_begin(m, ps, pk, total, &a, &z);
   else z.add(m + ps.col_hist, kColPasses * kRadix * 4);
   if ((rc = cu(launch_zero_batch(z, st), "memset")) ||

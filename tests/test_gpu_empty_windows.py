@@ -48,3 +48,40 @@ def test_nothing_is_written_behind_the_last_tile(lens, tuning, monkeypatch):
         for device in (False, True):
             _check(ans, ctx, src, dst, offs, flags, device)
     ctx.close()
+
+
+class _Dirty:
+    """Allocator hooks whose blocks come filled with 0x55."""
+
+    def __init__(self, ans):
+        self.live = {}
+
+        def _alloc(nbytes, stream, user):
+            t = torch.full((int(nbytes),), 0x55, dtype=torch.uint8, device="cuda")
+            torch.cuda.synchronize()
+            self.live[t.data_ptr()] = t
+            return t.data_ptr()
+
+        def _free(ptr, stream, user):
+            if ptr:
+                torch.cuda.synchronize()
+                del self.live[ptr]
+
+        self.alloc_fn = ans.ALLOC_FN(_alloc)
+        self.free_fn = ans.FREE_FN(_free)
+
+
+@pytest.mark.parametrize("tuning", [{}, {"sum_path": 1}, {"sum_path": 2}, {"agg_path": 1}, {"agg_path": 3}])
+@pytest.mark.parametrize("lens", [(0,), (0, 0, 0)])
+def test_only_empty_windows(lens, tuning):
+    from paper_2510_14050_gb300 import ans
+    offs = np.full(len(lens) + 1, 3, dtype=np.uint64)
+    src, dst = _packets(5, 1)
+    ctx = ans.Context(0, allocator=_Dirty(ans))
+    ctx.set_tuning(**tuning)
+    for cap in (0, 2 * TILE):
+        ctx.set_batch_capacity(cap)
+        for device in (False, True):
+            for flags in (ans.BATCH_SUM, ans.BATCH_MATRICES | ans.BATCH_SUM):
+                _check(ans, ctx, src, dst, offs, flags, device)
+    ctx.close()
