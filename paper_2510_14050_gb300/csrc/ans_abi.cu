@@ -2035,7 +2035,9 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
   uint64_t total_cap = 0;
   bool any_neg = false;
   // every count of the result stays below 2^32 if the inputs hold fewer
-  // packets in all (known once they have been computed)
+  // packets in all (known once they have been computed).  An input's packets
+  // are counted modulo 2^62: they are taken at their word only where its links
+  // times its largest count cannot reach that (imported counts may)
   uint64_t packets = 0;
   bool narrow = true;
   for (size_t i = 0; i < k; ++i) {
@@ -2055,8 +2057,10 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
     if (cudaEventQuery(b->done) == cudaSuccess) {
       ANS_TRY(block_fill_cache(const_cast<Block*>(b)));
       cap = std::min<uint64_t>(cap, b->h_hdr[2 * (size_t)x->seg + 1]);
-      const uint64_t held = b->h_q[x->seg].valid_packets;
-      narrow = narrow && held < (1ull << 32) - packets;
+      const ans_quantities& hq = b->h_q[x->seg];
+      const uint64_t held = hq.valid_packets;
+      narrow = narrow && held < (1ull << 32) - packets &&
+               (!hq.unique_links || hq.max_link_packets < (1ull << 62) / hq.unique_links);
       if (narrow) packets += held;
     } else {
       cudaGetLastError();
