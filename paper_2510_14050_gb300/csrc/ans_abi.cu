@@ -1866,14 +1866,9 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   end.err = c->d_err;
   if (blk) end.status[0] = blk->status;
   if (sblk) end.status[1] = sblk->status;
-  if (out && nseg) {
-    end.dst = (uint64_t*)addressable(out);
-    if (end.dst) {
-      end.src = (const uint64_t*)sb.q;
-      end.words = (uint64_t)nseg * sizeof(ans_quantities) / 8;
-    } else {
-      ANS_CUDA(cudaMemcpyAsync(out, sb.q, (size_t)nseg * sizeof(ans_quantities), cudaMemcpyDefault, st));
-    }
+  if (out && nseg && (end.dst = (uint64_t*)addressable(out))) {
+    end.src = (const uint64_t*)sb.q;
+    end.words = (uint64_t)nseg * sizeof(ans_quantities) / 8;
   }
   uint32_t slot = 0;
   if (ticket) {
@@ -1881,14 +1876,16 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
     end.status[2] = c->h_err_slots + slot;
   }
   if ((rc = cu(launch_batch_end(end, st), "batch end"))) return bail(rc);
+  if (!end.dst && (rc = copy_quantities_out(out, sb.q, nseg, st))) return bail(rc);
+  // (nothing may fail once the first handle has been given out)
+  for (Block* b : {blk, sblk})
+    if (b && (rc = cu(cudaEventRecord(b->done, st), "record"))) return bail(rc);
   if (ticket && (rc = add_ticket(c, st, slot, ticket))) return bail(rc);
   if (blk) {
-    if ((rc = cu(cudaEventRecord(blk->done, st), "record"))) return bail(rc);
     blk->refs = (int)nseg;
     for (uint32_t s = 0; s < nseg; ++s) per_window[s] = new ans_matrix{blk, s};
   }
   if (sblk) {
-    ANS_CUDA(cudaEventRecord(sblk->done, st));
     sblk->refs = 1;
     *sum = new ans_matrix{sblk, 0};
   }
