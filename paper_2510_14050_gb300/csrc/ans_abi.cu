@@ -1866,7 +1866,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   end.err = c->d_err;
   if (blk) end.status[0] = blk->status;
   if (sblk) end.status[1] = sblk->status;
-  if (out && nseg && (end.dst = (uint64_t*)addressable(out))) {
+  // (whole words; an array off their alignment is copied by copy_quantities_out)
+  if (out && nseg && (uintptr_t)out % 8 == 0 && (end.dst = (uint64_t*)addressable(out))) {
     end.src = (const uint64_t*)sb.q;
     end.words = (uint64_t)nseg * sizeof(ans_quantities) / 8;
   }

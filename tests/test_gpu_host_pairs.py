@@ -122,3 +122,24 @@ def test_budget_without_room_for_the_copy(device):
     ctx.set_tuning(sum_path=2)
     _check(ans, ctx, src, dst, ps, pd, offs, device)
     ctx.close()
+
+
+@pytest.mark.parametrize("where", ["device", "pinned", "pageable"])
+@pytest.mark.parametrize("shift", [0, 1, 4, 8])
+def test_quantities_at_any_address(where, shift):
+    """The array of quantities is written byte by byte where its address is
+    no multiple of a word."""
+    from paper_2510_14050_gb300 import ans
+    lens = (20_000, 0, 3)
+    offs = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
+    src, dst, ps, pd = _pinned(int(offs[-1]), 4)
+    room = torch.full((len(lens) * 72 + 16,), 7, dtype=torch.uint8)
+    room = room.cuda() if where == "device" else room.pin_memory() if where == "pinned" else room
+    ctx = ans.Context(0)
+    out = room[shift:shift + len(lens) * 72]
+    _, _, tk = ctx.batch_submit(ps.cuda(), pd.cuda(), offs, out=out)
+    ctx.wait(tk)
+    got = np.frombuffer(bytes(out.cpu().numpy()), dtype=np.int64)
+    assert ans.quantities_from_tensor(got) == oracle.batch(src, dst, offs, want_sum=False)[1]
+    assert bool((room[:shift].cpu() == 7).all()) and bool((room[shift + len(lens) * 72:].cpu() == 7).all())
+    ctx.close()
