@@ -17,6 +17,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <string>
@@ -1454,12 +1455,15 @@ struct WinLayout {
   }
 };
 
-// The batch pipeline (also serves ans_build_window with nwin == 1).
+// The batch pipeline (also serves ans_build_window with nwin == 1).  feed (or
+// empty) queues on `st` what fills the packet arrays, once all the batch's
+// memory is held: a batch refused for memory leaves nothing queued that reads
+// the caller's arrays.
 int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const uint64_t* h_offsets,
                 size_t nwin, uint32_t flags, ans_quantities* out, ans_matrix** per_window, ans_matrix** sum,
                 ans_ticket* ticket, cudaStream_t st, const uint32_t* const* h_srcs = nullptr,
                 const uint32_t* const* h_dsts = nullptr, const uint64_t* d_offsets = nullptr,
-                uint64_t dev_cap = 0) {
+                uint64_t dev_cap = 0, const std::function<int()>& feed = {}) {
   // dev: the offsets live on the device and the batch is planned there
   // (launch_plan); the host sizes everything for dev_cap packets.
   const bool dev = d_offsets != nullptr;
@@ -1571,7 +1575,9 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   }
   SumPlan sump;
   Block* sblk = nullptr;
+  bool queued = false;  // work that reads the caller's arrays
   auto bail = [&](int rc) {
+    if (queued) cudaStreamSynchronize(st);
     block_discard(blk, st);
     block_discard(sump.blk, st);
     block_discard(sblk, st);
@@ -1850,6 +1856,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
                           std::to_string(wl.ss_two_win) + std::to_string(wl.ss_two_pk) +
                           std::to_string(ss_shape(hp.ntiles)) + std::to_string(ss_shape(wl.ss.ntiles2)) +
                           std::to_string(ss_shape((uint32_t)pk_tiles));
+  queued = true;
+  if (feed && (rc = feed())) return bail(rc);
   if ((rc = run_launches(c, st, sig, launch_all))) return bail(rc);
   if (sump.blk) {  // the time sum's block is filled
     sblk = sump.blk;
@@ -2203,15 +2211,15 @@ int run_pairs(ans_ctx* c, const uint32_t* src, const uint32_t* dst, const uint64
     if (rc == ANS_OK) {
       uint32_t *gsrc = (uint32_t*)mem, *gdst = (uint32_t*)((char*)mem + pairs);
       uint64_t* span = (uint64_t*)((char*)mem + 2 * pairs);  // first packet, packets, offsets from the first
-      cudaError_t e = d_offsets ? launch_gather_offsets(d_offsets, nwin, total, span, st) : cudaSuccess;
-      if (e == cudaSuccess)
-        e = launch_gather_span(src, dst, h_offsets ? h_offsets[0] : 0, total, d_offsets ? span : nullptr, gsrc, gdst, st);
       std::vector<uint64_t> rel(h_offsets ? nwin + 1 : 0);
       for (size_t w = 0; w < rel.size(); ++w) rel[w] = h_offsets[w] - h_offsets[0];
-      rc = e != cudaSuccess ? fail(ANS_ERR_CUDA, std::string("gather: ") + cudaGetErrorString(e))
-                            : run_windows(c, gsrc, gdst, h_offsets ? rel.data() : nullptr, nwin, flags, out, per_window,
-                                          sum, ticket, st, nullptr, nullptr, d_offsets ? span + 2 : nullptr,
-                                          d_offsets ? total : 0);
+      const auto feed = [&]() -> int {
+        if (d_offsets) ANS_CUDA(launch_gather_offsets(d_offsets, nwin, total, span, st));
+        ANS_CUDA(launch_gather_span(src, dst, h_offsets ? h_offsets[0] : 0, total, d_offsets ? span : nullptr, gsrc, gdst, st));
+        return ANS_OK;
+      };
+      rc = run_windows(c, gsrc, gdst, h_offsets ? rel.data() : nullptr, nwin, flags, out, per_window, sum, ticket, st,
+                       nullptr, nullptr, d_offsets ? span + 2 : nullptr, d_offsets ? total : 0, feed);
       dev_free(c, mem, bytes, st);
     }
     if (rc != ANS_ERR_OOM && rc != ANS_ERR_BUDGET) return rc;
@@ -2487,14 +2495,15 @@ int ans_batch_submit_windows(ans_ctx* c, const uint32_t* const* srcs, const uint
       uint32_t* gsrc = (uint32_t*)gm;
       uint32_t* gdst = (uint32_t*)(gm + pairs);
       GatherWin* gw = (GatherWin*)(gm + 2 * pairs);
-      UploadSet us;
-      us.add(gw, table.data(), table.size() * sizeof(GatherWin));
-      int rc = us.flush(c, st);
-      if (rc == ANS_OK) {
-        const cudaError_t e = launch_gather_windows(gw, (uint32_t)table.size(), gsrc, gdst, st);
-        if (e != cudaSuccess) rc = fail(ANS_ERR_CUDA, std::string("gather: ") + cudaGetErrorString(e));
-      }
-      if (rc == ANS_OK) rc = run_windows(c, gsrc, gdst, offs.data(), nwin, flags, out, per_window, sum, ticket, st);
+      const auto feed = [&]() -> int {
+        UploadSet us;
+        us.add(gw, table.data(), table.size() * sizeof(GatherWin));
+        ANS_TRY(us.flush(c, st));
+        ANS_CUDA(launch_gather_windows(gw, (uint32_t)table.size(), gsrc, gdst, st));
+        return ANS_OK;
+      };
+      const int rc = run_windows(c, gsrc, gdst, offs.data(), nwin, flags, out, per_window, sum, ticket, st, nullptr,
+                                 nullptr, nullptr, 0, feed);
       if (!twice) return rc;
       dev_free(c, mem, need, st);
       if (rc != ANS_ERR_OOM && rc != ANS_ERR_BUDGET) return rc;

@@ -143,3 +143,39 @@ def test_quantities_at_any_address(where, shift):
     assert ans.quantities_from_tensor(got) == oracle.batch(src, dst, offs, want_sum=False)[1]
     assert bool((room[:shift].cpu() == 7).all()) and bool((room[shift + len(lens) * 72:].cpu() == 7).all())
     ctx.close()
+
+
+@pytest.mark.parametrize("call", ["host", "device", "windows", "windows_one_segment"])
+def test_a_refused_batch_reads_nothing(call):
+    """A budget that holds the copy of the pairs and not the batch: refused
+    with nothing on the stream that reads them (their copy alone would take 2.5
+    ms over the host link)."""
+    from paper_2510_14050_gb300 import ans
+    n = 1 << 26
+    ps, pd = (torch.zeros(n, dtype=torch.int32).pin_memory() for _ in range(2))
+    offs = np.array([0, n // 2, n], dtype=np.uint64)
+    o = torch.from_numpy(offs.astype(np.int64)).cuda() if call == "device" else offs
+    ctx = ans.Context(0, budget_bytes=9 * n)
+    if call == "windows_one_segment":
+        ctx.set_tuning(sum_path=2)
+    if call == "device":
+        ctx.set_batch_capacity(n)  # (its offsets are not read back)
+
+    def refused():
+        with pytest.raises(ans.AnsError) as e:
+            if call.startswith("windows"):
+                ctx.batch_submit_windows([(ps[:n // 2], pd[:n // 2]), (ps[n // 2:], pd[n // 2:])], ans.BATCH_SUM)
+            else:
+                ctx.batch_submit(ps, pd, o, ans.BATCH_SUM)
+        assert e.value.code == ans.ERR_BUDGET
+
+    refused()  # (its memory is mapped now)
+    before, after = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(100_000_000)  # about 50 ms of device time: the host's is hidden behind it
+    before.record()
+    refused()
+    after.record()
+    torch.cuda.synchronize()
+    assert before.elapsed_time(after) < 1.0
+    ctx.close()
