@@ -11,9 +11,16 @@
 //            partition and tile -- no order to keep, no look-back;
 //   count    one CTA per partition counts its destinations in a shared-memory
 //            table and adds the table's three quantities to the segment's.
-// A partition with more destinations than the table holds is read again in
-// 2, 4, ... classes by another mix of the destination, so every input ends
-// here and no sort stands behind.
+// A partition with more destinations than the table takes (a segment of more
+// than 2048 tables' worth of them, or destinations crowded into one) is cut by
+// its CTA into parts of about kColPart links, by another mix of the
+// destination, in memory, and the parts are counted one by one: two readings
+// and a writing of its links more.  A part with too many still, or the
+// partition where there is no such memory, is read again in 2, 4, ... classes.
+// So every input ends here and no sort stands behind.  (9 million links of as
+// many destinations: count 174 us, 225 with 64-bit counts, against 464 and 495
+// for the four passes of a column sort; 2^25: 584 and 763 against 1588 and 1682.
+// Reading all of it in classes, after tables filled to the brim: 5.0 ms and 10.6.)
 //
 // A destination with a large share of the links would make one partition, and
 // one table slot, a queue.  In segments of kColHeavyLinks links or more those
@@ -32,7 +39,9 @@ namespace ans {
 namespace {
 
 constexpr uint32_t kColSlots = 4096;               // table slots of one CTA
-constexpr uint32_t kColFill = kColSlots / 8 * 7;   // give up above this
+constexpr uint32_t kColFill = kColSlots / 4 * 3;   // give up above this
+constexpr uint32_t kColEarly = 920;                // or above this after 1024 links
+constexpr uint32_t kColSubs = 512;                 // most parts of a cut partition
 constexpr uint32_t kColNone = 0xFFFFFFFFu;         // empty slot (that destination is counted apart)
 constexpr int kColThreads = 256;
 
@@ -85,6 +94,12 @@ __global__ void __launch_bounds__(kColHeavyThreads) k_col_heavy(SegPlan p, ColPa
   if (threadIdx.x < kColHeavySlots) c.hkey[(uint64_t)p.first_tile[s] * kColHeavyPerTile + threadIdx.x] = s_key[threadIdx.x];
 }
 static_assert(1u << 3 == kColHeavyMin, "the lowest count listed");
+
+// The part of destination d among `subs` of its partition (its class comes
+// from another mix).
+__device__ __forceinline__ uint32_t col_sub(uint32_t d, uint32_t subs) {
+  return __umulhi(fmix32(fmix32(d) ^ 0x7F4A7C15u), subs);
+}
 
 struct ColSeg {
   uint32_t ft, parts;
@@ -214,20 +229,62 @@ __global__ void __launch_bounds__(kT, kP == 16 ? (kWide ? 1 : 2) : kT == 512 ? 3
   }
 }
 
+// The links kd, vd[0 .. m) of an overfull partition moved to sd, sv, grouped
+// into `subs` parts; start[0 .. subs] gets the parts' places.  Every thread of
+// the CTA calls it; cur: `subs` shared words.
+template <typename V>
+__device__ __forceinline__ void col_cut(const uint32_t* kd, const V* vd, uint32_t m, uint32_t subs, uint32_t* sd, V* sv,
+                                        uint32_t* start, uint32_t* cur) {
+  static_assert(kColSubs == 2 * kColThreads, "two parts per thread in the scan");
+  __shared__ uint32_t s_w[kColThreads / 32];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (uint32_t i = tid; i < subs; i += kColThreads) cur[i] = 0;
+  __syncthreads();
+#pragma unroll 4
+  for (uint32_t u = tid; u < m; u += kColThreads) atomicAdd(&cur[col_sub(kd[u], subs)], 1u);
+  __syncthreads();
+  const uint32_t a = 2 * tid < subs ? cur[2 * tid] : 0u, b = 2 * tid + 1 < subs ? cur[2 * tid + 1] : 0u;
+  uint32_t x = a + b;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  uint32_t off = x - a - b;
+  for (uint32_t w = 0; w < warp; ++w) off += s_w[w];
+  if (2 * tid < subs) start[2 * tid] = cur[2 * tid] = off;
+  if (2 * tid + 1 < subs) start[2 * tid + 1] = cur[2 * tid + 1] = off + a;
+  if (tid == 0) start[subs] = m;
+  __syncthreads();
+#pragma unroll 4
+  for (uint32_t u = tid; u < m; u += kColThreads) {
+    const uint32_t d = kd[u];
+    const V v = vd[u];
+    const uint32_t at = atomicAdd(&cur[col_sub(d, subs)], 1u);
+    sd[at] = d;
+    sv[at] = v;
+  }
+  __syncthreads();
+}
+
 // One partition per CTA (one that was never split is the whole segment).
 template <bool kWide>
-__global__ void __launch_bounds__(kColThreads) k_col_count(SegPlan p, ColParts c, const uint32_t* __restrict__ col_ids,
-                                                           const uint32_t* __restrict__ vals32,
-                                                           const uint64_t* __restrict__ vals64,
-                                                           const uint32_t* __restrict__ pdst,
-                                                           const void* __restrict__ pval,
-                                                           ans_quantities* __restrict__ q) {
+__global__ void __launch_bounds__(kColThreads, kWide ? 3 : 4) k_col_count(SegPlan p, ColParts c,
+                                                                          const uint32_t* __restrict__ col_ids,
+                                                                          const uint32_t* __restrict__ vals32,
+                                                                          const uint64_t* __restrict__ vals64,
+                                                                          const uint32_t* __restrict__ pdst,
+                                                                          const void* __restrict__ pval,
+                                                                          ans_quantities* __restrict__ q) {
   using V = typename std::conditional<kWide, uint64_t, uint32_t>::type;
   extern __shared__ __align__(16) uint32_t t_key[];
   uint32_t* t_cnt = t_key + kColSlots;
   uint32_t* t_lo = t_cnt + kColSlots;
   uint32_t* t_hi = t_lo + kColSlots;  // kWide only
   __shared__ uint32_t s_fill, s_over, s_spec_cnt, s_spec_lo, s_spec_hi;
+  __shared__ uint32_t s_start[kColSubs + 1];
   __shared__ unsigned long long s_red[3][kColThreads / 32];
   const uint32_t t = blockIdx.x / kColPerTile;
   const uint32_t s = find_seg(p, t);
@@ -238,8 +295,9 @@ __global__ void __launch_bounds__(kColThreads) k_col_count(SegPlan p, ColParts c
   const uint32_t* kd = col_ids + base;
   const V* vd = (kWide ? (const V*)vals64 : (const V*)vals32) + base;
   uint64_t m = g.n;
+  uint32_t at = 0;
   if (g.parts > 1) {
-    const uint32_t at = c.start[blockIdx.x];
+    at = c.start[blockIdx.x];
     m = c.cnt[blockIdx.x];
     kd = pdst + base + at;
     vd = reinterpret_cast<const V*>(pval) + base + at;
@@ -247,87 +305,129 @@ __global__ void __launch_bounds__(kColThreads) k_col_count(SegPlan p, ColParts c
   const bool heavy = b == 0 && g.n >= kColHeavyLinks;  // this CTA adds the heavy destinations
   if (m == 0 && !heavy) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t slots = 256;
-  while (slots < m + m / 2 && slots < kColSlots) slots <<= 1;
   auto add = [&](uint32_t* lo, uint32_t* hi, V x) {
     if constexpr (kWide) add64_shared(lo, hi, x);
     else atomicAdd(lo, x);
   };
   auto sum_of = [&](uint32_t lo, const uint32_t* hi) -> uint64_t { return kWide ? (uint64_t)*hi << 32 | lo : lo; };
   unsigned long long uniq = 0, mfan = 0, mpk = 0;
-  for (uint32_t R = 1, cls = 0; cls < R;) {
-    for (uint32_t i = threadIdx.x; i < slots; i += kColThreads) {
-      t_key[i] = kColNone;
-      t_cnt[i] = 0;
-      t_lo[i] = 0;
-      if (kWide) t_hi[i] = 0;
-    }
-    if (threadIdx.x == 0) s_fill = s_over = s_spec_cnt = s_spec_lo = s_spec_hi = 0;
-    __syncthreads();
-    constexpr int kU = 4;  // links per thread in flight
-    for (uint64_t u0 = 0; u0 < m; u0 += (uint64_t)kU * kColThreads) {
-      if (*(volatile uint32_t*)&s_over) break;
-      uint32_t d[kU];
-      V v[kU];
-#pragma unroll
-      for (int k = 0; k < kU; ++k) {
-        const uint64_t u = u0 + (uint64_t)k * kColThreads + threadIdx.x;
-        d[k] = u < m ? kd[u] : 0u;
-        v[k] = u < m ? vd[u] : V(0);
+  uint32_t subs = 0;  // parts of a cut partition, 0: whole
+  for (uint32_t sub = 0; sub < (subs ? subs : 1u); ++sub) {
+    unsigned long long found = 0;
+    uint32_t slots = 256;
+    while (slots < m + m / 2 && slots < kColSlots) slots <<= 1;
+    const bool watch = m > kColFill;  // it may hold too many destinations
+    // (a first round of links with hardly a destination twice is one of far more
+    // of them: cut at once)
+    const uint32_t early = !subs && g.parts > 1 && c.sdst && m > kColFill / 5 * 6 ? kColEarly : kColFill;
+    for (uint32_t R = 1, cls = 0; cls < R;) {
+      for (uint32_t i = threadIdx.x; i < slots; i += kColThreads) {
+        t_key[i] = kColNone;
+        t_cnt[i] = 0;
+        t_lo[i] = 0;
+        if (kWide) t_hi[i] = 0;
       }
+      if (threadIdx.x == 0) s_fill = s_over = s_spec_cnt = s_spec_lo = s_spec_hi = 0;
+      __syncthreads();
+      constexpr int kU = 4;  // links per thread in flight
+      for (uint64_t u0 = 0; u0 < m; u0 += (uint64_t)kU * kColThreads) {
+        if (__any_sync(0xffffffffu, *(volatile uint32_t*)&s_over)) break;  // (the warp as one)
+        uint32_t d[kU], claimed = 0;
+        V v[kU];
 #pragma unroll
-      for (int k = 0; k < kU; ++k) {
-        if (u0 + (uint64_t)k * kColThreads + threadIdx.x >= m) continue;
-        if (d[k] == kColNone) {
-          if (cls == 0) {
-            atomicAdd(&s_spec_cnt, 1u);
-            add(&s_spec_lo, &s_spec_hi, v[k]);
-          }
-          continue;
+        for (int k = 0; k < kU; ++k) {
+          const uint64_t u = u0 + (uint64_t)k * kColThreads + threadIdx.x;
+          d[k] = u < m ? kd[u] : 0u;
+          v[k] = u < m ? vd[u] : V(0);
         }
-        const uint32_t h = fmix32(d[k]);
-        if (R > 1 && (fmix32(h ^ 0x9E3779B9u) & (R - 1)) != cls) continue;
-        uint32_t i = h & (slots - 1);
-        for (uint32_t probe = 0; probe < slots; ++probe) {
-          uint32_t cur = *(volatile uint32_t*)&t_key[i];
-          if (cur == kColNone) {
-            cur = atomicCAS(&t_key[i], kColNone, d[k]);
-            if (cur == kColNone) {
-              cur = d[k];
-              if (atomicAdd(&s_fill, 1u) >= kColFill) s_over = 1;
+#pragma unroll
+        for (int k = 0; k < kU; ++k) {
+          if (u0 + (uint64_t)k * kColThreads + threadIdx.x < m) {
+            if (d[k] == kColNone) {
+              if (cls == 0) {
+                atomicAdd(&s_spec_cnt, 1u);
+                add(&s_spec_lo, &s_spec_hi, v[k]);
+              }
+            } else {
+              const uint32_t h = fmix32(d[k]);
+              if (R == 1 || (fmix32(h ^ 0x9E3779B9u) & (R - 1)) == cls) {
+                uint32_t i = h & (slots - 1);
+                for (uint32_t probe = 0; probe < slots; ++probe) {
+                  uint32_t cur = *(volatile uint32_t*)&t_key[i];
+                  if (cur == kColNone) {
+                    cur = atomicCAS(&t_key[i], kColNone, d[k]);
+                    if (cur == kColNone) {
+                      cur = d[k];
+                      ++claimed;
+                    }
+                  }
+                  if (cur == d[k]) {
+                    atomicAdd(&t_cnt[i], 1u);
+                    add(&t_lo[i], &t_hi[i], v[k]);
+                    break;
+                  }
+                  i = (i + 1) & (slots - 1);
+                }
+              }
             }
           }
-          if (cur == d[k]) {
-            atomicAdd(&t_cnt[i], 1u);
-            add(&t_lo[i], &t_hi[i], v[k]);
-            break;
+          // Given up before the table is nearly full: every second link the
+          // warps add up their new destinations, so that searches stay short (an
+          // addition for every new destination made the count of 6 million
+          // different ones 169 instead of 143 us; looking once a round of links,
+          // overfull partitions took 18 times as long; after every link, ones of
+          // few destinations 5% longer).
+          if (watch && k % 2 == 1 && __any_sync(0xffffffffu, claimed)) {
+            const uint32_t claims = __reduce_add_sync(0xffffffffu, claimed);
+            claimed = 0;
+            uint32_t fill = 0;
+            if (lane == 0) fill = atomicAdd(&s_fill, claims) + claims;
+            if (__shfl_sync(0xffffffffu, fill, 0) > (u0 ? kColFill : early)) {
+              s_over = 1;
+              break;
+            }
           }
-          i = (i + 1) & (slots - 1);
         }
       }
-    }
-    __syncthreads();
-    if (s_over) {  // more destinations than the table takes: twice the classes, from the start
-      R <<= 1;
-      cls = 0;
-      uniq = mfan = mpk = 0;
       __syncthreads();
-      continue;
-    }
-    for (uint32_t i = threadIdx.x; i < slots; i += kColThreads) {
-      if (t_key[i] != kColNone) {
-        ++uniq;
-        mfan = umax64(mfan, t_cnt[i]);
-        mpk = umax64(mpk, sum_of(t_lo[i], &t_hi[i]));
+      if (s_over) {
+        __syncthreads();
+        if (!subs && g.parts > 1 && c.sdst) break;  // cut below
+        R <<= 1;  // twice the classes, from the start
+        cls = 0;
+        found = 0;
+        continue;
       }
+      for (uint32_t i = threadIdx.x; i < slots; i += kColThreads) {
+        if (t_key[i] != kColNone) {
+          ++found;
+          mfan = umax64(mfan, t_cnt[i]);
+          mpk = umax64(mpk, sum_of(t_lo[i], &t_hi[i]));
+        }
+      }
+      if (threadIdx.x == 0 && s_spec_cnt) {
+        ++found;
+        mfan = umax64(mfan, s_spec_cnt);
+        mpk = umax64(mpk, sum_of(s_spec_lo, &s_spec_hi));
+      }
+      ++cls;
+      __syncthreads();  // the table is cleared for the next class
     }
-    if (threadIdx.x == 0 && s_spec_cnt) {
-      ++uniq;
-      mfan = umax64(mfan, s_spec_cnt);
-      mpk = umax64(mpk, sum_of(s_spec_lo, &s_spec_hi));
+    uniq += found;
+    if (!subs && s_over) {
+      subs = (uint32_t)umin64(kColSubs, (m + kColPart - 1) / kColPart);
+      uint32_t* sd = c.sdst + base + at;
+      V* sv = reinterpret_cast<V*>(c.sval) + base + at;
+      col_cut<V>(kd, vd, (uint32_t)m, subs, sd, sv, s_start, t_key);
+      kd = sd;
+      vd = sv;
+      m = s_start[1];
+      sub = ~0u;  // from part 0 on
+    } else if (sub + 1 < subs) {
+      kd += s_start[sub + 1] - s_start[sub];
+      vd += s_start[sub + 1] - s_start[sub];
+      m = s_start[sub + 2] - s_start[sub + 1];
     }
-    ++cls;
-    __syncthreads();  // the table is cleared for the next class
   }
   if (heavy && threadIdx.x < kColHeavySlots) {
     const size_t at = (size_t)g.ft * kColHeavyPerTile + threadIdx.x;

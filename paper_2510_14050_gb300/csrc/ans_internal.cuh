@@ -107,6 +107,12 @@ struct ColParts {
   uint32_t* start = nullptr;
   uint32_t* hkey = nullptr;
   unsigned long long* hsum = nullptr;
+  // Where overfull partitions are cut, at the segments' bases (null: not):
+  // links' destinations, and counts as wide as the column pass's.  The counts
+  // may take the place of vals32, which a segment of several partitions has
+  // left by then.
+  uint32_t* sdst = nullptr;
+  void* sval = nullptr;
   uint32_t max_parts = 0;  // most partitions of a segment
 };
 struct StatsArgs {
