@@ -995,12 +995,13 @@ int column_pass(ans_ctx* c, const StatsArgs& a, const PipeScratch& ps, char* m, 
 }
 
 // A time sum (one segment at base 0) takes the hash-group column statistics
-// when its counts are 32-bit, the column hashes are on, it may hold 2^24
+// when its counts are 32-bit, the column hashes are on, it may hold `least`
 // or more links (smaller sums sort their 2^16 groups' worth of work faster)
 // and the scratch holds the buffers for that many.
-bool hgroup_ok(const ans_ctx* c, const SegPlan& p, bool narrow, const PipeScratch& ps) {
+bool hgroup_ok(const ans_ctx* c, const SegPlan& p, bool narrow, const PipeScratch& ps,
+               uint64_t least = kHGroupMinLinks) {
   const uint64_t links = (uint64_t)p.ntiles * kTile;
-  return narrow && c->col_hash && p.nseg == 1 && links >= kHGroupMinLinks && ps.hgroup_cap > 0 &&
+  return narrow && c->col_hash && p.nseg == 1 && links >= least && ps.hgroup_cap > 0 &&
          links <= ps.hgroup_links;
 }
 
@@ -1054,7 +1055,8 @@ void zero_empty(Block* blk, ZeroBatch* z) {
 // caller at `m` / `ps` (which must provide vals buffers).  Only queues work
 // on `st` (it may be capturing); on failure the caller discards plan->blk.
 int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s, const uint64_t* fk,
-                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow = false, bool cols = true);
+                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow = false, bool cols = true,
+                   uint64_t group_links = kHGroupMinLinks);
 
 // First half of the time sum: the input links gathered and ordered (merge
 // rounds, or the kv passes with sum_path 1), left in (*fk, *fv).  Touches
@@ -1145,19 +1147,19 @@ int sum_order(ans_ctx* c, char* m, const PipeScratch& ps, const MatDesc* d_mats,
 // pass then carries 32-bit counts).
 int sum_launch(ans_ctx* c, char* m, const PipeScratch& ps, const MatDesc* d_mats, uint32_t k, SumPlan* plan,
                size_t off_catoff, size_t off_lens, size_t off_total, cudaStream_t st, bool narrow = false,
-               bool cols = true) {
+               bool cols = true, uint64_t group_links = kHGroupMinLinks) {
   const uint64_t *fk = nullptr, *fv = nullptr;
   ANS_TRY(sum_order(c, m, ps, d_mats, k, plan, off_catoff, off_lens, off_total, st, &fk, &fv));
-  return links_to_block(c, m, ps, plan->s, fk, fv, plan->blk, st, narrow, cols);
+  return links_to_block(c, m, ps, plan->s, fk, fv, plan->blk, st, narrow, cols, group_links);
 }
 
 // From sorted (key, value) links (equal keys adjacent) of the single segment
 // of `s` to a DCSR block: value prefix, run-length reduction, values as
 // prefix differences, row statistics and the column pass (the time sum's
 // statistics half).  cols false: without column statistics (a block that is
-// only gathered again).  Only queues work on `st`.
+// only gathered again); group_links: as hgroup_ok's.  Only queues work on `st`.
 int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s, const uint64_t* fk,
-                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow, bool cols) {
+                   const uint64_t* fv, Block* blk, cudaStream_t st, bool narrow, bool cols, uint64_t group_links) {
   uint32_t* tickets = at<uint32_t>(m, ps.tickets) + 32;
   auto fail_blk = [&](cudaError_t e, const char* what) {
     return fail(ANS_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
@@ -1190,7 +1192,7 @@ int links_to_block(ans_ctx* c, char* m, const PipeScratch& ps, const SegPlan& s,
   a.mode = kModeSum;
   if (narrow) a.vals32 = (uint32_t*)at<uint64_t>(m, ps.cv_b);
   a.no_cols = !cols;
-  if (cols && hgroup_ok(c, s, narrow, ps)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
+  if (cols && hgroup_ok(c, s, narrow, ps, group_links)) a.col_hkeys = at<uint32_t>(m, ps.ck_b);
   const uint64_t most = (uint64_t)s.ntiles * kTile;
   ZeroBatch z;
   z.add(blk->q, sizeof(ans_quantities));
@@ -2026,7 +2028,7 @@ int drop_zeros(ans_ctx* c, Block* blk, uint64_t cap, bool narrow, cudaStream_t s
     return bail(rc);
   SegPlan s2 = s;
   s2.len = count;
-  if ((rc = links_to_block(c, m, ps, s2, kb, vb, plan.blk, st, narrow))) return bail(rc);
+  if ((rc = links_to_block(c, m, ps, s2, kb, vb, plan.blk, st, narrow, true, kHGroupGivenLinks))) return bail(rc);
   *out = plan.blk;
   return ANS_OK;
 }
@@ -2113,7 +2115,7 @@ int combine_matrices(ans_ctx* c, const ans_matrix* const* mats, const int* signs
       return rc;
     }
     rc = sum_launch(c, m, ps, at<MatDesc>(m, off_mats), (uint32_t)k, &sump, off_catoff, off_lens, off_total, st,
-                    narrow && !any_neg, !any_neg);
+                    narrow && !any_neg, !any_neg, kHGroupGivenLinks);
     if (rc) {
       block_discard(sump.blk, st);
       return rc;
