@@ -763,8 +763,8 @@ struct PipeScratch {
     lb = L.add((size_t)ntiles * 8);
     lb2 = L.add((size_t)ntiles * 8);
     tickets = L.add(kTicketBlocks * 32 * 4);
-    run_start = L.add((pad + nseg) * 8);
-    row_pos = L.add((pad + nseg) * 8);
+    run_start = L.add((pad + nseg) * 4);
+    row_pos = L.add((pad + nseg) * 4);
     pre = with_vals ? L.add((pad + nseg) * 8) : 0;
   }
 };
@@ -2007,8 +2007,8 @@ int drop_zeros(ans_ctx* c, Block* blk, uint64_t cap, bool narrow, cudaStream_t s
   uint64_t* va = at<uint64_t>(m, ps.vals_a);
   uint64_t* vb = at<uint64_t>(m, ps.vals_b);
   uint32_t* tickets = at<uint32_t>(m, ps.tickets) + 32;
-  uint64_t* flags = at<uint64_t>(m, ps.run_start);
-  uint64_t* pos = at<uint64_t>(m, ps.row_pos);
+  uint64_t* flags = at<uint64_t>(m, ps.cv_a);  // free until the column pass
+  uint64_t* pos = at<uint64_t>(m, ps.pre);     // and until the result's prefix
   uint64_t* count = at<uint64_t>(m, off_count);
   const uint64_t* cat_off = at<uint64_t>(m, off_catoff);
   const SegPlan& s = plan.s;
