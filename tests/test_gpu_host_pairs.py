@@ -179,3 +179,65 @@ def test_a_refused_batch_reads_nothing(call):
     torch.cuda.synchronize()
     assert before.elapsed_time(after) < 1.0
     ctx.close()
+
+
+class _RefuseOnce:
+    """Allocator hooks that refuse the first allocation once armed."""
+
+    def __init__(self, ans):
+        self.live, self.armed, self.refused = {}, False, []
+
+        def _alloc(nbytes, stream, user):
+            if self.armed:
+                self.armed = False
+                self.refused.append(int(nbytes))
+                return None
+            t = torch.empty(int(nbytes), dtype=torch.uint8, device="cuda")
+            self.live[t.data_ptr()] = t
+            return t.data_ptr()
+
+        def _free(ptr, stream, user):
+            if ptr:
+                torch.cuda.synchronize()
+                del self.live[ptr]
+
+        self.alloc_fn = ans.ALLOC_FN(_alloc)
+        self.free_fn = ans.FREE_FN(_free)
+
+
+@pytest.mark.parametrize("tuning", [{}, {"sum_path": 2}, {"sum_path": 1, "agg_path": 2}, {"agg_path": 3}])
+@pytest.mark.parametrize("lens", [(1,), (0, PIECE - 1, 0, 2), (3 * PIECE + 7,) * 3, (7, CHIP + 1)])
+def test_windows_in_place_when_their_copy_is_refused(lens, tuning):
+    """The tuning is kept on the way to the fallback, which is seen to run: a
+    sum by re-sorting the packets is merged instead when they lie apart."""
+    from paper_2510_14050_gb300 import ans
+    offs = np.concatenate([[3], 3 + np.cumsum(lens)]).astype(np.uint64)
+    src, dst, ps, pd = _pinned(int(offs[-1]), len(lens))
+    wins = [(ps[int(a):int(b)], pd[int(a):int(b)]) for a, b in zip(offs[:-1], offs[1:])]
+    emats, eq, esum = oracle.batch(src[3:], dst[3:], offs - offs[0])
+    hooks = _RefuseOnce(ans)
+    ctx = ans.Context(0, allocator=hooks)
+    ctx.set_tuning(**tuning)
+    for refuse in (False, True, False):
+        hooks.armed = refuse
+        ctx.profile(True)
+        out = torch.zeros((len(lens), 9), dtype=torch.int64, device="cuda")
+        mats, summ, tk = ctx.batch_submit_windows(wins, ans.BATCH_MATRICES | ans.BATCH_SUM, out=out)
+        ctx.wait(tk)
+        ran = set(ctx.profile_read())
+        ctx.profile(False)
+        assert ans.quantities_from_tensor(out) == eq
+        for m, e in [*zip(mats, emats), (summ, esum)]:
+            for x, y in zip(m.to_numpy(), e):
+                np.testing.assert_array_equal(x, y)
+            m.free()
+        if len(lens) > 1 and tuning in ({"sum_path": 2}, {"agg_path": 3}):
+            assert ("merge" in ran) == refuse
+        if refuse:  # the copy: the call's first allocation where no larger one is kept
+            assert hooks.refused and hooks.refused[-1] >= 8 * int(offs[-1] - offs[0])
+        if not refuse and tuning:  # the next copy is asked for again
+            ctx.close()
+            ctx = ans.Context(0, allocator=hooks)
+            ctx.set_tuning(**tuning)
+    ctx.close()
+    assert not hooks.live
