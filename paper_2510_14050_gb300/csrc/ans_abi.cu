@@ -2882,6 +2882,8 @@ int ans_batch_bytes(ans_ctx* c, const uint64_t* h_offsets, size_t nwin, uint32_t
   const bool want_mats = (flags & ANS_BATCH_MATRICES) != 0, want_sum = (flags & ANS_BATCH_SUM) != 0;
   std::lock_guard<std::mutex> g(c->mu);
   const bool hash = c->agg_path == 1 && nwin > 0;
+  std::vector<size_t> guards;  // (debug mode: their bytes count too)
+  GuardSink gs(c->guards ? &guards : nullptr);
   WinLayout wl;
   wl.reserve(hp, (uint32_t)nwin, want_mats, want_sum, total, max_len, hash);
   size_t need = 0;

@@ -57,3 +57,21 @@ def test_signed_combinations(n):
     for x in (*ms, total, got):
         x.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("guards", ["0", "1"])
+@pytest.mark.parametrize("lens", [(1,), (5000, 0, 9000)])
+def test_batch_bytes_is_what_a_batch_takes(lens, guards, monkeypatch):
+    """In the debug mode too, whose guards take memory of their own."""
+    from paper_2510_14050_gb300 import ans
+    monkeypatch.setenv("ANS_SCRATCH_GUARDS", guards)
+    offs = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
+    src, dst = (torch.randint(0, 99, (int(offs[-1]),), dtype=torch.int32, device="cuda") for _ in range(2))
+    ctx = ans.Context(0)
+    need, held = ctx.batch_bytes(offs, ans.BATCH_MATRICES | ans.BATCH_SUM), ctx.memory()[0]
+    mats, summ, tk = ctx.batch_submit(src, dst, offs, ans.BATCH_MATRICES | ans.BATCH_SUM)
+    ctx.wait(tk)
+    assert ctx.memory()[0] - held == need
+    for m in [*mats, summ]:
+        m.free()
+    ctx.close()
