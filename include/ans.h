@@ -133,8 +133,8 @@ int ans_combine(ans_ctx* ctx, const ans_matrix* const* mats, const int* signs, s
 
 /* The nine quantities of a matrix (Table I, Sec. IV-C), recomputed on the
  * device from its DCSR arrays: row statistics by segmented reductions over
- * rows, column statistics by a transpose-free pass that sorts the stored links
- * by destination and reduces the destination runs.
+ * rows, column statistics by a transpose-free pass that groups the stored links
+ * by destination (hash partitions counted on chip, or a sort by destination).
  * out: host or device pointer to one ans_quantities.  With a device pointer
  * (or pinned host memory) the call is asynchronous; with pageable host memory
  * it returns once the result has been written. */
@@ -193,7 +193,7 @@ int ans_batch_submit_host(ans_ctx* ctx, const uint32_t* d_src, const uint32_t* d
 
 /* Capacity, in packets, of batches submitted with device-resident offsets
  * (ans_batch_submit): scratch, output blocks and grids are sized for it, so
- * a larger capacity costs memory (about 100 bytes per packet of scratch,
+ * a larger capacity costs memory (about 80 bytes per packet of scratch,
  * and the per-window and time-sum blocks at 24 bytes per packet each) and
  * some empty tiles.  0 (the default) sizes each batch by reading its first
  * and last offset back.  Errors: ANS_ERR_INVALID_ARG. */
@@ -206,8 +206,8 @@ int ans_set_batch_capacity(ans_ctx* ctx, uint64_t max_packets);
  * buffers), or in any host memory if the device reads pageable memory
  * (cudaDevAttrPageableMemoryAccess).  srcs, dsts and lens are host arrays of
  * nwin entries, read during the call; the windows' arrays must stay valid
- * until the batch completes.  On the paths that sort a batch's packets as one
- * segment (agg_path 2 or 3, sum_path 2) a kernel first gathers every window's
+ * until the batch completes.  With the paths that sort a batch's packets as one
+ * segment (agg_path 3, sum_path 2), and with agg_path 2, a kernel first gathers every window's
  * pairs, read in place, into one context-owned device buffer (8 bytes per
  * packet, kept for later calls and counted against the budget) and the batch
  * is analysed from there; if that buffer cannot be allocated the windows are
@@ -312,7 +312,9 @@ int ans_window_quantities_noalloc(const uint32_t* d_src, const uint32_t* d_dst, 
  * device bytes the context holds now (scratch plus live matrices) and its
  * budget (0 = none).  ans_batch_bytes gives the additional device bytes that
  * ans_batch_submit_host with these offsets and flags would allocate if called now
- * (scratch growth plus output matrices); nothing is allocated. */
+ * (scratch growth plus output matrices); nothing is allocated.  The copy of
+ * page-locked pairs, which is made only where it fits beside these, is not in
+ * them. */
 int ans_ctx_memory(ans_ctx* ctx, size_t* live_bytes, size_t* budget_bytes);
 int ans_batch_bytes(ans_ctx* ctx, const uint64_t* h_offsets, size_t nwin, uint32_t flags, size_t* bytes);
 
@@ -340,8 +342,9 @@ int ans_batch_bytes(ans_ctx* ctx, const uint64_t* h_offsets, size_t nwin, uint32
  * own time sum, windows stored back to back) every packet of the batch
  * sorted again as one segment and reduced like a window
  * -- the sum of Table I's A_t is the matrix of the concatenated packets;
- * batches of windows in their own arrays then take the kv_* passes, and sums
- * of k given matrices merge them (k <= 256) or take the kv_* passes.  agg_path: how
+ * batches of windows in their own arrays are gathered first, or where that
+ * does not fit merge (k <= 256) or take the kv_* passes, as sums
+ * of k given matrices do.  agg_path: how
  * a window's equal packets are grouped, 0 = sorting every packet's link key,
  * 1 = counting links in a per-window hash table (2^k >= 2 x packets slots of
  * 12 bytes, kept by the context between calls) and sorting only the distinct
@@ -352,13 +355,12 @@ int ans_batch_bytes(ans_ctx* ctx, const uint64_t* h_offsets, size_t nwin, uint32
  * agg_path 0 waits for the device and releases the tables.  graph: 1 = a batch's launch sequence is recorded into a CUDA
  * graph and replayed through a cached executable graph of the same shape
  * (updated in place with the call's pointers), 0 = launched directly; per-
- * kernel profiling always launches directly.  col_hash: 1 = each window's
- * column statistics are first counted in a shared-memory hash of its
- * destinations (one CTA, or a cluster, per window; up to 12288 distinct
- * destinations), then windows with more destinations and at most 2^18 links
- * in shared-memory hashes of destination partitions (up to 32 CTAs per
- * window, one partition each), and only windows neither fits take the
- * column sort; 0 = the column sort for every window.  merge_tile: output positions per CTA of the time sum's merge
+ * kernel profiling always launches directly.  col_hash: 1 = column statistics
+ * by hash partitions of the destinations, each counted in a shared-memory
+ * table, for matrices of up to 2^25 links and for batches with device-resident
+ * offsets; by hash groups for time sums that may hold 2^24 links or more (2^26
+ * for sums of given matrices); by the column sort for the rest; 0 = the column
+ * sort for every matrix.  merge_tile: output positions per CTA of the time sum's merge
  * rounds, 4096 or 2048 (more resident CTAs per SM, twice the merge-path
  * searches).  Results never depend on the configuration. */
 typedef struct {

@@ -1,14 +1,16 @@
 // C ABI of libans.so: contexts, memory budget, scratch, matrices, the batch
-// pipeline and completion tickets.  Host code only; the kernels live in
-// ans_sort.cu and ans_stats.cu.
+// pipeline and completion tickets.  Host code only; the kernels live in the
+// other ans_*.cu files.
 //
 // Pipeline of one batch of windows (every window of the batch in one fixed
 // sequence of launches, independent of the number of windows):
-//   pack + digit histograms -> 8 onesweep digit passes -> run-length reduce
-//   to DCSR -> values and row statistics -> column pass (4 destination-key
-//   passes, run reduction)
-//   [-> time sum: gather links -> histograms -> 8 key/value passes -> value
-//   prefix -> run-length reduce -> statistics -> column pass].
+//   sample sort of the packets (sample, count, scatter, local; long windows
+//   split twice) -> run-length reduce to DCSR -> values, row statistics and
+//   destination partition counts -> column pass (links scattered into the
+//   partitions, each counted)
+//   [-> time sum: the windows' links merged pairwise, or gathered and sorted
+//   by 8 key/value passes, then their value prefix; or the packets sorted
+//   again as one segment -> run-length reduce -> statistics -> column pass].
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -172,7 +174,8 @@ struct ans_ctx {
   int win_path = 1;
   SortCfg cfg_win{1024, kRankMatch, 1};
   // Time sum: 0 = merge the matrices' sorted links pairwise, 1 = radix-sort
-  // the gathered links (kv passes).
+  // the gathered links (kv passes), 2 = sort a batch's packets again as one
+  // segment (sums of given matrices: merged up to 256 of them).
   int sum_path = 0;
   int merge_tile = 4096;  // merge rounds: output positions per CTA (4096 or 2048)
   // Window aggregation: 0 = sort every packet's key, 1 = count links in
@@ -180,8 +183,8 @@ struct ans_ctx {
   // their own arena, left empty by every call that used them (hash_dirty
   // marks one that may not have been).
   int agg_path = 0;
-  // Window column statistics: 1 = a shared-memory hash of destinations per
-  // window first (windows that fit skip the column sort), 0 = sort only.
+  // Column statistics: 1 = links in hash partitions (or, large time sums,
+  // hash groups) of their destinations, 0 = the column sort.
   int col_hash = 1;
   int pageable = -1;  // does the device read pageable host memory (-1: not asked yet)
   // Packets a batch with device-resident offsets may hold (0: the call reads
@@ -1600,7 +1603,8 @@ int run_windows(ans_ctx* c, const uint32_t* d_src, const uint32_t* d_dst, const 
   int rc = ANS_OK;
   if (want_sum && nseg && (rc = sum_block(c, total, st, &sump))) return bail(rc);
   // (all the batch's memory is held; the rest of the planning runs beside the
-  // filling: a served batch of 100 windows 827 us, 845 with the filling after it)
+  // filling: a served batch of 100 windows 845 us with the filling after it, 835
+  // so; 827 with the filling before anything is asked for)
   if (feed) {
     queued = true;
     if ((rc = feed())) return bail(rc);

@@ -486,6 +486,9 @@ template <bool kWide>
 cudaError_t run_scatter(const SegPlan& p, const ColParts& c, const uint32_t* col_ids, const uint32_t* vals32,
                         const uint64_t* vals64, uint32_t* odst, void* oval, cudaStream_t st) {
   if (c.max_parts <= 1) return cudaSuccess;
+  // (c.max_parts: of the longest segment, or, in batches planned on the device,
+  // of one that holds the whole batch, whose shape every window then takes: 2^27
+  // packets in windows of 2^17 0.62 against 0.58 ms.)
   // With many partitions a CTA pays an atomic for nearly every one of them, so
   // it takes a whole tile (3 million links, 1108 partitions, 64-bit counts: 48
   // us, 85 by 2048 links); else 4096 links per CTA are faster (2^28 packets in

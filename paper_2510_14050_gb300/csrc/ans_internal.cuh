@@ -282,9 +282,13 @@ cudaError_t launch_count_prefix(const MatDesc* mats, uint32_t k, uint64_t* cat_o
 // segments longer than one_level.
 constexpr uint32_t kSsPerTile = 6;  // buckets per tile of keys
 // Longest segment that one split takes, in a plan of `total` keys.  One CTA
-// sorts a segment's sample: 23 us for 2^17 keys, 148 us for 2^20 (measured),
-// which a large batch hides behind its other segments and a small one does
-// not; a second split costs two more reads and a write of the keys.
+// sorts a segment's sample: 24 us for 2^17 keys, 39 us for 2^18, 207 us for 2^20
+// (measured), which a large batch hides behind its other segments and a small
+// one does not; a second split costs two more reads and a write of the keys.
+// (A split makes at most 1024 buckets: from 1.4 million keys on they grow beyond
+// the 1366 aimed at, up to 2048 for 2^21, and more of them exceed what one CTA
+// sorts on chip.  k_ss_local takes 12.2 ps a key for windows of 1.36 million, 14.6
+// for 1.7 million, 16.4 for 2^21; the digit passes took 58 for all of the sort.)
 constexpr uint64_t ss_one_level(uint64_t total) { return total >= (1ull << 24) ? 1ull << 21 : 1ull << 18; }
 struct SsArgs {
   SegPlan plan;                         // raw packets: window_inputs(plan, s, src, dst)

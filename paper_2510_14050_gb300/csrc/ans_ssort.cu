@@ -14,8 +14,11 @@
 //   scatter  keys moved to their buckets: ranks by one shared-memory atomic
 //            per key, space by one global atomic per bucket and tile -- no
 //            chain of tiles waiting for one another;
-//   local    every bucket (~1366 keys) sorted by one CTA on chip: 16 keys per
-//            thread in registers, then merge-path rounds in shared memory.
+//   local    every bucket (~1366 keys, up to 2048 in segments of 1.4 to 2.1
+//            million) sorted by one CTA on chip: 16 keys per thread in
+//            registers, then merge-path rounds in shared memory; one of more
+//            than 2048 keys (16 samples a bucket misjudge about one in forty;
+//            half of them at 2^21) in pieces merged through global memory.
 //
 // Buckets hold equal numbers of packets whatever the addresses look like, so
 // heavy sources and links cost nothing extra.  A segment too long for one
@@ -738,7 +741,8 @@ cudaError_t launch_ss_sample(const SsArgs& a0, uint64_t max_len, cudaStream_t st
   a.sample_max = 1024;
   const uint64_t want = (uint64_t)umin64(kSsSampleMax, (uint64_t)umax64(1, ss_buckets(max_len, a.level1, a.one_level)) * kSsOversample);
   while (a.sample_max < want) a.sample_max <<= 1;
-  // (nb - 1 splitters are compacted in the same buffer: sample_max >= 32 nb)
+  // (the splitters are compacted in the same buffer, which is as long as a
+  // split's most buckets at least)
   const uint32_t grid = a.nseg < 65536u ? a.nseg : 65536u;
   k_ss_sample<<<grid, kSsSampleThreads, (size_t)a.sample_max * 8, st>>>(a);
   return cudaGetLastError();

@@ -789,9 +789,9 @@ __global__ void __launch_bounds__(1024) k_hgroup_plan(HGroupBufs b, uint32_t max
 }
 
 // Count (key, links, packets) into the group's table; true if this call took
-// a new slot.  The fill stays below the table size (the callers give up at
-// three quarters, and each thread takes at most one slot meanwhile), so a
-// slot is always found.
+// a new slot.  (A table given up at three quarters may fill meanwhile, as warps
+// under way take more slots each; a key that then finds none is dropped with
+// the whole result.)
 __device__ __forceinline__ bool hg_insert(uint32_t* t_key, uint32_t* t_cnt, uint32_t* t_sum, uint32_t slots,
                                           uint32_t key, uint32_t cnt, uint32_t sum) {
   uint32_t h = (key >> 16) & (slots - 1);  // the group fixes the low 16 bits
