@@ -28,6 +28,11 @@
  *     (the time sum's merge rounds beside the window column pass); that work
  *     is forked from and joined back into `stream`, so completion on
  *     `stream` covers it.
+ *   - Contexts may be used from different threads at once.  While one submits a
+ *     batch with graph = 1 (a recording of some 30 us), no other thread may wait
+ *     for the whole device on its own (cudaDeviceSynchronize): the runtime
+ *     refuses that during a capture.  The library's own waits (destroying or
+ *     retuning a context, a wait limit) keep clear of recordings.
  *   - Matrices are owned by the caller once returned and released with
  *     ans_matrix_free().  A matrix keeps its memory alive independently of
  *     the context's scratch.
@@ -96,7 +101,8 @@ int ans_ctx_create(ans_ctx** out, int device, size_t mem_budget_bytes,
                    ans_alloc_fn alloc, ans_free_fn free_fn, void* user);
 
 /* Wait for the context's outstanding work and release its scratch and
- * tickets; the handle is invalid afterwards.  Matrices created from the
+ * tickets; the handle is invalid afterwards (unless the call fails: ANS_ERR_CUDA
+ * while a stream of the caller's is being captured, which rules the wait out).  Matrices created from the
  * context stay valid: the context's remaining state (its free hook and user
  * pointer included, which must stay usable) is released with the last of
  * them.  Destroying a context twice is ANS_ERR_INVALID_ARG (while matrices

@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <atomic>
 #include <chrono>
+#include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -322,6 +323,37 @@ struct ans_matrix {
 
 namespace {
 
+// Recordings of batches (run_launches) and waits for the whole device exclude
+// one another across contexts and threads: the runtime refuses such a wait while
+// a stream is being captured, and breaks the capture off.
+struct Recordings {
+  std::mutex mu;
+  std::condition_variable cv;
+  int running = 0, waits = 0;  // recordings under way; waits asked for or under way
+};
+Recordings g_rec;
+struct RecordGuard {
+  RecordGuard() {
+    std::unique_lock<std::mutex> l(g_rec.mu);
+    g_rec.cv.wait(l, [] { return g_rec.waits == 0; });
+    ++g_rec.running;
+  }
+  ~RecordGuard() {
+    std::lock_guard<std::mutex> l(g_rec.mu);
+    --g_rec.running;
+    g_rec.cv.notify_all();
+  }
+};
+cudaError_t device_wait() {
+  std::unique_lock<std::mutex> l(g_rec.mu);
+  ++g_rec.waits;
+  g_rec.cv.wait(l, [] { return g_rec.running == 0; });
+  const cudaError_t e = cudaDeviceSynchronize();
+  --g_rec.waits;
+  g_rec.cv.notify_all();
+  return e;
+}
+
 int dev_alloc(ans_ctx* c, size_t bytes, cudaStream_t st, void** out) {
   *out = nullptr;
   if (bytes == 0) return ANS_OK;
@@ -340,7 +372,7 @@ int dev_alloc(ans_ctx* c, size_t bytes, cudaStream_t st, void** out) {
       // to the device once everything queued has finished, and retry.
       cudaGetLastError();
       cudaMemPool_t pool = nullptr;
-      if (cudaDeviceSynchronize() == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, c->device) == cudaSuccess)
+      if (device_wait() == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, c->device) == cudaSuccess)
         cudaMemPoolTrimTo(pool, 0);
       cudaGetLastError();
       e = cudaMallocAsync(&p, bytes, st);
@@ -1355,14 +1387,22 @@ int run_launches(ans_ctx* c, cudaStream_t st, const std::string& key, F&& fn) {
   if (!c->ev_join) ANS_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
   if (!c->graph || c->prof.on) return fn(st);
   if (!c->cap) ANS_CUDA(cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking));
-  ANS_CUDA(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal));
-  const int rc = fn(c->cap);
   cudaGraph_t g = nullptr;
-  const cudaError_t e = cudaStreamEndCapture(c->cap, &g);
+  int rc = ANS_OK;
+  cudaError_t e = cudaSuccess;
+  {
+    RecordGuard rg;
+    ANS_CUDA(cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal));
+    rc = fn(c->cap);
+    e = cudaStreamEndCapture(c->cap, &g);
+  }
   if (rc != ANS_OK || e != cudaSuccess) {
+    // (the caller's own wait for the device in another thread breaks a recording
+    // off, too; nothing of it has run: launched directly, which reports what
+    // else may be wrong)
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
-    return rc != ANS_OK ? rc : fail(ANS_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+    return fn(st);
   }
   auto it = c->graphs.find(key);
   if (it != c->graphs.end()) {
@@ -2338,7 +2378,10 @@ int ans_ctx_destroy(ans_ctx* c) {
     std::lock_guard<std::mutex> g(c->mu);
     if (c->closed) return fail(ANS_ERR_INVALID_ARG, "context already destroyed");
     DeviceGuard dg(c->device);
-    cudaDeviceSynchronize();
+    if (device_wait() == cudaErrorStreamCaptureUnsupported) {  // the caller's own capture
+      cudaGetLastError();
+      return fail(ANS_ERR_CUDA, "a stream is being captured: the context's work cannot be waited for");
+    }
     for (auto& kv : c->tickets) cudaEventDestroy(kv.second.ev);
     c->tickets.clear();
     dev_free(c, c->scratch, c->scratch_size, c->aux);
@@ -2656,7 +2699,7 @@ int ans_set_wait_limit(ans_ctx* c, uint32_t polls) {
   std::lock_guard<std::mutex> g(c->mu);
   DeviceGuard dg(c->device);
   // the limit is read by kernels: change it only with nothing in flight
-  ANS_CUDA(cudaDeviceSynchronize());
+  ANS_CUDA(device_wait());
   ANS_CUDA(cudaMemcpy(c->d_err + 1, &polls, 4, cudaMemcpyHostToDevice));
   return ANS_OK;
 }
@@ -2957,7 +3000,7 @@ int ans_set_tuning(ans_ctx* c, const ans_tuning* t) {
   c->merge_tile = (int)t->merge_tile;
   if (c->agg_path != 1 && c->hash_mem) {  // the hash tables are no longer needed
     DeviceGuard dg(c->device);
-    ANS_CUDA(cudaDeviceSynchronize());
+    ANS_CUDA(device_wait());
     dev_free(c, c->hash_mem, c->hash_slots * 12, c->aux);
     c->hash_mem = nullptr;
     c->hash_slots = 0;
