@@ -77,9 +77,9 @@ REFERENCE_SAMPLE = {1: 1, 2: 64, 3: 96, 4: 256}
 # for the library sources it was captured with and the paths and launch
 # shapes that decide the traffic (else the bench reports null).
 NCU_TRAFFIC = {
-    4: {"library": "3633e1125f1ad841", "matrices": False,
+    4: {"library": "f3479bb325110c50", "matrices": False,
         "paths": {"agg_path": 0, "sum_path": 2, "col_hash": 1},
-        "step": 233.8, "kernels": {"ss_local": 14.41, "ss_scatter": 16.64, "ss_count": 9.42, "rle": 17.53}},
+        "step": 233.8, "kernels": {"ss_local": 14.41, "ss_scatter": 16.63, "ss_count": 9.42, "rle": 17.53}},
 }
 
 
